@@ -17,14 +17,13 @@
 // Warp roles: warp 0 = TMA producer of the weight tiles, warp 1 = TMEM owner and MMA issuer,
 // warp 2 = second MMA issuer (two-slab units only), warps 3-6 (and 7-10 for the second slab) =
 // epilogue (warp w reads TMEM lanes 32*(w%4) .. +31), last warp = TMA producer of the activation
-// tiles.  The loads have two issuing threads because one thread needs ~170 cycles per TMA
-// instruction, and a k-block of a two-slab unit takes three of them plus an L2 prefetch; the weight
-// producer depends on no earlier kernel and starts while the previous kernel is still running.
+// tiles.  The weight producer depends on no earlier kernel and starts while the previous kernel is
+// still running.
 //
-// One thread can issue a tcgen05.mma (K = 16) only every ~132 cycles, whatever its N, while the
-// tensor pipe needs N/2 cycles for it: a single issuer keeps the pipe busy only for N = 256.
-// A unit of two row slabs has two independent accumulators, each fed by its own issuing thread,
-// so the pipe sees two instructions per 132 cycles and stays busy for any N >= 132.
+// The producer and issuer warps run their loops with all 32 lanes and elect one lane around the TMA and
+// MMA instructions (ptx::elect_one): one warp then issues a k-block's four MMAs in the tensor pipe's own
+// time for N >= 128 (240 cycles; 477 when lane 0 alone runs the loop).  Stand-alone, lane-0 loops against
+// this form: QKV at 32 rows 23.9 -> 20.6 us, down 23.3 -> 21.1, gate/up at 512 rows 77.5 -> 76.6.
 #include <math.h>
 #include <stdio.h>
 
@@ -50,7 +49,7 @@ template <int EPI, int CG>
 __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensorMap *tmB, const CUtensorMap *tmB2,
                                           const CUtensorMap *tmC, const KParams &p, uint8_t *smem_raw, uint64_t *bars, uint32_t *tmem_slot,
                                           int *abort_flag) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = (CG == 2) ? ptx::cluster_ctarank() : 0u;
   const bool leader = rank == 0;
   const int group = (CG == 2) ? (blockIdx.x >> 1) : blockIdx.x;
@@ -125,78 +124,78 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      const uint64_t pol_w = ptx::policy_evict_first();   // weights are read once per step
-      const uint32_t b_bytes = (CG == 2) ? (uint32_t)half_n * 128u : (uint32_t)p.tile_n * 128u;
-      const uint32_t tx = (CG == 2 ? (1 + p.a_peer_loads) : 1) * (uint32_t)slabs * p.a_box_bytes + CG * b_bytes;
-      auto issue_b = [&](int stage, int kb, int nt) {   // weight tile of k-block kb (and the stage's byte count)
-        const uint32_t dstB = sB + stage * p.b_stage_bytes;
-        if (CG == 1) {
-          ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
-          if (EPI == EPI_SWIGLU) {
-            ptx::tma_load_2d_hint(dstB, tmB, full_bar(stage), kb * TILE_K, nt * half_n, pol_w);
-            ptx::tma_load_2d_hint(dstB + half_n * 128, tmB2, full_bar(stage), kb * TILE_K, nt * half_n, pol_w);
-          } else {
-            ptx::tma_load_2d_hint(dstB, tmB, full_bar(stage), kb * TILE_K, nt * p.tile_n, pol_w);
-          }
+    const uint64_t pol_w = ptx::policy_evict_first();   // weights are read once per step
+    const uint32_t b_bytes = (CG == 2) ? (uint32_t)half_n * 128u : (uint32_t)p.tile_n * 128u;
+    const uint32_t tx = (CG == 2 ? (1 + p.a_peer_loads) : 1) * (uint32_t)slabs * p.a_box_bytes + CG * b_bytes;
+    auto issue_b = [&](int stage, int kb, int nt) {   // weight tile of k-block kb (and the stage's byte count)
+      const uint32_t dstB = sB + stage * p.b_stage_bytes;
+      if (CG == 1) {
+        ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
+        if (EPI == EPI_SWIGLU) {
+          ptx::tma_load_2d_hint(dstB, tmB, full_bar(stage), kb * TILE_K, nt * half_n, pol_w);
+          ptx::tma_load_2d_hint(dstB + half_n * 128, tmB2, full_bar(stage), kb * TILE_K, nt * half_n, pol_w);
         } else {
-          if (leader) ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
-          const uint32_t lead_full = ptx::mapa(full_bar(stage), 0);
-          if (EPI == EPI_SWIGLU)
-            ptx::tma_load_2d_pair_hint(dstB, leader ? tmB : tmB2, lead_full, kb * TILE_K, nt * half_n, pol_w);
-          else
-            ptx::tma_load_2d_pair_hint(dstB, tmB, lead_full, kb * TILE_K, nt * p.tile_n + (int)rank * half_n, pol_w);
+          ptx::tma_load_2d_hint(dstB, tmB, full_bar(stage), kb * TILE_K, nt * p.tile_n, pol_w);
         }
-      };
-      // Weights come from HBM exactly once and the ring holds only a few k-blocks, fewer than HBM's latency
-      // under load is worth: the tile PF_AHEAD k-blocks further on is asked into L2 with every load.
-      constexpr int PF_AHEAD = 8;
-      auto prefetch_b = [&](int kb, int nt) {
-        if (EPI == EPI_LMHEAD) return;   // HBM-bound already: asking tiles into L2 early only adds re-reads (measured +15 % traffic)
-        if (CG == 1) {
-          if (EPI == EPI_SWIGLU) {
-            ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * half_n);
-            ptx::tma_prefetch_l2_2d(tmB2, kb * TILE_K, nt * half_n);
-          } else {
-            ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * p.tile_n);
-          }
-        } else if (EPI == EPI_SWIGLU) {
-          ptx::tma_prefetch_l2_2d(leader ? tmB : tmB2, kb * TILE_K, nt * half_n);
+      } else {
+        if (leader) ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
+        const uint32_t lead_full = ptx::mapa(full_bar(stage), 0);
+        if (EPI == EPI_SWIGLU)
+          ptx::tma_load_2d_pair_hint(dstB, leader ? tmB : tmB2, lead_full, kb * TILE_K, nt * half_n, pol_w);
+        else
+          ptx::tma_load_2d_pair_hint(dstB, tmB, lead_full, kb * TILE_K, nt * p.tile_n + (int)rank * half_n, pol_w);
+      }
+    };
+    // Weights come from HBM exactly once and the ring holds only a few k-blocks, fewer than HBM's latency
+    // under load is worth: the tile PF_AHEAD k-blocks further on is asked into L2 with every load.
+    constexpr int PF_AHEAD = 8;
+    auto prefetch_b = [&](int kb, int nt) {
+      if (EPI == EPI_LMHEAD) return;   // HBM-bound already: asking tiles into L2 early only adds re-reads (measured +15 % traffic)
+      if (CG == 1) {
+        if (EPI == EPI_SWIGLU) {
+          ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * half_n);
+          ptx::tma_prefetch_l2_2d(tmB2, kb * TILE_K, nt * half_n);
         } else {
-          ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * p.tile_n + (int)rank * half_n);
+          ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * p.tile_n);
         }
-      };
-      // one producer thread for the weights (this warp), one for the activations (last warp): both walk the
-      // same units, k-blocks and stages; every unit starts at stage 0 (so the staging area is what a unit
-      // fills last), with one phase bit per stage.  No kernel writes weights, so this thread does not wait
-      // for the previous kernel of the stream.
-      uint32_t phases = 0;
-      int lt = 0;
-      bool ok = true;
-      for (int u = group; u < num_units && ok; u += n_groups, ++lt) {
-        int mt, nt, kb0, kb1;
-        decode(u, mt, nt, kb0, kb1);
-        int stage = 0;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (kb + p.n_stages + PF_AHEAD < kb1) prefetch_b(kb + p.n_stages + PF_AHEAD, nt);
-          if (p.gate && lt > 0 && kb - kb0 == p.n_stages - 2 &&
-              !ptx::mbar_wait(sfree_bar, (uint32_t)(lt - 1) & 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-          if (!ptx::mbar_wait(empty_bar(stage), ((phases >> stage) & 1u) ^ 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
+      } else if (EPI == EPI_SWIGLU) {
+        ptx::tma_prefetch_l2_2d(leader ? tmB : tmB2, kb * TILE_K, nt * half_n);
+      } else {
+        ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * p.tile_n + (int)rank * half_n);
+      }
+    };
+    // one producer thread for the weights (this warp), one for the activations (last warp): both walk the
+    // same units, k-blocks and stages; every unit starts at stage 0 (so the staging area is what a unit
+    // fills last), with one phase bit per stage.  No kernel writes weights, so this thread does not wait
+    // for the previous kernel of the stream.
+    uint32_t phases = 0;
+    int lt = 0;
+    bool ok = true;
+    for (int u = group; u < num_units && ok; u += n_groups, ++lt) {
+      int mt, nt, kb0, kb1;
+      decode(u, mt, nt, kb0, kb1);
+      int stage = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (p.gate && lt > 0 && kb - kb0 == p.n_stages - 2 &&
+            !ptx::mbar_wait_warp(sfree_bar, (uint32_t)(lt - 1) & 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
+        if (!ptx::mbar_wait_warp(empty_bar(stage), ((phases >> stage) & 1u) ^ 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
+        if (ptx::elect_one()) {
           issue_b(stage, kb, nt);
+          if (kb + p.n_stages + PF_AHEAD < kb1) prefetch_b(kb + p.n_stages + PF_AHEAD, nt);
           if (kb - kb0 == p.n_stages - 1)   // the ring is primed: ask for the tiles between it and the running prefetch
             for (int i = p.n_stages; i < min(kb1 - kb0, p.n_stages + PF_AHEAD); ++i) prefetch_b(kb0 + i, nt);
-          phases ^= 1u << stage;
-          if (++stage == p.n_stages) stage = 0;
         }
+        phases ^= 1u << stage;
+        if (++stage == p.n_stages) stage = 0;
       }
-      if (!ok) *abort_flag = 1;
     }
+    if (!ok) *abort_flag = 1;
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------------ MMA issuers (leader CTA only when paired)
     // warp 1 feeds slab 0, warp 2 slab 1: each slab has its own accumulator columns, so the two
     // instruction streams need no ordering between them; both count on the stage's `empty` barrier.
     const int sl = warp - 1;
-    if (lane == 0 && leader && (sl < slabs || p.kil)) {
+    if (leader && (sl < slabs || p.kil)) {
       const uint32_t idesc = ptx::idesc_bf16(TILE_M * CG, (uint32_t)p.tile_n);
       uint32_t phases = 0;
       int lt = 0;
@@ -206,7 +205,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
         decode(u, mt, nt, kb0, kb1);
         const int ab = lt % nbuf;
         const uint32_t aphase = (lt / nbuf) & 1;
-        if (!ptx::mbar_wait(tempty_bar(ab), aphase ^ 1u)) { fail(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
+        if (!ptx::mbar_wait_warp(tempty_bar(ab), aphase ^ 1u)) { fail(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
         ptx::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + (ab + sl) * ACC_COLS;   // slab sl of a two-slab unit: column sl * ACC_COLS
         int stage = 0;
@@ -218,22 +217,25 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
             if (++stage == p.n_stages) stage = 0;
             continue;
           }
-          if (!ptx::mbar_wait(full_bar(stage), (phases >> stage) & 1u)) { fail(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
+          if (!ptx::mbar_wait_warp(full_bar(stage), (phases >> stage) & 1u)) { fail(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
           ptx::tc_fence_after_sync();
           const uint64_t a_desc = ptx::smem_desc_sw128(sA + stage * p.a_stage_bytes + (p.kil ? 0 : sl * A_STAGE_BYTES));
           const uint64_t b_desc = ptx::smem_desc_sw128(sB + stage * p.b_stage_bytes);
+          const bool first = kb == kb0 + (p.kil ? sl : 0);
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int k = 0; k < TILE_K / 16; ++k) {   // 16 bf16 = 32 bytes per MMA: descriptor address += 2
-            const uint32_t acc = (kb > kb0 + (p.kil ? sl : 0) || k > 0) ? 1u : 0u;
-            if (CG == 2) ptx::mma_bf16_ss_pair(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, acc);
-            else ptx::mma_bf16_ss(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, acc);
+            for (int k = 0; k < TILE_K / 16; ++k) {   // 16 bf16 = 32 bytes per MMA: descriptor address += 2
+              const uint32_t acc = (!first || k > 0) ? 1u : 0u;
+              if (CG == 2) ptx::mma_bf16_ss_pair(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, acc);
+              else ptx::mma_bf16_ss(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, acc);
+            }
+            if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3);
+            else ptx::mma_commit(empty_bar(stage));
           }
-          if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3);
-          else ptx::mma_commit(empty_bar(stage));
           phases ^= 1u << stage;
           if (++stage == p.n_stages) stage = 0;
         }
-        if (ok) {
+        if (ok && ptx::elect_one()) {
           if (CG == 2) ptx::mma_commit_pair(tfull_bar(ab), 3);
           else ptx::mma_commit(tfull_bar(ab));
         }
@@ -242,40 +244,38 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
     }
   } else if (warp == 3 + 4 * slabs) {
     // ------------------------------------------------------------------ TMA producer of the activation tiles
-    if (lane == 0) {
-      const uint64_t pol_a = ptx::policy_evict_last();    // activations are re-read by every column tile
-      auto issue_a = [&](int stage, int kb, int m0) {   // activation rows of k-block kb, one box per slab
-        const uint32_t dstA = sA + stage * p.a_stage_bytes;
-        if (CG == 1) {
-          for (int sl = 0; sl < slabs; ++sl)
-            ptx::tma_load_2d_hint(dstA + sl * A_STAGE_BYTES, tmA, full_bar(stage), kb * TILE_K, m0 + sl * TILE_M, pol_a);
-        } else {
-          const uint32_t lead_full = ptx::mapa(full_bar(stage), 0);
-          for (int sl = 0; sl < slabs; ++sl)
-            ptx::tma_load_2d_pair_hint(dstA + sl * A_STAGE_BYTES, tmA, lead_full, kb * TILE_K, m0 + sl * TILE_M * CG, pol_a);
-        }
-      };
-      grid_dep_wait();   // the activations are the previous kernel's output
-      uint32_t phases = 0;
-      int lt = 0;
-      bool ok = true;
-      const bool loads_a = leader || p.a_peer_loads;   // few rows: the second CTA of a pair has none
-      for (int u = group; u < num_units && ok && loads_a; u += n_groups, ++lt) {
-        int mt, nt, kb0, kb1;
-        decode(u, mt, nt, kb0, kb1);
-        const int m0 = mt * unit_rows + (int)rank * TILE_M;
-        int stage = 0;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (p.gate && lt > 0 && kb - kb0 == p.n_stages - 2 &&
-              !ptx::mbar_wait(sfree_bar, (uint32_t)(lt - 1) & 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-          if (!ptx::mbar_wait(empty_bar(stage), ((phases >> stage) & 1u) ^ 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-          issue_a(stage, kb, m0);
-          phases ^= 1u << stage;
-          if (++stage == p.n_stages) stage = 0;
-        }
+    const uint64_t pol_a = ptx::policy_evict_last();    // activations are re-read by every column tile
+    auto issue_a = [&](int stage, int kb, int m0) {   // activation rows of k-block kb, one box per slab
+      const uint32_t dstA = sA + stage * p.a_stage_bytes;
+      if (CG == 1) {
+        for (int sl = 0; sl < slabs; ++sl)
+          ptx::tma_load_2d_hint(dstA + sl * A_STAGE_BYTES, tmA, full_bar(stage), kb * TILE_K, m0 + sl * TILE_M, pol_a);
+      } else {
+        const uint32_t lead_full = ptx::mapa(full_bar(stage), 0);
+        for (int sl = 0; sl < slabs; ++sl)
+          ptx::tma_load_2d_pair_hint(dstA + sl * A_STAGE_BYTES, tmA, lead_full, kb * TILE_K, m0 + sl * TILE_M * CG, pol_a);
       }
-      if (!ok) *abort_flag = 1;
+    };
+    grid_dep_wait();   // the activations are the previous kernel's output
+    uint32_t phases = 0;
+    int lt = 0;
+    bool ok = true;
+    const bool loads_a = leader || p.a_peer_loads;   // few rows: the second CTA of a pair has none
+    for (int u = group; u < num_units && ok && loads_a; u += n_groups, ++lt) {
+      int mt, nt, kb0, kb1;
+      decode(u, mt, nt, kb0, kb1);
+      const int m0 = mt * unit_rows + (int)rank * TILE_M;
+      int stage = 0;
+      for (int kb = kb0; kb < kb1; ++kb) {
+        if (p.gate && lt > 0 && kb - kb0 == p.n_stages - 2 &&
+            !ptx::mbar_wait_warp(sfree_bar, (uint32_t)(lt - 1) & 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
+        if (!ptx::mbar_wait_warp(empty_bar(stage), ((phases >> stage) & 1u) ^ 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
+        if (ptx::elect_one()) issue_a(stage, kb, m0);
+        phases ^= 1u << stage;
+        if (++stage == p.n_stages) stage = 0;
+      }
     }
+    if (!ok) *abort_flag = 1;
   } else {
     // ------------------------------------------------------------------ epilogue
     // warps 3-6 drain slab 0, warps 7-10 (two-slab units only) slab 1; warp w may touch TMEM lanes 32 (w % 4) ..
@@ -288,7 +288,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
       decode(u, mt, nt, kb0, kb1);
       const int ab = lt % nbuf;
       const uint32_t aphase = (lt / nbuf) & 1;
-      if (!ptx::mbar_wait(tfull_bar(ab), aphase)) { fail(p.status, DEV_TIMEOUT_EPILOGUE); ok = false; break; }
+      if (!ptx::mbar_wait_warp(tfull_bar(ab), aphase)) { fail(p.status, DEV_TIMEOUT_EPILOGUE); ok = false; break; }
       ptx::tc_fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (ab + sl) * ACC_COLS;
       const int row0 = mt * unit_rows + sl * (TILE_M * CG) + (int)rank * TILE_M + q * 32;

@@ -19,6 +19,22 @@ __device__ __forceinline__ uint64_t globaltimer() {
   return t;
 }
 
+// True in exactly one lane of a converged warp.  The roles that issue TMA and tcgen05 instructions run their loops with the
+// whole warp (waits included) and enter elect_one() around the instructions alone: the operands are then values the whole
+// warp agrees on.  A loop that only lane 0 runs costs 477 cycles per k-block of four N = 32 MMAs where this form takes 152
+// (N = 128: 477 against 240, the tensor pipe's own time), and a TMA load issued that way lands after 537 cycles, not 362.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t is;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(is)::"memory");
+  return is != 0;
+}
+// The warp's number within the block, the same register value in every lane.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // ---- mbarrier -------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
@@ -53,6 +69,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
   uint32_t spins = 0;
   while (!mbar_try_wait(bar, parity)) {
     if ((++spins & 0x3ffu) == 0 && globaltimer() - t0 > limit_ns) return false;
+  }
+  return true;
+}
+
+// The same for a whole converged warp: every lane gets the same answer, so that the warp stays together behind it (the
+// warp-wide instructions that follow would wait for ever for a lane that gave up on its own).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t limit_ns = 2000000000ull) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = globaltimer();
+  uint32_t spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if ((++spins & 0x3ffu) == 0 && __any_sync(0xffffffffu, globaltimer() - t0 > limit_ns)) return false;
   }
   return true;
 }
