@@ -235,6 +235,10 @@ GemmArgs make_gemm_args(l2pd_ctx *c, int epi, const TmaDesc *a, const TmaDesc *b
   g.epi = epi; g.a = a; g.b = b; g.b2 = b2; g.c = cm; g.M = M; g.N = N; g.K = K; g.tile_n = pl.tile_n; g.out = out;
   g.cta_group = pl.cta_group; g.k_splits = pl.k_splits; g.slabs = pl.slabs; g.k_interleave = pl.k_interleave;
   g.status = c->d_status;
+  // the row's last, narrower column tile
+  const TmaDesc *ct = cm == &c->tc_qkv ? &c->tct_qkv : cm == &c->tc_o ? &c->tct_o : cm == &c->tc_h ? &c->tct_h : cm == &c->tc_down ? &c->tct_down : nullptr;
+  const int tail = cm == &c->tc_qkv ? c->tail_qkv : cm == &c->tc_o ? c->tail_o : cm == &c->tc_h ? c->tail_h : cm == &c->tc_down ? c->tail_down : 0;
+  if (ct && tail > 0) { g.c_tail = ct; g.tail_cols = tail; }
   if (M <= 128 && pl.slabs == 1 && c->a_box > 0 && c->a_box < 128) {   // few rows: the map of the same buffer with the small box
     g.a = a == &c->ta_n ? &c->ta_n_s : a == &c->ta_att ? &c->ta_att_s : a == &c->ta_h ? &c->ta_h_s : a;
     if (g.a != a) g.a_box_rows = c->a_box;
@@ -264,9 +268,10 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
   if (tc) {
     // the tiling follows the row count of this step; weight tensor maps are re-encoded when the
     // box (rows of the weight tile one CTA loads) changes
-    // contexts that can chain the projections of a layer into one launch keep every tile at most CHAIN_TILE_N wide:
-    // the chained kernel has one ring for all of them, and that width leaves it five stages
-    const int max_tn = (c->chain_clusters > 0 && T_rows > 256 && T_rows <= CHAIN_MAX_ROWS && T_rows <= c->ksum_rows) ? CHAIN_TILE_N : 256;
+    // A step that chains the projections of a layer into one launch has two row slabs per unit and tiles at most
+    // CHAIN_TILE_N wide (the chained kernel has one ring for all of them, and that width leaves it five stages); its K slices
+    // are those of the single launches, so that both forms add in the same order.
+    const bool big_chain = c->chain_mode != 0 && c->chain_clusters > 0 && T_rows > 256 && T_rows <= CHAIN_MAX_ROWS && T_rows <= c->ksum_rows;
     // steps of at most 256 rows chain with one row slab per unit (key/value-cache configurations: the rotation is a kernel
     // of its own there); their tiling is used only when chaining is asked for
     const bool small_chain = c->chain_mode != 0 && c->chain_clusters > 0 && c->ksum && T_rows <= 256 && !c->fuse_rope;
@@ -290,10 +295,16 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
       c->pl_down = plan_gemm_pair_one_slab(EPI_RESIDUAL, T_rows, d, F, c->num_sms, max_ks, CHAIN_TILE_N);
       c->pl_gu = plan_gemm_pair_one_slab(EPI_SWIGLU, T_rows, F, d, c->num_sms, 1, CHAIN_TILE_N);
     } else {
-      c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0, 4, max_tn);
-      c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks, max_tn);
-      c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks, max_tn);
-      c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0, 4, max_tn);
+      c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0);
+      c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks);
+      c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks);
+      c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0);
+      if (big_chain) {
+        c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0, 1, CHAIN_TILE_N, 2);
+        c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks, CHAIN_TILE_N, 2, c->pl_o.k_splits);
+        c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks, CHAIN_TILE_N, 2, c->pl_down.k_splits);
+        c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0, 1, CHAIN_TILE_N, 2);
+      }
     }
     int box = c->pl_qkv.tile_n / c->pl_qkv.cta_group;
     if (box != c->box_qkv) { l2pd_status r = encode_weight_maps(c, c->tb_qkv, c->wqkv, 3 * hd, d, box); if (r) return r; c->box_qkv = box; }
@@ -333,8 +344,8 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     r = out_map_x(c->tc_o, c->tcw_o, ks_o, c->pl_o.tile_n); if (r) return r;
     r = out_map(c->tc_h, c->tcw_h, c->h, false, F, c->pl_gu.tile_n / 2); if (r) return r;
     r = out_map_x(c->tc_down, c->tcw_down, ks_d, c->pl_down.tile_n); if (r) return r;
-    if (c->tc_rows != T_rows && c->chain_clusters > 0 && T_rows <= CHAIN_MAX_ROWS) {
-      // maps of the last, narrower column tiles (-1: a tail the staged epilogue cannot take; the step then does not chain)
+    if (c->tc_rows != T_rows) {
+      // maps of the last, narrower column tiles (-1: a tail the staged epilogue cannot take: direct stores, and the step does not chain)
       auto tail_map = [&](TmaDesc &m, int &tail, void *ptr, bool fp32, int64_t rows, int64_t N, int w, int mult = 16) {
         tail = (int)(N % w);
         if (tail && ((tail % mult) || make_tma_out_tail(&m, ptr, fp32, rows, N, tail) != L2PD_OK)) tail = -1;
@@ -369,13 +380,13 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     ChainStep st{};
     switch (which) {
       case 0: st.g = make_gemm_args(c, epi_qkv, &c->ta_n, &c->tb_qkv[l], nullptr, &c->tc_qkv, qkv, T_rows, 3 * hd, d, c->pl_qkv);
-              st.g.c_tail = c->tail_qkv > 0 ? &c->tct_qkv : nullptr; st.g.tail_cols = c->tail_qkv; break;
+              break;
       case 1: st.g = make_gemm_args(c, EPI_RESIDUAL, &c->ta_att, &c->tb_o[l], nullptr, &c->tc_o, c->x, T_rows, d, hd, c->pl_o);
-              st.g.c_tail = c->tail_o > 0 ? &c->tct_o : nullptr; st.g.tail_cols = c->tail_o; break;
+              break;
       case 2: st.g = make_gemm_args(c, EPI_SWIGLU, &c->ta_n, &c->tb_gate[l], &c->tb_up[l], &c->tc_h, hbuf, T_rows, F, d, c->pl_gu);
-              st.g.c_tail = c->tail_h > 0 ? &c->tct_h : nullptr; st.g.tail_cols = c->tail_h; break;
+              break;
       default: st.g = make_gemm_args(c, EPI_RESIDUAL, &c->ta_h, &c->tb_down[l], nullptr, &c->tc_down, c->x, T_rows, d, F, c->pl_down);
-              st.g.c_tail = c->tail_down > 0 ? &c->tct_down : nullptr; st.g.tail_cols = c->tail_down; break;
+              break;
     }
     return st;
   };
@@ -1158,7 +1169,12 @@ static l2pd_status gemm_common(void *stream, int epi, const void *A, const void 
   TmaDesc tcm;
   const int out_w = epi == EPI_SWIGLU ? pl.tile_n / 2 : pl.tile_n;
   const bool staged = !direct && N >= out_w && make_tma_out_3d(&tcm, out, epi == EPI_RESIDUAL, M, N, out_w) == L2PD_OK;
+  TmaDesc tct;
+  const int tail = N % out_w;
   GemmArgs g{};
+  if (staged && tail && tail % (epi == EPI_SWIGLU ? 8 : 16) == 0 && make_tma_out_tail(&tct, out, epi == EPI_RESIDUAL, M, N, tail) == L2PD_OK) {
+    g.c_tail = &tct; g.tail_cols = tail;
+  }
   g.c = staged ? &tcm : nullptr;
   g.epi = epi; g.a = &ta; g.b = &tb; g.b2 = epi == EPI_SWIGLU ? &tb2 : nullptr;
   g.M = M; g.N = N; g.K = K; g.tile_n = pl.tile_n; g.cta_group = pl.cta_group; g.k_splits = pl.k_splits;

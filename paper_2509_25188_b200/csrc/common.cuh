@@ -173,14 +173,16 @@ void set_standalone_error(const char *fmt, ...);
 // unit into two accumulators that the epilogue adds — halves the K loop where instruction issue bounds it
 struct GemmPlan { int cta_group, tile_n, k_splits, slabs, k_interleave; };
 // max_tile_n caps the tile width (a kernel that chains several projections keeps one ring geometry for all of them)
-GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits = 4, int max_tile_n = 256);
+// force_slabs / force_ks: 0 = chosen
+GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits = 4, int max_tile_n = 256,
+                   int force_slabs = 0, int force_ks = 0);
 GemmPlan plan_gemm_pair_one_slab(int epi, int M, int N, int K, int num_sms, int max_k_splits, int max_tile_n);
 int effective_k_splits(int K, int k_splits);   // what the launcher makes of a requested K split
 struct GemmArgs {
   int epi;                 // EPI_STORE, EPI_RESIDUAL, EPI_SWIGLU, or EPI_LMHEAD
   const TmaDesc *a, *b, *b2;
   const TmaDesc *c;        // output map from make_tma_out_3d (rows = M, tile_w matching tile_n), or null: direct stores
-  const TmaDesc *c_tail;   // optional (chained launches): map of the row's last, narrower tile alone, from make_tma_out_tail
+  const TmaDesc *c_tail;   // optional: map of the row's last, narrower tile alone, from make_tma_out_tail
   int tail_cols;           // its output columns (a multiple of 16)
   int M, N, K, tile_n;
   int cta_group, k_splits; // 0 / 1 = single CTA, no split

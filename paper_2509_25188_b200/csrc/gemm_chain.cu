@@ -38,6 +38,7 @@ constexpr int CHAIN_MAX_PHASES = 6;
 constexpr int CHAIN_MAX_GEMMS = 4;
 constexpr int MAPS_PER_GEMM = 5;
 constexpr int CG = 2, SLABS = 2;
+constexpr int CHAIN_MAX_STAGES = 8;
 constexpr int EPI_THREADS = 256;          // warps 4-11
 constexpr int REGS_LAUNCH = 168, REGS_LEAN = 56, REGS_EPI = 224;   // registers per thread: at launch, producers / issuers, epilogue
 static_assert(128 * REGS_LEAN + 256 * REGS_EPI <= 384 * REGS_LAUNCH, "register split exceeds what the block is launched with");
@@ -565,7 +566,7 @@ bool chain_step_supported(const ChainStep &s) {
   const int ks = effective_k_splits(g.K, g.k_splits);
   const int num_kb = ceil_div(g.K, TILE_K);
   if (ceil_div(num_kb, ks) * (ks - 1) >= num_kb) return false;
-  if (num_kb - ceil_div(num_kb, ks) * (ks - 1) < MAX_STAGES) return false;
+  if (num_kb - ceil_div(num_kb, ks) * (ks - 1) < CHAIN_MAX_STAGES) return false;
   if (g.epi == EPI_RESIDUAL && ks > 1 && !g.part) return false;   // K slices must store partial sums (fixed order)
   // every tile is stored through the TMA unit: an output map, and one for the last tile if it is narrower
   const int n_per_tile = g.epi == EPI_SWIGLU ? g.tile_n / 2 : g.tile_n;
@@ -593,7 +594,7 @@ cudaError_t chain_build_table(const ChainStep *steps, int n_steps, unsigned int 
   max_b = (max_b + 1023) & ~1023;
   const int stage_bytes = SLABS * A_STAGE_BYTES + max_b;
   int stages = (SMEM_BUDGET - 4096) / stage_bytes;   // the kernel's static shared memory (phase table, barriers) is ~2 KB
-  if (stages > MAX_STAGES) stages = MAX_STAGES;
+  if (stages > CHAIN_MAX_STAGES) stages = CHAIN_MAX_STAGES;
   if (stages < 4) return cudaErrorInvalidValue;   // two stages double as the staging area
   c.n_phases = n_steps; c.n_stages = stages; c.b_stage_bytes = max_b; c.pad_ = 0;
   c.bar = bar; c.status = status;

@@ -13,7 +13,7 @@ namespace gemm_dev {
 constexpr int TILE_M = 128;
 constexpr int TILE_K = 64;                       // 64 bf16 = 128 bytes = one swizzle row
 constexpr int A_STAGE_BYTES = TILE_M * TILE_K * 2;
-constexpr int MAX_STAGES = 8;
+constexpr int MAX_STAGES = 12;                   // few-row units: 96 and more KB of weights in flight per SM
 constexpr int TMEM_COLS = 512;
 constexpr int ACC_COLS = 256;                    // columns per accumulator buffer
 constexpr int SMEM_BUDGET = 227 * 1024;
@@ -43,6 +43,12 @@ struct KParams {
   // instead of a whole 128-row tile; the MMA still reads 128 rows, the rest being whatever shared memory holds, into
   // accumulator rows that are never stored.  a_peer_loads = 0: the second CTA of a pair has no rows and loads none.
   int a_box_bytes, a_peer_loads;
+  int out_ring;         // 1: the epilogue's staging tiles have shared memory of their own behind the ring (one-slab units); the
+                        // ring then runs on from unit to unit
+  int out_stage_off;    // where they are (bytes from the ring's start)
+  int last_bufs;        // > 0: a CTA's last unit drains through this many staging tiles per warp over the (then idle) ring, one
+                        // for every flush, so that no flush waits for an earlier one to have been read
+  int tail_slabs;       // live row slabs of the last row tile (1 where a two-slab tile's second slab has no rows)
 };
 
 __device__ __forceinline__ void fail(int32_t *status, int code) {
@@ -305,8 +311,9 @@ struct StagedOut {
   uint32_t stage0, stage, sw;
   int lane, n_flush, map_nt, row0;
   bool add;                      // fp32 residual added into X by the TMA unit (no K slices' partial sums)
-  __device__ __forceinline__ StagedOut(const CUtensorMap *m, uint32_t s0, int ln, int mnt, int r0, bool add_)
-      : tmC(m), stage0(s0), stage(s0), sw((uint32_t)(ln & 7)), lane(ln), n_flush(0), map_nt(mnt), row0(r0), add(add_) {}
+  int bufs;                      // staging tiles: STAGE_BUFS used in turn, or one for every flush of the unit
+  __device__ __forceinline__ StagedOut(const CUtensorMap *m, uint32_t s0, int ln, int mnt, int r0, bool add_, int bufs_)
+      : tmC(m), stage0(s0), stage(s0), sw((uint32_t)(ln & 7)), lane(ln), n_flush(0), map_nt(mnt), row0(r0), add(add_), bufs(bufs_) {}
   __device__ __forceinline__ uint32_t chunk_addr(int ch) const { return stage + lane * 128 + (((uint32_t)ch ^ sw) << 4); }
   __device__ __forceinline__ void st16(int ch, uint32_t a, uint32_t b, uint32_t c, uint32_t d) const {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(chunk_addr(ch)), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -324,6 +331,7 @@ struct StagedOut {
   }
   // pick the next staging tile; the flush that used it STAGE_BUFS turns ago has read it
   __device__ __forceinline__ void reuse() {
+    if (bufs > STAGE_BUFS) { stage = stage0 + (uint32_t)n_flush * 4096u; return; }
     stage = stage0 + (uint32_t)(n_flush % STAGE_BUFS) * 4096u;
     if (n_flush >= STAGE_BUFS) {
       if (lane == 0) ptx::bulk_wait_read_n<STAGE_BUFS - 1>();
@@ -405,9 +413,9 @@ __device__ __forceinline__ void emit_swiglu_cols(StagedOut &o, const uint32_t (&
 template <int EPI>
 __device__ __forceinline__ void drain_tile_staged(const KParams &p, const CUtensorMap *tmC, uint32_t taddr, int row0,
                                                   int nt, uint32_t stage0, int lane, bool res_store, int tail_cols = 0,
-                                                  bool two_acc = false) {
+                                                  bool two_acc = false, int bufs = STAGE_BUFS) {
   const int half_n = p.tile_n >> 1;
-  StagedOut o(tmC, stage0, lane, tail_cols > 0 ? 0 : nt, row0, EPI == EPI_RESIDUAL && !res_store);
+  StagedOut o(tmC, stage0, lane, tail_cols > 0 ? 0 : nt, row0, EPI == EPI_RESIDUAL && !res_store, bufs);
   if (EPI == EPI_QKV_ROPE) {
     // 16 columns at a time; the angles of a chunk are requested together with its accumulator columns, one chunk
     // ahead of their use

@@ -21,11 +21,18 @@
 // still running.
 //
 // The producer and issuer warps run their loops with all 32 lanes and elect one lane around the TMA and
-// MMA instructions (ptx::elect_one): one warp then issues a k-block's four MMAs in the tensor pipe's own
-// time for N >= 128 (240 cycles; 477 when lane 0 alone runs the loop).  Stand-alone, lane-0 loops against
-// this form: QKV at 32 rows 23.9 -> 20.6 us, down 23.3 -> 21.1, gate/up at 512 rows 77.5 -> 76.6.
+// MMA instructions (ptx::elect_one).  What such a warp costs per k-block is its own instruction latency, so
+// the loops hold nothing that can be decided per unit: 250-280 cycles per k-block for narrow tiles, the
+// tensor pipe's own time from N = 128 (paired) on; with lane-0 loops and the case distinctions inside it
+// was 480-620 for any width.
+// Stand-alone at 32 rows, before -> now (us): QKV 23.9 -> 20.2, O 11.8 -> 9.9, gate/up 42.1 -> 33.5
+// (6.0 TB/s), down 23.3 -> 19.4; at 256 rows gate/up 48.2 -> 41.3; at 512 rows gate/up 77.5 -> 70.6, and the
+// output projections without K slices as fast as with three (41.1 against 41.2), which spares the partial
+// sums.  Sustained at 16384 rows (power-capped) 1330-1400 TFLOP/s where cuBLAS reaches 1340-1370.
 #include <math.h>
 #include <stdio.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "gemm_device.cuh"
@@ -47,7 +54,7 @@ namespace {
 //         release the accumulator on the leader's `tmem empty` barrier.
 template <int EPI, int CG>
 __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensorMap *tmB, const CUtensorMap *tmB2,
-                                          const CUtensorMap *tmC, const KParams &p, uint8_t *smem_raw, uint64_t *bars, uint32_t *tmem_slot,
+                                          const CUtensorMap *tmC, const CUtensorMap *tmCT, const KParams &p, uint8_t *smem_raw, uint64_t *bars, uint32_t *tmem_slot,
                                           int *abort_flag) {
   const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = (CG == 2) ? ptx::cluster_ctarank() : 0u;
@@ -58,13 +65,14 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
   const uint32_t base = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;
   const uint32_t sA = base;
   const uint32_t sB = base + p.n_stages * p.a_stage_bytes;
-  const uint32_t sOut = sA + (uint32_t)(p.n_stages - 2) * p.a_stage_bytes;   // output staging: see drain_tile_staged
+  // output staging (see drain_tile_staged): behind the ring, or over the A operands of its last two stages
+  const uint32_t sOut = p.out_ring ? base + p.out_stage_off : sA + (uint32_t)(p.n_stages - 2) * p.a_stage_bytes;
   const int slabs = p.slabs;
   const int nbuf = (slabs == 1 && !p.kil) ? 2 : 1;   // accumulator buffers a unit can alternate between
   const int unit_rows = TILE_M * CG * slabs;
   const uint32_t bar0 = ptx::smem_u32(bars);
   auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };
+  auto empty_bar = [&](int s) { return bar0 + 8u * (MAX_STAGES + s); };   // = full_bar(s) + 8 MAX_STAGES
   auto tfull_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + b); };
   auto tempty_bar = [&](int b) { return bar0 + 8u * (2 * MAX_STAGES + 2 + b); };
   const uint32_t sfree_bar = bar0 + 8u * (2 * MAX_STAGES + 4);
@@ -81,7 +89,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
     ptx::prefetch_tensormap(tmA);
     ptx::prefetch_tensormap(tmB);
     if (EPI == EPI_SWIGLU) ptx::prefetch_tensormap(tmB2);
-    if (EPI != EPI_LMHEAD && p.out_tma) ptx::prefetch_tensormap(tmC);
+    if (EPI != EPI_LMHEAD && p.out_tma) { ptx::prefetch_tensormap(tmC); ptx::prefetch_tensormap(tmCT); }
   }
   if (warp == 1) {
     if (CG == 2) { ptx::tmem_alloc_pair(ptx::smem_u32(tmem_slot), TMEM_COLS); ptx::tmem_relinquish_pair(); }
@@ -106,176 +114,184 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
   // group_m row tiles; inside a group the row tiles of one column tile are adjacent, then the next
   // column tile follows.  The CTAs running at the same time thus share a few weight tiles, and a
   // group's activation rows (sized to a fraction of L2) stay resident while its column tiles stream by.
-  int unit_ks = 0;   // K slice of the unit decoded last
+  // A last row tile with fewer live slabs comes after all others: its units are short and fill up the last wave.
+  const int m_full = p.tail_slabs < slabs ? p.m_tiles - 1 : p.m_tiles;
+  const int full_units = m_full * p.n_tiles * p.k_splits;
+  int unit_ks = 0;        // K slice of the unit decoded last
+  int unit_slabs = slabs; // and its live slabs
   auto decode = [&](int u, int &mt, int &nt, int &kb0, int &kb1) {
-    const int per_slice = p.m_tiles * p.n_tiles;
-    const int ks = u / per_slice;
+    int ks;
+    if (u < full_units) {
+      const int per_slice = m_full * p.n_tiles;
+      ks = u / per_slice;
+      const int r = u - ks * per_slice;
+      const int per_group = p.group_m * p.n_tiles;
+      const int g = r / per_group;
+      const int w = r - g * per_group;
+      const int gm = min(p.group_m, m_full - g * p.group_m);   // the last group may be smaller
+      nt = w / gm;
+      mt = g * p.group_m + (w - nt * gm);
+      unit_slabs = slabs;
+    } else {
+      const int r = u - full_units;
+      ks = r / p.n_tiles;
+      nt = r - ks * p.n_tiles;
+      mt = m_full;
+      unit_slabs = p.tail_slabs;
+    }
     unit_ks = ks;
-    const int r = u - ks * per_slice;
-    const int per_group = p.group_m * p.n_tiles;
-    const int g = r / per_group;
-    const int w = r - g * per_group;
-    const int gm = min(p.group_m, p.m_tiles - g * p.group_m);   // the last group may be smaller
-    nt = w / gm;
-    mt = g * p.group_m + (w - nt * gm);
     kb0 = ks * kb_per;
     kb1 = min(num_kb, kb0 + kb_per);
   };
+  const bool restart = p.gate || p.kil;   // units start at ring stage 0; otherwise the ring runs on from unit to unit
+  const int n_stages = p.n_stages;
+  int32_t *const status = p.status;
+  auto wait = [&](uint32_t bar, uint32_t parity, int code) { return ptx::mbar_wait_or_abort(bar, parity, abort_flag, status, code); };
 
-  if (warp == 0) {
-    // ------------------------------------------------------------------ TMA producer
-    const uint64_t pol_w = ptx::policy_evict_first();   // weights are read once per step
-    const uint32_t b_bytes = (CG == 2) ? (uint32_t)half_n * 128u : (uint32_t)p.tile_n * 128u;
-    const uint32_t tx = (CG == 2 ? (1 + p.a_peer_loads) : 1) * (uint32_t)slabs * p.a_box_bytes + CG * b_bytes;
-    auto issue_b = [&](int stage, int kb, int nt) {   // weight tile of k-block kb (and the stage's byte count)
-      const uint32_t dstB = sB + stage * p.b_stage_bytes;
-      if (CG == 1) {
-        ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
-        if (EPI == EPI_SWIGLU) {
-          ptx::tma_load_2d_hint(dstB, tmB, full_bar(stage), kb * TILE_K, nt * half_n, pol_w);
-          ptx::tma_load_2d_hint(dstB + half_n * 128, tmB2, full_bar(stage), kb * TILE_K, nt * half_n, pol_w);
-        } else {
-          ptx::tma_load_2d_hint(dstB, tmB, full_bar(stage), kb * TILE_K, nt * p.tile_n, pol_w);
-        }
-      } else {
-        if (leader) ptx::mbar_arrive_expect_tx(full_bar(stage), tx);
-        const uint32_t lead_full = ptx::mapa(full_bar(stage), 0);
-        if (EPI == EPI_SWIGLU)
-          ptx::tma_load_2d_pair_hint(dstB, leader ? tmB : tmB2, lead_full, kb * TILE_K, nt * half_n, pol_w);
-        else
-          ptx::tma_load_2d_pair_hint(dstB, tmB, lead_full, kb * TILE_K, nt * p.tile_n + (int)rank * half_n, pol_w);
-      }
-    };
-    // Weights come from HBM exactly once and the ring holds only a few k-blocks, fewer than HBM's latency
-    // under load is worth: the tile PF_AHEAD k-blocks further on is asked into L2 with every load.
-    constexpr int PF_AHEAD = 8;
-    auto prefetch_b = [&](int kb, int nt) {
-      if (EPI == EPI_LMHEAD) return;   // HBM-bound already: asking tiles into L2 early only adds re-reads (measured +15 % traffic)
-      if (CG == 1) {
-        if (EPI == EPI_SWIGLU) {
-          ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * half_n);
-          ptx::tma_prefetch_l2_2d(tmB2, kb * TILE_K, nt * half_n);
-        } else {
-          ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * p.tile_n);
-        }
-      } else if (EPI == EPI_SWIGLU) {
-        ptx::tma_prefetch_l2_2d(leader ? tmB : tmB2, kb * TILE_K, nt * half_n);
-      } else {
-        ptx::tma_prefetch_l2_2d(tmB, kb * TILE_K, nt * p.tile_n + (int)rank * half_n);
-      }
-    };
-    // one producer thread for the weights (this warp), one for the activations (last warp): both walk the
-    // same units, k-blocks and stages; every unit starts at stage 0 (so the staging area is what a unit
-    // fills last), with one phase bit per stage.  No kernel writes weights, so this thread does not wait
-    // for the previous kernel of the stream.
-    uint32_t phases = 0;
-    int lt = 0;
-    bool ok = true;
-    for (int u = group; u < num_units && ok; u += n_groups, ++lt) {
+  // One warp walks its ring: stage address, barrier and parity advance together.  The loops below are what the issuing
+  // warps' latency is made of (a warp that issues four MMAs or two loads per k-block executes one instruction after
+  // another), so nothing is decided inside them that can be decided per unit: with the case distinctions inside, a k-block
+  // took an issuer 355 cycles whatever its width.  RST: units start at ring stage 0, and the parity comes from one bit per
+  // stage; otherwise the ring runs on and one parity flips at every wrap.
+  auto produce = [&](auto rst, uint32_t dst0, uint32_t stage_bytes, bool gated, auto &&unit_begin, auto &&load) {
+    constexpr bool RST = decltype(rst)::value;
+    uint32_t phases = 0, par = 1, full = bar0, dst = dst0;
+    int lt = 0, stage = 0;
+    for (int u = group; u < num_units; u += n_groups, ++lt) {
       int mt, nt, kb0, kb1;
       decode(u, mt, nt, kb0, kb1);
-      int stage = 0;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (p.gate && lt > 0 && kb - kb0 == p.n_stages - 2 &&
-            !ptx::mbar_wait_warp(sfree_bar, (uint32_t)(lt - 1) & 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-        if (!ptx::mbar_wait_warp(empty_bar(stage), ((phases >> stage) & 1u) ^ 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-        if (ptx::elect_one()) {
-          issue_b(stage, kb, nt);
-          if (kb + p.n_stages + PF_AHEAD < kb1) prefetch_b(kb + p.n_stages + PF_AHEAD, nt);
-          if (kb - kb0 == p.n_stages - 1)   // the ring is primed: ask for the tiles between it and the running prefetch
-            for (int i = p.n_stages; i < min(kb1 - kb0, p.n_stages + PF_AHEAD); ++i) prefetch_b(kb0 + i, nt);
+      unit_begin(mt, nt);
+      if (RST) { stage = 0; full = bar0; dst = dst0; }
+      int k = kb0 * TILE_K;
+      const int k_end = kb1 * TILE_K;
+      auto run = [&](int k_stop) {
+        for (; k < k_stop; k += TILE_K) {
+          const bool ok = wait(full + 8u * MAX_STAGES, RST ? ((phases >> stage) & 1u) ^ 1u : par, DEV_TIMEOUT_PRODUCER);
+          if (ptx::elect_one() && ok) load(full, dst, k);
+          if (RST) phases ^= 1u << stage;
+          full += 8u; dst += stage_bytes;
+          if (++stage == n_stages) { stage = 0; full = bar0; dst = dst0; par ^= 1u; }
         }
-        phases ^= 1u << stage;
-        if (++stage == p.n_stages) stage = 0;
+      };
+      if (RST && gated && lt > 0) {   // the last two stages double as the staging area of the unit before
+        run(min(k_end, k + (n_stages - 2) * TILE_K));
+        if (k < k_end) wait(sfree_bar, (uint32_t)(lt - 1) & 1u, DEV_TIMEOUT_PRODUCER);
+      }
+      run(k_end);
+    }
+  };
+  // STEP = 2: alternating issuers (p.kil).  The ring then has an even number of stages and every unit starts at stage 0, so
+  // the stages of even k-blocks are the even ones: each stage's barriers have one consumer, which sees all of their phases
+  // in order (a thread that skipped phases could not tell a parity from the one two phases on).
+  auto issue = [&](auto rst, auto step, int sl) {
+    constexpr bool RST = decltype(rst)::value;
+    constexpr int STEP = decltype(step)::value;
+    const uint32_t idesc = ptx::idesc_bf16(TILE_M * CG, (uint32_t)p.tile_n);
+    const int s0 = STEP == 2 ? sl : 0;      // first k-block and stage of a unit
+    const uint32_t a_step = ((uint32_t)p.a_stage_bytes >> 4) * STEP, b_step = ((uint32_t)p.b_stage_bytes >> 4) * STEP;   // descriptor units
+    const uint64_t a_desc0 = ptx::smem_desc_sw128(sA + (STEP == 2 ? s0 * p.a_stage_bytes : sl * A_STAGE_BYTES));
+    const uint64_t b_desc0 = ptx::smem_desc_sw128(sB + s0 * p.b_stage_bytes);
+    const uint32_t full0 = bar0 + 8u * s0;
+    uint32_t phases = 0, par = 0, full = full0;
+    uint64_t a_desc = a_desc0, b_desc = b_desc0;
+    int lt = 0, stage = s0;
+    for (int u = group; u < num_units; u += n_groups, ++lt) {
+      int mt, nt, kb0, kb1;
+      decode(u, mt, nt, kb0, kb1);
+      const int ab = lt % nbuf;
+      const uint32_t aphase = (lt / nbuf) & 1;
+      const uint32_t d_tmem = tmem_base + (ab + sl) * ACC_COLS;   // slab sl of a two-slab unit: column sl * ACC_COLS
+      if (RST) { stage = s0; full = full0; a_desc = a_desc0; b_desc = b_desc0; }
+      bool ok = wait(tempty_bar(ab), aphase ^ 1u, DEV_TIMEOUT_MMA);
+      ptx::tc_fence_after_sync();
+      auto run = [&](auto live) {
+        uint32_t acc = 0;
+        for (int i = kb0 + s0; i < kb1; i += STEP) {
+          ok = wait(full, RST ? (phases >> stage) & 1u : par, DEV_TIMEOUT_MMA);
+          ptx::tc_fence_after_sync();
+          if (ptx::elect_one() && ok) {
+            if (decltype(live)::value) {
+#pragma unroll
+              for (int k = 0; k < TILE_K / 16; ++k) {   // 16 bf16 = 32 bytes per MMA: descriptor address += 2
+                if (CG == 2) ptx::mma_bf16_ss_pair(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, k ? 1u : acc);
+                else ptx::mma_bf16_ss(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, k ? 1u : acc);
+              }
+            }
+            if (CG == 2) ptx::mma_commit_pair(full + 8u * MAX_STAGES, 3);
+            else ptx::mma_commit(full + 8u * MAX_STAGES);
+          }
+          acc = 1;
+          if (RST) phases ^= 1u << stage;
+          full += 8u * STEP; a_desc += a_step; b_desc += b_step;
+          if ((stage += STEP) >= n_stages) { stage = s0; full = full0; a_desc = a_desc0; b_desc = b_desc0; par ^= 1u; }
+        }
+      };
+      if (STEP == 2 || sl < unit_slabs) run(std::true_type{});
+      else run(std::false_type{});          // a slab without rows: the barriers only
+      if (ptx::elect_one() && ok) {
+        if (CG == 2) ptx::mma_commit_pair(tfull_bar(ab), 3);
+        else ptx::mma_commit(tfull_bar(ab));
       }
     }
-    if (!ok) *abort_flag = 1;
+  };
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ TMA producer of the weight tiles
+    // No kernel writes weights, so this warp does not wait for the previous kernel of the stream.
+    const uint64_t pol_w = ptx::policy_evict_first();   // weights are read once per step
+    const uint32_t b_bytes = (CG == 2) ? (uint32_t)half_n * 128u : (uint32_t)p.tile_n * 128u;
+    const uint32_t a_bytes = (CG == 2 ? (1 + p.a_peer_loads) : 1) * (uint32_t)p.a_box_bytes;
+    const CUtensorMap *const tmW = (CG == 2 && EPI == EPI_SWIGLU && !leader) ? tmB2 : tmB;
+    const uint32_t to_leader = CG == 2 ? ptx::mapa(bar0, 0) - bar0 : 0;   // a barrier's address here -> in the leader CTA
+    uint32_t tx = 0;
+    int brow = 0;
+    auto unit_begin = [&](int, int nt) {
+      tx = (uint32_t)unit_slabs * a_bytes + CG * b_bytes;
+      brow = EPI == EPI_SWIGLU ? nt * half_n : nt * p.tile_n + (CG == 2 ? (int)rank * half_n : 0);
+    };
+    auto load = [&](uint32_t full, uint32_t dst, int k) {
+      if (CG == 1) {
+        ptx::mbar_arrive_expect_tx(full, tx);
+        ptx::tma_load_2d_hint(dst, tmW, full, k, brow, pol_w);
+        if (EPI == EPI_SWIGLU) ptx::tma_load_2d_hint(dst + half_n * 128, tmB2, full, k, brow, pol_w);
+      } else {
+        if (leader) ptx::mbar_arrive_expect_tx(full, tx);
+        ptx::tma_load_2d_pair_hint(dst, tmW, full + to_leader, k, brow, pol_w);
+      }
+    };
+    if (restart) produce(std::true_type{}, sB, p.b_stage_bytes, p.gate, unit_begin, load);
+    else produce(std::false_type{}, sB, p.b_stage_bytes, false, unit_begin, load);
   } else if (warp == 1 || warp == 2) {
     // ------------------------------------------------------------------ MMA issuers (leader CTA only when paired)
     // warp 1 feeds slab 0, warp 2 slab 1: each slab has its own accumulator columns, so the two
     // instruction streams need no ordering between them; both count on the stage's `empty` barrier.
     const int sl = warp - 1;
     if (leader && (sl < slabs || p.kil)) {
-      const uint32_t idesc = ptx::idesc_bf16(TILE_M * CG, (uint32_t)p.tile_n);
-      uint32_t phases = 0;
-      int lt = 0;
-      bool ok = true;
-      for (int u = group; u < num_units && ok; u += n_groups, ++lt) {
-        int mt, nt, kb0, kb1;
-        decode(u, mt, nt, kb0, kb1);
-        const int ab = lt % nbuf;
-        const uint32_t aphase = (lt / nbuf) & 1;
-        if (!ptx::mbar_wait_warp(tempty_bar(ab), aphase ^ 1u)) { fail(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
-        ptx::tc_fence_after_sync();
-        const uint32_t d_tmem = tmem_base + (ab + sl) * ACC_COLS;   // slab sl of a two-slab unit: column sl * ACC_COLS
-        int stage = 0;
-        for (int kb = kb0; kb < kb1; ++kb) {
-          // Alternating issuers: the ring has an even number of stages and every unit starts at stage 0, so the
-          // stages of even k-blocks are the even ones.  Each stage's barriers thus have one consumer, which sees all of
-          // their phases in order (a thread that skipped phases could not tell a parity from the one two phases on).
-          if (p.kil && ((kb - kb0) & 1) != sl) {
-            if (++stage == p.n_stages) stage = 0;
-            continue;
-          }
-          if (!ptx::mbar_wait_warp(full_bar(stage), (phases >> stage) & 1u)) { fail(p.status, DEV_TIMEOUT_MMA); ok = false; break; }
-          ptx::tc_fence_after_sync();
-          const uint64_t a_desc = ptx::smem_desc_sw128(sA + stage * p.a_stage_bytes + (p.kil ? 0 : sl * A_STAGE_BYTES));
-          const uint64_t b_desc = ptx::smem_desc_sw128(sB + stage * p.b_stage_bytes);
-          const bool first = kb == kb0 + (p.kil ? sl : 0);
-          if (ptx::elect_one()) {
-#pragma unroll
-            for (int k = 0; k < TILE_K / 16; ++k) {   // 16 bf16 = 32 bytes per MMA: descriptor address += 2
-              const uint32_t acc = (!first || k > 0) ? 1u : 0u;
-              if (CG == 2) ptx::mma_bf16_ss_pair(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, acc);
-              else ptx::mma_bf16_ss(d_tmem, a_desc + 2u * k, b_desc + 2u * k, idesc, acc);
-            }
-            if (CG == 2) ptx::mma_commit_pair(empty_bar(stage), 3);
-            else ptx::mma_commit(empty_bar(stage));
-          }
-          phases ^= 1u << stage;
-          if (++stage == p.n_stages) stage = 0;
-        }
-        if (ok && ptx::elect_one()) {
-          if (CG == 2) ptx::mma_commit_pair(tfull_bar(ab), 3);
-          else ptx::mma_commit(tfull_bar(ab));
-        }
-      }
-      if (!ok) *abort_flag = 1;
+      if (p.kil) issue(std::true_type{}, std::integral_constant<int, 2>{}, sl);
+      else if (restart) issue(std::true_type{}, std::integral_constant<int, 1>{}, sl);
+      else issue(std::false_type{}, std::integral_constant<int, 1>{}, sl);
     }
   } else if (warp == 3 + 4 * slabs) {
     // ------------------------------------------------------------------ TMA producer of the activation tiles
     const uint64_t pol_a = ptx::policy_evict_last();    // activations are re-read by every column tile
-    auto issue_a = [&](int stage, int kb, int m0) {   // activation rows of k-block kb, one box per slab
-      const uint32_t dstA = sA + stage * p.a_stage_bytes;
-      if (CG == 1) {
-        for (int sl = 0; sl < slabs; ++sl)
-          ptx::tma_load_2d_hint(dstA + sl * A_STAGE_BYTES, tmA, full_bar(stage), kb * TILE_K, m0 + sl * TILE_M, pol_a);
-      } else {
-        const uint32_t lead_full = ptx::mapa(full_bar(stage), 0);
-        for (int sl = 0; sl < slabs; ++sl)
-          ptx::tma_load_2d_pair_hint(dstA + sl * A_STAGE_BYTES, tmA, lead_full, kb * TILE_K, m0 + sl * TILE_M * CG, pol_a);
-      }
-    };
+    const uint32_t to_leader = CG == 2 ? ptx::mapa(bar0, 0) - bar0 : 0;
     grid_dep_wait();   // the activations are the previous kernel's output
-    uint32_t phases = 0;
-    int lt = 0;
-    bool ok = true;
-    const bool loads_a = leader || p.a_peer_loads;   // few rows: the second CTA of a pair has none
-    for (int u = group; u < num_units && ok && loads_a; u += n_groups, ++lt) {
-      int mt, nt, kb0, kb1;
-      decode(u, mt, nt, kb0, kb1);
-      const int m0 = mt * unit_rows + (int)rank * TILE_M;
-      int stage = 0;
-      for (int kb = kb0; kb < kb1; ++kb) {
-        if (p.gate && lt > 0 && kb - kb0 == p.n_stages - 2 &&
-            !ptx::mbar_wait_warp(sfree_bar, (uint32_t)(lt - 1) & 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-        if (!ptx::mbar_wait_warp(empty_bar(stage), ((phases >> stage) & 1u) ^ 1u)) { fail(p.status, DEV_TIMEOUT_PRODUCER); ok = false; break; }
-        if (ptx::elect_one()) issue_a(stage, kb, m0);
-        phases ^= 1u << stage;
-        if (++stage == p.n_stages) stage = 0;
-      }
+    if (leader || p.a_peer_loads) {   // few rows: the second CTA of a pair has none
+      int m0 = 0;
+      bool two = false;
+      auto unit_begin = [&](int mt, int) { m0 = mt * unit_rows + (int)rank * TILE_M; two = unit_slabs == 2; };
+      auto load = [&](uint32_t full, uint32_t dst, int k) {   // activation rows of the k-block, one box per live slab
+        if (CG == 1) {
+          ptx::tma_load_2d_hint(dst, tmA, full, k, m0, pol_a);
+          if (two) ptx::tma_load_2d_hint(dst + A_STAGE_BYTES, tmA, full, k, m0 + TILE_M, pol_a);
+        } else {
+          ptx::tma_load_2d_pair_hint(dst, tmA, full + to_leader, k, m0, pol_a);
+          if (two) ptx::tma_load_2d_pair_hint(dst + A_STAGE_BYTES, tmA, full + to_leader, k, m0 + TILE_M * CG, pol_a);
+        }
+      };
+      if (restart) produce(std::true_type{}, sA, p.a_stage_bytes, p.gate, unit_begin, load);
+      else produce(std::false_type{}, sA, p.a_stage_bytes, false, unit_begin, load);
     }
-    if (!ok) *abort_flag = 1;
   } else {
     // ------------------------------------------------------------------ epilogue
     // warps 3-6 drain slab 0, warps 7-10 (two-slab units only) slab 1; warp w may touch TMEM lanes 32 (w % 4) ..
@@ -288,7 +304,7 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
       decode(u, mt, nt, kb0, kb1);
       const int ab = lt % nbuf;
       const uint32_t aphase = (lt / nbuf) & 1;
-      if (!ptx::mbar_wait_warp(tfull_bar(ab), aphase)) { fail(p.status, DEV_TIMEOUT_EPILOGUE); ok = false; break; }
+      if (!ptx::mbar_wait_idle(tfull_bar(ab), aphase, 20)) { fail(p.status, DEV_TIMEOUT_EPILOGUE); ok = false; break; }
       ptx::tc_fence_after_sync();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (ab + sl) * ACC_COLS;
       const int row0 = mt * unit_rows + sl * (TILE_M * CG) + (int)rank * TILE_M + q * 32;
@@ -297,10 +313,19 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
       const bool last_unit = u + n_groups >= num_units;
       const bool res_store = EPI == EPI_RESIDUAL && p.part != nullptr && p.k_splits > 1;
       const int slice_row0 = res_store ? unit_ks * p.part_rows : 0;   // partial sums: the slice's own rows
-      if (EPI != EPI_LMHEAD && p.out_tma && nt < p.out_full_tiles && (last_unit || p.gate))
-        drain_tile_staged<EPI>(p, tmC, taddr, slice_row0 + row0, nt, sOut + (uint32_t)(warp - 3) * (4096u * STAGE_BUFS), lane,
-                               res_store);
-      else
+      if (sl >= unit_slabs || row0 >= p.M) {
+        // no rows here
+      } else if (EPI != EPI_LMHEAD && p.out_tma && (nt < p.out_full_tiles || p.out_tail_cols) && (last_unit || p.gate || p.out_ring)) {
+        const int tail = nt < p.out_full_tiles ? 0 : p.out_tail_cols;   // the row's last, narrower tile has a map of its own
+        const bool wide = last_unit && p.last_bufs > 0;
+        if (p.out_ring && lt > 0 && !wide) {   // the unit before has left this warp's staging tiles
+          if (lane == 0) ptx::bulk_wait_read();
+          __syncwarp();
+        }
+        drain_tile_staged<EPI>(p, tail ? tmCT : tmC, taddr, slice_row0 + row0, nt,
+                               wide ? base + (uint32_t)(warp - 3) * (4096u * p.last_bufs) : sOut + (uint32_t)(warp - 3) * (4096u * STAGE_BUFS),
+                               lane, res_store, tail, false, wide ? p.last_bufs : STAGE_BUFS);
+      } else
         drain_tile<EPI>(p, taddr, row0 + lane, nt, res_store ? 2 : (p.k_splits > 1 ? 1 : 0),
                         res_store ? p.part + (int64_t)slice_row0 * p.N : reinterpret_cast<float *>(p.out),
                         p.kil && kb1 - kb0 >= 2);
@@ -343,23 +368,25 @@ __device__ __forceinline__ void gemm_body(const CUtensorMap *tmA, const CUtensor
 template <int EPI>
 __global__ void __launch_bounds__(384, 1)
 gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmC, const KParams p) {
+                    const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmC,
+                         const __grid_constant__ CUtensorMap tmCT, const KParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 5];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  gemm_body<EPI, 1>(&tmA, &tmB, &tmB2, &tmC, p, smem_raw, bars, &tmem_slot, &abort_flag);
+  gemm_body<EPI, 1>(&tmA, &tmB, &tmB2, &tmC, &tmCT, p, smem_raw, bars, &tmem_slot, &abort_flag);
 }
 
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(384, 1)
 gemm_tcgen05_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                         const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmC, const KParams p) {
+                         const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmC,
+                         const __grid_constant__ CUtensorMap tmCT, const KParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bars[2 * MAX_STAGES + 5];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  gemm_body<EPI, 2>(&tmA, &tmB, &tmB2, &tmC, p, smem_raw, bars, &tmem_slot, &abort_flag);
+  gemm_body<EPI, 2>(&tmA, &tmB, &tmB2, &tmC, &tmCT, p, smem_raw, bars, &tmem_slot, &abort_flag);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -464,30 +491,40 @@ l2pd_status make_tma_out_tail(TmaDesc *out, void *ptr, bool fp32, int64_t rows, 
   return r == CUDA_SUCCESS ? L2PD_OK : L2PD_ERR_CUDA;
 }
 
-// Modelled cycles of one GEMM for a tile width / K split / slab count.  Per 64-deep k-block a CTA
-// needs the largest of: the tensor pipe's 2 * tile_n cycles per slab; the ~620 cycles one thread
-// takes to issue its four MMAs and the stage hand-over; the bytes it must take in at INGEST bytes
-// per cycle.  A unit adds a fixed fill part and, when its accumulators are not double-buffered
-// (two slabs), the drain of the accumulator; times the number of waves over the SMs (or SM pairs).
-static double plan_cost(int M, int N, int K, int num_sms, int cg, int slabs, int unit_n, int tile_n, int ks, bool is_residual, bool kil) {
-  const double INGEST = cg == 2 ? 58.0 : 68.0;   // measured: bytes per cycle an SM takes in from L2 through TMA
+// Modelled cycles of one GEMM for a tile width / K split / slab count, from traces of the kernel on the 8B layer shapes.
+//   k-block   a 64-deep k-block takes the largest of the tensor pipe's 2 * tile_n cycles per slab, the 250 cycles its
+//             issuer needs at least (300 with two slabs), and the bytes a CTA takes in at 95 B per cycle (measured alone:
+//             79-117 B, by how many CTAs share a tile).  A sixth of the ingest time comes on top of the rest: between two
+//             tilings that keep the pipe equally busy the one that moves fewer bytes lets the power cap hold a higher clock.
+//   unit      one slab: two accumulator buffers, ~400 cycles between units; two slabs: the drain is exposed.
+//   launch    7000 cycles from the CTA's start to its first MMA, and the last unit's drain.
+//   memory    the weights are read from HBM once, at 3450 B per cycle of the whole chip.
+//   K slices  store fp32 partial sums that the next RMSNorm reads: ~2000 B per cycle both ways together.
+static double plan_cost(int M, int N, int K, int num_sms, int cg, int slabs, int unit_n, int tile_n, int ks, bool is_residual) {
   const int groups = num_sms / cg;
-  const int m_tiles = ceil_div(M, TILE_M * cg * slabs);
+  const int n_slabs = ceil_div(M, TILE_M * cg);
   const int n_tiles = ceil_div(N, unit_n);
-  const int units = m_tiles * n_tiles * ks;
-  const int waves = ceil_div(units, groups);
+  const int full = (n_slabs / slabs) * n_tiles * ks, tail = (n_slabs % slabs) ? n_tiles * ks : 0;
   const int kb = ceil_div(ceil_div(K, TILE_K), ks);
-  const double bytes = (double)slabs * A_STAGE_BYTES + 128.0 * tile_n / cg;
-  const double per_kb = fmax(fmax(2.0 * tile_n * slabs, kil ? 330.0 : 620.0), bytes / INGEST) * 1.06;
-  // emptying the accumulators: bf16 stores leave an SM at ~34 B per cycle; fp32 additions into X are bound
-  // by L2's atomic units, ~2500 B per cycle for the whole chip, i.e. ~17 B per cycle and SM when all drain at once
-  // (K slices store their partial sums plainly: twice the rate of the additions)
-  const double drain = (double)TILE_M * slabs * unit_n * (is_residual ? (ks > 1 ? 4.0 / 34.0 : 4.0 / 17.0) : 2.0 / 34.0) + 1500.0;
-  const double exposed = slabs == 2 ? drain : 0.3 * drain;
-  return waves * (kb * per_kb + 6000.0 + exposed) + (slabs == 2 ? 0.0 : 0.7 * drain);
+  auto drain = [&](int sl) { return 1000.0 + (is_residual ? 32.0 : 20.0) * tile_n * (sl == 2 ? 1.6 : 1.0); };
+  auto unit = [&](int sl) {
+    const double bytes = (double)sl * A_STAGE_BYTES + 128.0 * tile_n / cg;
+    const double pipe = 2.0 * tile_n * sl * (cg == 1 ? 1.13 : 1.0);
+    return kb * (fmax(fmax(pipe, sl == 2 ? 300.0 : 250.0), bytes / 95.0) + 0.15 * bytes / 95.0) + (slabs == 2 ? drain(sl) : 400.0);
+  };
+  // units go round the CTA groups in order, the full ones first
+  const double uf = unit(slabs), ut = tail ? unit(n_slabs % slabs) : 0.0;
+  const int q = full / groups, r = full % groups, a = tail / groups, b = tail % groups;
+  double span;
+  if (r == 0) span = q * uf + (a + (b ? 1 : 0)) * ut;
+  else span = fmax((q + 1) * uf + (a + (r + b > groups ? 1 : 0)) * ut, q * uf + (a + (b ? 1 : 0)) * ut);
+  span += 7000.0 + (slabs == 2 ? 0.0 : drain(1));
+  span = fmax(span, 2.0 * (double)n_tiles * tile_n * K / 3450.0 + 7000.0) + 0.05 * span;
+  if (ks > 1) span += 8.0 * ks * (double)M * N / 2000.0 * (M > 128 ? 1.0 : 0.25);
+  return span;
 }
 
-GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits, int max_tile_n) {
+GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits, int max_tile_n, int force_slabs, int force_ks) {
   GemmPlan best{1, 256, 1, 1, 0};
   double best_cost = 1e300;
   const bool swiglu = epi == EPI_SWIGLU;
@@ -495,19 +532,19 @@ GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, 
   for (int cg = 1; cg <= 2; ++cg) {
     if (cg == 2 && (M <= TILE_M || epi == EPI_LMHEAD || num_sms < 2)) continue;
     for (int slabs = 1; slabs <= 2; ++slabs) {
-      // a second slab: the weight tile is read once for twice the rows, and a second thread issues MMAs
+      // a second slab: the weight tile is read once for twice the rows
       if (slabs == 2 && (cg == 1 || epi == EPI_LMHEAD || M <= TILE_M * cg)) continue;
+      if (force_slabs && slabs != force_slabs) continue;
       for (int tn = 256; tn >= 64; tn -= step) {
         if (force_tile_n && tn != force_tile_n) continue;
         if (!force_tile_n && tn > max_tile_n) continue;
         const int unit_n = swiglu ? tn / 2 : tn;
         const int max_ks = (epi == EPI_RESIDUAL) ? (max_k_splits < 4 ? max_k_splits : 4) : 1;
         for (int ks = 1; ks <= max_ks; ++ks) {
-          if (ceil_div(K, TILE_K) < 8 * ks) break;
-          // few rows: one 128-row MMA per 132 cycles and issuer bounds the K loop; the idle second issuer takes every other k-block
-          const bool kil = M <= TILE_M * cg && slabs == 1 && epi != EPI_LMHEAD;
-          const double c = plan_cost(M, N, K, num_sms, cg, slabs, unit_n, tn, ks, epi == EPI_RESIDUAL, kil);
-          if (c < best_cost - 1e-9) { best_cost = c; best = GemmPlan{cg, tn, ks, slabs, kil ? 1 : 0}; }
+          if (force_ks && ks != force_ks) continue;
+          if (ks > 1 && ceil_div(K, TILE_K) < 8 * ks) break;
+          const double c = plan_cost(M, N, K, num_sms, cg, slabs, unit_n, tn, ks, epi == EPI_RESIDUAL);
+          if (c < best_cost - 1e-9) { best_cost = c; best = GemmPlan{cg, tn, ks, slabs, 0}; }
         }
       }
     }
@@ -527,7 +564,7 @@ GemmPlan plan_gemm_pair_one_slab(int epi, int M, int N, int K, int num_sms, int 
     const int max_ks = (epi == EPI_RESIDUAL) ? (max_k_splits < 4 ? max_k_splits : 4) : 1;
     for (int ks = 1; ks <= max_ks; ++ks) {
       if (ceil_div(K, TILE_K) < 8 * ks) break;
-      const double c = plan_cost(M, N, K, num_sms, 2, 1, unit_n, tn, ks, epi == EPI_RESIDUAL, true);
+      const double c = plan_cost(M, N, K, num_sms, 2, 1, unit_n, tn, ks, epi == EPI_RESIDUAL);
       if (c < best_cost - 1e-9) { best_cost = c; best = GemmPlan{2, tn, ks, 1, 1}; }
     }
   }
@@ -561,17 +598,25 @@ cudaError_t fill_kparams(const GemmArgs &g, int stages, int b_stage_bytes, KPara
   if (g.a_box_rows > 0 && g.a_box_rows < TILE_M) {
     if (g.M > TILE_M || p.slabs != 1 || g.a_box_rows < g.M || (g.a_box_rows % 8)) return cudaErrorInvalidValue;
     p.a_box_bytes = g.a_box_rows * TILE_K * 2;
+    // The ring keeps only the rows there are.  The MMA's 128 rows then run into the next stages and, from the last ones, into
+    // the weight ring behind: in bounds, and into accumulator rows that are never stored.
+    if (cg == 1 && !chained) p.a_stage_bytes = p.a_box_bytes;
   }
   if (cg == 2 && g.M <= TILE_M) p.a_peer_loads = 0;
   const int stage_bytes = p.a_stage_bytes + p.b_stage_bytes;
+  // one-slab units overlap their drain with the next unit's main loop: staging tiles of their own, four warps' worth
+  p.out_ring = (!chained && p.slabs == 1 && g.c != nullptr && g.epi != EPI_LMHEAD && !g.k_interleave) ? 1 : 0;
+  const int out_bytes = p.out_ring ? 4 * STAGE_BUFS * 4096 : 0;
   if (stages <= 0) {
-    stages = (SMEM_BUDGET - 2048) / stage_bytes;
+    stages = (SMEM_BUDGET - 2048 - out_bytes) / stage_bytes;
     if (stages > MAX_STAGES) stages = MAX_STAGES;
     if (g.k_interleave) stages &= ~1;   // alternate k-blocks <-> alternate stages
   }
-  if (stages < 2 || stages > MAX_STAGES || (size_t)stages * stage_bytes + 2048 > (size_t)SMEM_BUDGET) return cudaErrorInvalidValue;
+  if (stages < 2 || stages > MAX_STAGES || (size_t)stages * stage_bytes + out_bytes + 2048 > (size_t)SMEM_BUDGET) return cudaErrorInvalidValue;
   p.n_stages = stages;
+  p.out_stage_off = (stages * stage_bytes + 1023) & ~1023;
   p.m_tiles = ceil_div(g.M, TILE_M * cg * p.slabs);
+  p.tail_slabs = ceil_div(g.M - (p.m_tiles - 1) * TILE_M * cg * p.slabs, TILE_M * cg);
   const int n_per_tile = (g.epi == EPI_SWIGLU) ? g.tile_n / 2 : g.tile_n;
   // staged output: needs the output map and a staging area (the A part of the ring's last two stages)
   p.kil = g.k_interleave ? 1 : 0;
@@ -584,6 +629,13 @@ cudaError_t fill_kparams(const GemmArgs &g, int stages, int b_stage_bytes, KPara
   if (p.out_tma && g.c_tail && g.tail_cols > 0) {
     if (g.tail_cols != g.N - p.out_full_tiles * n_per_tile || (g.tail_cols % (g.epi == EPI_SWIGLU ? 8 : 16))) return cudaErrorInvalidValue;
     p.out_tail_cols = g.tail_cols;
+  }
+  {
+    const int num_kb = ceil_div(g.K, TILE_K);
+    const int flush_cols = g.epi == EPI_RESIDUAL ? 32 : 64;
+    const int bufs = ceil_div(n_per_tile, flush_cols);
+    p.last_bufs = (p.out_tma && !chained && bufs > STAGE_BUFS && bufs * 4096 * 4 * p.slabs <= stages * stage_bytes &&
+                   num_kb - ceil_div(num_kb, ks) * (ks - 1) >= stages) ? bufs : 0;   // (a whole ring of loads lies between two drains)
   }
   p.gate = (p.out_tma && p.slabs == 2 && stages >= 4) ? 1 : 0;
   p.n_tiles = ceil_div(g.N, n_per_tile);
@@ -614,14 +666,15 @@ cudaError_t launch_gemm_tcgen05(cudaStream_t st, const GemmArgs &g, int num_sms)
   if (units <= 0) return cudaSuccess;
   const int groups = num_sms / cg;
   const int grid = cg * (units < groups ? units : groups);
-  const size_t smem = (size_t)stages * stage_bytes + 1024;
+  const size_t smem = p.out_ring ? (size_t)p.out_stage_off + 4 * STAGE_BUFS * 4096 + 1024 : (size_t)stages * stage_bytes + 1024;
   const CUtensorMap &b2 = g.b2 ? g.b2->map : g.b->map;
   const CUtensorMap &cm = p.out_tma ? g.c->map : g.a->map;
+  const CUtensorMap &cmt = p.out_tail_cols ? g.c_tail->map : cm;
   cudaError_t e;
 #define L2PD_LAUNCH(KERNEL, EPI)                                                                      \
   e = cudaFuncSetAttribute(KERNEL<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET - 1024); \
   if (e != cudaSuccess) return e;                                                                    \
-  e = launch_kernel(KERNEL<EPI>, dim3(grid), dim3(128 + 128 * p.slabs), smem, st, g.a->map, g.b->map, b2, cm, p);                \
+  e = launch_kernel(KERNEL<EPI>, dim3(grid), dim3(128 + 128 * p.slabs), smem, st, g.a->map, g.b->map, b2, cm, cmt, p);                \
   if (e != cudaSuccess) return e;
   if (cg == 1) {
     switch (g.epi) {

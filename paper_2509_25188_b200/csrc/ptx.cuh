@@ -85,6 +85,40 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, ui
   return true;
 }
 
+// As mbar_wait_warp, for a wait that lasts thousands of cycles (an accumulator, while the main loop runs): the warp sleeps
+// between polls, which otherwise compete with the producers' and issuers' barrier and TMA instructions.
+__device__ __forceinline__ bool mbar_wait_idle(uint32_t bar, uint32_t parity, uint32_t sleep_ns, uint64_t limit_ns = 2000000000ull) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const uint64_t t0 = globaltimer();
+  uint32_t spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    __nanosleep(sleep_ns);
+    if ((++spins & 0x3fu) == 0 && __any_sync(0xffffffffu, globaltimer() - t0 > limit_ns)) return false;
+  }
+  return true;
+}
+
+// The wait of a producer or issuer loop.  It does not end the loop: when the wait runs out, or another role of the CTA has
+// failed (`abort_flag`, in shared memory), it returns false and the caller goes on without issuing anything, all later waits
+// returning false at once.  A loop without an early exit lets the assembler see that its stage, address and descriptor
+// values are the same in every lane (k-block of four N = 64 MMAs: 278 cycles with the exit, 215 without).
+__device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity, int *abort_flag, int32_t *status, int code,
+                                                   uint64_t limit_ns = 2000000000ull) {
+  if (mbar_try_wait(bar, parity)) return true;
+  volatile int *const ab = abort_flag;
+  const uint64_t t0 = globaltimer();
+  uint32_t spins = 0;
+  while (!mbar_try_wait(bar, parity)) {
+    if (*ab) return false;
+    if ((++spins & 0x3ffu) == 0 && globaltimer() - t0 > limit_ns) {
+      if (status) atomicCAS(status, 0, code);
+      *ab = 1;
+      return false;
+    }
+  }
+  return true;
+}
+
 // ---- thread-block clusters (pairs of CTAs sharing one MMA tile) -----------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
