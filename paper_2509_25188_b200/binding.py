@@ -465,6 +465,23 @@ def attention_bf16(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, H: int, dh
     return out
 
 
+def _flat_params(arrays, dev):
+    """The arrays as fp32 in one device tensor (one transfer each way): the tensor, each array's address in it, and a
+    function that brings the tensor back as numpy arrays of the arrays' shapes."""
+    arrays = [np.asarray(a, dtype=np.float32) for a in arrays]
+    ends = np.cumsum([0] + [-(-a.size // 4) * 4 for a in arrays])       # every array starts on 16 bytes
+    host = np.zeros(max(int(ends[-1]), 1), np.float32)
+    for a, lo in zip(arrays, ends):
+        host[lo:lo + a.size] = a.ravel()
+    flat = torch.from_numpy(host).to(dev)
+    ptrs = [flat.data_ptr() + 4 * int(lo) for lo in ends[:-1]]
+
+    def split(t):
+        back = t.cpu().numpy()
+        return [back[lo:lo + a.size].reshape(a.shape).copy() for a, lo in zip(arrays, ends)]
+    return flat, ptrs, split
+
+
 def filter_train(filt: Dict[str, np.ndarray], C_in, Y_in, epochs: int, lr: float = 1e-3, beta1: float = 0.9,
                  beta2: float = 0.999, eps: float = 1e-8, weight_decay: float = 0.01, batch_size: int = 0,
                  device: int = 0):
@@ -475,13 +492,12 @@ def filter_train(filt: Dict[str, np.ndarray], C_in, Y_in, epochs: int, lr: float
     tc = (C_in if isinstance(C_in, torch.Tensor) else torch.from_numpy(np.ascontiguousarray(C_in))).to(dev, torch.float32).contiguous()
     ty = (Y_in if isinstance(Y_in, torch.Tensor) else torch.from_numpy(np.ascontiguousarray(Y_in))).to(dev, torch.uint8).contiguous()
     N, s = int(tc.shape[0]), int(tc.shape[1])
-    p = {k: torch.from_numpy(np.ascontiguousarray(filt[k], dtype=np.float32)).to(dev) for k in ("w1", "b1", "w2", "b2")}
+    flat, ptrs, split = _flat_params([filt[k] for k in ("w1", "b1", "w2", "b2")], dev)
     bs = N if batch_size <= 0 else batch_size
     losses = np.zeros(max(epochs * (-(-N // bs)), 1), np.float32)
     cfg = TrainConfig(lr, beta1, beta2, eps, weight_decay, epochs, batch_size)
-    _check(lib.l2pd_filter_train(_stream(), s, N, tc.data_ptr(), ty.data_ptr(), p["w1"].data_ptr(), p["b1"].data_ptr(),
-                                 p["w2"].data_ptr(), p["b2"].data_ptr(), C.byref(cfg), losses.ctypes.data), None)
-    return {k: v.cpu().numpy() for k, v in p.items()}, losses[: epochs * (-(-N // bs))]
+    _check(lib.l2pd_filter_train(_stream(), s, N, tc.data_ptr(), ty.data_ptr(), *ptrs, C.byref(cfg), losses.ctypes.data), None)
+    return dict(zip(("w1", "b1", "w2", "b2"), split(flat))), losses[: epochs * (-(-N // bs))]
 
 
 def filter_train_layers(layers, C_in, Y_in, epochs: int, lr: float = 1e-3, beta1: float = 0.9, beta2: float = 0.999,
@@ -492,15 +508,14 @@ def filter_train_layers(layers, C_in, Y_in, epochs: int, lr: float = 1e-3, beta1
     tc = (C_in if isinstance(C_in, torch.Tensor) else torch.from_numpy(np.ascontiguousarray(C_in))).to(dev, torch.float32).contiguous()
     ty = (Y_in if isinstance(Y_in, torch.Tensor) else torch.from_numpy(np.ascontiguousarray(Y_in))).to(dev, torch.uint8).contiguous()
     N, s = int(tc.shape[0]), int(tc.shape[1])
-    ws = [torch.from_numpy(np.ascontiguousarray(w, dtype=np.float32)).to(dev) for w, _ in layers]
-    bs_ = [torch.from_numpy(np.ascontiguousarray(b_, dtype=np.float32)).to(dev) for _, b_ in layers]
     n = len(layers)
-    pw = (C.c_void_p * max(n, 1))(*[t.data_ptr() for t in ws])
-    pb = (C.c_void_p * max(n, 1))(*[t.data_ptr() for t in bs_])
+    flat, ptrs, split = _flat_params([a for layer in layers for a in layer], dev)
+    pw, pb = (C.c_void_p * max(n, 1))(*ptrs[0::2]), (C.c_void_p * max(n, 1))(*ptrs[1::2])
     bsz = N if batch_size <= 0 else batch_size
     updates = epochs * (-(-N // bsz))
     losses = np.zeros(max(updates, 1), np.float32)
     cfg = TrainConfig(lr, beta1, beta2, eps, weight_decay, epochs, batch_size)
     _check(lib.l2pd_filter_train_layers(_stream(), s, n, N, tc.data_ptr(), ty.data_ptr(), pw, pb, C.byref(cfg),
                                         losses.ctypes.data), None)
-    return [(w.cpu().numpy(), b_.cpu().numpy()) for w, b_ in zip(ws, bs_)], losses[:updates]
+    out = split(flat)
+    return list(zip(out[0::2], out[1::2])), losses[:updates]

@@ -953,6 +953,27 @@ l2pd_status l2pd_set_collect(l2pd_ctx *c, float *d_c, uint8_t *d_y, int64_t capa
 }
 int64_t l2pd_collect_count(const l2pd_ctx *c) { return c ? c->collect_n : 0; }
 
+// Scratch of the filter training: stream-ordered, from a pool of the library's own for each device that keeps at most 32 MB
+// between calls (a cudaMalloc and cudaFree pair took 0.7 ms of every call) and gives it back when a context is destroyed.
+static cudaMemPool_t train_pool(int dev) {
+  static cudaMemPool_t pools[64] = {};
+  static std::mutex mu;
+  if (dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lock(mu);
+  if (!pools[dev]) {
+    cudaMemPoolProps pr = {};
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    pr.location.id = dev;
+    uint64_t keep = 32u << 20;
+    cudaMemPool_t q = nullptr;
+    if (cudaMemPoolCreate(&q, &pr) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) { cudaMemPoolDestroy(q); cudaGetLastError(); return nullptr; }
+    pools[dev] = q;
+  }
+  return pools[dev];
+}
+
 static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t N, const float *d_c, const uint8_t *d_y,
                                      float *const *w, float *const *b, const l2pd_train_config *t, float *h_losses) {
   if (!d_c || !d_y || !w || !b || !t) return L2PD_ERR_ARG;
@@ -967,31 +988,37 @@ static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t
   const int per = s * s + s, P = L * per;
   const int64_t bs = t->batch_size > 0 ? t->batch_size : N;
   const int64_t per_epoch = (N + bs - 1) / bs, updates = per_epoch * t->epochs;
-  float *theta = nullptr, *gpart = nullptr, *losses = nullptr;
-  auto cleanup = [&]() { cudaFree(theta); cudaFree(gpart); cudaFree(losses); };
-  if (cudaMalloc(&theta, sizeof(float) * 3 * P) != cudaSuccess || cudaMalloc(&gpart, sizeof(float) * (size_t)sms * (P + 1)) != cudaSuccess ||
-      cudaMalloc(&losses, sizeof(float) * (size_t)(updates > 0 ? updates : 1)) != cudaSuccess) { cleanup(); return L2PD_ERR_OOM; }
-  float *m = theta + P, *v = theta + 2 * P;
-  const size_t ss = sizeof(float) * s * s, sv = sizeof(float) * s;
-  bool ok = cudaMemsetAsync(m, 0, sizeof(float) * 2 * P, st) == cudaSuccess;
-  for (int k = 0; ok && k < L; ++k)
-    ok = cudaMemcpyAsync(theta + k * per, w[k], ss, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-         cudaMemcpyAsync(theta + k * per + s * s, b[k], sv, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-  FilterTrainHyper h{t->lr, t->beta1, t->beta2, t->eps, t->weight_decay};
-  double p1 = 1.0, p2 = 1.0;   // beta^t, carried in double
-  int64_t u = 0;
-  for (int e = 0; ok && e < t->epochs; ++e)
-    for (int64_t lo = 0; ok && lo < N; lo += bs, ++u) {
-      p1 *= t->beta1; p2 *= t->beta2;
-      ok = launch_filter_update(st, d_c, d_y, lo, (N - lo < bs ? N - lo : bs), s, L, theta, m, v, gpart, sms, h, 1.0 - p1, 1.0 - p2,
-                                losses + u) == cudaSuccess;
-    }
-  for (int k = 0; ok && k < L; ++k)
-    ok = cudaMemcpyAsync(w[k], theta + k * per, ss, cudaMemcpyDeviceToDevice, st) == cudaSuccess &&
-         cudaMemcpyAsync(b[k], theta + k * per + s * s, sv, cudaMemcpyDeviceToDevice, st) == cudaSuccess;
-  if (ok && h_losses && updates > 0) ok = cudaMemcpyAsync(h_losses, losses, sizeof(float) * updates, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+  // one allocation: theta, m, v | the blocks' gradient sums | losses | meeting counter, status
+  const size_t n_sums = (size_t)filter_train_max_rows(N < bs ? N : bs, sms) * filter_train_row_floats(P), n_loss = (size_t)(updates > 0 ? updates : 1);
+  float *theta = nullptr;
+  cudaMemPool_t pool = train_pool(dev);
+  if (!pool || cudaMallocFromPoolAsync((void **)&theta, sizeof(float) * (3 * (size_t)P + n_sums + n_loss + 8), pool, st) != cudaSuccess) return L2PD_ERR_OOM;
+  float *m = theta + P, *v = theta + 2 * P, *gpart = theta + ((3 * P + 3) & ~3), *losses = gpart + n_sums;
+  unsigned *bar = reinterpret_cast<unsigned *>(losses + n_loss);
+  int32_t *d_status = reinterpret_cast<int32_t *>(bar + 1);
+  bool ok = launch_filter_pack(st, w, b, s, L, theta, d_status, true) == cudaSuccess;
+  FilterTrainArgs fa{d_c, d_y, N, bs, s, L, theta, m, v, gpart, losses, {t->lr, t->beta1, t->beta2, t->eps, t->weight_decay}, bar, d_status};
+  // updates per launch: some 50 ms of work, so that no launch holds the device for long
+  const double per_update = (double)(N < bs ? N : bs) * s * s * L + 1e7;
+  int64_t chunk = (int64_t)(3.5e11 / per_update);
+  chunk = chunk < 1 ? 1 : (chunk > 4096 ? 4096 : chunk);
+  double p1 = 1.0, p2 = 1.0;   // beta^u, carried in double
+  for (int64_t u = 0; ok && u < updates; u += chunk) {
+    const int64_t u1 = updates - u < chunk ? updates : u + chunk;
+    ok = cudaMemsetAsync(bar, 0, 4, st) == cudaSuccess && launch_filter_train(st, fa, u, u1, p1, p2, sms) == cudaSuccess;
+    for (int64_t i = u; i < u1; ++i) { p1 *= t->beta1; p2 *= t->beta2; }
+  }
+  if (ok) ok = launch_filter_pack(st, w, b, s, L, theta, d_status, false) == cudaSuccess;
+  // losses and status in one copy: they lie behind one another
+  const size_t n_back = h_losses ? n_loss + 2 : 2;
+  std::vector<float> back(n_back);
+  if (ok) ok = cudaMemcpyAsync(back.data(), losses + (n_loss + 2 - n_back), sizeof(float) * n_back, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+  ok = (cudaFreeAsync(theta, st) == cudaSuccess) && ok;
   ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;
-  cleanup();
+  int32_t h_stat = DEV_OK;
+  memcpy(&h_stat, &back[n_back - 1], 4);
+  if (ok && h_stat != DEV_OK) return L2PD_ERR_TIMEOUT;
+  if (ok && h_losses && updates > 0) memcpy(h_losses, back.data(), sizeof(float) * updates);
   return ok ? L2PD_OK : L2PD_ERR_CUDA;
 }
 
@@ -1088,6 +1115,7 @@ void l2pd_destroy(l2pd_ctx *c) {
   if (!c) return;
   cudaSetDevice(c->device);
   cudaDeviceSynchronize();
+  if (cudaMemPool_t pool = train_pool(c->device)) cudaMemPoolTrimTo(pool, 0);
   free_all(c);
   delete c;
 }

@@ -144,9 +144,21 @@ cudaError_t launch_decide(cudaStream_t st, const DecideArgs &a, int n_slots);
 // theta / m / v: packed per layer W_k [s*s], b_k [s] (n_layers of them, 1 .. 4); gpart: [grid, n_layers*(s*s+s) + 1] scratch;
 // bc1 / bc2 = 1 - beta^t for this update's step count t; loss_out receives the batch's loss before the update.
 struct FilterTrainHyper { float lr, beta1, beta2, eps, weight_decay; };
-cudaError_t launch_filter_update(cudaStream_t st, const float *C, const uint8_t *Y, int64_t n0, int64_t n, int s, int n_layers,
-                                 float *theta, float *m, float *v, float *gpart, int grid, const FilterTrainHyper &h,
-                                 double bc1, double bc2, float *loss_out);
+inline __host__ __device__ int filter_train_row_floats(int P) { return (P + 4) & ~3; }   // P sums and the loss, padded to 16 bytes
+struct FilterTrainArgs {
+  const float *C; const uint8_t *Y; int64_t N, batch;   // samples [N, s] and targets; samples per update
+  int s, n_layers;                                       // 1 to 4 Linear(s, s) layers
+  float *theta, *m, *v;                                  // packed per layer: W [s*s], b [s]
+  float *gpart;                                          // [filter_train_max_rows][filter_train_row_floats], 16-byte aligned
+  float *losses;                                         // [updates]
+  FilterTrainHyper h;
+  unsigned *bar; int32_t *status;                        // meeting counter (0 before every launch), status word
+};
+int filter_train_max_rows(int64_t batch, int sms);   // rows of gpart a launch may write
+// pack: the layers' arrays -> theta (moments m, v behind it set to 0, status cleared); otherwise theta -> the arrays
+cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, bool pack);
+// updates [u0, u1) in one cooperative launch; p1 = beta1^u0, p2 = beta2^u0
+cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms);
 
 // gemm_tcgen05.cu
 struct TmaDesc { CUtensorMap map; };

@@ -1,363 +1,457 @@
 // Filter training, stage 2 of Algorithm 1: minimise Eq. 6, the mean binary cross-entropy between
-// sigmoid(f_theta(conf)) and the EGP targets, over theta = (W1, b1, W2, b2) of the two-layer filter
-// (Section 3.2; 2 * (s*s + s) parameters) with AdamW (Section 4.1: learning rate 0.001).
+// sigmoid(f_theta(conf)) and the EGP targets, over the weights of the filter (Section 3.2: two Linear(s, s)
+// layers; Section 4.4: one to four, ReLU between consecutive layers) with AdamW (Section 4.1: learning rate 0.001).
 //
-// One update = two launches:
-//   filter_grad_warp_kernel (s <= 32)  a warp per sample, lane j = block position j: the lane keeps row j of W1 and
-//                        W2 and the accumulators of row j of both gradients in registers; the sample's vectors
-//                        (c, h, dz) pass between lanes through 128-byte shared-memory slots read as broadcasts;
-//   filter_grad_kernel (s > 32, or the depth variants of Section 4.4: 1 to 4 layers)  every block walks tiles of
-//                        32 samples: forward through the layers, dz = sigmoid(z) - y, then layer by layer
-//                        downwards dW_k += delta_k^T x_k, db_k += sum delta_k, delta_{k-1} = (delta_k W_k) [x_k > 0],
-//                        into accumulators its threads own; a block ends by writing its sums (not yet divided
-//                        by the batch's element count) and its loss sum to its own row of `gpart`;
-//   filter_adamw_kernel  one thread per parameter adds the rows in block order (so a run is bit-reproducible), scales by
-//                        1 / (samples * s) and applies AdamW: decoupled weight decay, bias-corrected moments.
-// The whole problem (a few thousand parameters, samples of s floats) lives in shared memory and L2; the
-// arithmetic is fp32 on CUDA cores: K = s <= 64 is far too short a contraction for the tensor cores to matter.
+// filter_train_kernel runs many updates in one cooperative launch.  One update:
+//   gradient   every block walks tiles of T samples held in shared memory: forward through the layers, dz = sigmoid(z) - y, delta of the layers below
+//              (delta_{k-1} = (delta_k W_k) [x_k > 0]), then dW_k += delta_k^T x_k into accumulators its threads own;
+//              it ends by writing its sums (not yet divided by the batch's element count) and its loss sum to its own
+//              row of `gpart`;
+//   meeting    all blocks meet at a counter in global memory (cooperative launch: all are resident; bounded wait);
+//   AdamW      a block takes 8 parameters at a time, its threads shares of the rows that are then added in order (a run is
+//              bit-reproducible on a given GPU), scales by 1 / (samples * s) and applies the update: decoupled weight
+//              decay, bias-corrected moments;
+//   meeting    and every block reads the new weights.
+// K = s <= 64 is too short a contraction, and fp32 too wide a type, for the tensor cores; what bounds the kernel is the
+// fp32 pipe (432 M multiply-adds for 84,480 samples of 32: 12 us) and, for small batches, the two meetings (~2 us each) and
+// the phases' latency.  A thread computes 4 samples x C positions (dW: 4 x 4 elements) from 16-byte shared-memory
+// vectors, 16 C multiply-adds for 4 + C loads; rows are padded to 4 mod 32 words and positions dealt out so that the
+// vectors of a warp lie in different banks.  The next tile arrives (cp.async) while one is worked on.
+// Measured, one update, two launches of per-sample warps before -> this: 84,480 samples of 32 positions, two layers 100 -> 40 us
+// (tiles 30 us, which are bound by shared-memory loads at 40 % of the fp32 pipe); 1,024 samples of 64, four layers
+// 95 -> 21 us; a call without updates 1.0 -> 0.15 ms.
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace l2pd {
 
 namespace {
 
-constexpr int TB = 32;               // samples per tile
-constexpr int GRAD_THREADS = 512;
+constexpr int MAX_LAYERS = 4;
 constexpr int MAX_S = 64;
-constexpr int MAX_OWN = (MAX_S * MAX_S + GRAD_THREADS - 1) / GRAD_THREADS;   // accumulator elements per thread and matrix
 
-struct GradArgs {
+struct TrainArgs {
   const float *C;          // [N, s] filter inputs
   const uint8_t *Y;        // [N, s] targets (0 / 1)
-  int64_t n0, n;           // the batch: samples [n0, n0 + n)
-  int s;
-  int n_layers;            // 1 .. 4 Linear(s, s) layers, ReLU between consecutive layers
-  const float *theta;      // packed per layer: W_k [s*s], b_k [s]
-  float *gpart;            // [gridDim.x, P + 1]: gradient sums, then the loss sum
-};
-
-constexpr int MAX_LAYERS = 4;
-
-// Any depth, any s <= 64: every block walks tiles of 32 samples held in shared memory.
-__global__ void __launch_bounds__(GRAD_THREADS) filter_grad_kernel(GradArgs a) {
-  extern __shared__ float sm[];
-  const int s = a.s, sp = s + 1, L = a.n_layers;   // padded row stride: rows read side by side fall into different banks
-  float *W = sm;                      // [L][s][sp]
-  float *Bv = W + L * s * sp;         // [L][s]
-  float *X = Bv + L * s;              // [L][TB][sp]: X[0] the inputs, X[k] = relu(output of layer k - 1)
-  float *D0 = X + L * TB * sp;        // [TB][sp] delta of the layer being differentiated
-  float *D1 = D0 + TB * sp;           // [TB][sp] delta of the layer below
-  __shared__ float red[GRAD_THREADS / 32];
-
-  grid_dep_launch();
-  grid_dep_wait();
-  const int tid = threadIdx.x;
-  const int per = s * s + s, P = L * per;
-  for (int k = 0; k < L; ++k) {
-    for (int e = tid; e < s * s; e += GRAD_THREADS) W[(k * s + e / s) * sp + e % s] = a.theta[k * per + e];
-    if (tid < s) Bv[k * s + tid] = a.theta[k * per + s * s + tid];
-  }
-
-  float acc[MAX_LAYERS][MAX_OWN], gb[MAX_LAYERS];
-#pragma unroll
-  for (int k = 0; k < MAX_LAYERS; ++k) {
-    gb[k] = 0.f;
-#pragma unroll
-    for (int q = 0; q < MAX_OWN; ++q) acc[k][q] = 0.f;
-  }
-  float loss = 0.f;
-
-  const int64_t n_tiles = (a.n + TB - 1) / TB;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t base = a.n0 + tile * TB;
-    const int rows = (int)((a.n - tile * TB) < TB ? (a.n - tile * TB) : TB);
-    __syncthreads();                                   // the previous tile's buffers are no longer read
-    for (int e = tid; e < TB * s; e += GRAD_THREADS) {
-      const int n = e / s, i = e - n * s;
-      X[n * sp + i] = n < rows ? a.C[(base + n) * s + i] : 0.f;
-    }
-    __syncthreads();
-    // forward: layer k maps X[k] to X[k + 1] = relu(.), the last layer to dz = sigmoid(z) - y in D0
-    for (int k = 0; k < L; ++k) {
-      const float *xin = X + k * TB * sp, *wk = W + k * s * sp;
-      for (int o = tid; o < TB * s; o += GRAD_THREADS) {
-        const int n = o / s, j = o - n * s;
-        float v = Bv[k * s + j];
-        for (int i = 0; i < s; ++i) v = fmaf(wk[j * sp + i], xin[n * sp + i], v);
-        if (k + 1 < L) {
-          X[(k + 1) * TB * sp + n * sp + j] = fmaxf(v, 0.f);
-        } else {
-          float dz = 0.f;
-          if (n < rows) {
-            const float y = (float)a.Y[(base + n) * s + j];
-            dz = 1.0f / (1.0f + expf(-v)) - y;
-            loss += fmaxf(v, 0.f) - v * y + log1pf(expf(-fabsf(v)));
-          }
-          D0[n * sp + j] = dz;
-        }
-      }
-      __syncthreads();
-    }
-    // backward: dW_k += delta_k^T X[k], db_k += sum delta_k, delta_{k-1} = (delta_k W_k) [X[k] > 0]
-    float *dcur = D0, *dnxt = D1;
-#pragma unroll
-    for (int kk = 0; kk < MAX_LAYERS; ++kk) {
-      const int k = L - 1 - kk;
-      if (k < 0) break;
-      const float *xin = X + k * TB * sp, *wk = W + k * s * sp;
-#pragma unroll
-      for (int q = 0; q < MAX_OWN; ++q) {
-        const int e = tid + q * GRAD_THREADS;
-        if (e < s * s) {
-          const int j = e / s, i = e - j * s;
-          float v = acc[kk][q];
-          for (int n = 0; n < TB; ++n) v = fmaf(dcur[n * sp + j], xin[n * sp + i], v);
-          acc[kk][q] = v;
-        }
-      }
-      if (tid < s) {
-        float v = gb[kk];
-        for (int n = 0; n < TB; ++n) v += dcur[n * sp + tid];
-        gb[kk] = v;
-      }
-      if (k > 0) {
-        for (int o = tid; o < TB * s; o += GRAD_THREADS) {
-          const int n = o / s, i = o - n * s;
-          float v = 0.f;
-          for (int j = 0; j < s; ++j) v = fmaf(dcur[n * sp + j], wk[j * sp + i], v);
-          dnxt[n * sp + i] = xin[n * sp + i] > 0.f ? v : 0.f;
-        }
-      }
-      __syncthreads();
-      float *t = dcur; dcur = dnxt; dnxt = t;
-    }
-  }
-
-  float *out = a.gpart + (int64_t)blockIdx.x * (P + 1);
-#pragma unroll
-  for (int kk = 0; kk < MAX_LAYERS; ++kk) {       // acc[kk] belongs to layer L - 1 - kk
-    const int k = L - 1 - kk;
-    if (k < 0) break;
-#pragma unroll
-    for (int q = 0; q < MAX_OWN; ++q) {
-      const int e = tid + q * GRAD_THREADS;
-      if (e < s * s) out[k * per + e] = acc[kk][q];
-    }
-    if (tid < s) out[k * per + s * s + tid] = gb[kk];
-  }
-  for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-  if ((tid & 31) == 0) red[tid >> 5] = loss;
-  __syncthreads();
-  if (tid == 0) {
-    float t = 0.f;
-    for (int w = 0; w < GRAD_THREADS / 32; ++w) t += red[w];
-    out[P] = t;
-  }
-}
-
-// ---- s <= 32: a warp per sample ------------------------------------------------------------------------------
-constexpr int WG_WARPS = 8;
-constexpr int WG_ROW = 33;   // padded row of the W2 copy that is read by columns
-
-__global__ void __launch_bounds__(WG_WARPS * 32) filter_grad_warp_kernel(GradArgs a) {
-  extern __shared__ __align__(16) float wsm[];
-  float *W2s = wsm;                               // [32][33], zero beyond s
-  float *vc = W2s + 32 * WG_ROW;                  // [warps][32]; 32 * 33 floats = 4224 bytes, a multiple of 16
-  float *vh = vc + WG_WARPS * 32;
-  float *vd = vh + WG_WARPS * 32;
-  float *red = vd + WG_WARPS * 32;                // [warps][2 * 1024 + 64] at the end of the kernel
-
-  grid_dep_launch();
-  grid_dep_wait();
-  const int s = a.s, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int P = 2 * (s * s + s);
-  for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
-    const int j = e >> 5, i = e & 31;
-    W2s[j * WG_ROW + i] = (j < s && i < s) ? a.theta[s * s + s + j * s + i] : 0.f;
-  }
-  float w1[32], w2[32], acc1[32], acc2[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const bool in = lane < s && i < s;
-    w1[i] = in ? a.theta[lane * s + i] : 0.f;
-    w2[i] = in ? a.theta[s * s + s + lane * s + i] : 0.f;
-    acc1[i] = 0.f; acc2[i] = 0.f;
-  }
-  const float b1 = lane < s ? a.theta[s * s + lane] : 0.f, b2 = lane < s ? a.theta[2 * s * s + s + lane] : 0.f;
-  float gb1 = 0.f, gb2 = 0.f, loss = 0.f;
-  __syncthreads();
-
-  float *mc = vc + warp * 32, *mh = vh + warp * 32, *md = vd + warp * 32;
-  const int64_t stride = (int64_t)gridDim.x * WG_WARPS;
-  // the next sample's row is requested before the current one is worked on (a warp has no other loads to hide it behind)
-  int64_t n = (int64_t)blockIdx.x * WG_WARPS + warp;
-  float c_nx = 0.f, y_nx = 0.f;
-  if (n < a.n && lane < s) { c_nx = a.C[(a.n0 + n) * s + lane]; y_nx = (float)a.Y[(a.n0 + n) * s + lane]; }
-  for (; n < a.n; n += stride) {
-    const float c = c_nx, y = y_nx;
-    if (n + stride < a.n && lane < s) {
-      const int64_t row = (a.n0 + n + stride) * s;
-      c_nx = a.C[row + lane]; y_nx = (float)a.Y[row + lane];
-    }
-    mc[lane] = c;
-    __syncwarp();
-    // the dot products run as four interleaved partial sums (a single chain of 32 dependent multiply-adds would
-    // leave the two warps a scheduler has here waiting on latency); the order of the additions is fixed
-    float p0 = b1, p1 = 0.f, p2 = 0.f, p3 = 0.f;           // pre_j = W1[j,:] c + b1_j
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 v = *reinterpret_cast<const float4 *>(mc + 4 * q);
-      p0 = fmaf(w1[4 * q], v.x, p0); p1 = fmaf(w1[4 * q + 1], v.y, p1);
-      p2 = fmaf(w1[4 * q + 2], v.z, p2); p3 = fmaf(w1[4 * q + 3], v.w, p3);
-    }
-    const float pre = (p0 + p1) + (p2 + p3);
-    const float h = fmaxf(pre, 0.f);
-    mh[lane] = lane < s ? h : 0.f;
-    __syncwarp();
-    p0 = b2; p1 = 0.f; p2 = 0.f; p3 = 0.f;                 // z_j = W2[j,:] h + b2_j
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 v = *reinterpret_cast<const float4 *>(mh + 4 * q);
-      p0 = fmaf(w2[4 * q], v.x, p0); p1 = fmaf(w2[4 * q + 1], v.y, p1);
-      p2 = fmaf(w2[4 * q + 2], v.z, p2); p3 = fmaf(w2[4 * q + 3], v.w, p3);
-    }
-    const float z = (p0 + p1) + (p2 + p3);
-    float dz = 0.f;
-    if (lane < s) {
-      dz = 1.0f / (1.0f + expf(-z)) - y;
-      loss += fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
-    }
-    md[lane] = dz;
-    __syncwarp();
-    p0 = 0.f; p1 = 0.f; p2 = 0.f; p3 = 0.f;                // dh_i = sum_j W2[j, i] dz_j  (lane = i)
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 v = *reinterpret_cast<const float4 *>(md + 4 * q);
-      p0 = fmaf(W2s[(4 * q) * WG_ROW + lane], v.x, p0); p1 = fmaf(W2s[(4 * q + 1) * WG_ROW + lane], v.y, p1);
-      p2 = fmaf(W2s[(4 * q + 2) * WG_ROW + lane], v.z, p2); p3 = fmaf(W2s[(4 * q + 3) * WG_ROW + lane], v.w, p3);
-    }
-    const float dh = (p0 + p1) + (p2 + p3);
-    const float dpre = pre > 0.f ? dh : 0.f;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {                          // rows j of dW2 += dz_j h, of dW1 += dpre_j c
-      const float4 vh4 = *reinterpret_cast<const float4 *>(mh + 4 * q);
-      const float4 vc4 = *reinterpret_cast<const float4 *>(mc + 4 * q);
-      acc2[4 * q] = fmaf(dz, vh4.x, acc2[4 * q]); acc2[4 * q + 1] = fmaf(dz, vh4.y, acc2[4 * q + 1]);
-      acc2[4 * q + 2] = fmaf(dz, vh4.z, acc2[4 * q + 2]); acc2[4 * q + 3] = fmaf(dz, vh4.w, acc2[4 * q + 3]);
-      acc1[4 * q] = fmaf(dpre, vc4.x, acc1[4 * q]); acc1[4 * q + 1] = fmaf(dpre, vc4.y, acc1[4 * q + 1]);
-      acc1[4 * q + 2] = fmaf(dpre, vc4.z, acc1[4 * q + 2]); acc1[4 * q + 3] = fmaf(dpre, vc4.w, acc1[4 * q + 3]);
-    }
-    gb2 += dz; gb1 += dpre;
-    __syncwarp();                                          // the slots are rewritten by the next sample
-  }
-
-  // the block's sums: every warp parks its rows, then each element is added over the warps in warp order
-  float *mine = red + warp * (2 * 1024 + 64);
-#pragma unroll
-  for (int i = 0; i < 32; ++i) { mine[i * 32 + lane] = acc1[i]; mine[1024 + i * 32 + lane] = acc2[i]; }   // [column][row]: no bank conflicts
-  mine[2048 + lane] = gb1; mine[2048 + 32 + lane] = gb2;
-  for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
-  __shared__ float wloss[WG_WARPS];
-  if (lane == 0) wloss[warp] = loss;
-  __syncthreads();
-  float *out = a.gpart + (int64_t)blockIdx.x * (P + 1);
-  for (int e = threadIdx.x; e < 2 * 1024 + 64; e += blockDim.x) {
-    float t = 0.f;
-    for (int w = 0; w < WG_WARPS; ++w) t += red[w * (2 * 1024 + 64) + e];
-    if (e < 2048) {
-      const int mat = e >> 10, i = (e >> 5) & 31, j = e & 31;
-      if (j < s && i < s) out[mat * (s * s + s) + j * s + i] = t;
-    } else {
-      const int which = (e - 2048) >> 5, j = e & 31;
-      if (j < s) out[which * (s * s + s) + s * s + j] = t;
-    }
-  }
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < WG_WARPS; ++w) t += wloss[w];
-    out[P] = t;
-  }
-}
-
-struct AdamArgs {
-  const float *gpart;
-  int n_blocks, P;
-  float inv_count;                 // 1 / (samples in the batch * s)
+  int64_t N, batch;        // samples; samples per update (the last batch of an epoch may be shorter)
+  int64_t u0, u1;          // this launch's updates
+  int per_epoch;           // updates per epoch
+  int s, n_layers, P;      // P parameters
+  float *theta, *m, *v;    // packed per layer: W_k [s*s], b_k [s]
+  float *gpart;            // a row per block: gradient sums, then the loss sum
+  float *losses;           // [updates]: the batch's loss, measured before the update
   float lr, beta1, beta2, eps, weight_decay;
-  float bc1, bc2;                  // 1 - beta1^t, 1 - beta2^t
-  float *theta, *m, *v;
-  float *loss_out;                 // the batch's loss, measured before this update
+  double p1, p2;           // beta1^u0, beta2^u0
+  unsigned *bar;           // meeting counter, 0 at launch
+  int32_t *status;
 };
 
-constexpr int ADAM_THREADS = 128;
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
 
-__global__ void __launch_bounds__(ADAM_THREADS) filter_adamw_kernel(AdamArgs a) {
-  grid_dep_launch();
-  grid_dep_wait();
-  const int p = blockIdx.x * ADAM_THREADS + threadIdx.x;   // one parameter per thread; entry P is the loss
-  if (p <= a.P) {
-    // the rows are added in block order whatever the batching of the loads: 32 loads in flight, then 32 adds
-    float g = 0.f;
-    int b = 0;
-    for (; b + 32 <= a.n_blocks; b += 32) {
-      float t[32];
-#pragma unroll
-      for (int i = 0; i < 32; ++i) t[i] = a.gpart[(int64_t)(b + i) * (a.P + 1) + p];
-#pragma unroll
-      for (int i = 0; i < 32; ++i) g += t[i];
+// All blocks of the launch meet: `target` arrivals on the counter.  False (for the whole block) when the wait ran out.
+__device__ __forceinline__ bool meet(unsigned *bar, unsigned target, int32_t *status, int *s_ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(bar), "r"(1u) : "memory");
+    int ok = 1;
+    const uint64_t t0 = ptx::globaltimer();
+    uint32_t spins = 0;
+    while ((int)(ld_acquire(bar) - target) < 0) {
+      if ((++spins & 0x3fu) == 0) {
+        if (*reinterpret_cast<volatile int32_t *>(status) != DEV_OK) { ok = 0; break; }
+        if (ptx::globaltimer() - t0 > 2000000000ull) { atomicCAS(status, 0, DEV_TIMEOUT_EPILOGUE); ok = 0; break; }
+      }
     }
-    for (; b < a.n_blocks; ++b) g += a.gpart[(int64_t)b * (a.P + 1) + p];
-    g *= a.inv_count;
-    if (p == a.P) { *a.loss_out = g; return; }
-    const float th = a.theta[p] * (1.0f - a.lr * a.weight_decay);
-    const float m = a.beta1 * a.m[p] + (1.0f - a.beta1) * g;
-    const float v = a.beta2 * a.v[p] + (1.0f - a.beta2) * g * g;
-    a.m[p] = m; a.v[p] = v;
-    a.theta[p] = th - a.lr * (m / a.bc1) / (sqrtf(v / a.bc2) + a.eps);
+    *s_ok = ok;
   }
+  __syncthreads();
+  return *s_ok != 0;
+}
+
+// Words of the tile buffers: X[0] twice (the next tile arrives while this one is worked on), X[1 .. L - 1], and the deltas of
+// the layer being differentiated and of the one below.  They also hold the end of an update's sums (4096 + 256 words where
+// threads share a gradient).
+template <int S, int T>
+__host__ __device__ constexpr int train_tile_floats(int L) {
+  return (L + 1 + (L < 2 ? L : 2)) * T * (S + 4) < 4096 + 256 ? 4096 + 256 : (L + 1 + (L < 2 ? L : 2)) * T * (S + 4);
+}
+template <int S, int T>
+constexpr int train_smem_floats(int L) { return L * (S * (S + 4) + S) + train_tile_floats<S, T>(L) + 2 * T * S / 4 + 64; }
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, int bytes) {   // the rest of the 16 bytes is zero
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+
+// S: positions padded to 32 or 64; T: samples per tile; LM: most layers (accumulators in registers); TH threads per block,
+// OCC blocks per SM.
+template <int S, int T, int LM, int TH, int OCC>
+__global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a) {
+  constexpr int TRAIN_THREADS = TH, TRAIN_WARPS = TH / 32;
+  constexpr int C = T * S / (4 * TRAIN_THREADS);      // positions per thread (x 4 samples)
+  constexpr int NCG = S / C, NSG = T / 4;
+  static_assert(C >= 1 && NCG % 8 == 0 && NCG * NSG == TRAIN_THREADS, "thread tiling");
+  constexpr int RS = S + 4;                           // row stride of every matrix: 4 mod 32 words
+  constexpr int G = 16 * TH / (S * S);                  // groups of threads that share a gradient, each with T / G of the samples
+  constexpr int GT = TRAIN_THREADS / G, GA = S / 4;   // threads per group = GA x GA
+  extern __shared__ __align__(16) float sm[];
+  __shared__ int s_ok;
+  const int s = a.s, L = a.n_layers, per = s * s + s, P = a.P, gs = filter_train_row_floats(P), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float *W = sm;                          // [L][S][RS]
+  float *Bv = W + L * S * RS;             // [L][S]
+  float *X0 = Bv + L * S;                 // [2][T][RS]: inputs of this tile and the next
+  float *X1 = X0 + 2 * T * RS;            // [L - 1][T][RS]: relu(output of layer k - 1) at k - 1
+  float *D = X1 + (L - 1) * T * RS;       // [min(L, 2)][T][RS]: gradient of the loss with respect to a layer's output
+  float *X = X0;                          // (the sums at the end of an update)
+  uint8_t *Ys = reinterpret_cast<uint8_t *>(X0 + train_tile_floats<S, T>(L));   // [2][T][S]
+  float *red = reinterpret_cast<float *>(Ys + 2 * T * S);                       // [64]
+  // outputs of a thread: samples sg + NSG e, positions cg + NCG c (forward) or C cg + c (backward); a warp has 8 position
+  // groups x 4 sample groups
+  const int cg = (tid & 7) + 8 * (tid / (8 * NSG)), sg = (tid >> 3) % NSG;
+  const int grp = tid / GT, ga = (tid % GT) / GA, gb_ = tid % GA;            // dW: elements (4 ga + r, 4 gb_ + q) of group grp
+  constexpr int DBP = TRAIN_THREADS / S;                                     // db: position tid % S, one of DBP parts of the samples
+  // rows that fill their padded width and start on 16 bytes come by cp.async
+  const bool vec = s == S && ((reinterpret_cast<uintptr_t>(a.C) | reinterpret_cast<uintptr_t>(a.Y)) & 15) == 0;
+  double p1 = a.p1, p2 = a.p2;
+  unsigned target = 0;
+
+  for (int64_t u = a.u0; u < a.u1; ++u) {
+    const int64_t n0 = (u % a.per_epoch) * a.batch, nb = a.N - n0 < a.batch ? a.N - n0 : a.batch;
+    const int64_t n_tiles = (nb + T - 1) / T;
+    const int rows = (int)(n_tiles < gridDim.x ? n_tiles : gridDim.x);       // blocks that have tiles
+    if (blockIdx.x < rows) {
+      if (s == S) {
+        for (int k = 0; k < L; ++k) {
+          constexpr int NV = S * S / 4 / TRAIN_THREADS;     // 16-byte vectors per thread and layer, all in flight together
+          float4 t[NV];
+#pragma unroll
+          for (int q = 0; q < NV; ++q) t[q] = __ldcg(reinterpret_cast<const float4 *>(a.theta + k * per) + tid + q * TRAIN_THREADS);
+#pragma unroll
+          for (int q = 0; q < NV; ++q) {
+            const int e = 4 * (tid + q * TRAIN_THREADS);
+            *reinterpret_cast<float4 *>(W + (k * S + e / S) * RS + e % S) = t[q];
+          }
+        }
+      } else {
+#pragma unroll 8
+        for (int e = tid; e < L * S * S; e += TRAIN_THREADS) {
+          const int k = e / (S * S), j = (e / S) % S, i = e % S;
+          W[(k * S + j) * RS + i] = (j < s && i < s) ? __ldcg(a.theta + k * per + j * s + i) : 0.f;
+        }
+      }
+      for (int e = tid; e < L * S; e += TRAIN_THREADS) Bv[e] = (e % S) < s ? __ldcg(a.theta + (e / S) * per + s * s + e % S) : 0.f;
+      float acc[LM][16], gb[LM], loss = 0.f;
+#pragma unroll
+      for (int k = 0; k < LM; ++k) {
+        gb[k] = 0.f;
+#pragma unroll
+        for (int q = 0; q < 16; ++q) acc[k][q] = 0.f;
+      }
+      auto fetch = [&](int64_t tile, int buf) {
+        const int64_t base = n0 + tile * T;
+        const int live = (int)(nb - tile * T < T ? nb - tile * T : T);
+        float *xd = X0 + buf * T * RS;
+        uint8_t *yd = Ys + buf * T * S;
+        if (vec) {
+          for (int e = tid; e < T * S / 4; e += TRAIN_THREADS) {
+            const int n = e / (S / 4), i = 4 * (e % (S / 4));
+            const bool in = n < live;
+            cp_async16(xd + n * RS + i, a.C + (in ? (base + n) * s + i : 0), in ? 16 : 0);
+          }
+          for (int e = tid; e < T * S / 16; e += TRAIN_THREADS) {
+            const bool in = 16 * e < live * S;
+            cp_async16(yd + 16 * e, a.Y + (in ? base * s + 16 * e : 0), in ? 16 : 0);
+          }
+          asm volatile("cp.async.commit_group;" ::: "memory");
+        } else {
+          for (int e = tid; e < T * S; e += TRAIN_THREADS) {
+            const int n = e / S, i = e % S;
+            const bool in = n < live && i < s;
+            xd[n * RS + i] = in ? a.C[(base + n) * s + i] : 0.f;
+            yd[e] = in ? a.Y[(base + n) * s + i] : 0;
+          }
+        }
+      };
+      int buf = 0;
+      fetch(blockIdx.x, 0);
+      for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, buf ^= 1) {
+        const int live = (int)(nb - tile * T < T ? nb - tile * T : T);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();                                   // this tile has arrived; the previous one is no longer read
+        if (tile + gridDim.x < n_tiles) fetch(tile + gridDim.x, buf ^ 1);
+        float *const x0 = X0 + buf * T * RS;
+        // forward: layer k maps X[k] to X[k + 1] = relu(.), the last layer to dz = sigmoid(z) - y in D
+        for (int k = 0; k < L; ++k) {
+          const float *xin = (k ? X1 + (k - 1) * T * RS : x0) + sg * RS, *wk = W + (k * S + cg) * RS;
+          float o[C][4];
+#pragma unroll
+          for (int c = 0; c < C; ++c) o[c][0] = o[c][1] = o[c][2] = o[c][3] = Bv[k * S + cg + NCG * c];
+#pragma unroll 4
+          for (int i = 0; i < S; i += 4) {
+            float4 w[C], x[4];
+#pragma unroll
+            for (int c = 0; c < C; ++c) w[c] = *reinterpret_cast<const float4 *>(wk + NCG * c * RS + i);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = *reinterpret_cast<const float4 *>(xin + NSG * e * RS + i);
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+              for (int e = 0; e < 4; ++e)
+                o[c][e] = fmaf(w[c].w, x[e].w, fmaf(w[c].z, x[e].z, fmaf(w[c].y, x[e].y, fmaf(w[c].x, x[e].x, o[c][e]))));
+          }
+          if (k + 1 < L) {
+            float *xo = X1 + k * T * RS + sg * RS + cg;
+#pragma unroll
+            for (int c = 0; c < C; ++c)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) xo[NSG * e * RS + NCG * c] = fmaxf(o[c][e], 0.f);
+          } else {
+            // loss = max(z, 0) - z y + log(1 + t), t = exp(-|z|): the logarithms of this thread's outputs are taken as one,
+            // of the product of the (1 + t), carried as pm = product - 1
+            float pm = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int n = sg + NSG * e;
+#pragma unroll
+              for (int c = 0; c < C; ++c) {
+                const int j = cg + NCG * c;
+                const bool on = n < live && j < s;
+                const float z = o[c][e], y = Ys[(buf * T + n) * S + j] ? 1.f : 0.f;
+                const float t = expf(-fabsf(z)), sig = __fdividef(z >= 0.f ? 1.f : t, 1.f + t);
+                if (on) { loss += fmaxf(z, 0.f) - z * y; pm = fmaf(pm, t, pm + t); }
+                D[n * RS + j] = on ? sig - y : 0.f;
+              }
+            }
+            loss += log1pf(pm);
+          }
+          __syncthreads();
+        }
+        // backward, layer by layer: dW_k += D[k]^T X[k], db_k += sum D[k], D[k - 1] = (D[k] W_k) [X[k] > 0]
+        float *dcur = D, *dnxt = D + T * RS;
+#pragma unroll
+        for (int kk = 0; kk < LM; ++kk) {                  // acc[kk] belongs to layer L - 1 - kk
+          const int k = L - 1 - kk;
+          if (k < 0) break;
+          const float *xin = k ? X1 + (k - 1) * T * RS : x0;
+          const float *dk = dcur + grp * (T / G) * RS + 4 * ga, *xk = xin + grp * (T / G) * RS + 4 * gb_;
+#pragma unroll 4
+          for (int n = 0; n < T / G; ++n) {
+            const float4 dv = *reinterpret_cast<const float4 *>(dk + n * RS), xv = *reinterpret_cast<const float4 *>(xk + n * RS);
+            const float dr[4] = {dv.x, dv.y, dv.z, dv.w}, xr[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+              for (int q = 0; q < 4; ++q) acc[kk][4 * r + q] = fmaf(dr[r], xr[q], acc[kk][4 * r + q]);
+          }
+          const float *db = dcur + (tid / S) * (T / DBP) * RS + tid % S;
+#pragma unroll
+          for (int n = 0; n < T / DBP; ++n) gb[kk] += db[n * RS];
+          if (k > 0) {
+            const float *din = dcur + sg * RS, *wk = W + k * S * RS + C * cg;
+            float o[C][4];
+#pragma unroll
+            for (int c = 0; c < C; ++c) o[c][0] = o[c][1] = o[c][2] = o[c][3] = 0.f;
+#pragma unroll 2
+            for (int j = 0; j < S; j += 4) {
+              float4 d[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) d[e] = *reinterpret_cast<const float4 *>(din + NSG * e * RS + j);
+#pragma unroll
+              for (int r = 0; r < 4; ++r) {
+                float w[C];
+                if constexpr (C == 4) *reinterpret_cast<float4 *>(w) = *reinterpret_cast<const float4 *>(wk + (j + r) * RS);
+                else if constexpr (C == 2) *reinterpret_cast<float2 *>(w) = *reinterpret_cast<const float2 *>(wk + (j + r) * RS);
+                else w[0] = wk[(j + r) * RS];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const float dr = r == 0 ? d[e].x : r == 1 ? d[e].y : r == 2 ? d[e].z : d[e].w;
+#pragma unroll
+                  for (int c = 0; c < C; ++c) o[c][e] = fmaf(w[c], dr, o[c][e]);
+                }
+              }
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+#pragma unroll
+              for (int c = 0; c < C; ++c) {
+                const int at = (sg + NSG * e) * RS + C * cg + c;
+                dnxt[at] = xin[at] > 0.f ? o[c][e] : 0.f;
+              }
+            __syncthreads();
+            float *t = dcur; dcur = dnxt; dnxt = t;
+          }
+        }
+      }
+      // the block's sums: groups and parts are added in order through shared memory (over the tile buffers)
+      float *out = a.gpart + (int64_t)blockIdx.x * gs;
+#pragma unroll
+      for (int kk = 0; kk < LM; ++kk) {
+        const int k = L - 1 - kk;
+        if (k < 0) break;
+        __syncthreads();
+        if (G > 1) {
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            *reinterpret_cast<float4 *>(X + (grp * S + 4 * ga + r) * S + 4 * gb_) =
+                make_float4(acc[kk][4 * r], acc[kk][4 * r + 1], acc[kk][4 * r + 2], acc[kk][4 * r + 3]);
+        }
+        X[G * S * S * (G > 1) + tid] = gb[kk];
+        __syncthreads();
+        if (G > 1) {
+          // (the groups' sums lie as [group][position][position])
+#pragma unroll
+          for (int q = 0; q < S * S / TRAIN_THREADS; ++q) {
+            const int e = tid + q * TRAIN_THREADS, j = e / S, i = e % S;
+            float t = X[e];
+#pragma unroll
+            for (int g = 1; g < G; ++g) t += X[g * S * S + e];
+            if (j < s && i < s) __stcg(out + k * per + j * s + i, t);
+          }
+        } else {
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if (s == S)
+              __stcg(reinterpret_cast<float4 *>(out + k * per + (4 * ga + r) * S + 4 * gb_),
+                     make_float4(acc[kk][4 * r], acc[kk][4 * r + 1], acc[kk][4 * r + 2], acc[kk][4 * r + 3]));
+            else
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int j = 4 * ga + r, i = 4 * gb_ + q;
+              if (j < s && i < s) __stcg(out + k * per + j * s + i, acc[kk][4 * r + q]);
+            }
+        }
+        if (tid < s) {
+          float t = 0.f;
+#pragma unroll
+          for (int q = 0; q < DBP; ++q) t += X[G * S * S * (G > 1) + q * S + tid];
+          __stcg(out + k * per + s * s + tid, t);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      if (lane == 0) red[warp] = loss;
+      __syncthreads();
+      if (tid == 0) {
+        float t = 0.f;
+        for (int w = 0; w < TRAIN_WARPS; ++w) t += red[w];
+        __stcg(out + P, t);
+      }
+    }
+    target += gridDim.x;
+    if (!meet(a.bar, target, a.status, &s_ok)) return;
+
+    // AdamW: 32 parameters per block and pass, a share of the rows per warp; entry P is the loss
+    p1 *= (double)a.beta1; p2 *= (double)a.beta2;
+    const float bc1 = (float)(1.0 - p1), bc2 = (float)(1.0 - p2), inv_count = (float)(1.0 / ((double)nb * s));
+    // A block's pass: PW parameters x RG shares of the rows.  Few parameters and many rows: a sector of a row per load and
+    // many shares; many parameters: wider passes, whose number costs more than their length.
+    const int PW = P < 16 * (int)gridDim.x ? 8 : rows > 64 ? 32 : TRAIN_THREADS, RG = TRAIN_THREADS / PW;
+    const int pl = tid % PW, rg = tid / PW, share = (rows + RG - 1) / RG, b0 = rg * share, b1 = min(rows, b0 + share);
+    for (int c = blockIdx.x; c * PW <= P; c += gridDim.x) {
+      const int p = c * PW + pl;
+      float g = 0.f;
+      if (p <= P) {
+        for (int b = b0; b < b1; b += 16) {                // up to 16 rows in flight; adding zero at the end changes nothing
+          float t[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) t[i] = b + i < b1 ? __ldcg(a.gpart + (int64_t)(b + i) * gs + p) : 0.f;
+#pragma unroll
+          for (int i = 0; i < 16; ++i) g += t[i];
+        }
+      }
+      if (RG > 1) {
+        __syncthreads();
+        X[tid] = g;
+        __syncthreads();
+      }
+      if (tid < PW && p <= P) {
+        for (int w = 1; w < RG; ++w) g += X[w * PW + tid];
+        g *= inv_count;
+        if (p == P) {
+          a.losses[u] = g;
+        } else {
+          const float th = __ldcg(a.theta + p) * (1.0f - a.lr * a.weight_decay);
+          const float m = a.beta1 * a.m[p] + (1.0f - a.beta1) * g;
+          const float v = a.beta2 * a.v[p] + (1.0f - a.beta2) * g * g;
+          a.m[p] = m; a.v[p] = v;
+          __stcg(a.theta + p, th - a.lr * (m / bc1) / (sqrtf(v / bc2) + a.eps));
+        }
+      }
+    }
+    if (u + 1 < a.u1) {
+      target += gridDim.x;
+      if (!meet(a.bar, target, a.status, &s_ok)) return;
+    }
+  }
+}
+
+struct PackArgs { float *w[MAX_LAYERS], *b[MAX_LAYERS]; float *theta; int s, n_layers; };
+
+// The caller's arrays -> theta, moments 0, status 0 (pack), and theta -> the caller's arrays.
+__global__ void filter_pack_kernel(PackArgs a, int pack, int32_t *status) {
+  const int per = a.s * a.s + a.s, P = a.n_layers * per;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < P; e += gridDim.x * blockDim.x) {
+    const int k = e / per, r = e - k * per;
+    float *q = r < a.s * a.s ? a.w[k] + r : a.b[k] + (r - a.s * a.s);
+    if (pack) { a.theta[e] = *q; a.theta[P + e] = 0.f; a.theta[2 * P + e] = 0.f; }
+    else *q = a.theta[e];
+  }
+  if (pack && blockIdx.x == 0 && threadIdx.x == 0) *status = DEV_OK;
+}
+
+template <int S, int T, int LM, int TH, int OCC>
+cudaError_t launch_train(cudaStream_t st, TrainArgs &a, int sms) {
+  const size_t smem = sizeof(float) * (size_t)train_smem_floats<S, T>(a.n_layers);
+  cudaError_t e = cudaFuncSetAttribute(filter_train_kernel<S, T, LM, TH, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int occ = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, filter_train_kernel<S, T, LM, TH, OCC>, TH, smem);
+  if (e != cudaSuccess) return e;
+  if (occ < 1) return cudaErrorInvalidConfiguration;
+  if (occ > OCC) occ = OCC;
+  const int64_t tiles = ((a.N < a.batch ? a.N : a.batch) + T - 1) / T;
+  // one block per SM at least takes part in the parameters' update, tiles or not; more only for their own tiles
+  int grid = sms * occ;
+  if (tiles < grid) grid = (int)(tiles > sms ? tiles : sms);
+  void *args[] = {&a};
+  return cudaLaunchCooperativeKernel((const void *)filter_train_kernel<S, T, LM, TH, OCC>, dim3(grid), dim3(TH), args, smem, st);
 }
 
 }  // namespace
 
-size_t filter_grad_smem(int s, int L) { return sizeof(float) * (size_t)(L * s * (s + 1) + L * s + (L + 2) * TB * (s + 1)); }
-constexpr size_t WG_SMEM = sizeof(float) * (32 * WG_ROW + 3 * WG_WARPS * 32 + WG_WARPS * (2 * 1024 + 64));
+cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, bool pack) {
+  PackArgs a = {};
+  for (int k = 0; k < n_layers; ++k) { a.w[k] = w[k]; a.b[k] = b[k]; }
+  a.theta = theta; a.s = s; a.n_layers = n_layers;
+  filter_pack_kernel<<<(n_layers * (s * s + s) + 255) / 256, 256, 0, st>>>(a, pack ? 1 : 0, status);
+  return cudaGetLastError();
+}
 
-cudaError_t launch_filter_update(cudaStream_t st, const float *C, const uint8_t *Y, int64_t n0, int64_t n, int s, int n_layers,
-                                 float *theta, float *m, float *v, float *gpart, int grid, const FilterTrainHyper &h,
-                                 double bc1, double bc2, float *loss_out) {
-  if (n_layers < 1 || n_layers > MAX_LAYERS || s < 1 || s > MAX_S) return cudaErrorInvalidValue;
-  GradArgs g{C, Y, n0, n, s, n_layers, theta, gpart};
-  int blocks;
-  cudaError_t e;
-  if (s <= 32 && n_layers == 2) {
-    static bool attr_w = false;
-    if (!attr_w) {
-      e = cudaFuncSetAttribute(filter_grad_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WG_SMEM);
-      if (e != cudaSuccess) return e;
-      attr_w = true;
-    }
-    const int64_t want = (n + WG_WARPS - 1) / WG_WARPS;
-    blocks = (int)(want < grid ? want : grid);
-    e = launch_kernel(filter_grad_warp_kernel, dim3(blocks), dim3(WG_WARPS * 32), WG_SMEM, st, g);
-  } else {
-    static bool attr = false;
-    if (!attr) {
-      e = cudaFuncSetAttribute(filter_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)filter_grad_smem(MAX_S, MAX_LAYERS));
-      if (e != cudaSuccess) return e;
-      attr = true;
-    }
-    const int64_t n_tiles = (n + TB - 1) / TB;
-    blocks = (int)(n_tiles < grid ? n_tiles : grid);
-    e = launch_kernel(filter_grad_kernel, dim3(blocks), dim3(GRAD_THREADS), filter_grad_smem(s, n_layers), st, g);
+int filter_train_max_rows(int64_t batch, int sms) { return (int)(ceil_div64(batch, 16) < 3 * sms ? ceil_div64(batch, 16) : 3 * sms); }
+
+cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms) {
+  if (f.n_layers < 1 || f.n_layers > MAX_LAYERS || f.s < 1 || f.s > MAX_S) return cudaErrorInvalidValue;
+  TrainArgs a;
+  a.C = f.C; a.Y = f.Y; a.N = f.N; a.batch = f.batch; a.u0 = u0; a.u1 = u1;
+  a.per_epoch = (int)((f.N + f.batch - 1) / f.batch);
+  a.s = f.s; a.n_layers = f.n_layers; a.P = f.n_layers * (f.s * f.s + f.s);
+  a.theta = f.theta; a.m = f.m; a.v = f.v; a.gpart = f.gpart; a.losses = f.losses;
+  a.lr = f.h.lr; a.beta1 = f.h.beta1; a.beta2 = f.h.beta2; a.eps = f.h.eps; a.weight_decay = f.h.weight_decay;
+  a.p1 = p1; a.p2 = p2; a.bar = f.bar; a.status = f.status;
+  const int64_t nb = f.N < f.batch ? f.N : f.batch;
+  // Large batches: tiles of 64 samples, 4 x 4 outputs per thread.  With fewer than one such tile for every SM smaller tiles
+  // spread the batch over more blocks (1,024 samples of 64, four layers: tiles of 16 take 19.5 k cycles, of 32 30 k; 84,480
+  // of 32: 128 threads with 4 x 4 outputs 56 k, 256 threads with 2 x 4 65 k).
+  const bool small = nb < (int64_t)(f.s <= 32 ? 64 : 32) * sms;
+  if (f.s <= 32) {
+    if (f.n_layers <= 2) return small ? launch_train<32, 32, 2, 256, 2>(st, a, sms) : launch_train<32, 64, 2, 128, 3>(st, a, sms);
+    return small ? launch_train<32, 32, 4, 256, 1>(st, a, sms) : launch_train<32, 64, 4, 128, 2>(st, a, sms);
   }
-  if (e != cudaSuccess) return e;
-  AdamArgs a{};
-  a.gpart = gpart; a.n_blocks = blocks; a.P = n_layers * (s * s + s);
-  a.inv_count = (float)(1.0 / ((double)n * s));
-  a.lr = h.lr; a.beta1 = h.beta1; a.beta2 = h.beta2; a.eps = h.eps; a.weight_decay = h.weight_decay;
-  a.bc1 = (float)bc1; a.bc2 = (float)bc2;
-  a.theta = theta; a.m = m; a.v = v; a.loss_out = loss_out;
-  return launch_kernel(filter_adamw_kernel, dim3((a.P + 1 + ADAM_THREADS - 1) / ADAM_THREADS), dim3(ADAM_THREADS), 0, st, a);
+  if (f.n_layers <= 2) return small ? launch_train<64, 16, 2, 256, 2>(st, a, sms) : launch_train<64, 64, 2, 256, 1>(st, a, sms);
+  return small ? launch_train<64, 16, 4, 256, 1>(st, a, sms) : launch_train<64, 64, 4, 256, 1>(st, a, sms);
 }
 
 }  // namespace l2pd

@@ -147,3 +147,24 @@ def test_depth_variant_training_matches_the_oracle(depth, s, n, batch):
     with pytest.raises(b_.L2pdError) as e:
         b_.filter_train_layers(layers0 * 5, C, Y, 1)          # more than four layers
     assert e.value.status == -1
+
+
+@pytest.mark.parametrize("s,n,depth,batch", [
+    (1, 1, 1, 0), (31, 31, 2, 0), (32, 33, 1, 0), (33, 65, 2, 64),          # one position; edges of 32-sample tiles and of the padding to 32 / 64
+    (32, 64 * 148 - 1, 2, 0), (32, 64 * 148 + 65, 2, 0),                     # either side of the step from tiles of 32 to tiles of 64
+    (64, 64 * 148 + 1, 4, 0), (40, 9600, 3, 9500), (32, 20000, 4, 0)])       # the deepest filters on large tiles, a ragged last batch
+def test_training_at_the_edges_of_its_tiles(s, n, depth, batch):
+    """Parameters after 3 epochs and the losses against the oracle.  An update moves a parameter by at most about lr
+    = 1e-3; where a gradient component sits at fp32 rounding level Adam can take either sign, 2 lr per update apart, so
+    single parameters may differ by 2 lr x updates <= 1.2e-2; all others agree to 1e-5 (fp32 sums of n terms)."""
+    C, Y = _data(s, n, seed=7 * s + n)
+    rng = np.random.default_rng(5)
+    layers = [(np.eye(s) + rng.normal(size=(s, s)) * 0.5 / np.sqrt(s), rng.normal(size=s) * 0.02) for _ in range(depth)]
+    layers = [(w.astype(np.float32), b.astype(np.float32)) for w, b in layers]
+    want, want_losses = orc.train_filter_layers(layers, C.astype(np.float64), Y.astype(np.float64), 3, lr=1e-3, batch_size=batch)
+    got, losses = _b().filter_train_layers(layers, C, Y, 3, lr=1e-3, batch_size=batch)
+    assert np.abs(losses - want_losses).max() < 1e-5
+    for (gw, gb), (ww, wb) in zip(got, want):
+        d = np.concatenate([np.abs(gw - ww).ravel(), np.abs(gb - wb).ravel()])
+        assert d.max() <= 2e-3 * len(losses) + 1e-6
+        assert np.mean(d > 1e-5) <= 0.01 + 1.0 / d.size
