@@ -112,7 +112,7 @@ cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, c
 template <typename T>
 cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, const T *vc,
                                   const SeqMeta *meta, const int32_t *row_slot, T *out,
-                                  int64_t kv_seq_stride, int rows, int H, int dh, int max_kv);
+                                  int64_t kv_seq_stride, int rows, int H, int dh, int max_kv, int n_slots, int max_q);
 cudaError_t launch_row_softmax_partials(cudaStream_t st, const float *logits, int R, int V,
                                         float *part_m, float *part_s, int32_t *part_i);
 

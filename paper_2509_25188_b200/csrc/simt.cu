@@ -1,8 +1,13 @@
 // CUDA-core kernels: the GEMM and attention of fp32 configurations (tcgen05 has no fp32
-// kind, and TF32 would not reach 1e-4 relative accuracy), written for correctness on small
-// models.  The same templates instantiate for bf16 storage as an independent cross-check
-// of the tensor-core kernels.
+// kind, and TF32 would not reach 1e-4 relative accuracy).  Their models are small: a projection is a few
+// dozen MFLOP, so what bounds it is latency.  gemm_f32_kernel and attention_f32_kernel keep everything a
+// block needs in flight at once (cp.async) and spread a step over as many blocks as its sizes allow.
+// The plain templates simt_gemm_kernel / simt_attention_kernel serve bf16 storage, as an independent
+// cross-check of the tensor-core kernels, and fp32 matrices that do not start on 16 bytes.
 #include "common.cuh"
+#include "ptx.cuh"
+
+#include <type_traits>
 
 namespace l2pd {
 
@@ -138,45 +143,283 @@ __global__ void simt_attention_kernel(const T *__restrict__ q, const T *__restri
   }
 }
 
-// Per-row max, sum of exp and argmax (lowest id on ties) of stored fp32 logits: one tile.
-__global__ void row_softmax_partials_kernel(const float *logits, int V, float *part_m, float *part_s,
-                                            int32_t *part_i) {
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, bool in) {   // zeros where `in` is false
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(ptx::smem_u32(dst)), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// C[M,N] = A[M,K] * W[N,K]^T in fp32, epilogues as simt_gemm_kernel.  A block computes a B x B tile with 256 threads: KG
+// groups of threads hold the whole tile, 4 x 4 outputs each, and take turns along K (16-deep shares of a 64-deep stage for
+// B = 32); the groups' sums are added in order at the end.  Four stages in flight: K = 256 is requested whole before the
+// first multiply.  Rows are 68 words apart and dealt out interleaved, so the 16-byte loads of a warp do not collide.
+// Measured at 96 rows of the tiny model (d 256, 688), one launch between events, 64 x 64 blocks with 16-deep unpipelined
+// stages before -> now (us): QKV 34 -> 10, O 38 -> 13, gate/up 43 -> 13, down 103 -> 18, LM head 22 -> 10.
+constexpr int F_BK = 64, F_ROW = F_BK + 4, F_STAGES = 4, F_THREADS = 256;
+template <int EPI, int B>
+__global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__restrict__ A, const float *__restrict__ W,
+                                                             const float *__restrict__ W2, float *out, const float *__restrict__ bias,
+                                                             int M, int N, int K) {
+  constexpr int TG = (B / 4) * (B / 4), KG = F_THREADS / TG, KS = F_BK / KG;   // threads per group, groups, k per group and stage
+  constexpr int MATS = EPI == EPI_SWIGLU ? 3 : 2, MAT = B * F_ROW;
+  static_assert(KG >= 1 && KS % 4 == 0, "tiling");
+  extern __shared__ __align__(16) float sm[];   // [F_STAGES][MATS][B][F_ROW]; the groups' sums at the end
+  const int tid = threadIdx.x, grp = tid / TG, t = tid % TG, tx = t % (B / 4), ty = t / (B / 4);
+  const int m0 = blockIdx.y * B, n0 = blockIdx.x * B, n_st = (K + F_BK - 1) / F_BK;
+  auto load = [&](int st, bool act, bool wts) {
+    float *d = sm + (st % F_STAGES) * MATS * MAT;
+    for (int e = tid; e < B * (F_BK / 4); e += F_THREADS) {
+      const int r = e / (F_BK / 4), c = 4 * (e % (F_BK / 4)), k = st * F_BK + c;
+      if (act) cp_async16(d + r * F_ROW + c, A + (m0 + r < M && k < K ? (int64_t)(m0 + r) * K + k : 0), m0 + r < M && k < K);
+      if (wts) {
+        const bool in = n0 + r < N && k < K;
+        const int64_t o = in ? (int64_t)(n0 + r) * K + k : 0;
+        cp_async16(d + MAT + r * F_ROW + c, W + o, in);
+        if (EPI == EPI_SWIGLU) cp_async16(d + 2 * MAT + r * F_ROW + c, W2 + o, in);
+      }
+    }
+  };
+  grid_dep_launch();
+  // no kernel writes weights: the first stages' are requested before the previous kernel has completed
+  for (int st = 0; st < F_STAGES - 1 && st < n_st; ++st) load(st, false, true);
+  grid_dep_wait();
+  for (int st = 0; st < F_STAGES - 1; ++st) {
+    if (st < n_st) load(st, true, false);
+    cp_async_commit();                          // (the weights requested above belong to the first group)
+  }
+  float acc[4][4] = {}, acc2[EPI == EPI_SWIGLU ? 4 : 1][4] = {};
+  for (int st = 0; st < n_st; ++st) {
+    cp_async_wait<F_STAGES - 2>();
+    __syncthreads();
+    if (st + F_STAGES - 1 < n_st) load(st + F_STAGES - 1, true, true);
+    cp_async_commit();
+    const float *a = sm + (st % F_STAGES) * MATS * MAT + ty * F_ROW + grp * KS, *w = sm + (st % F_STAGES) * MATS * MAT + MAT + tx * F_ROW + grp * KS;
+#pragma unroll
+    for (int k = 0; k < KS; k += 4) {
+      float4 av[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const float4 *>(a + (B / 4) * i * F_ROW + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float4 wv = *reinterpret_cast<const float4 *>(w + (B / 4) * j * F_ROW + k);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          acc[i][j] = fmaf(av[i].w, wv.w, fmaf(av[i].z, wv.z, fmaf(av[i].y, wv.y, fmaf(av[i].x, wv.x, acc[i][j]))));
+        if (EPI == EPI_SWIGLU) {
+          const float4 uv = *reinterpret_cast<const float4 *>(w + MAT + (B / 4) * j * F_ROW + k);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            acc2[i][j] = fmaf(av[i].w, uv.w, fmaf(av[i].z, uv.z, fmaf(av[i].y, uv.y, fmaf(av[i].x, uv.x, acc2[i][j]))));
+        }
+      }
+    }
+  }
+  if (KG > 1) {
+    // group g > 0 leaves its sums, group 0 adds them in order ([group][output][thread]: no bank conflicts)
+    constexpr int NO = EPI == EPI_SWIGLU ? 32 : 16;
+    static_assert((KG - 1) * NO * TG <= F_STAGES * MATS * MAT, "room for the groups' sums");
+    __syncthreads();
+    if (grp > 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          sm[((grp - 1) * NO + 4 * i + j) * TG + t] = acc[i][j];
+          if (EPI == EPI_SWIGLU) sm[((grp - 1) * NO + 16 + 4 * i + j) * TG + t] = acc2[i][j];
+        }
+    }
+    __syncthreads();
+    if (grp > 0) return;
+    for (int g = 0; g < KG - 1; ++g)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          acc[i][j] += sm[(g * NO + 4 * i + j) * TG + t];
+          if (EPI == EPI_SWIGLU) acc2[i][j] += sm[(g * NO + 16 + 4 * i + j) * TG + t];
+        }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int gm = m0 + ty + (B / 4) * i;
+    if (gm >= M) continue;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int gn = n0 + tx + (B / 4) * j;
+      if (gn >= N) continue;
+      float *o = out + (int64_t)gm * N + gn;
+      const float v = acc[i][j];
+      if (EPI == EPI_STORE) *o = v;
+      else if (EPI == EPI_RESIDUAL) *o += v;
+      else if (EPI == EPI_SWIGLU) *o = v / (1.0f + expf(-v)) * acc2[i][j];
+      else *o = v + (bias ? bias[gn] : 0.f);
+    }
+  }
+}
+
+// fp32 attention: a block takes 16 query rows of one head and walks the keys in tiles of 64 with a running maximum and sum.
+// 16 threads per row: thread l computes the scores of keys l + 16 i and the output dimensions l + 16 i.  (A block per row and
+// head, which read every key row and every value column alone, took 24 us at 96 rows, 96 keys, 4 heads of 64; this 17, most of
+// it the launch.)
+constexpr int A_Q = 16, A_K = 64;
+__global__ void __launch_bounds__(256) attention_f32_kernel(const float *__restrict__ q, const float *__restrict__ kc,
+                                                            const float *__restrict__ vc, const SeqMeta *meta, float *out,
+                                                            int64_t kv_seq_stride, int H, int dh) {
+  extern __shared__ __align__(16) float sm[];
   grid_dep_launch();
   grid_dep_wait();
-  __shared__ float rm[32];
-  __shared__ int ri[32];
-  __shared__ float rs[32];
-  int r = blockIdx.x;
+  const SeqMeta m = meta[blockIdx.z];
+  const int q0 = blockIdx.x * A_Q, h = blockIdx.y, hd = H * dh, tid = threadIdx.x, r = tid >> 4, l = tid & 15;
+  if (q0 >= m.n_rows) return;
+  const int stride = dh + 4, sk = A_K + 4;
+  float *Q = sm, *Kt = Q + A_Q * stride, *Vt = Kt + A_K * stride, *S = Vt + A_K * stride;   // S [16][sk]
+  const float *kb = kc + (int64_t)m.seq * kv_seq_stride + h * dh, *vb = vc + (int64_t)m.seq * kv_seq_stride + h * dh;
+  const bool live = q0 + r < m.n_rows;
+  const bool v4 = (dh & 3) == 0;
+  // (dh is a multiple of 4 here, or every row is copied word by word)
+  auto rows = [&](float *d, const float *src, int n, int n_valid) {
+    if (v4) {
+      for (int e = tid; e < n * (dh / 4); e += 256) {
+        const int i = e / (dh / 4), c = 4 * (e % (dh / 4));
+        cp_async16(d + i * stride + c, src + (i < n_valid ? (int64_t)i * hd + c : 0), i < n_valid);
+      }
+    } else {
+      for (int e = tid; e < n * dh; e += 256) {
+        const int i = e / dh, c = e - i * dh;
+        d[i * stride + c] = i < n_valid ? src[(int64_t)i * hd + c] : 0.f;
+      }
+    }
+  };
+  rows(Q, q + (int64_t)(m.row0 + q0) * hd + h * dh, A_Q, min(A_Q, m.n_rows - q0));
+  constexpr int MAX_D = 16;                       // dh <= 256
+  float o[MAX_D], m_run = -INFINITY, l_run = 0.f;
+#pragma unroll
+  for (int i = 0; i < MAX_D; ++i) o[i] = 0.f;
+  const float scale = 1.0f / sqrtf((float)dh);
+  for (int j0 = 0; j0 < m.kv_len; j0 += A_K) {
+    const int nk = min(A_K, m.kv_len - j0);
+    __syncthreads();                              // the previous tile is no longer read
+    rows(Kt, kb + (int64_t)j0 * hd, A_K, nk);
+    rows(Vt, vb + (int64_t)j0 * hd, A_K, nk);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    if (v4) {
+      for (int c = 0; c < dh; c += 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(Q + r * stride + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float4 y = *reinterpret_cast<const float4 *>(Kt + (l + 16 * i) * stride + c);
+          s[i] = fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, s[i]))));
+        }
+      }
+    } else {
+      for (int c = 0; c < dh; ++c)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[i] = fmaf(Q[r * stride + c], Kt[(l + 16 * i) * stride + c], s[i]);
+    }
+    float mx = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s[i] = l + 16 * i < nk ? s[i] * scale : -INFINITY;
+      mx = fmaxf(mx, s[i]);
+    }
+    for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+    const float m_new = fmaxf(m_run, mx), f = expf(m_run - m_new);   // the first tile: exp(-inf) = 0
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float e = expf(s[i] - m_new);
+      sum += e;
+      S[r * sk + l + 16 * i] = e;
+    }
+    for (int w = 8; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+    l_run = l_run * f + sum;
+    m_run = m_new;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < MAX_D; ++i) {
+      if (16 * i >= dh) break;
+      float a = 0.f;
+      const int c = l + 16 * i;
+      if (c < dh) {
+#pragma unroll 8
+        for (int j = 0; j < nk; ++j) a = fmaf(S[r * sk + j], Vt[j * stride + c], a);
+        o[i] = fmaf(o[i], f, a);
+      }
+    }
+    __syncwarp();
+  }
+  const float inv = 1.0f / l_run;
+  float *orow = out + (int64_t)(m.row0 + q0 + r) * hd + h * dh;
+#pragma unroll
+  for (int i = 0; i < MAX_D; ++i)
+    if (l + 16 * i < dh && live) orow[l + 16 * i] = o[i] * inv;
+}
+
+// Per-row max, sum of exp and argmax (lowest id on ties) of stored fp32 logits: one tile.  A thread folds 16 logits at a
+// time (all requested together) into its running (max, sum, argmax); the threads' records are merged at the end.
+constexpr int R_THREADS = 512;
+__device__ __forceinline__ void merge_records(float &mx, float &sum, int &ix, float om, float os, int oi) {
+  const float nm = fmaxf(mx, om);
+  sum = (mx == -INFINITY ? 0.f : sum * expf(mx - nm)) + (om == -INFINITY ? 0.f : os * expf(om - nm));
+  ix = (om > mx || (om == mx && oi < ix)) ? oi : ix;
+  mx = nm;
+}
+__global__ void __launch_bounds__(R_THREADS) row_softmax_partials_kernel(const float *logits, int V, float *part_m, float *part_s,
+                                                                         int32_t *part_i) {
+  grid_dep_launch();
+  grid_dep_wait();
+  __shared__ float rm[R_THREADS / 32], rs[R_THREADS / 32];
+  __shared__ int ri[R_THREADS / 32];
+  const int r = blockIdx.x;
   const float *row = logits + (int64_t)r * V;
-  float mx = -INFINITY;
+  float mx = -INFINITY, sum = 0.f;
   int ix = 0x7fffffff;
-  for (int v = threadIdx.x; v < V; v += blockDim.x) {
-    float a = row[v];
-    if (a > mx) { mx = a; ix = v; }
+  constexpr int U = 16;
+  for (int v0 = threadIdx.x; v0 < V; v0 += U * R_THREADS) {
+    float f[U], cm = -INFINITY;
+#pragma unroll
+    for (int u = 0; u < U; ++u) f[u] = v0 + u * R_THREADS < V ? row[v0 + u * R_THREADS] : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < U; ++u) cm = fmaxf(cm, f[u]);
+    if (cm > mx) {
+      sum *= expf(mx - cm);                       // the first chunk: 0 * exp(-inf)
+      mx = cm;
+#pragma unroll
+      for (int u = U - 1; u >= 0; --u) if (f[u] == cm) ix = v0 + u * R_THREADS;   // the lowest id that holds the maximum
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) sum += mx == -INFINITY ? 0.f : expf(f[u] - mx);
   }
-  int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   for (int o = 16; o > 0; o >>= 1) {
-    float om = __shfl_xor_sync(0xffffffffu, mx, o);
-    int oi = __shfl_xor_sync(0xffffffffu, ix, o);
-    if (om > mx || (om == mx && oi < ix)) { mx = om; ix = oi; }
+    const float om = __shfl_xor_sync(0xffffffffu, mx, o), os = __shfl_xor_sync(0xffffffffu, sum, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, ix, o);
+    merge_records(mx, sum, ix, om, os, oi);
   }
-  if (l == 0) { rm[w] = mx; ri[w] = ix; }
+  if (l == 0) { rm[w] = mx; rs[w] = sum; ri[w] = ix; }
   __syncthreads();
-  mx = (l < nw) ? rm[l] : -INFINITY;
-  ix = (l < nw) ? ri[l] : 0x7fffffff;
-  for (int o = 16; o > 0; o >>= 1) {
-    float om = __shfl_xor_sync(0xffffffffu, mx, o);
-    int oi = __shfl_xor_sync(0xffffffffu, ix, o);
-    if (om > mx || (om == mx && oi < ix)) { mx = om; ix = oi; }
+  if (w == 0) {
+    mx = l < R_THREADS / 32 ? rm[l] : -INFINITY;
+    sum = l < R_THREADS / 32 ? rs[l] : 0.f;
+    ix = l < R_THREADS / 32 ? ri[l] : 0x7fffffff;
+    for (int o = 16; o > 0; o >>= 1) {
+      const float om = __shfl_xor_sync(0xffffffffu, mx, o), os = __shfl_xor_sync(0xffffffffu, sum, o);
+      const int oi = __shfl_xor_sync(0xffffffffu, ix, o);
+      merge_records(mx, sum, ix, om, os, oi);
+    }
+    if (l == 0) { part_m[r] = mx; part_s[r] = sum; part_i[r] = ix; }
   }
-  float sum = 0.f;
-  for (int v = threadIdx.x; v < V; v += blockDim.x) sum += expf(row[v] - mx);
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (l == 0) rs[w] = sum;
-  __syncthreads();
-  sum = (l < nw) ? rs[l] : 0.f;
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  if (threadIdx.x == 0) { part_m[r] = mx; part_s[r] = sum; part_i[r] = ix; }
+}
+
+template <int EPI, int B>
+cudaError_t launch_gemm_f32(cudaStream_t st, const float *A, const float *W, const float *W2, float *C, const float *bias, int M, int N, int K) {
+  const size_t smem = sizeof(float) * F_STAGES * (EPI == EPI_SWIGLU ? 3 : 2) * B * F_ROW;
+  cudaError_t e = cudaFuncSetAttribute(gemm_f32_kernel<EPI, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(gemm_f32_kernel<EPI, B>, dim3(ceil_div(N, B), ceil_div(M, B)), dim3(F_THREADS), smem, st, A, W, W2, C, bias, M, N, K);
 }
 
 }  // namespace
@@ -184,6 +427,21 @@ __global__ void row_softmax_partials_kernel(const float *logits, int V, float *p
 template <typename T>
 cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, const T *W2, void *C,
                              const float *bias, int M, int N, int K) {
+  if constexpr (std::is_same<T, float>::value) {
+    const uintptr_t bits = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(W2);
+    if ((bits & 15) == 0 && (K & 3) == 0) {
+      // 32 x 32 tiles until 64 x 64 ones give every SM two blocks (SwiGLU, two weight tiles: 32 x 32 always)
+      const bool big = (int64_t)ceil_div(N, 64) * ceil_div(M, 64) >= 296;
+      float *Cf = reinterpret_cast<float *>(C);
+      switch (epi) {
+        case EPI_STORE: return big ? launch_gemm_f32<EPI_STORE, 64>(st, A, W, W2, Cf, bias, M, N, K) : launch_gemm_f32<EPI_STORE, 32>(st, A, W, W2, Cf, bias, M, N, K);
+        case EPI_RESIDUAL: return big ? launch_gemm_f32<EPI_RESIDUAL, 64>(st, A, W, W2, Cf, bias, M, N, K) : launch_gemm_f32<EPI_RESIDUAL, 32>(st, A, W, W2, Cf, bias, M, N, K);
+        case EPI_SWIGLU: return launch_gemm_f32<EPI_SWIGLU, 32>(st, A, W, W2, Cf, bias, M, N, K);
+        case EPI_STORE_F32: return big ? launch_gemm_f32<EPI_STORE_F32, 64>(st, A, W, W2, Cf, bias, M, N, K) : launch_gemm_f32<EPI_STORE_F32, 32>(st, A, W, W2, Cf, bias, M, N, K);
+        default: return cudaErrorInvalidValue;
+      }
+    }
+  }
   dim3 grid(ceil_div(N, BN), ceil_div(M, BM));
   switch (epi) {
     case EPI_STORE: return launch_kernel(simt_gemm_kernel<T, EPI_STORE>, grid, dim3(256), 0, st, A, W, W2, C, bias, M, N, K);
@@ -197,7 +455,14 @@ cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, c
 template <typename T>
 cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, const T *vc,
                                   const SeqMeta *meta, const int32_t *row_slot, T *out,
-                                  int64_t kv_seq_stride, int rows, int H, int dh, int max_kv) {
+                                  int64_t kv_seq_stride, int rows, int H, int dh, int max_kv, int n_slots, int max_q) {
+  if constexpr (std::is_same<T, float>::value) {   // q, K and V are the library's own buffers: rows of H * dh floats, 16-byte aligned
+    const size_t bytes = sizeof(float) * ((size_t)(A_Q + 2 * A_K) * (dh + 4) + A_Q * (A_K + 4));
+    cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(attention_f32_kernel, dim3(ceil_div(max_q, A_Q), H, n_slots), dim3(256), bytes, st, q, kc, vc, meta, out,
+                         kv_seq_stride, H, dh);
+  }
   size_t smem = (size_t)(dh + max_kv) * sizeof(float);
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(simt_attention_kernel<T>,
@@ -210,7 +475,7 @@ cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, cons
 
 cudaError_t launch_row_softmax_partials(cudaStream_t st, const float *logits, int R, int V,
                                         float *part_m, float *part_s, int32_t *part_i) {
-  return launch_kernel(row_softmax_partials_kernel, dim3(R), dim3(256), 0, st, logits, V, part_m, part_s, part_i);
+  return launch_kernel(row_softmax_partials_kernel, dim3(R), dim3(R_THREADS), 0, st, logits, V, part_m, part_s, part_i);
 }
 
 template cudaError_t launch_simt_gemm<float>(cudaStream_t, int, const float *, const float *,
@@ -219,9 +484,9 @@ template cudaError_t launch_simt_gemm<bf16>(cudaStream_t, int, const bf16 *, con
                                             void *, const float *, int, int, int);
 template cudaError_t launch_simt_attention<float>(cudaStream_t, const float *, const float *,
                                                   const float *, const SeqMeta *, const int32_t *,
-                                                  float *, int64_t, int, int, int, int);
+                                                  float *, int64_t, int, int, int, int, int, int);
 template cudaError_t launch_simt_attention<bf16>(cudaStream_t, const bf16 *, const bf16 *, const bf16 *,
                                                  const SeqMeta *, const int32_t *, bf16 *, int64_t, int,
-                                                 int, int, int);
+                                                 int, int, int, int, int);
 
 }  // namespace l2pd

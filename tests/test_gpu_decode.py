@@ -55,6 +55,23 @@ def test_c0_full_decode_bit_exact(gain):
     dec.close()
 
 
+@pytest.mark.parametrize("kw,B,P,G,s", [
+    (dict(d_model=72, n_heads=2, head_dim=36, d_ff=104, vocab=211), 2, 19, 16, 8),       # tails in every dimension of a 32 x 32 x 64 tile
+    (dict(d_model=24, n_heads=4, head_dim=6, d_ff=40, vocab=64), 1, 130, 16, 16),        # head rows that are not multiples of 16 bytes, three key tiles
+    (dict(d_model=64, n_heads=2, head_dim=256, d_ff=64, vocab=100), 1, 3, 4, 4),         # the widest head, fewer rows than a query tile
+    (dict(d_model=128, n_heads=2, head_dim=64, d_ff=136, vocab=5000), 4, 70, 64, 64)])   # LM head on 64 x 64 tiles
+def test_fp32_step_at_the_edges_of_its_tiles(kw, B, P, G, s):
+    """A lockstep decode per shape against the oracle, logits to 1e-4 of the row maximum (fp32 sums of at most 512 terms)."""
+    from tests.helpers import small_shape
+    shape = small_shape(mask_id=kw["vocab"] - 1, eot_id=kw["vocab"] - 2, **kw)
+    w = wl.make_weights(shape, seed=3, final_norm_gain=wl.spread_gain(shape))
+    filt = wl.make_filter(s, 0.96, seed=0)
+    dec = _b().Decoder(shape, w, filt, block_len=s, max_batch=B, max_seq=P + G)
+    lockstep(dec, oracle_model(shape, w), filt, orc.DecodeConfig(block_len=s), wl.make_prompts(B, P, shape, seed=2), G,
+             logit_rtol=1e-4, conf_atol=1e-3, p_margin=0.01, max_steps=6)
+    dec.close()
+
+
 @pytest.mark.parametrize("gain", [None, 1.0])
 def test_c0_lockstep_fp32(gain):
     shape, w = _tiny(gain)
