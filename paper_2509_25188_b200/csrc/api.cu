@@ -442,7 +442,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     for (int l = 0; l < f.n_layers; ++l) {
       if (c->fuse_rope) {
         CKLK(L2PD_K_ATTENTION, launch_attention_tc(s, c->tq_packed, c->tk_packed, c->tv_packed, c->d_meta, (bf16 *)att, hd, 0, 0, 1,
-                                  n_slots, max_q_rows, H, c->d_status));
+                                  n_slots, max_q_rows, H, c->num_sms, c->d_status));
       } else {
         // key/value-cache configurations: rotation + scatter into the store, then attention over the store
         T *kc = (T *)c->kc + (f.kv_cache_mode ? (int64_t)l * c->kv_layer_stride : 0);
@@ -450,7 +450,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
         CKLK(L2PD_K_ROPE, launch_rope_scatter<T>(s, qkv, c->d_meta, c->d_row_slot, c->cs_table, q, kc, vc, c->kv_seq_stride, T_rows, H, dh));
         const int kv_row_base = f.kv_cache_mode ? l * f.max_batch * f.max_seq : 0;
         CKLK(L2PD_K_ATTENTION, launch_attention_tc(s, c->ta_q, c->t_kstore, c->t_vstore, c->d_meta, (bf16 *)att, hd, f.max_seq,
-                                  kv_row_base, 0, n_slots, max_q_rows, H, c->d_status));
+                                  kv_row_base, 0, n_slots, max_q_rows, H, c->num_sms, c->d_status));
       }
       l2pd_status r = launch_chain(l + 1);
       if (r) return r;
@@ -470,11 +470,11 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
       CKLK(L2PD_K_ROPE, launch_rope_scatter<T>(s, qkv, c->d_meta, c->d_row_slot, c->cs_table, q, kc, vc, c->kv_seq_stride, T_rows, H, dh));
     if (tc && c->fuse_rope) {
       CKLK(L2PD_K_ATTENTION, launch_attention_tc(s, c->tq_packed, c->tk_packed, c->tv_packed, c->d_meta, (bf16 *)att, hd, 0, 0, 1,
-                                n_slots, max_q_rows, H, c->d_status));
+                                n_slots, max_q_rows, H, c->num_sms, c->d_status));
     } else if (tc && c->attn_tc) {
       const int kv_row_base = f.kv_cache_mode ? l * f.max_batch * f.max_seq : 0;
       CKLK(L2PD_K_ATTENTION, launch_attention_tc(s, c->ta_q, c->t_kstore, c->t_vstore, c->d_meta, (bf16 *)att, hd, f.max_seq,
-                                kv_row_base, 0, n_slots, max_q_rows, H, c->d_status));
+                                kv_row_base, 0, n_slots, max_q_rows, H, c->num_sms, c->d_status));
     } else if (tc) {
       CKLK(L2PD_K_ATTENTION, launch_attention_bf16(s, (const bf16 *)q, (const bf16 *)kc, (const bf16 *)vc, c->d_meta, (bf16 *)att, hd, hd,
                                 c->kv_seq_stride, hd, n_slots, max_q_rows, H, dh));
@@ -1271,7 +1271,9 @@ l2pd_status l2pd_attention_bf16(void *stream, const void *q, const void *k, cons
   if (q_stride < (int64_t)H * dh || kv_stride < (int64_t)H * dh || out_stride < (int64_t)H * dh) return L2PD_ERR_SHAPE;
   if (impl == 0 && attention_tc_supported(dh, q_stride, kv_stride, out_stride)) {
     int32_t *status = standalone_status();
-    if (!status) return L2PD_ERR_CUDA;
+    int dev = 0, sms = 0;
+    if (!status || cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return L2PD_ERR_CUDA;
     TmaDesc tq, tk, tv;
     l2pd_status r = make_tma_2d_bf16_strided(&tq, q, Tq, (int64_t)H * dh, q_stride, 128);
     if (r) return r;
@@ -1279,8 +1281,8 @@ l2pd_status l2pd_attention_bf16(void *stream, const void *q, const void *k, cons
     if (r) return r;
     r = make_tma_2d_bf16_strided(&tv, v, Tk, (int64_t)H * dh, kv_stride, 128);
     if (r) return r;
-    if (launch_attention_tc((cudaStream_t)stream, tq, tk, tv, nullptr, (bf16 *)out, out_stride, 0, 0, 0, Tk, Tq, H, status) !=
-        cudaSuccess)
+    if (launch_attention_tc((cudaStream_t)stream, tq, tk, tv, nullptr, (bf16 *)out, out_stride, 0, 0, 0, Tk, Tq, H, sms,
+                            status) != cudaSuccess)
       return L2PD_ERR_CUDA;
     return finish_standalone((cudaStream_t)stream, status, check);
   }

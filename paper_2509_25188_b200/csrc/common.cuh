@@ -254,6 +254,7 @@ cudaError_t launch_attention_bf16(cudaStream_t st, const bf16 *q, const bf16 *kc
 bool attention_tc_supported(int dh, int64_t q_stride, int64_t kv_row_stride, int64_t out_stride);
 cudaError_t launch_attention_tc(cudaStream_t st, const TmaDesc &tq, const TmaDesc &tk, const TmaDesc &tv,
                                 const SeqMeta *meta, bf16 *out, int64_t out_stride, int kv_rows_per_seq,
-                                int kv_row_base, int kv_packed, int n_slots, int max_q_rows, int H, int32_t *status);
+                                int kv_row_base, int kv_packed, int n_slots, int max_q_rows, int H, int num_sms,
+                                int32_t *status);
 
 }  // namespace l2pd

@@ -205,6 +205,23 @@ def test_attention_scores_that_grow_along_the_keys(impl):
     assert np.sqrt(((got - want) ** 2).mean()) < 6e-3
 
 
+@pytest.mark.parametrize("Tq,Tk,H", [(200, 40, 200), (128, 128, 149), (33, 129, 300), (129, 300, 100), (257, 769, 60)])
+def test_attention_with_several_tiles_per_block(Tq, Tk, H):
+    """More query tiles than SMs, so that a block runs one behind the other, with 1, 2, 3 and 7 key tiles: odd and even
+    numbers move the groups and score buffers against the tiles, and warps and last rows without queries come between."""
+    b = _b()
+    dh = 128
+    q = _bf16(8, 0, (Tq, H * dh), 1.0)
+    k = orc.widen(_bf16(8, 1, (Tk, H * dh), 1.0)) * (0.2 + np.arange(Tk)[:, None] / Tk)   # later keys score higher: rescaling
+    k = wl.f32_to_bf16_bits(k.astype(np.float32))
+    v = _bf16(8, 2, (Tk, H * dh), 1.0)
+    got = b.attention_bf16(b.to_device(q), b.to_device(k), b.to_device(v), H, dh).float().cpu().numpy()
+    want = orc.attention(orc.widen(q).reshape(Tq, H, dh), orc.widen(k).reshape(Tk, H, dh),
+                         orc.widen(v).reshape(Tk, H, dh)).reshape(Tq, H * dh)
+    # each weight and then the result is rounded to bf16, 2^-9 relative; the weights of a row sum to one
+    assert np.abs(got - want).max() < 1.02 * 2.0 ** -8 * np.abs(orc.widen(v)).max()
+
+
 def test_shape_errors_are_reported_not_launched():
     b = _b()
     A = b.to_device(_bf16(6, 0, (16, 64), 1.0))
