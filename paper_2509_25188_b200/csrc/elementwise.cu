@@ -113,57 +113,78 @@ __device__ __forceinline__ void store4(bf16 *p, float a, float b, float c, float
 // One block per row; rows up to 4 * 4 * blockDim floats stay in registers between the two passes.
 // n_part > 0: the row first takes in the partial sums of a K-split projection, slice after slice, and
 // the summed row is written back to x.
-// NPART is a compile-time count so that all loads of a row chunk are issued before the first addition.
-template <typename T, int NPART>
-__global__ void __launch_bounds__(256) rmsnorm_kernel(float *x, const float *gain, float eps, T *n, int d,
-                                                      const float *part, int64_t part_stride) {
+// Bound by the chain of latencies between two projections.  NPART is a compile-time count and a row's loads are issued before
+// its first store (which may alias them), the gain's before the wait for the kernel before: one trip to memory where five
+// followed one another.  ONE: at most a block to an SM, up to 80 registers; else 48 or 40, so that the blocks of an SM leave
+// the next projection the registers to start beside them (512 rows: with 88 it, and its first weights, started 7 us later).
+// From the previous kernel's end to the last store, slices to add: 125 rows 4.6 -> 3.1 us, 32 rows (beside the next weights'
+// stream) 5.0 -> 4.3, 512 rows 4.1 as before; a whole step of 306 rows at d = 1024, with the rotation below: 224 -> 212 us.
+template <typename T, int NPART, bool ONE>
+__global__ void __launch_bounds__(256, ONE ? 3 : NPART ? 5 : 6) rmsnorm_kernel(float *x, const float *gain, float eps, T *n, int d,
+                                                                              const float *part, int64_t part_stride) {
   grid_dep_launch();
-  grid_dep_wait();
   __shared__ float red[32];
   const int row = blockIdx.x;
   float4 *xr = reinterpret_cast<float4 *>(x + (int64_t)row * d);
+  const float4 *pr = reinterpret_cast<const float4 *>(part + (int64_t)row * d), *g4 = reinterpret_cast<const float4 *>(gain);
   const int d4 = d >> 2;
-  constexpr int CACHE = 4;
-  float4 v[CACHE];
-  float ss = 0.f;
-  auto fetch = [&](int i) {
-    float4 w = xr[i];
-    if (NPART > 0) {
-      float4 q[NPART > 0 ? NPART : 1];
-#pragma unroll
-      for (int s = 0; s < NPART; ++s) q[s] = reinterpret_cast<const float4 *>(part + s * part_stride + (int64_t)row * d)[i];
-#pragma unroll
-      for (int s = 0; s < NPART; ++s) { w.x += q[s].x; w.y += q[s].y; w.z += q[s].z; w.w += q[s].w; }
-      xr[i] = w;
-    }
-    return w;
-  };
+  const int64_t p4 = part_stride >> 2;
+  constexpr int CACHE = 4, NP = NPART > 0 ? NPART : 1;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 v[CACHE], g[ONE ? CACHE : 1], q[NP][CACHE];
 #pragma unroll
   for (int k = 0; k < CACHE; ++k) {
     const int i = threadIdx.x + k * blockDim.x;
-    v[k] = (i < d4) ? fetch(i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ONE) g[k] = i < d4 ? __ldg(g4 + i) : zero;
+    else if (i < d4) asm volatile("prefetch.global.L1 [%0];" ::"l"(g4 + i));
+  }
+  grid_dep_wait();
+#pragma unroll
+  for (int k = 0; k < CACHE; ++k) {
+    const int i = threadIdx.x + k * blockDim.x;
+    v[k] = i < d4 ? xr[i] : zero;
+#pragma unroll
+    for (int s = 0; s < NPART; ++s) q[s][k] = i < d4 ? pr[s * p4 + i] : zero;
+  }
+  float ss = 0.f;
+#pragma unroll
+  for (int k = 0; k < CACHE; ++k) {
+#pragma unroll
+    for (int s = 0; s < NPART; ++s) { v[k].x += q[s][k].x; v[k].y += q[s][k].y; v[k].z += q[s][k].z; v[k].w += q[s][k].w; }
     ss += v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z + v[k].w * v[k].w;
   }
+  if (NPART > 0) {
+#pragma unroll
+    for (int k = 0; k < CACHE; ++k) {
+      const int i = threadIdx.x + k * blockDim.x;
+      if (i < d4) xr[i] = v[k];
+    }
+  }
   for (int i = threadIdx.x + CACHE * blockDim.x; i < d4; i += blockDim.x) {
-    float4 w = fetch(i);
+    float4 w = xr[i];
+#pragma unroll
+    for (int s = 0; s < NPART; ++s) {
+      const float4 a = pr[s * p4 + i];
+      w.x += a.x; w.y += a.y; w.z += a.z; w.w += a.w;
+    }
+    if (NPART > 0) xr[i] = w;
     ss += w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
   }
   const float tot = block_sum(ss, red);
   const float inv = 1.0f / sqrtf(tot / (float)d + eps);
-  const float4 *g4 = reinterpret_cast<const float4 *>(gain);
   T *nr = n + (int64_t)row * d;
 #pragma unroll
   for (int k = 0; k < CACHE; ++k) {
     const int i = threadIdx.x + k * blockDim.x;
     if (i < d4) {
-      const float4 g = g4[i];
-      store4(nr + 4 * i, v[k].x * g.x * inv, v[k].y * g.y * inv, v[k].z * g.z * inv, v[k].w * g.w * inv);
+      const float4 a = ONE ? g[ONE ? k : 0] : __ldg(g4 + i);
+      store4(nr + 4 * i, v[k].x * a.x * inv, v[k].y * a.y * inv, v[k].z * a.z * inv, v[k].w * a.w * inv);
     }
   }
   for (int i = threadIdx.x + CACHE * blockDim.x; i < d4; i += blockDim.x) {
     const float4 w = xr[i];          // already summed and written back above, by this same thread
-    const float4 g = g4[i];
-    store4(nr + 4 * i, w.x * g.x * inv, w.y * g.y * inv, w.z * g.z * inv, w.w * g.w * inv);
+    const float4 a = g4[i];
+    store4(nr + 4 * i, w.x * a.x * inv, w.y * a.y * inv, w.z * a.z * inv, w.w * a.w * inv);
   }
 }
 
@@ -184,6 +205,9 @@ __global__ void __launch_bounds__(256) add_partials_kernel(float *x, const float
 // Rotates q and k (pair (i, i+dh/2) by the tabulated angle of the row's position) and writes
 // q to the packed query buffer and k, v to the key/value store at [sequence, position].
 // One work item = 8 consecutive pair indices of one head (16-byte accesses); needs dh % 16 == 0.
+// Few rows: bound by its chain of loads, row -> slot -> position -> angles; the row itself is loaded beside it, all of it
+// before the first store (which may alias it).  32 rows: 2.3 us from the previous kernel's end to the last store.
+// Many rows: bound by memory, 5.9 TB/s at 16384.
 template <typename T>
 __global__ void __launch_bounds__(256) rope_scatter_vec_kernel(const T *qkv, const SeqMeta *meta,
                                                                 const int32_t *row_slot, const float2 *cs_table,
@@ -192,40 +216,41 @@ __global__ void __launch_bounds__(256) rope_scatter_vec_kernel(const T *qkv, con
   grid_dep_launch();
   grid_dep_wait();
   const int row = blockIdx.x;
-  const SeqMeta m = meta[row_slot[row]];
-  const int pos = m.pos0 + (row - m.row0);
+  const int slot = row_slot[row];
   const int half = dh >> 1, hd = H * dh, per_head = half >> 3;
   const T *src = qkv + (int64_t)row * 3 * hd;
   T *qd = q + (int64_t)row * hd;
-  T *kd = kc + (int64_t)m.seq * kv_seq_stride + (int64_t)pos * hd;
-  T *vd = vc + (int64_t)m.seq * kv_seq_stride + (int64_t)pos * hd;
-  const float2 *cs = cs_table + (int64_t)pos * half;
   for (int item = threadIdx.x; item < H * per_head; item += blockDim.x) {
     const int h = item / per_head, c = item - h * per_head;
     const int a = h * dh + c * 8, b = a + half;
+    Vec8<T> q1, q2, k1, k2, v1, v2, y1, y2;
+    q1.load(src + a); q2.load(src + b);
+    k1.load(src + hd + a); k2.load(src + hd + b);
+    v1.load(src + 2 * hd + a); v2.load(src + 2 * hd + b);
+    const SeqMeta m = meta[slot];
+    const int pos = m.pos0 + (row - m.row0);
+    T *kd = kc + (int64_t)m.seq * kv_seq_stride + (int64_t)pos * hd;
+    T *vd = vc + (int64_t)m.seq * kv_seq_stride + (int64_t)pos * hd;
+    const float2 *cs = cs_table + (int64_t)pos * half;
     float2 t[8];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
       *reinterpret_cast<float4 *>(&t[2 * i]) = *reinterpret_cast<const float4 *>(&cs[c * 8 + 2 * i]);
-    Vec8<T> x1, x2, y1, y2;
-    x1.load(src + a); x2.load(src + b);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float u = x1.get(i), w = x2.get(i);
+      const float u = q1.get(i), w = q2.get(i);
       y1.set(i, u * t[i].x - w * t[i].y);
       y2.set(i, w * t[i].x + u * t[i].y);
     }
     y1.store(qd + a); y2.store(qd + b);
-    x1.load(src + hd + a); x2.load(src + hd + b);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const float u = x1.get(i), w = x2.get(i);
+      const float u = k1.get(i), w = k2.get(i);
       y1.set(i, u * t[i].x - w * t[i].y);
       y2.set(i, w * t[i].x + u * t[i].y);
     }
     y1.store(kd + a); y2.store(kd + b);
-    x1.load(src + 2 * hd + a); x2.load(src + 2 * hd + b);
-    x1.store(vd + a); x2.store(vd + b);
+    v1.store(vd + a); v2.store(vd + b);
   }
 }
 
@@ -393,10 +418,10 @@ template <typename T>
 cudaError_t launch_rmsnorm(cudaStream_t st, float *x, const float *gain, float eps, T *n,
                            int rows, int d, const float *part, int n_part, int64_t part_stride) {
   switch (n_part) {
-    case 0: return launch_kernel(rmsnorm_kernel<T, 0>, dim3(rows), dim3(256), 0, st, x, gain, eps, n, d, part, part_stride);
-    case 2: return launch_kernel(rmsnorm_kernel<T, 2>, dim3(rows), dim3(256), 0, st, x, gain, eps, n, d, part, part_stride);
-    case 3: return launch_kernel(rmsnorm_kernel<T, 3>, dim3(rows), dim3(256), 0, st, x, gain, eps, n, d, part, part_stride);
-    case 4: return launch_kernel(rmsnorm_kernel<T, 4>, dim3(rows), dim3(256), 0, st, x, gain, eps, n, d, part, part_stride);
+#define L2PD_NORM(NP) \
+    case NP: return launch_kernel(rows <= 128 ? rmsnorm_kernel<T, NP, true> : rmsnorm_kernel<T, NP, false>, dim3(rows), dim3(256), 0, st, x, gain, eps, n, d, part, part_stride);
+    L2PD_NORM(0) L2PD_NORM(2) L2PD_NORM(3) L2PD_NORM(4)
+#undef L2PD_NORM
     default: return cudaErrorInvalidValue;
   }
 }

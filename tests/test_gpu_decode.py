@@ -331,6 +331,18 @@ def test_bf16_small_model_lockstep(spread, kv_cache):
     dec.close()
 
 
+@pytest.mark.parametrize("d_model,P,kv_cache", [(512, 96, 0), (512, 97, 1), (4608, 97, 0), (4608, 65, 2)])
+def test_bf16_rows_around_a_block_per_sm(d_model, P, kv_cache):
+    """RMSNorm with up to 128 rows and with more, K slices to take in, and rows that do not fit a block's registers."""
+    shape = _bf16_shape(d_model=d_model, n_heads=4, d_ff=8192, vocab=1000, mask_id=999, eot_id=998)
+    w = wl.make_weights(shape, seed=5)
+    filt = wl.make_filter(32, 0.96, seed=0)
+    dec = _b().Decoder(shape, w, filt, block_len=32, max_batch=1, max_seq=P + 32, kv_cache=kv_cache)
+    lockstep(dec, oracle_model(shape, w), filt, orc.DecodeConfig(block_len=32, kv_cache=kv_cache > 0, dual_cache=kv_cache == 2),
+             wl.make_prompts(1, P, shape, seed=6), 32, logit_rtol=2e-2, conf_atol=1e-3, p_margin=0.02, max_steps=3)
+    dec.close()
+
+
 @pytest.mark.parametrize("kv_cache", [1, 2])
 def test_bf16_six_layers_three_sequences_cached_lockstep(kv_cache):
     """The key/value store at depth: six layers and three sequences, so that layer strides (layers 2..5) and sequence
