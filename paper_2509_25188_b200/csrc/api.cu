@@ -67,7 +67,7 @@ struct l2pd_ctx {
   float *logits_f32 = nullptr;       // fp32 configurations: [max_lm_rows, V]
   SeqMeta *d_meta = nullptr, *h_meta = nullptr;
   int32_t *d_row_slot = nullptr;
-  StepSummary *d_summary = nullptr, *h_summary = nullptr;
+  StepSummary *h_summary = nullptr;
   int32_t *d_status = nullptr, *h_status = nullptr;
   float2 *cs_table = nullptr;
   // partial sums of the K slices of the O and down projections, [4][ksum_rows][d] fp32: summed in slice order by the
@@ -358,7 +358,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     c->tc_rows = T_rows;
   }
 
-  CKLK(L2PD_K_OTHER, launch_build_row_map(s, c->d_meta, n_slots, c->d_row_slot, c->d_row_pos));
+  CKLK(L2PD_K_OTHER, launch_build_row_map(s, c->h_meta, c->d_meta, n_slots, c->d_row_slot, c->d_row_pos));
   CKLK(L2PD_K_EMBED, launch_embed_rmsnorm<T>(s, c->d_tokens, c->P + c->G, c->d_meta, c->d_row_slot, (const T *)c->tok_emb,
                               c->norm1[0], f.rms_eps, c->x, n, T_rows, d));
   if (c->cap) CK(cudaMemcpyAsync(c->cap, c->x, (size_t)T_rows * d * 4, cudaMemcpyDeviceToDevice, s));
@@ -565,7 +565,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
   a.tokens = c->d_tokens; a.tok_stride = c->P + c->G; a.masked = c->d_masked; a.st = c->st;
   a.w1 = c->fw1; a.b1 = c->fb1; a.w2 = c->fw2; a.b2 = c->fb2; a.tau = f.tau;
   a.use_filter = f.use_filter; a.use_eotp = f.use_eotp; a.committed_conf_mode = f.committed_conf_mode;
-  a.eot_id = f.eot_id; a.summary = c->d_summary;
+  a.eot_id = f.eot_id; a.summary = c->h_summary; a.status = c->d_status; a.status_out = c->h_status;
   a.rule = c->rule; a.conf_threshold = c->conf_threshold; a.ref = c->d_ref;
   a.n_filter_layers = c->n_filter_layers;
   for (int k = 0; k < 4; ++k) { a.fw[k] = c->flt_w[k]; a.fb[k] = c->flt_b[k]; }
@@ -587,7 +587,7 @@ void free_all(l2pd_ctx *c) {
   cudaFree(c->d_row_pos); cudaFree(c->cs_table_t); cudaFree(c->ksum);
   cudaFree(c->d_chain_bar); cudaFree(c->d_chain_trace); cudaFree(c->d_chain_tabs);
   if (c->h_chain_tabs) cudaFreeHost(c->h_chain_tabs);
-  cudaFree(c->d_meta); cudaFree(c->d_row_slot); cudaFree(c->d_summary); cudaFree(c->d_status); cudaFree(c->cs_table);
+  cudaFree(c->d_meta); cudaFree(c->d_row_slot); cudaFree(c->d_status); cudaFree(c->cs_table);
   if (c->h_meta) cudaFreeHost(c->h_meta);
   if (c->h_summary) cudaFreeHost(c->h_summary);
   if (c->h_status) cudaFreeHost(c->h_status);
@@ -715,7 +715,6 @@ l2pd_status l2pd_init(const l2pd_config *cfg, const l2pd_weights *w, int device,
       if (r == L2PD_OK && cudaMallocHost((void **)&c->h_chain_tabs, (size_t)(f.n_layers + 1) * chain_table_bytes()) != cudaSuccess) r = L2PD_ERR_OOM;
     }
   }
-  A(dev_alloc(c, &c->d_summary, (int64_t)f.max_batch));
   A(dev_alloc(c, &c->d_status, (int64_t)1));
   A(dev_alloc(c, &c->cs_table, (int64_t)f.max_seq * (f.head_dim / 2)));
   if (r != L2PD_OK) return fail(r);
@@ -851,12 +850,9 @@ l2pd_status l2pd_denoise_step(l2pd_ctx *c, void *stream, const l2pd_step_out *ou
   if (c->collect_c && c->collect_n + n_slots > c->collect_cap)   // a full sink: nothing is launched, nothing appended
     return set_err(c, L2PD_ERR_SHAPE, "sample sink full (%lld of %lld)", (long long)c->collect_n, (long long)c->collect_cap);
   CK(cudaEventRecord(c->ev0, s));
-  CK(cudaMemcpyAsync(c->d_meta, c->h_meta, sizeof(SeqMeta) * n_slots, cudaMemcpyHostToDevice, s));
   l2pd_status r = (f.dtype == L2PD_BF16) ? forward_and_decide<bf16>(c, s, n_slots, T_rows, max_q, max_kv, out)
                                          : forward_and_decide<float>(c, s, n_slots, T_rows, max_q, max_kv, out);
   if (r != L2PD_OK) return r;
-  CK(cudaMemcpyAsync(c->h_summary, c->d_summary, sizeof(StepSummary) * c->B, cudaMemcpyDeviceToHost, s));
-  CK(cudaMemcpyAsync(c->h_status, c->d_status, 4, cudaMemcpyDeviceToHost, s));
   CK(cudaEventRecord(c->ev1, s));
   CK(cudaStreamSynchronize(s));
   CK(cudaEventElapsedTime(&c->last_ms, c->ev0, c->ev1));

@@ -94,7 +94,7 @@ template <typename T>
 cudaError_t launch_final_norm_gather(cudaStream_t st, const float *x, const SeqMeta *meta,
                                      const float *gain, float eps, T *nf, int n_slots, int s,
                                      int rows_padded, int d);
-cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *meta, int n_slots, int32_t *row_slot, int32_t *row_pos);
+cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, SeqMeta *meta, int n_slots, int32_t *row_slot, int32_t *row_pos);
 // Library-owned copy of a QKV weight [3*H*dh, d] whose q and k rows are reordered inside each head so that the
 // rotary pair (i, i + dh/2) sits in adjacent rows (2i, 2i + 1); the v rows are copied as they are.
 cudaError_t launch_permute_qkv_rows(cudaStream_t st, const bf16 *src, bf16 *dst, int H, int dh, int d);
@@ -135,7 +135,8 @@ struct DecideArgs {
   float conf_threshold;           // rule 1
   const int32_t *ref;             // rule 2: reference answers [B, G]
   float *collect_c; uint8_t *collect_y; int64_t collect_base;   // optional: slot k appends (filter input, pred == ref) as sample collect_base + k
-  StepSummary *summary;           // [max_batch], indexed by sequence
+  StepSummary *summary;           // [max_batch], indexed by sequence (pinned host memory)
+  const int32_t *status; int32_t *status_out;   // the device status word and its copy (pinned host memory)
   float *o_conf; int32_t *o_pred; float *o_p; uint8_t *o_unmask;   // optional [B, s]
 };
 cudaError_t launch_decide(cudaStream_t st, const DecideArgs &a, int n_slots);

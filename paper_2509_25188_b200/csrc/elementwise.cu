@@ -345,12 +345,17 @@ __global__ void final_norm_gather_kernel(const float *x, const SeqMeta *meta, co
   for (int i = threadIdx.x; i < d; i += blockDim.x) out[i] = from_f32<T>(xr[i] * gain[i] * inv);
 }
 
-__global__ void build_row_map_kernel(const SeqMeta *meta, int32_t *row_slot, int32_t *row_pos) {
+// A step's first kernel.  The descriptions of its sequences come as an argument, META_BATCH at a time, and are stored for
+// the kernels that follow, instead of a copy from host memory in front.
+constexpr int META_BATCH = 64;
+struct MetaBatch { SeqMeta m[META_BATCH]; };
+__global__ void build_row_map_kernel(const __grid_constant__ MetaBatch b, int slot0, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos) {
   grid_dep_launch();
-  grid_dep_wait();
-  SeqMeta m = meta[blockIdx.x];
+  const SeqMeta m = b.m[blockIdx.x];
+  const int slot = slot0 + blockIdx.x;
+  if (threadIdx.x == 0) meta[slot] = m;
   for (int i = threadIdx.x; i < m.n_rows; i += blockDim.x) {
-    row_slot[m.row0 + i] = blockIdx.x;
+    row_slot[m.row0 + i] = slot;
     row_pos[m.row0 + i] = m.pos0 + i;
   }
 }
@@ -446,8 +451,18 @@ cudaError_t launch_final_norm_gather(cudaStream_t st, const float *x, const SeqM
                                      int rows_padded, int d) {
   return launch_kernel(final_norm_gather_kernel<T>, dim3(rows_padded), dim3(256), 0, st, x, meta, gain, eps, nf, n_slots, s, d);
 }
-cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *meta, int n_slots, int32_t *row_slot, int32_t *row_pos) {
-  return launch_kernel(build_row_map_kernel, dim3(n_slots), dim3(256), 0, st, meta, row_slot, row_pos);
+cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, SeqMeta *meta, int n_slots, int32_t *row_slot, int32_t *row_pos) {
+  for (int slot0 = 0; slot0 < n_slots; slot0 += META_BATCH) {
+    const int n = n_slots - slot0 < META_BATCH ? n_slots - slot0 : META_BATCH;
+    MetaBatch b;
+    for (int i = 0; i < n; ++i) b.m[i] = h_meta[slot0 + i];
+    // an ordinary launch, which starts when all earlier work of the stream is complete: the kernels behind it read weights
+    // before their own wait
+    build_row_map_kernel<<<n, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 cudaError_t launch_permute_qkv_rows(cudaStream_t st, const bf16 *src, bf16 *dst, int H, int dh, int d) {
   permute_qkv_rows_kernel<<<3 * H * dh, 256, 0, st>>>(src, dst, H, dh, d);

@@ -331,6 +331,18 @@ def test_bf16_small_model_lockstep(spread, kv_cache):
     dec.close()
 
 
+@pytest.mark.parametrize("B,s", [(64, 4), (65, 16), (130, 64)])
+def test_batches_around_the_descriptions_of_one_launch(B, s):
+    """More sequences than one launch's argument describes, with the smallest and the largest filter."""
+    shape, w = _tiny()
+    filt = wl.make_filter(s, 0.96, seed=0)
+    dec = _b().Decoder(shape, w, filt, block_len=s, max_batch=B, max_seq=3 + s)
+    st = lockstep(dec, oracle_model(shape, w), filt, orc.DecodeConfig(block_len=s), wl.make_prompts(B, 3, shape, seed=4), s,
+                  logit_rtol=1e-4, conf_atol=1e-3, p_margin=0.01, max_steps=2, oracle_when=lambda i, k, state: i in (0, 63, 64, B - 1))
+    assert st["replay_checked"] >= 0.9 * sum(st["seq_steps"])
+    dec.close()
+
+
 @pytest.mark.parametrize("d_model,P,kv_cache", [(512, 96, 0), (512, 97, 1), (4608, 97, 0), (4608, 65, 2)])
 def test_bf16_rows_around_a_block_per_sm(d_model, P, kv_cache):
     """RMSNorm with up to 128 rows and with more, K slices to take in, and rows that do not fit a block's registers."""
