@@ -496,6 +496,8 @@ l2pd_status make_tma_out_tail(TmaDesc *out, void *ptr, bool fp32, int64_t rows, 
 //             issuer needs at least (300 with two slabs), and the bytes a CTA takes in at 95 B per cycle (measured alone:
 //             79-117 B, by how many CTAs share a tile).  A sixth of the ingest time comes on top of the rest: between two
 //             tilings that keep the pipe equally busy the one that moves fewer bytes lets the power cap hold a higher clock.
+//             From 4096 rows on, where the cap holds all the time, nearly a half: the down projection (K = 12288) then takes
+//             two slabs, whose exposed drain its long main loop outweighs (16384-row step: 0.15 195, 0.45 191, 0.8 197 ms).
 //   unit      one slab: two accumulator buffers, ~400 cycles between units; two slabs: the drain is exposed.
 //   launch    7000 cycles from the CTA's start to its first MMA, and the last unit's drain.
 //   memory    the weights are read from HBM once, at 3450 B per cycle of the whole chip.
@@ -506,11 +508,12 @@ static double plan_cost(int M, int N, int K, int num_sms, int cg, int slabs, int
   const int n_tiles = ceil_div(N, unit_n);
   const int full = (n_slabs / slabs) * n_tiles * ks, tail = (n_slabs % slabs) ? n_tiles * ks : 0;
   const int kb = ceil_div(ceil_div(K, TILE_K), ks);
+  const double traffic = M >= 4096 ? 0.45 : 0.15;
   auto drain = [&](int sl) { return 1000.0 + (is_residual ? 32.0 : 20.0) * tile_n * (sl == 2 ? 1.6 : 1.0); };
   auto unit = [&](int sl) {
     const double bytes = (double)sl * A_STAGE_BYTES + 128.0 * tile_n / cg;
     const double pipe = 2.0 * tile_n * sl * (cg == 1 ? 1.13 : 1.0);
-    return kb * (fmax(fmax(pipe, sl == 2 ? 300.0 : 250.0), bytes / 95.0) + 0.15 * bytes / 95.0) + (slabs == 2 ? drain(sl) : 400.0);
+    return kb * (fmax(fmax(pipe, sl == 2 ? 300.0 : 250.0), bytes / 95.0) + traffic * bytes / 95.0) + (slabs == 2 ? drain(sl) : 400.0);
   };
   // units go round the CTA groups in order, the full ones first
   const double uf = unit(slabs), ut = tail ? unit(n_slabs % slabs) : 0.0;
@@ -640,9 +643,10 @@ cudaError_t fill_kparams(const GemmArgs &g, int stages, int b_stage_bytes, KPara
   p.gate = (p.out_tma && p.slabs == 2 && stages >= 4) ? 1 : 0;
   p.n_tiles = ceil_div(g.N, n_per_tile);
   p.k_splits = ks;
-  {   // a raster group's activation rows: about 32 MB, a quarter of L2
+  {   // A raster group's activation rows: about 46 MB of L2's 126, which also holds the weights in use and the output on its
+      // way out.  Steps of 16384 / 20000 rows: 32 MB 192.4-196 / 239-243 ms, 46 MB 190-192 / 235-236, 64 MB 201 / 245, 90 MB 207 / 259
     const double tile_bytes = (double)TILE_M * cg * p.slabs * ((double)g.K / ks) * 2.0;
-    int gm = (int)(32.0e6 / tile_bytes);
+    int gm = (int)(46.0e6 / tile_bytes);
     p.group_m = gm < 1 ? 1 : (gm > p.m_tiles ? p.m_tiles : gm);
   }
   p.out = g.out; p.bias = g.bias; p.part_m = g.part_m; p.part_s = g.part_s; p.part_i = g.part_i;
