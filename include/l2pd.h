@@ -283,14 +283,14 @@ l2pd_status l2pd_profile_read(const l2pd_ctx *ctx, int32_t kind, double *ms_tota
  * attention kernel (preceded by the rotation / scatter kernel in the key/value-cache configurations) and ONE persistent
  * launch that holds the output projection, the RMSNorm before the MLP, the gate/up and down projections and the next
  * layer's RMSNorm and QKV projection: the weight loads of a projection then start while the one before it is still
- * draining, which is what the small steps of the dual cache (a few dozen rows, bound by weight streaming) gain from.
+ * draining.
  * l2pd_set_chain(ctx, mode): 0 (the state after l2pd_init) one launch per projection; 1 chained launches where the step's
  * shapes allow, one launch per projection elsewhere; 2 the chained form's tiling in single launches (for comparisons:
- * modes 1 and 2 give bit-identical results).  With more than 256 rows the tiling does not depend on the mode, and all
- * three modes agree bit for bit; with at most 256 rows modes 1 and 2 use one 256-row slab per unit with the two
- * MMA-issuing threads on alternate k-blocks (key/value-cache configurations only).  May be called between steps.
- * Measured at 512 rows the chained and the single-launch form take the same time within a few percent (programmatic
- * dependent launch already hides the launch and the ring fill of a projection behind the one before it).
+ * modes 1 and 2 give bit-identical results).  With more than 256 rows modes 1 and 2 use two row slabs per unit, tiles of at
+ * most 176 columns and mode 0's K slices: all three modes agree bit for bit.  With at most 256 rows they use one 256-row slab
+ * per unit with the two MMA-issuing warps on alternate k-blocks (key/value-cache configurations only).  May be called between
+ * steps.  Single launches are the faster form (8B step, mode 0 / 1: 32 rows 3.5 / 5.8 ms, 125 rows 3.7 / 3.8, 512 rows 6.6 / 9.7):
+ * programmatic dependent launch hides the launch and the ring fill of a projection behind the one before it.
  * l2pd_chain_trace_enable(ctx, 1) makes every chained launch of the following steps record, per phase and CTA,
  * the nanosecond timer at which the CTA opened the phase, had its first and its last accumulator ready (for an
  * RMSNorm phase both equal the opening) and finished the phase; l2pd_chain_trace_read copies the last step's
@@ -333,7 +333,7 @@ void l2pd_destroy(l2pd_ctx *ctx);                   /* NULL is allowed */
  * slices K, the slices adding into X with floating-point reductions whose order is not fixed; slabs 2
  * (pairs only) lets one unit cover two 256-row slabs against one load of the weight tile; k_interleave
  * 1 (one slab only) has two threads issue the MMAs of alternate k-blocks into two accumulators that the
- * epilogue adds (chosen automatically when the rows fit one slab), 2 switches it off.
+ * epilogue adds (never chosen automatically), 2 says that it is not wanted.
  * A and the output follow stream order.  The weights W are requested before the kernel launched
  * just ahead of this one in the stream has completed (programmatic dependent launch): that kernel
  * must not be the one that writes them. */

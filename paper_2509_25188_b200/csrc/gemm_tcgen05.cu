@@ -1,6 +1,6 @@
 // bf16 GEMM on the 5th-generation tensor cores:  acc[M,N] = A[M,K] * W[N,K]^T, fp32 accumulation
-// in tensor memory, operands brought to shared memory by TMA (128-byte swizzle), one thread
-// issuing tcgen05.mma, four warps draining the accumulator.  Persistent CTAs (one per SM) walk
+// in tensor memory, operands brought to shared memory by TMA (128-byte swizzle), one warp per
+// slab issuing tcgen05.mma, four draining its accumulator.  Persistent CTAs (one per SM) walk
 // the output tiles; the accumulator is double-buffered in TMEM so a tile's epilogue overlaps the
 // next tile's main loop.
 //

@@ -122,6 +122,24 @@ def test_gemm_bf16_swiglu(M, F, K, tile_n):
     _close_bf16(got, want)
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 104, 4096), (8, 2064, 192), (33, 1040, 840), (127, 4096, 520), (128, 176, 64), (129, 528, 1024),
+                                   (257, 1040, 832), (513, 2064, 320), (1029, 784, 512), (4100, 1040, 1088)])
+def test_gemm_plans_at_the_edges_of_rows_and_tiles(M, N, K):
+    """Automatic plans: a ring that holds only the rows there are (M <= 128), a last unit whose second slab is empty, one-slab
+    units that stage their output beside the ring, narrow last column tiles; the three epilogues of a layer."""
+    b = _b()
+    A, W, W2 = _bf16(9, 0, (M, K), 1.0), _bf16(9, 1, (N, K), 0.05), _bf16(9, 2, (N, K), 0.05)
+    a, dA, dW = orc.widen(A), b.to_device(A), b.to_device(W)
+    want = orc.linear(a, W)
+    _close_bf16(b.gemm_bf16(dA, dW).float().cpu().numpy(), want)
+    _close_bf16(b.gemm_bf16_swiglu(dA, dW, b.to_device(W2)).float().cpu().numpy(), orc.silu(want) * orc.linear(a, W2))
+    X = wl.make_activations(9, 3, (M, N), 1.0, "fp32")
+    got = b.gemm_bf16_residual(dA, dW, b.to_device(X.copy())).cpu().numpy()
+    # fp32 sums of K exact products in any order, and of at most four slices: K 2^-24 of the sum of magnitudes
+    bound = (K + 4) * 2.0 ** -24 * (np.abs(a) @ np.abs(orc.widen(W)).T + np.abs(X))
+    assert (np.abs(got - (X.astype(np.float64) + want)) <= bound).all()
+
+
 @pytest.mark.parametrize("R,V,K,with_bias", [(32, 4096, 256, False), (16, 5000, 136, True), (200, 1000, 512, True),
                                              (1, 70, 64, False), (32, 20000, 1024, True)])
 def test_lm_head_fused_confidence(R, V, K, with_bias):
