@@ -75,10 +75,12 @@ template <> __device__ __forceinline__ bf16 from_f32<bf16>(float v) { return __f
 // ---- launchers implemented in the .cu files -------------------------------------------------------
 
 // elementwise.cu
+// A step's first kernels: the descriptions of its sequences (host memory) -> meta, the maps row -> slot and row -> position,
+// x = the rows' embeddings, n = RMSNorm(x)
 template <typename T>
-cudaError_t launch_embed_rmsnorm(cudaStream_t st, const int32_t *tokens, int64_t tok_stride,
-                                 const SeqMeta *meta, const int32_t *row_slot, const T *emb,
-                                 const float *gain, float eps, float *x, T *n, int rows, int d);
+cudaError_t launch_step_begin(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
+                              int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
+                              const float *gain, float eps, float *x, T *n, int rows, int d);
 // n = RMSNorm(x).  With n_part > 0, first x += part[0] + part[1] + ... (slice s at part + s * part_stride elements,
 // added in that order) and x is written back: the fixed-order end of a K-split projection.
 template <typename T>
@@ -94,7 +96,6 @@ template <typename T>
 cudaError_t launch_final_norm_gather(cudaStream_t st, const float *x, const SeqMeta *meta,
                                      const float *gain, float eps, T *nf, int n_slots, int s,
                                      int rows_padded, int d);
-cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, SeqMeta *meta, int n_slots, int32_t *row_slot, int32_t *row_pos);
 // Library-owned copy of a QKV weight [3*H*dh, d] whose q and k rows are reordered inside each head so that the
 // rotary pair (i, i + dh/2) sits in adjacent rows (2i, 2i + 1); the v rows are copied as they are.
 cudaError_t launch_permute_qkv_rows(cudaStream_t st, const bf16 *src, bf16 *dst, int H, int dh, int d);

@@ -46,16 +46,35 @@ template <> struct Vec8<float> {
   __device__ __forceinline__ void set(int i, float f) { reinterpret_cast<float *>(&a)[i] = f; }
 };
 
+constexpr int META_BATCH = 64;
+struct MetaBatch { SeqMeta m[META_BATCH]; };
+
 // x[row,:] = emb[token,:];  n[row,:] = x * g / sqrt(mean(x^2) + eps)
+// A step's first kernel when n_arg > 0: the descriptions of its n_arg sequences come as an argument, in place of a copy from
+// host memory and a kernel of its own that builds the row maps (3 us of a small model's step); the blocks store them, and the
+// maps, for the kernels that follow.
 template <typename T>
-__global__ void embed_rmsnorm_kernel(const int32_t *tokens, int64_t tok_stride, const SeqMeta *meta,
-                                     const int32_t *row_slot, const T *emb, const float *gain,
+__global__ void embed_rmsnorm_kernel(const __grid_constant__ MetaBatch b, int n_arg, const int32_t *tokens, int64_t tok_stride,
+                                     SeqMeta *meta, int32_t *row_slot, int32_t *row_pos, const T *emb, const float *gain,
                                      float eps, float *x, T *n, int d) {
   grid_dep_launch();
-  grid_dep_wait();
   __shared__ float red[32];
   int row = blockIdx.x;
-  SeqMeta m = meta[row_slot[row]];
+  SeqMeta m;
+  if (n_arg > 0) {
+    int slot = 0;
+    for (int step = META_BATCH / 2; step > 0; step >>= 1)   // the last sequence that starts at or before this row
+      if (slot + step < n_arg && b.m[slot + step].row0 <= row) slot += step;
+    m = b.m[slot];
+    if (threadIdx.x == 0) {
+      row_slot[row] = slot;
+      row_pos[row] = m.pos0 + (row - m.row0);
+      if (row == m.row0) meta[slot] = m;
+    }
+  } else {
+    grid_dep_wait();
+    m = meta[row_slot[row]];
+  }
   int pos = m.pos0 + (row - m.row0);
   int tok = tokens[(int64_t)m.seq * tok_stride + pos];
   const T *e = emb + (int64_t)tok * d;
@@ -345,10 +364,8 @@ __global__ void final_norm_gather_kernel(const float *x, const SeqMeta *meta, co
   for (int i = threadIdx.x; i < d; i += blockDim.x) out[i] = from_f32<T>(xr[i] * gain[i] * inv);
 }
 
-// A step's first kernel.  The descriptions of its sequences come as an argument, META_BATCH at a time, and are stored for
-// the kernels that follow, instead of a copy from host memory in front.
-constexpr int META_BATCH = 64;
-struct MetaBatch { SeqMeta m[META_BATCH]; };
+// The first kernel of a step of more than META_BATCH sequences: stores their descriptions, META_BATCH to a launch, and the
+// maps from packed rows to them.  (Fewer: embed_rmsnorm_kernel does it.)
 __global__ void build_row_map_kernel(const __grid_constant__ MetaBatch b, int slot0, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos) {
   grid_dep_launch();
   const SeqMeta m = b.m[blockIdx.x];
@@ -414,10 +431,29 @@ __global__ void gather_response_kernel(const int32_t *tokens, int P, int G, int3
 }  // namespace
 
 template <typename T>
-cudaError_t launch_embed_rmsnorm(cudaStream_t st, const int32_t *tokens, int64_t tok_stride,
-                                 const SeqMeta *meta, const int32_t *row_slot, const T *emb,
-                                 const float *gain, float eps, float *x, T *n, int rows, int d) {
-  return launch_kernel(embed_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, tokens, tok_stride, meta, row_slot, emb, gain, eps, x, n, d);
+cudaError_t launch_step_begin(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
+                              int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
+                              const float *gain, float eps, float *x, T *n, int rows, int d) {
+  // The first launch is an ordinary one, which starts when all earlier work of the stream is complete: the kernels behind it
+  // read weights before their own wait.
+  MetaBatch b;
+  auto fill = [&](int slot0) {
+    const int k = n_slots - slot0 < META_BATCH ? n_slots - slot0 : META_BATCH;
+    for (int i = 0; i < k; ++i) b.m[i] = h_meta[slot0 + i];
+    return k;
+  };
+  if (n_slots <= META_BATCH) {
+    const int k = fill(0);
+    embed_rmsnorm_kernel<T><<<rows, 256, 0, st>>>(b, k, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
+    return cudaGetLastError();
+  }
+  for (int slot0 = 0; slot0 < n_slots; slot0 += META_BATCH) {
+    const int k = fill(slot0);
+    build_row_map_kernel<<<k, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return launch_kernel(embed_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, b, 0, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
 }
 template <typename T>
 cudaError_t launch_rmsnorm(cudaStream_t st, float *x, const float *gain, float eps, T *n,
@@ -451,19 +487,6 @@ cudaError_t launch_final_norm_gather(cudaStream_t st, const float *x, const SeqM
                                      int rows_padded, int d) {
   return launch_kernel(final_norm_gather_kernel<T>, dim3(rows_padded), dim3(256), 0, st, x, meta, gain, eps, nf, n_slots, s, d);
 }
-cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, SeqMeta *meta, int n_slots, int32_t *row_slot, int32_t *row_pos) {
-  for (int slot0 = 0; slot0 < n_slots; slot0 += META_BATCH) {
-    const int n = n_slots - slot0 < META_BATCH ? n_slots - slot0 : META_BATCH;
-    MetaBatch b;
-    for (int i = 0; i < n; ++i) b.m[i] = h_meta[slot0 + i];
-    // an ordinary launch, which starts when all earlier work of the stream is complete: the kernels behind it read weights
-    // before their own wait
-    build_row_map_kernel<<<n, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
 cudaError_t launch_permute_qkv_rows(cudaStream_t st, const bf16 *src, bf16 *dst, int H, int dh, int d) {
   permute_qkv_rows_kernel<<<3 * H * dh, 256, 0, st>>>(src, dst, H, dh, d);
   return cudaGetLastError();
@@ -484,9 +507,8 @@ cudaError_t launch_gather_response(cudaStream_t st, const int32_t *tokens, int B
 }
 
 #define INSTANTIATE(T)                                                                              \
-  template cudaError_t launch_embed_rmsnorm<T>(cudaStream_t, const int32_t *, int64_t,               \
-                                               const SeqMeta *, const int32_t *, const T *,          \
-                                               const float *, float, float *, T *, int, int);        \
+  template cudaError_t launch_step_begin<T>(cudaStream_t, const SeqMeta *, int, SeqMeta *, int32_t *, int32_t *, \
+                                            const int32_t *, int64_t, const T *, const float *, float, float *, T *, int, int); \
   template cudaError_t launch_rmsnorm<T>(cudaStream_t, float *, const float *, float, T *,           \
                                          int, int, const float *, int, int64_t);                     \
   template cudaError_t launch_rope_scatter<T>(cudaStream_t, const T *, const SeqMeta *,              \
