@@ -151,10 +151,10 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 // C[M,N] = A[M,K] * W[N,K]^T in fp32, epilogues as simt_gemm_kernel.  A block computes a B x B tile with 256 threads: KG
 // groups of threads hold the whole tile, 4 x 4 outputs each, and take turns along K (16-deep shares of a 64-deep stage for
-// B = 32); the groups' sums are added in order at the end.  Four stages in flight: K = 256 is requested whole before the
+// B = 32, 4-deep ones for B = 16); the groups' sums are added in order at the end, by all threads.  Four stages in flight: K = 256 is requested whole before the
 // first multiply.  Rows are 68 words apart and dealt out interleaved, so the 16-byte loads of a warp do not collide.
 // Measured at 96 rows of the tiny model (d 256, 688), one launch between events, 64 x 64 blocks with 16-deep unpipelined
-// stages before -> now (us): QKV 34 -> 10, O 38 -> 13, gate/up 43 -> 13, down 103 -> 18, LM head 22 -> 10.
+// stages before -> now (us, some 5 of them the events): QKV 34 -> 9, O 38 -> 8, gate/up 43 -> 11, down 103 -> 9, LM head 22 -> 10.
 constexpr int F_BK = 64, F_ROW = F_BK + 4, F_STAGES = 4, F_THREADS = 256;
 template <int EPI, int B>
 __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__restrict__ A, const float *__restrict__ W,
@@ -214,95 +214,101 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__rest
       }
     }
   }
-  if (KG > 1) {
-    // group g > 0 leaves its sums, group 0 adds them in order ([group][output][thread]: no bank conflicts)
+  auto emit = [&](int i, int j, int x, int y, float v, float u) {   // output (i, j) of thread (x, y) of the tile
+    const int gm = m0 + y + (B / 4) * i, gn = n0 + x + (B / 4) * j;
+    if (gm >= M || gn >= N) return;
+    float *o = out + (int64_t)gm * N + gn;
+    if (EPI == EPI_STORE) *o = v;
+    else if (EPI == EPI_RESIDUAL) *o += v;
+    else if (EPI == EPI_SWIGLU) *o = v / (1.0f + expf(-v)) * u;
+    else *o = v + (bias ? bias[gn] : 0.f);
+  };
+  if (KG == 1) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) emit(i, j, tx, ty, acc[i][j], EPI == EPI_SWIGLU ? acc2[i][j] : 0.f);
+  } else {
+    // the groups leave their sums ([group][output][thread]: no bank conflicts), all threads share out the outputs and add
+    // them in the order of the groups
     constexpr int NO = EPI == EPI_SWIGLU ? 32 : 16;
-    static_assert((KG - 1) * NO * TG <= F_STAGES * MATS * MAT, "room for the groups' sums");
+    static_assert(KG * NO * TG <= F_STAGES * MATS * MAT, "room for the groups' sums");
     __syncthreads();
-    if (grp > 0) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          sm[((grp - 1) * NO + 4 * i + j) * TG + t] = acc[i][j];
-          if (EPI == EPI_SWIGLU) sm[((grp - 1) * NO + 16 + 4 * i + j) * TG + t] = acc2[i][j];
-        }
-    }
+      for (int j = 0; j < 4; ++j) {
+        sm[(grp * NO + 4 * i + j) * TG + t] = acc[i][j];
+        if (EPI == EPI_SWIGLU) sm[(grp * NO + 16 + 4 * i + j) * TG + t] = acc2[i][j];
+      }
     __syncthreads();
-    if (grp > 0) return;
-    for (int g = 0; g < KG - 1; ++g)
+    for (int e = tid; e < B * B; e += F_THREADS) {
+      const int k = e / TG, th = e % TG;
+      float v = sm[k * TG + th], u = EPI == EPI_SWIGLU ? sm[(16 + k) * TG + th] : 0.f;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j] += sm[(g * NO + 4 * i + j) * TG + t];
-          if (EPI == EPI_SWIGLU) acc2[i][j] += sm[(g * NO + 16 + 4 * i + j) * TG + t];
-        }
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty + (B / 4) * i;
-    if (gm >= M) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx + (B / 4) * j;
-      if (gn >= N) continue;
-      float *o = out + (int64_t)gm * N + gn;
-      const float v = acc[i][j];
-      if (EPI == EPI_STORE) *o = v;
-      else if (EPI == EPI_RESIDUAL) *o += v;
-      else if (EPI == EPI_SWIGLU) *o = v / (1.0f + expf(-v)) * acc2[i][j];
-      else *o = v + (bias ? bias[gn] : 0.f);
+      for (int g = 1; g < KG; ++g) {
+        v += sm[(g * NO + k) * TG + th];
+        if (EPI == EPI_SWIGLU) u += sm[(g * NO + 16 + k) * TG + th];
+      }
+      emit(k / 4, k % 4, th % (B / 4), th / (B / 4), v, u);
     }
   }
 }
 
-// fp32 attention: a block takes 16 query rows of one head and walks the keys in tiles of 64 with a running maximum and sum.
-// 16 threads per row: thread l computes the scores of keys l + 16 i and the output dimensions l + 16 i.  (A block per row and
-// head, which read every key row and every value column alone, took 24 us at 96 rows, 96 keys, 4 heads of 64; this 17, most of
-// it the launch.)
-constexpr int A_Q = 16, A_K = 64;
-__global__ void __launch_bounds__(256) attention_f32_kernel(const float *__restrict__ q, const float *__restrict__ kc,
+// fp32 attention: a block takes 8 query rows of one head and walks the keys in tiles of 64 with a running maximum and sum;
+// the next tile is on its way meanwhile where two fit (`bufs`).  16 threads per row: thread l computes the scores of keys
+// l + 16 i and the output dimensions 4 l + 64 i ... + 3, four sums that share each probability and take a value row in
+// 16-byte pieces.  96 rows, 96 keys, 4 heads of 64 (some 5 us of it the events): a block per row and head 24 us; 16 rows to a
+// block, one tile at a time and one dimension after the other 17; this 13.
+constexpr int A_Q = 8, A_K = 64, A_THREADS = 16 * A_Q;
+__global__ void __launch_bounds__(A_THREADS) attention_f32_kernel(const float *__restrict__ q, const float *__restrict__ kc,
                                                             const float *__restrict__ vc, const SeqMeta *meta, float *out,
-                                                            int64_t kv_seq_stride, int H, int dh) {
+                                                            int64_t kv_seq_stride, int H, int dh, int bufs) {
   extern __shared__ __align__(16) float sm[];
   grid_dep_launch();
   grid_dep_wait();
   const SeqMeta m = meta[blockIdx.z];
   const int q0 = blockIdx.x * A_Q, h = blockIdx.y, hd = H * dh, tid = threadIdx.x, r = tid >> 4, l = tid & 15;
   if (q0 >= m.n_rows) return;
-  const int stride = dh + 4, sk = A_K + 4;
-  float *Q = sm, *Kt = Q + A_Q * stride, *Vt = Kt + A_K * stride, *S = Vt + A_K * stride;   // S [16][sk]
+  const int stride = (dh + 3) / 4 * 4 + 4, sk = A_K + 4;
+  float *const Q = sm, *const S = Q + A_Q * stride, *const KV = S + A_Q * sk;   // S [A_Q][sk], KV [bufs][K then V][A_K][stride]
   const float *kb = kc + (int64_t)m.seq * kv_seq_stride + h * dh, *vb = vc + (int64_t)m.seq * kv_seq_stride + h * dh;
   const bool live = q0 + r < m.n_rows;
   const bool v4 = (dh & 3) == 0;
   // (dh is a multiple of 4 here, or every row is copied word by word)
   auto rows = [&](float *d, const float *src, int n, int n_valid) {
     if (v4) {
-      for (int e = tid; e < n * (dh / 4); e += 256) {
+      for (int e = tid; e < n * (dh / 4); e += A_THREADS) {
         const int i = e / (dh / 4), c = 4 * (e % (dh / 4));
         cp_async16(d + i * stride + c, src + (i < n_valid ? (int64_t)i * hd + c : 0), i < n_valid);
       }
     } else {
-      for (int e = tid; e < n * dh; e += 256) {
+      for (int e = tid; e < n * dh; e += A_THREADS) {
         const int i = e / dh, c = e - i * dh;
         d[i * stride + c] = i < n_valid ? src[(int64_t)i * hd + c] : 0.f;
       }
     }
   };
   rows(Q, q + (int64_t)(m.row0 + q0) * hd + h * dh, A_Q, min(A_Q, m.n_rows - q0));
-  constexpr int MAX_D = 16;                       // dh <= 256
-  float o[MAX_D], m_run = -INFINITY, l_run = 0.f;
-#pragma unroll
-  for (int i = 0; i < MAX_D; ++i) o[i] = 0.f;
+  constexpr int MAX_D = 4;                        // dh <= 256: 64 dimensions at a time
+  float o[MAX_D][4] = {}, m_run = -INFINITY, l_run = 0.f;
   const float scale = 1.0f / sqrtf((float)dh);
-  for (int j0 = 0; j0 < m.kv_len; j0 += A_K) {
+  auto fetch = [&](int j0, int buf) {
     const int nk = min(A_K, m.kv_len - j0);
-    __syncthreads();                              // the previous tile is no longer read
-    rows(Kt, kb + (int64_t)j0 * hd, A_K, nk);
-    rows(Vt, vb + (int64_t)j0 * hd, A_K, nk);
-    cp_async_commit();
-    cp_async_wait<0>();
+    rows(KV + 2 * buf * A_K * stride, kb + (int64_t)j0 * hd, A_K, nk);
+    rows(KV + (2 * buf + 1) * A_K * stride, vb + (int64_t)j0 * hd, A_K, nk);
+  };
+  fetch(0, 0);
+  cp_async_commit();
+  for (int j0 = 0; j0 < m.kv_len; j0 += A_K) {
+    const int nk = min(A_K, m.kv_len - j0), buf = bufs == 2 ? (j0 / A_K) & 1 : 0;
+    const float *const Kt = KV + 2 * buf * A_K * stride, *const Vt = Kt + A_K * stride;
+    if (bufs == 2) {
+      if (j0 + A_K < m.kv_len) fetch(j0 + A_K, buf ^ 1);
+      cp_async_commit();
+      cp_async_wait<1>();
+    } else
+      cp_async_wait<0>();
     __syncthreads();
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     if (v4) {
@@ -338,25 +344,40 @@ __global__ void __launch_bounds__(256) attention_f32_kernel(const float *__restr
     l_run = l_run * f + sum;
     m_run = m_new;
     __syncwarp();
+    // each sum runs over the keys in order; probabilities of absent keys are zero, and so are their value rows
 #pragma unroll
     for (int i = 0; i < MAX_D; ++i) {
-      if (16 * i >= dh) break;
-      float a = 0.f;
-      const int c = l + 16 * i;
+      const int c = 4 * l + 64 * i;
+      if (64 * i >= dh) break;
       if (c < dh) {
-#pragma unroll 8
-        for (int j = 0; j < nk; ++j) a = fmaf(S[r * sk + j], Vt[j * stride + c], a);
-        o[i] = fmaf(o[i], f, a);
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int j = 0; j < nk; j += 4) {
+          const float4 p4 = *reinterpret_cast<const float4 *>(S + r * sk + j);
+          const float p[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const float4 y = *reinterpret_cast<const float4 *>(Vt + (j + u) * stride + c);
+            a[0] = fmaf(p[u], y.x, a[0]); a[1] = fmaf(p[u], y.y, a[1]);
+            a[2] = fmaf(p[u], y.z, a[2]); a[3] = fmaf(p[u], y.w, a[3]);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[i][e] = fmaf(o[i][e], f, a[e]);
       }
     }
-    __syncwarp();
+    __syncthreads();                              // this tile has been read: its place may be filled again
+    if (bufs == 1 && j0 + A_K < m.kv_len) { fetch(j0 + A_K, 0); cp_async_commit(); }
   }
   const float inv = 1.0f / l_run;
   float *orow = out + (int64_t)(m.row0 + q0 + r) * hd + h * dh;
 #pragma unroll
   for (int i = 0; i < MAX_D; ++i)
-    if (l + 16 * i < dh && live) orow[l + 16 * i] = o[i] * inv;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (4 * l + 64 * i + e < dh && live) orow[4 * l + 64 * i + e] = o[i][e] * inv;
 }
+
 
 // Per-row max, sum of exp and argmax (lowest id on ties) of stored fp32 logits: one tile.  A thread folds 16 logits at a
 // time (all requested together) into its running (max, sum, argmax); the threads' records are merged at the end.
@@ -430,14 +451,24 @@ cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, c
   if constexpr (std::is_same<T, float>::value) {
     const uintptr_t bits = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(W2);
     if ((bits & 15) == 0 && (K & 3) == 0) {
-      // 32 x 32 tiles until 64 x 64 ones give every SM two blocks (SwiGLU, two weight tiles: 32 x 32 always)
-      const bool big = (int64_t)ceil_div(N, 64) * ceil_div(M, 64) >= 296;
+      // 32 x 32 tiles until 64 x 64 ones give every SM two blocks (SwiGLU, two weight tiles: no more than 32 x 32); 16 x 16 tiles
+      // as long as 32 x 32 ones fill at most every second SM.  Tiny decode of 96 rows, 32 x 32 alone 4.00 ms, 16 x 16 up to 37 blocks
+      // (O, down) 3.36, up to 74 (QKV and gate/up too) 3.13
+      auto blocks = [&](int b) { return (int64_t)ceil_div(N, b) * ceil_div(M, b); };
+      const int tile = blocks(64) >= 296 && epi != EPI_SWIGLU ? 64 : (blocks(32) <= 74 ? 16 : 32);
       float *Cf = reinterpret_cast<float *>(C);
+#define L2PD_F32(E)                                                                                      \
+  case E: return tile == 16 ? launch_gemm_f32<E, 16>(st, A, W, W2, Cf, bias, M, N, K)                    \
+                            : launch_gemm_f32<E, 32>(st, A, W, W2, Cf, bias, M, N, K);
+      switch (tile == 64 ? epi : -1) {
+        case EPI_STORE: return launch_gemm_f32<EPI_STORE, 64>(st, A, W, W2, Cf, bias, M, N, K);
+        case EPI_RESIDUAL: return launch_gemm_f32<EPI_RESIDUAL, 64>(st, A, W, W2, Cf, bias, M, N, K);
+        case EPI_STORE_F32: return launch_gemm_f32<EPI_STORE_F32, 64>(st, A, W, W2, Cf, bias, M, N, K);
+        default: break;
+      }
       switch (epi) {
-        case EPI_STORE: return big ? launch_gemm_f32<EPI_STORE, 64>(st, A, W, W2, Cf, bias, M, N, K) : launch_gemm_f32<EPI_STORE, 32>(st, A, W, W2, Cf, bias, M, N, K);
-        case EPI_RESIDUAL: return big ? launch_gemm_f32<EPI_RESIDUAL, 64>(st, A, W, W2, Cf, bias, M, N, K) : launch_gemm_f32<EPI_RESIDUAL, 32>(st, A, W, W2, Cf, bias, M, N, K);
-        case EPI_SWIGLU: return launch_gemm_f32<EPI_SWIGLU, 32>(st, A, W, W2, Cf, bias, M, N, K);
-        case EPI_STORE_F32: return big ? launch_gemm_f32<EPI_STORE_F32, 64>(st, A, W, W2, Cf, bias, M, N, K) : launch_gemm_f32<EPI_STORE_F32, 32>(st, A, W, W2, Cf, bias, M, N, K);
+        L2PD_F32(EPI_STORE) L2PD_F32(EPI_RESIDUAL) L2PD_F32(EPI_SWIGLU) L2PD_F32(EPI_STORE_F32)
+#undef L2PD_F32
         default: return cudaErrorInvalidValue;
       }
     }
@@ -457,11 +488,12 @@ cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, cons
                                   const SeqMeta *meta, const int32_t *row_slot, T *out,
                                   int64_t kv_seq_stride, int rows, int H, int dh, int max_kv, int n_slots, int max_q) {
   if constexpr (std::is_same<T, float>::value) {   // q, K and V are the library's own buffers: rows of H * dh floats, 16-byte aligned
-    const size_t bytes = sizeof(float) * ((size_t)(A_Q + 2 * A_K) * (dh + 4) + A_Q * (A_K + 4));
-    cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    auto bytes = [&](int bufs) { return (int)(sizeof(float) * ((size_t)(A_Q + 2 * bufs * A_K) * ((dh + 3) / 4 * 4 + 4) + A_Q * (A_K + 4))); };
+    const int bufs = max_kv > A_K && bytes(2) <= 200 * 1024 ? 2 : 1;
+    cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(bufs));
     if (e != cudaSuccess) return e;
-    return launch_kernel(attention_f32_kernel, dim3(ceil_div(max_q, A_Q), H, n_slots), dim3(256), bytes, st, q, kc, vc, meta, out,
-                         kv_seq_stride, H, dh);
+    return launch_kernel(attention_f32_kernel, dim3(ceil_div(max_q, A_Q), H, n_slots), dim3(A_THREADS), (size_t)bytes(bufs), st, q, kc, vc,
+                         meta, out, kv_seq_stride, H, dh, bufs);
   }
   size_t smem = (size_t)(dh + max_kv) * sizeof(float);
   if (smem > 48 * 1024) {
