@@ -151,8 +151,9 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 
 // C[M,N] = A[M,K] * W[N,K]^T in fp32, epilogues as simt_gemm_kernel.  A block computes a B x B tile with 256 threads: KG
 // groups of threads hold the whole tile, 4 x 4 outputs each, and take turns along K (16-deep shares of a 64-deep stage for
-// B = 32, 4-deep ones for B = 16); the groups' sums are added in order at the end, by all threads.  Four stages in flight: K = 256 is requested whole before the
-// first multiply.  Rows are 68 words apart and dealt out interleaved, so the 16-byte loads of a warp do not collide.
+// B = 32, 4-deep ones for B = 16); the groups' sums are added in order at the end, by all threads.  Four stages in flight:
+// K = 256 is requested whole before the first multiply.  Rows are 68 words apart and dealt out interleaved, so the 16-byte
+// loads of a warp do not collide.
 // Measured at 96 rows of the tiny model (d 256, 688), one launch between events, 64 x 64 blocks with 16-deep unpipelined
 // stages before -> now (us, some 5 of them the events): QKV 34 -> 9, O 38 -> 8, gate/up 43 -> 11, down 103 -> 9, LM head 22 -> 10.
 constexpr int F_BK = 64, F_ROW = F_BK + 4, F_STAGES = 4, F_THREADS = 256;
