@@ -217,7 +217,8 @@ int64_t l2pd_collect_count(const l2pd_ctx *ctx);
  * d_c [N, s] float, d_y [N, s] uint8 (0 / 1): DEVICE.  d_w1 [s, s], d_b1 [s], d_w2 [s, s], d_b2 [s]: DEVICE fp32,
  * initial values in, trained values out.  h_losses: HOST [epochs * ceil(N / batch)] or NULL, the loss of every
  * update's batch measured before the update.  Runs on the current device, allocates and frees its scratch,
- * returns after the stream has finished.  s in [1, 64] (else L2PD_ERR_SHAPE); bad hyper-parameters L2PD_ERR_ARG.
+ * returns after the stream has finished.  s in [1, 64] (else L2PD_ERR_SHAPE); bad hyper-parameters L2PD_ERR_ARG;
+ * L2PD_ERR_TIMEOUT when a bounded device-side wait ran out: the weights then keep their initial values.
  */
 typedef struct {
   float lr, beta1, beta2, eps, weight_decay;   /* the paper gives lr = 0.001; AdamW's published defaults: 0.9, 0.999, 1e-8, 0.01 */
@@ -309,6 +310,13 @@ int64_t l2pd_chain_trace_read(l2pd_ctx *ctx, uint64_t *h_out, int64_t capacity, 
  * clears the word; the context stays usable.  code = 0 clears it.
  */
 l2pd_status l2pd_debug_set_device_status(l2pd_ctx *ctx, void *stream, int32_t code);
+/* The same for the filter training: l2pd_filter_train_layers with a given number of updates per launch (0: as usual) and a
+ * given bound on the wait at which the blocks of a launch meet; launch number short_launch (-1: none) expects one arrival
+ * more than there are blocks, so that its first wait runs out and the call returns L2PD_ERR_TIMEOUT. */
+l2pd_status l2pd_debug_filter_train(void *stream, int32_t s, int32_t n_layers, int64_t N, const float *d_c,
+                                    const uint8_t *d_y, float *const *d_w, float *const *d_b,
+                                    const l2pd_train_config *cfg, float *h_losses, int64_t updates_per_launch,
+                                    int64_t wait_ns, int64_t short_launch);
 
 /* Device time of the most recent step in milliseconds (CUDA events on the step's stream),
  * or a negative value if no step has run. */

@@ -64,7 +64,7 @@ EXPORTS = ["l2pd_init", "l2pd_state_reset", "l2pd_denoise_step", "l2pd_decode", 
            "l2pd_launch_count", "l2pd_last_step_ms", "l2pd_profile_enable", "l2pd_profile_read", "l2pd_last_error", "l2pd_destroy",
            "l2pd_gemm_bf16", "l2pd_gemm_bf16_residual", "l2pd_gemm_bf16_swiglu", "l2pd_lm_head_bf16",
            "l2pd_lm_head_scratch_elems", "l2pd_attention_bf16", "l2pd_lm_head_bf16_static",
-           "l2pd_set_chain", "l2pd_chain_trace_enable", "l2pd_chain_trace_read", "l2pd_debug_set_device_status"]
+           "l2pd_set_chain", "l2pd_chain_trace_enable", "l2pd_chain_trace_read", "l2pd_debug_set_device_status", "l2pd_debug_filter_train"]
 
 
 KINDS = ["embed", "gemm_qkv", "rope", "attention", "gemm_o", "rmsnorm", "gemm_gate_up", "gemm_down",
@@ -94,6 +94,7 @@ def _load() -> C.CDLL:
     lib.l2pd_collect_count.restype = i64
     lib.l2pd_filter_train.argtypes = [vp, i32, i64, vp, vp, vp, vp, vp, vp, C.POINTER(TrainConfig), vp]
     lib.l2pd_filter_train_layers.argtypes = [vp, i32, i32, i64, vp, vp, vp, vp, C.POINTER(TrainConfig), vp]
+    lib.l2pd_debug_filter_train.argtypes = [vp, i32, i32, i64, vp, vp, vp, vp, C.POINTER(TrainConfig), vp, i64, i64, i64]
     lib.l2pd_last_step_rows.argtypes = [vp]
     lib.l2pd_launch_count.argtypes = [vp]
     lib.l2pd_launch_count.restype = i64

@@ -969,8 +969,13 @@ static cudaMemPool_t train_pool(int dev) {
   return pools[dev];
 }
 
+// What the test hook sets: updates per launch (0: chosen), the bound of a meeting's wait, and a launch whose meetings are one
+// arrival short (-1: none).
+struct TrainLimits { int64_t chunk; uint64_t wait_ns; int64_t short_launch; };
+
 static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t N, const float *d_c, const uint8_t *d_y,
-                                     float *const *w, float *const *b, const l2pd_train_config *t, float *h_losses) {
+                                     float *const *w, float *const *b, const l2pd_train_config *t, float *h_losses,
+                                     const TrainLimits &lim = {0, 2000000000ull, -1}) {
   if (!d_c || !d_y || !w || !b || !t) return L2PD_ERR_ARG;
   if (L < 1 || L > 4) return L2PD_ERR_ARG;
   for (int k = 0; k < L; ++k) if (!w[k] || !b[k]) return L2PD_ERR_ARG;
@@ -992,15 +997,17 @@ static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t
   unsigned *bar = reinterpret_cast<unsigned *>(losses + n_loss);
   int32_t *d_status = reinterpret_cast<int32_t *>(bar + 1);
   bool ok = launch_filter_pack(st, w, b, s, L, theta, d_status, true) == cudaSuccess;
-  FilterTrainArgs fa{d_c, d_y, N, bs, s, L, theta, m, v, gpart, losses, {t->lr, t->beta1, t->beta2, t->eps, t->weight_decay}, bar, d_status};
+  FilterTrainArgs fa{d_c, d_y, N, bs, s, L, theta, m, v, gpart, losses, {t->lr, t->beta1, t->beta2, t->eps, t->weight_decay}, bar, d_status, lim.wait_ns};
   // updates per launch: some 50 ms of work, so that no launch holds the device for long
   const double per_update = (double)(N < bs ? N : bs) * s * s * L + 1e7;
   int64_t chunk = (int64_t)(3.5e11 / per_update);
   chunk = chunk < 1 ? 1 : (chunk > 4096 ? 4096 : chunk);
+  if (lim.chunk > 0) chunk = lim.chunk;
   double p1 = 1.0, p2 = 1.0;   // beta^u, carried in double
   for (int64_t u = 0; ok && u < updates; u += chunk) {
     const int64_t u1 = updates - u < chunk ? updates : u + chunk;
-    ok = cudaMemsetAsync(bar, 0, 4, st) == cudaSuccess && launch_filter_train(st, fa, u, u1, p1, p2, sms) == cudaSuccess;
+    const int start = u / chunk == lim.short_launch ? 0xff : 0;   // -1: the counter never reaches its target
+    ok = cudaMemsetAsync(bar, start, 4, st) == cudaSuccess && launch_filter_train(st, fa, u, u1, p1, p2, sms) == cudaSuccess;
     for (int64_t i = u; i < u1; ++i) { p1 *= t->beta1; p2 *= t->beta2; }
   }
   if (ok) ok = launch_filter_pack(st, w, b, s, L, theta, d_status, false) == cudaSuccess;
@@ -1026,6 +1033,13 @@ l2pd_status l2pd_filter_train(void *stream, int32_t s, int64_t N, const float *d
 l2pd_status l2pd_filter_train_layers(void *stream, int32_t s, int32_t n_layers, int64_t N, const float *d_c, const uint8_t *d_y,
                                      float *const *d_w, float *const *d_b, const l2pd_train_config *t, float *h_losses) {
   return filter_train_impl(stream, s, n_layers, N, d_c, d_y, d_w, d_b, t, h_losses);
+}
+
+l2pd_status l2pd_debug_filter_train(void *stream, int32_t s, int32_t n_layers, int64_t N, const float *d_c, const uint8_t *d_y,
+                                    float *const *d_w, float *const *d_b, const l2pd_train_config *t, float *h_losses,
+                                    int64_t updates_per_launch, int64_t wait_ns, int64_t short_launch) {
+  if (updates_per_launch < 0 || wait_ns < 1) return L2PD_ERR_ARG;
+  return filter_train_impl(stream, s, n_layers, N, d_c, d_y, d_w, d_b, t, h_losses, {updates_per_launch, (uint64_t)wait_ns, short_launch});
 }
 
 int32_t l2pd_num_active(const l2pd_ctx *c) { return c ? c->n_active : 0; }

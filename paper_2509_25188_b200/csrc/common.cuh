@@ -155,9 +155,11 @@ struct FilterTrainArgs {
   float *losses;                                         // [updates]
   FilterTrainHyper h;
   unsigned *bar; int32_t *status;                        // meeting counter (0 before every launch), status word
+  uint64_t limit_ns;                                     // bound of a meeting's wait
 };
 int filter_train_max_rows(int64_t batch, int sms);   // rows of gpart a launch may write
-// pack: the layers' arrays -> theta (moments m, v behind it set to 0, status cleared); otherwise theta -> the arrays
+// pack: the layers' arrays -> theta (moments m, v behind it set to 0, status cleared); otherwise theta -> the arrays, unless
+// the status says that a meeting ran out
 cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, bool pack);
 // updates [u0, u1) in one cooperative launch; p1 = beta1^u0, p2 = beta2^u0
 cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms);

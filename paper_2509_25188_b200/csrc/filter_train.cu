@@ -44,6 +44,7 @@ struct TrainArgs {
   double p1, p2;           // beta1^u0, beta2^u0
   unsigned *bar;           // meeting counter, 0 at launch
   int32_t *status;
+  uint64_t limit_ns;       // bound of a meeting's wait
 };
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
@@ -53,7 +54,7 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
 }
 
 // All blocks of the launch meet: `target` arrivals on the counter.  False (for the whole block) when the wait ran out.
-__device__ __forceinline__ bool meet(unsigned *bar, unsigned target, int32_t *status, int *s_ok) {
+__device__ __forceinline__ bool meet(unsigned *bar, unsigned target, int32_t *status, uint64_t limit_ns, int *s_ok) {
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -64,7 +65,7 @@ __device__ __forceinline__ bool meet(unsigned *bar, unsigned target, int32_t *st
     while ((int)(ld_acquire(bar) - target) < 0) {
       if ((++spins & 0x3fu) == 0) {
         if (*reinterpret_cast<volatile int32_t *>(status) != DEV_OK) { ok = 0; break; }
-        if (ptx::globaltimer() - t0 > 2000000000ull) { atomicCAS(status, 0, DEV_TIMEOUT_EPILOGUE); ok = 0; break; }
+        if (ptx::globaltimer() - t0 > limit_ns) { atomicCAS(status, 0, DEV_TIMEOUT_EPILOGUE); ok = 0; break; }
       }
     }
     *s_ok = ok;
@@ -118,6 +119,8 @@ __global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a
   const bool vec = s == S && ((reinterpret_cast<uintptr_t>(a.C) | reinterpret_cast<uintptr_t>(a.Y)) & 15) == 0;
   double p1 = a.p1, p2 = a.p2;
   unsigned target = 0;
+  // a meeting of an earlier launch ran out: the parameters are part old, part new, and nothing may be made of them
+  if (*reinterpret_cast<volatile int32_t *>(a.status) != DEV_OK) return;
 
   for (int64_t u = a.u0; u < a.u1; ++u) {
     const int64_t n0 = (u % a.per_epoch) * a.batch, nb = a.N - n0 < a.batch ? a.N - n0 : a.batch;
@@ -341,7 +344,7 @@ __global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a
       }
     }
     target += gridDim.x;
-    if (!meet(a.bar, target, a.status, &s_ok)) return;
+    if (!meet(a.bar, target, a.status, a.limit_ns, &s_ok)) return;
 
     // AdamW: 32 parameters per block and pass, a share of the rows per warp; entry P is the loss
     p1 *= (double)a.beta1; p2 *= (double)a.beta2;
@@ -383,15 +386,17 @@ __global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a
     }
     if (u + 1 < a.u1) {
       target += gridDim.x;
-      if (!meet(a.bar, target, a.status, &s_ok)) return;
+      if (!meet(a.bar, target, a.status, a.limit_ns, &s_ok)) return;
     }
   }
 }
 
 struct PackArgs { float *w[MAX_LAYERS], *b[MAX_LAYERS]; float *theta; int s, n_layers; };
 
-// The caller's arrays -> theta, moments 0, status 0 (pack), and theta -> the caller's arrays.
+// The caller's arrays -> theta, moments 0, status 0 (pack), and theta -> the caller's arrays, which stay as they were when a
+// meeting ran out (blocks leave it at different points, so theta is then part old, part new).
 __global__ void filter_pack_kernel(PackArgs a, int pack, int32_t *status) {
+  if (!pack && *status != DEV_OK) return;
   const int per = a.s * a.s + a.s, P = a.n_layers * per;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < P; e += gridDim.x * blockDim.x) {
     const int k = e / per, r = e - k * per;
@@ -440,7 +445,7 @@ cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64
   a.s = f.s; a.n_layers = f.n_layers; a.P = f.n_layers * (f.s * f.s + f.s);
   a.theta = f.theta; a.m = f.m; a.v = f.v; a.gpart = f.gpart; a.losses = f.losses;
   a.lr = f.h.lr; a.beta1 = f.h.beta1; a.beta2 = f.h.beta2; a.eps = f.h.eps; a.weight_decay = f.h.weight_decay;
-  a.p1 = p1; a.p2 = p2; a.bar = f.bar; a.status = f.status;
+  a.p1 = p1; a.p2 = p2; a.bar = f.bar; a.status = f.status; a.limit_ns = f.limit_ns;
   const int64_t nb = f.N < f.batch ? f.N : f.batch;
   // Large batches: tiles of 64 samples, 4 x 4 outputs per thread.  With fewer than one such tile for every SM smaller tiles
   // spread the batch over more blocks (1,024 samples of 64, four layers: tiles of 16 take 19.5 k cycles, of 32 30 k; 84,480

@@ -168,3 +168,36 @@ def test_training_at_the_edges_of_its_tiles(s, n, depth, batch):
         d = np.concatenate([np.abs(gw - ww).ravel(), np.abs(gb - wb).ravel()])
         assert d.max() <= 2e-3 * len(losses) + 1e-6
         assert np.mean(d > 1e-5) <= 0.01 + 1.0 / d.size
+
+
+def test_a_meeting_that_runs_out_leaves_the_weights_alone():
+    """One update to a launch, the third launch one arrival short (host-side hook; its wait gives up after 2 ms): the call
+    reports the time-out, the caller's arrays keep their initial values although two updates had been made, and the next
+    training on the same device is that of an untouched process."""
+    import ctypes
+    import torch
+    b = _b()
+    s, n, depth = 32, 3000, 2
+    C, Y = _data(s, n, seed=2)
+    c, y = torch.from_numpy(C).cuda(), torch.from_numpy(Y).cuda()
+    rng = np.random.default_rng(8)
+    layers = [((np.eye(s) + 0.1 * rng.normal(size=(s, s))).astype(np.float32), np.zeros(s, np.float32)) for _ in range(depth)]
+    cfg = b.TrainConfig(1e-3, 0.9, 0.999, 1e-8, 0.01, 5, 0)
+
+    def run(short_launch):
+        w, bias = [torch.from_numpy(q).cuda() for q, _ in layers], [torch.from_numpy(q).cuda() for _, q in layers]
+        pw, pb = ((ctypes.c_void_p * depth)(*[t.data_ptr() for t in ts]) for ts in (w, bias))
+        losses = np.zeros(5, np.float32)
+        r = b.lib.l2pd_debug_filter_train(torch.cuda.current_stream().cuda_stream, s, depth, n, c.data_ptr(), y.data_ptr(), pw, pb,
+                                          ctypes.byref(cfg), losses.ctypes.data, 1, 2_000_000, short_launch)
+        return r, [(u.cpu().numpy(), v.cpu().numpy()) for u, v in zip(w, bias)], losses
+
+    before, _ = b.filter_train_layers(layers, C, Y, 5)
+    r, got, _ = run(2)
+    assert r == -5
+    for (gw, gb), (w, bias) in zip(got, layers):
+        assert np.array_equal(gw, w) and np.array_equal(gb, bias)
+    r, got, losses = run(-1)                                      # the hook without a short launch: the ordinary training
+    assert r == 0 and losses[-1] < losses[0]
+    for (gw, gb), (w, bias) in zip(got, before):
+        assert np.array_equal(gw, w) and np.array_equal(gb, bias)
