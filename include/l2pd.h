@@ -217,7 +217,8 @@ int64_t l2pd_collect_count(const l2pd_ctx *ctx);
  * d_c [N, s] float, d_y [N, s] uint8 (0 / 1): DEVICE.  d_w1 [s, s], d_b1 [s], d_w2 [s, s], d_b2 [s]: DEVICE fp32,
  * initial values in, trained values out.  h_losses: HOST [epochs * ceil(N / batch)] or NULL, the loss of every
  * update's batch measured before the update.  Runs on the current device, allocates and frees its scratch,
- * returns after the stream has finished.  s in [1, 64] (else L2PD_ERR_SHAPE); bad hyper-parameters L2PD_ERR_ARG;
+ * returns after the stream has finished.  Its launches take every SM for some 100 us each (one update, where that is
+ * longer); kernels of other streams run between them.  s in [1, 64] (else L2PD_ERR_SHAPE); bad hyper-parameters L2PD_ERR_ARG;
  * L2PD_ERR_TIMEOUT when a bounded device-side wait ran out: the weights then keep their initial values.
  */
 typedef struct {

@@ -996,21 +996,27 @@ static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t
   float *m = theta + P, *v = theta + 2 * P, *gpart = theta + ((3 * P + 3) & ~3), *losses = gpart + n_sums;
   unsigned *bar = reinterpret_cast<unsigned *>(losses + n_loss);
   int32_t *d_status = reinterpret_cast<int32_t *>(bar + 1);
-  bool ok = launch_filter_pack(st, w, b, s, L, theta, d_status, true) == cudaSuccess;
-  FilterTrainArgs fa{d_c, d_y, N, bs, s, L, theta, m, v, gpart, losses, {t->lr, t->beta1, t->beta2, t->eps, t->weight_decay}, bar, d_status, lim.wait_ns};
-  // updates per launch: some 50 ms of work, so that no launch holds the device for long
-  const double per_update = (double)(N < bs ? N : bs) * s * s * L + 1e7;
-  int64_t chunk = (int64_t)(3.5e11 / per_update);
-  chunk = chunk < 1 ? 1 : (chunk > 4096 ? 4096 : chunk);
-  if (lim.chunk > 0) chunk = lim.chunk;
+  bool ok = launch_filter_pack(st, w, b, s, L, theta, d_status, bar, true) == cudaSuccess;
+  FilterTrainArgs fa{d_c, d_y, N, bs, s, L, theta, m, v, gpart, losses, {t->lr, t->beta1, t->beta2, t->eps, t->weight_decay}, bar, d_status, 0u, lim.wait_ns};
+  const int64_t chunk = lim.chunk > 0 ? lim.chunk : filter_train_updates_per_launch(N < bs ? N : bs, s, L);
   double p1 = 1.0, p2 = 1.0;   // beta^u, carried in double
-  for (int64_t u = 0; ok && u < updates; u += chunk) {
+  // At most 64 launches are in the queue: a launch call that finds it full (1024) waits in the driver, and the launches of
+  // other threads with it (a decode beside the training stood still until all its launches were queued).
+  constexpr int64_t GROUP = 32;
+  cudaEvent_t done[2] = {nullptr, nullptr};
+  for (int64_t u = 0, k = 0; ok && u < updates; u += chunk, ++k) {
     const int64_t u1 = updates - u < chunk ? updates : u + chunk;
-    const int start = u / chunk == lim.short_launch ? 0xff : 0;   // -1: the counter never reaches its target
-    ok = cudaMemsetAsync(bar, start, 4, st) == cudaSuccess && launch_filter_train(st, fa, u, u1, p1, p2, sms) == cudaSuccess;
+    if (k == lim.short_launch) ++fa.arrivals;   // the counter never reaches its target
+    ok = launch_filter_train(st, fa, u, u1, p1, p2, sms) == cudaSuccess;
     for (int64_t i = u; i < u1; ++i) { p1 *= t->beta1; p2 *= t->beta2; }
+    if (ok && (k + 1) % GROUP == 0) {
+      cudaEvent_t &mine = done[(k / GROUP) & 1], &before = done[(k / GROUP + 1) & 1];
+      ok = (mine || cudaEventCreateWithFlags(&mine, cudaEventDisableTiming) == cudaSuccess) && cudaEventRecord(mine, st) == cudaSuccess &&
+           (!before || cudaEventSynchronize(before) == cudaSuccess);
+    }
   }
-  if (ok) ok = launch_filter_pack(st, w, b, s, L, theta, d_status, false) == cudaSuccess;
+  for (cudaEvent_t e : done) if (e) cudaEventDestroy(e);
+  if (ok) ok = launch_filter_pack(st, w, b, s, L, theta, d_status, bar, false) == cudaSuccess;
   // losses and status in one copy: they lie behind one another
   const size_t n_back = h_losses ? n_loss + 2 : 2;
   std::vector<float> back(n_back);

@@ -154,15 +154,18 @@ struct FilterTrainArgs {
   float *gpart;                                          // [filter_train_max_rows][filter_train_row_floats], 16-byte aligned
   float *losses;                                         // [updates]
   FilterTrainHyper h;
-  unsigned *bar; int32_t *status;                        // meeting counter (0 before every launch), status word
+  unsigned *bar; int32_t *status;                        // meeting counter, status word
+  unsigned arrivals;                                     // what the counter holds before the next launch
   uint64_t limit_ns;                                     // bound of a meeting's wait
 };
 int filter_train_max_rows(int64_t batch, int sms);   // rows of gpart a launch may write
-// pack: the layers' arrays -> theta (moments m, v behind it set to 0, status cleared); otherwise theta -> the arrays, unless
+// pack: the layers' arrays -> theta (moments m, v behind it, status and counter set to 0); otherwise theta -> the arrays, unless
 // the status says that a meeting ran out
-cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, bool pack);
-// updates [u0, u1) in one cooperative launch; p1 = beta1^u0, p2 = beta2^u0
-cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms);
+cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, unsigned *bar, bool pack);
+// updates that one launch should run, so that it does not hold the device for long
+int64_t filter_train_updates_per_launch(int64_t batch, int s, int n_layers);
+// updates [u0, u1) in one cooperative launch, which advances f.arrivals; p1 = beta1^u0, p2 = beta2^u0
+cudaError_t launch_filter_train(cudaStream_t st, FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms);
 
 // gemm_tcgen05.cu
 struct TmaDesc { CUtensorMap map; };

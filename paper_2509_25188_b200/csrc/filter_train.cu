@@ -2,7 +2,7 @@
 // sigmoid(f_theta(conf)) and the EGP targets, over the weights of the filter (Section 3.2: two Linear(s, s)
 // layers; Section 4.4: one to four, ReLU between consecutive layers) with AdamW (Section 4.1: learning rate 0.001).
 //
-// filter_train_kernel runs many updates in one cooperative launch.  One update:
+// filter_train_kernel runs some 100 us of updates in one cooperative launch.  One update:
 //   gradient   every block walks tiles of T samples held in shared memory: forward through the layers, dz = sigmoid(z) - y, delta of the layers below
 //              (delta_{k-1} = (delta_k W_k) [x_k > 0]), then dW_k += delta_k^T x_k into accumulators its threads own;
 //              it ends by writing its sums (not yet divided by the batch's element count) and its loss sum to its own
@@ -42,7 +42,8 @@ struct TrainArgs {
   float *losses;           // [updates]: the batch's loss, measured before the update
   float lr, beta1, beta2, eps, weight_decay;
   double p1, p2;           // beta1^u0, beta2^u0
-  unsigned *bar;           // meeting counter, 0 at launch
+  unsigned *bar;           // meeting counter, `arrivals` at launch
+  unsigned arrivals;
   int32_t *status;
   uint64_t limit_ns;       // bound of a meeting's wait
 };
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a
   // rows that fill their padded width and start on 16 bytes come by cp.async
   const bool vec = s == S && ((reinterpret_cast<uintptr_t>(a.C) | reinterpret_cast<uintptr_t>(a.Y)) & 15) == 0;
   double p1 = a.p1, p2 = a.p2;
-  unsigned target = 0;
+  unsigned target = a.arrivals;
   // a meeting of an earlier launch ran out: the parameters are part old, part new, and nothing may be made of them
   if (*reinterpret_cast<volatile int32_t *>(a.status) != DEV_OK) return;
 
@@ -393,9 +394,9 @@ __global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a
 
 struct PackArgs { float *w[MAX_LAYERS], *b[MAX_LAYERS]; float *theta; int s, n_layers; };
 
-// The caller's arrays -> theta, moments 0, status 0 (pack), and theta -> the caller's arrays, which stay as they were when a
+// The caller's arrays -> theta, moments 0, status and meeting counter 0 (pack), and theta -> the caller's arrays, which stay as they were when a
 // meeting ran out (blocks leave it at different points, so theta is then part old, part new).
-__global__ void filter_pack_kernel(PackArgs a, int pack, int32_t *status) {
+__global__ void filter_pack_kernel(PackArgs a, int pack, int32_t *status, unsigned *bar) {
   if (!pack && *status != DEV_OK) return;
   const int per = a.s * a.s + a.s, P = a.n_layers * per;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < P; e += gridDim.x * blockDim.x) {
@@ -404,11 +405,11 @@ __global__ void filter_pack_kernel(PackArgs a, int pack, int32_t *status) {
     if (pack) { a.theta[e] = *q; a.theta[P + e] = 0.f; a.theta[2 * P + e] = 0.f; }
     else *q = a.theta[e];
   }
-  if (pack && blockIdx.x == 0 && threadIdx.x == 0) *status = DEV_OK;
+  if (pack && blockIdx.x == 0 && threadIdx.x == 0) { *status = DEV_OK; *bar = 0; }
 }
 
 template <int S, int T, int LM, int TH, int OCC>
-cudaError_t launch_train(cudaStream_t st, TrainArgs &a, int sms) {
+cudaError_t launch_train(cudaStream_t st, TrainArgs &a, int sms, int *blocks) {
   const size_t smem = sizeof(float) * (size_t)train_smem_floats<S, T>(a.n_layers);
   cudaError_t e = cudaFuncSetAttribute(filter_train_kernel<S, T, LM, TH, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -422,22 +423,35 @@ cudaError_t launch_train(cudaStream_t st, TrainArgs &a, int sms) {
   int grid = sms * occ;
   if (tiles < grid) grid = (int)(tiles > sms ? tiles : sms);
   void *args[] = {&a};
+  *blocks = grid;
   return cudaLaunchCooperativeKernel((const void *)filter_train_kernel<S, T, LM, TH, OCC>, dim3(grid), dim3(TH), args, smem, st);
 }
 
 }  // namespace
 
-cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, bool pack) {
+cudaError_t launch_filter_pack(cudaStream_t st, float *const *w, float *const *b, int s, int n_layers, float *theta, int32_t *status, unsigned *bar, bool pack) {
   PackArgs a = {};
   for (int k = 0; k < n_layers; ++k) { a.w[k] = w[k]; a.b[k] = b[k]; }
   a.theta = theta; a.s = s; a.n_layers = n_layers;
-  filter_pack_kernel<<<(n_layers * (s * s + s) + 255) / 256, 256, 0, st>>>(a, pack ? 1 : 0, status);
+  filter_pack_kernel<<<(n_layers * (s * s + s) + 255) / 256, 256, 0, st>>>(a, pack ? 1 : 0, status, bar);
   return cudaGetLastError();
 }
 
 int filter_train_max_rows(int64_t batch, int sms) { return (int)(ceil_div64(batch, 16) < 3 * sms ? ceil_div64(batch, 16) : 3 * sms); }
 
-cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms) {
+// A launch occupies every SM, and a kernel of another stream waits for it, so a launch takes about 100 us of updates, by a
+// model of their time that holds within a fifth (the fixed part: meetings and phases).  Beside training at 84,480 x 32, two
+// layers, a decode step of the tiny model (20 kernels, 0.12 ms alone) takes 0.48 ms and the 512-row step of four 8B layers
+// (0.85 ms alone) 2.5 ms; with launches of 400 us 2.0 and 9.1 ms, of 80 ms each stands still for a launch or two.  The
+// training itself pays 2 % (38.9 -> 39.9 us an update; four layers, 1,024 x 64: 19.3 -> 20.0).
+int64_t filter_train_updates_per_launch(int64_t batch, int s, int n_layers) {
+  const double S = s <= 32 ? 32.0 : 64.0, macs = (double)batch * S * S * (3 * n_layers - 1);
+  const double us = 5.0 + 3.0 * n_layers + macs / 14.4e6;
+  const int64_t n = (int64_t)(100.0 / us);
+  return n < 1 ? 1 : n;
+}
+
+cudaError_t launch_filter_train(cudaStream_t st, FilterTrainArgs &f, int64_t u0, int64_t u1, double p1, double p2, int sms) {
   if (f.n_layers < 1 || f.n_layers > MAX_LAYERS || f.s < 1 || f.s > MAX_S) return cudaErrorInvalidValue;
   TrainArgs a;
   a.C = f.C; a.Y = f.Y; a.N = f.N; a.batch = f.batch; a.u0 = u0; a.u1 = u1;
@@ -445,18 +459,23 @@ cudaError_t launch_filter_train(cudaStream_t st, const FilterTrainArgs &f, int64
   a.s = f.s; a.n_layers = f.n_layers; a.P = f.n_layers * (f.s * f.s + f.s);
   a.theta = f.theta; a.m = f.m; a.v = f.v; a.gpart = f.gpart; a.losses = f.losses;
   a.lr = f.h.lr; a.beta1 = f.h.beta1; a.beta2 = f.h.beta2; a.eps = f.h.eps; a.weight_decay = f.h.weight_decay;
-  a.p1 = p1; a.p2 = p2; a.bar = f.bar; a.status = f.status; a.limit_ns = f.limit_ns;
+  a.p1 = p1; a.p2 = p2; a.bar = f.bar; a.arrivals = f.arrivals; a.status = f.status; a.limit_ns = f.limit_ns;
   const int64_t nb = f.N < f.batch ? f.N : f.batch;
   // Large batches: tiles of 64 samples, 4 x 4 outputs per thread.  With fewer than one such tile for every SM smaller tiles
   // spread the batch over more blocks (1,024 samples of 64, four layers: tiles of 16 take 19.5 k cycles, of 32 30 k; 84,480
   // of 32: 128 threads with 4 x 4 outputs 56 k, 256 threads with 2 x 4 65 k).
   const bool small = nb < (int64_t)(f.s <= 32 ? 64 : 32) * sms;
+  int blocks = 0;
+  cudaError_t e;
   if (f.s <= 32) {
-    if (f.n_layers <= 2) return small ? launch_train<32, 32, 2, 256, 2>(st, a, sms) : launch_train<32, 64, 2, 128, 3>(st, a, sms);
-    return small ? launch_train<32, 32, 4, 256, 1>(st, a, sms) : launch_train<32, 64, 4, 128, 2>(st, a, sms);
+    if (f.n_layers <= 2) e = small ? launch_train<32, 32, 2, 256, 2>(st, a, sms, &blocks) : launch_train<32, 64, 2, 128, 3>(st, a, sms, &blocks);
+    else e = small ? launch_train<32, 32, 4, 256, 1>(st, a, sms, &blocks) : launch_train<32, 64, 4, 128, 2>(st, a, sms, &blocks);
+  } else {
+    if (f.n_layers <= 2) e = small ? launch_train<64, 16, 2, 256, 2>(st, a, sms, &blocks) : launch_train<64, 64, 2, 256, 1>(st, a, sms, &blocks);
+    else e = small ? launch_train<64, 16, 4, 256, 1>(st, a, sms, &blocks) : launch_train<64, 64, 4, 256, 1>(st, a, sms, &blocks);
   }
-  if (f.n_layers <= 2) return small ? launch_train<64, 16, 2, 256, 2>(st, a, sms) : launch_train<64, 64, 2, 256, 1>(st, a, sms);
-  return small ? launch_train<64, 16, 4, 256, 1>(st, a, sms) : launch_train<64, 64, 4, 256, 1>(st, a, sms);
+  f.arrivals += (unsigned)blocks * (unsigned)(2 * (u1 - u0) - 1);   // two meetings an update, but for the launch's last one
+  return e;
 }
 
 }  // namespace l2pd

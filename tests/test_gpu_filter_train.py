@@ -201,3 +201,43 @@ def test_a_meeting_that_runs_out_leaves_the_weights_alone():
     assert r == 0 and losses[-1] < losses[0]
     for (gw, gb), (w, bias) in zip(got, before):
         assert np.array_equal(gw, w) and np.array_equal(gb, bias)
+
+
+def test_a_decode_on_another_stream_runs_beside_the_training():
+    """The training's launches are short and few are queued: while 4,000 updates (some 160 ms) run in a thread on one stream,
+    a decode on another gets its steps (0.1 ms each alone) between them, and both results are those of runs on their own.
+    With one launch for all updates the decode got a single step."""
+    import threading
+    import torch
+    b = _b()
+    shape, d = wl.TINY, wl.DECODES["C0"]
+    w = wl.make_weights(shape, seed=0, final_norm_gain=wl.spread_gain(shape))
+    f0 = wl.make_filter(d.block_len, d.tau, seed=0)
+    prompts = wl.make_prompts(1, d.prompt_len, shape, seed=1)
+    dec = b.Decoder(shape, w, f0, block_len=d.block_len, tau=d.tau, max_batch=1, max_seq=d.prompt_len + d.gen_len)
+    want_tokens, _, want_steps, _ = dec.decode(prompts, d.gen_len)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    c = torch.rand(84480, 32, generator=g, device="cuda")
+    y = (c > 0.6).to(torch.uint8)
+    start = wl.make_filter(32, seed=3)
+    want, want_losses = b.filter_train(start, c, y, 4000)
+    got = []
+
+    def train():
+        torch.cuda.set_device(0)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            got.append(b.filter_train(start, c, y, 4000))
+
+    torch.cuda.synchronize()
+    th = threading.Thread(target=train)
+    th.start()
+    steps = 0
+    with torch.cuda.stream(torch.cuda.Stream()):
+        while th.is_alive():
+            tokens, _, n, _ = dec.decode(prompts, d.gen_len)
+            assert np.array_equal(tokens, want_tokens) and np.array_equal(n, want_steps)
+            steps += int(n[0])
+    th.join()
+    dec.close()
+    assert np.array_equal(got[0][1], want_losses) and all(np.array_equal(got[0][0][k], want[k]) for k in want)
+    assert steps >= 2 * int(want_steps[0])
