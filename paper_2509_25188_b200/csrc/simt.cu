@@ -333,11 +333,12 @@ __global__ void __launch_bounds__(A_THREADS) attention_f32_kernel(const float *_
       mx = fmaxf(mx, s[i]);
     }
     for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-    const float m_new = fmaxf(m_run, mx), f = expf(m_run - m_new);   // the first tile: exp(-inf) = 0
+    // while every score so far is -inf (dot products beyond the range), the reference is 0: their probabilities are then 0
+    const float m_new = fmaxf(m_run, mx), m_ref = m_new == -INFINITY ? 0.f : m_new, f = expf(m_run - m_ref);   // the first tile: exp(-inf) = 0
     float sum = 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float e = expf(s[i] - m_new);
+      const float e = expf(s[i] - m_ref);
       sum += e;
       S[r * sk + l + 16 * i] = e;
     }

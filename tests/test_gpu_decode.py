@@ -376,3 +376,21 @@ def test_bf16_six_layers_three_sequences_cached_lockstep(kv_cache):
     assert cached_steps >= 3                      # most steps read the store
     assert st["replay_checked"] >= 0.9 * sum(st["seq_steps"])
     dec.close()
+
+
+def test_fp32_scores_beyond_the_range_in_a_whole_key_tile():
+    """The first 64 keys score -inf (a dot product below -3.4e38) with every masked row, the others are finite: their
+    probabilities are 0, as in the oracle, whose 64-bit scores are finite, and not 0 / 0."""
+    shape = wl.ModelShape(n_layers=1, d_model=32, n_heads=1, head_dim=16, d_ff=40, vocab=50, rms_eps=1e-5, rope_theta=1e30,
+                          mask_id=49, eot_id=48, dtype="fp32")
+    w = wl.make_weights(shape, seed=3, final_norm_gain=wl.spread_gain(shape))
+    layer = w["layers"][0]
+    w["tok_emb"][0], w["tok_emb"][shape.mask_id] = 0.0, 0.0
+    w["tok_emb"][0, 0] = w["tok_emb"][shape.mask_id, 1] = 1.0     # prompt rows: unit vector 0; masked rows: unit vector 1
+    layer["wqkv"][7], layer["wqkv"][16 + 7] = 0.0, 0.0            # pair 7 turns by less than 1e-23 per position
+    layer["wqkv"][7, 1], layer["wqkv"][16 + 7, 0] = 1e20, -1e20   # q . k = -3e41 for a masked row and a prompt key, else small
+    filt = wl.make_filter(16, 0.96, seed=0)
+    dec = _b().Decoder(shape, w, filt, block_len=16, max_batch=1, max_seq=96)
+    lockstep(dec, oracle_model(shape, w), filt, orc.DecodeConfig(block_len=16), np.zeros((1, 80), np.int32), 16,
+             logit_rtol=1e-4, conf_atol=1e-3, p_margin=0.01, max_steps=1)
+    dec.close()
