@@ -14,6 +14,7 @@ namespace l2pd {
 namespace {
 
 constexpr int BM = 64, BN = 64, BK = 16;
+constexpr int MAX_GRID_YZ = 65535;   // blocks along the y and z of a grid
 
 // C[M,N] = A[M,K] * W[N,K]^T with fp32 accumulation in k order; 256 threads, 4x4 outputs each.
 //   EPI_STORE      C (T)    = acc
@@ -264,12 +265,15 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__rest
 constexpr int A_Q = 8, A_K = 64, A_THREADS = 16 * A_Q;
 __global__ void __launch_bounds__(A_THREADS) attention_f32_kernel(const float *__restrict__ q, const float *__restrict__ kc,
                                                             const float *__restrict__ vc, const SeqMeta *meta, float *out,
-                                                            int64_t kv_seq_stride, int H, int dh, int bufs) {
+                                                            int64_t kv_seq_stride, int H, int dh, int bufs, int n_slots, int n_qt) {
   extern __shared__ __align__(16) float sm[];
   grid_dep_launch();
+  int slot = blockIdx.z, qt = blockIdx.x;
+  while (qt >= n_qt) { qt -= n_qt; slot += MAX_GRID_YZ; }   // more sequences than the grid's z has room for
+  if (slot >= n_slots) return;
   grid_dep_wait();
-  const SeqMeta m = meta[blockIdx.z];
-  const int q0 = blockIdx.x * A_Q, h = blockIdx.y, hd = H * dh, tid = threadIdx.x, r = tid >> 4, l = tid & 15;
+  const SeqMeta m = meta[slot];
+  const int q0 = qt * A_Q, h = blockIdx.y, hd = H * dh, tid = threadIdx.x, r = tid >> 4, l = tid & 15;
   if (q0 >= m.n_rows) return;
   const int stride = (dh + 3) / 4 * 4 + 4, sk = A_K + 4;
   float *const Q = sm, *const S = Q + A_Q * stride, *const KV = S + A_Q * sk;   // S [A_Q][sk], KV [bufs][K then V][A_K][stride]
@@ -494,8 +498,9 @@ cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, cons
     const int bufs = max_kv > A_K && bytes(2) <= 200 * 1024 ? 2 : 1;
     cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(bufs));
     if (e != cudaSuccess) return e;
-    return launch_kernel(attention_f32_kernel, dim3(ceil_div(max_q, A_Q), H, n_slots), dim3(A_THREADS), (size_t)bytes(bufs), st, q, kc, vc,
-                         meta, out, kv_seq_stride, H, dh, bufs);
+    const int n_qt = ceil_div(max_q, A_Q), z = n_slots < MAX_GRID_YZ ? n_slots : MAX_GRID_YZ;
+    return launch_kernel(attention_f32_kernel, dim3(n_qt * ceil_div(n_slots, z), H, z), dim3(A_THREADS), (size_t)bytes(bufs), st, q, kc, vc,
+                         meta, out, kv_seq_stride, H, dh, bufs, n_slots, n_qt);
   }
   size_t smem = (size_t)(dh + max_kv) * sizeof(float);
   if (smem > 48 * 1024) {

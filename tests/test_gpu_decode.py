@@ -394,3 +394,20 @@ def test_fp32_scores_beyond_the_range_in_a_whole_key_tile():
     lockstep(dec, oracle_model(shape, w), filt, orc.DecodeConfig(block_len=16), np.zeros((1, 80), np.int32), 16,
              logit_rtol=1e-4, conf_atol=1e-3, p_margin=0.01, max_steps=1)
     dec.close()
+
+
+@pytest.mark.parametrize("B", [65600])
+def test_fp32_batches_beyond_a_grid_dimension(B):
+    """More sequences than the y and z of a grid count (65,535).  All have the same prompt, so every row equals the first."""
+    shape = wl.ModelShape(n_layers=1, d_model=8, n_heads=1, head_dim=8, d_ff=8, vocab=16, rms_eps=1e-5, rope_theta=1e4,
+                          mask_id=15, eot_id=14, dtype="fp32")
+    w = wl.make_weights(shape, seed=4, final_norm_gain=wl.spread_gain(shape))
+    m = oracle_model(shape, w)
+    dec = _b().Decoder(shape, w, const_filter(1, 10.0), block_len=1, max_batch=B, max_seq=2)
+    dec.state_reset(np.full((B, 1), 3, np.int32), 1)
+    out = dec.denoise_step(want_logits=True)
+    dec.close()
+    want = orc.block_logits(m, orc.init_state(m, np.array([3]), 1), orc.DecodeConfig(block_len=1))[0]
+    assert np.abs(out["logits"][0, 0] - want).max() <= 1e-4 * np.abs(want).max()
+    assert np.array_equal(out["logits"], np.broadcast_to(out["logits"][:1], out["logits"].shape))
+    assert (out["pred"] == want.argmax()).all() and out["unmask"].all() and (out["done"] == 1).all()
