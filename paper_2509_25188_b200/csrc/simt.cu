@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__rest
   static_assert(KG >= 1 && KS % 4 == 0, "tiling");
   extern __shared__ __align__(16) float sm[];   // [F_STAGES][MATS][B][F_ROW]; the groups' sums at the end
   const int tid = threadIdx.x, grp = tid / TG, t = tid % TG, tx = t % (B / 4), ty = t / (B / 4);
-  const int m0 = blockIdx.y * B, n0 = blockIdx.x * B, n_st = (K + F_BK - 1) / F_BK;
+  const int m0 = (blockIdx.y + MAX_GRID_YZ * blockIdx.z) * B, n0 = blockIdx.x * B, n_st = (K + F_BK - 1) / F_BK;
+  if (m0 >= M) return;                          // row tiles beyond the grid's y go on in z
   auto load = [&](int st, bool act, bool wts) {
     float *d = sm + (st % F_STAGES) * MATS * MAT;
     for (int e = tid; e < B * (F_BK / 4); e += F_THREADS) {
@@ -446,7 +447,8 @@ cudaError_t launch_gemm_f32(cudaStream_t st, const float *A, const float *W, con
   const size_t smem = sizeof(float) * F_STAGES * (EPI == EPI_SWIGLU ? 3 : 2) * B * F_ROW;
   cudaError_t e = cudaFuncSetAttribute(gemm_f32_kernel<EPI, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_kernel(gemm_f32_kernel<EPI, B>, dim3(ceil_div(N, B), ceil_div(M, B)), dim3(F_THREADS), smem, st, A, W, W2, C, bias, M, N, K);
+  const int mt = ceil_div(M, B), y = mt < MAX_GRID_YZ ? mt : MAX_GRID_YZ;
+  return launch_kernel(gemm_f32_kernel<EPI, B>, dim3(ceil_div(N, B), y, ceil_div(mt, y)), dim3(F_THREADS), smem, st, A, W, W2, C, bias, M, N, K);
 }
 
 }  // namespace

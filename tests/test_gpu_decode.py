@@ -396,9 +396,9 @@ def test_fp32_scores_beyond_the_range_in_a_whole_key_tile():
     dec.close()
 
 
-@pytest.mark.parametrize("B", [65600])
+@pytest.mark.parametrize("B", [65600, 1048600])
 def test_fp32_batches_beyond_a_grid_dimension(B):
-    """More sequences than the y and z of a grid count (65,535).  All have the same prompt, so every row equals the first."""
+    """More sequences than the y and z of a grid count (65,535), then also more 32-row tiles (two rows a sequence).  All have the same prompt, so every row equals the first."""
     shape = wl.ModelShape(n_layers=1, d_model=8, n_heads=1, head_dim=8, d_ff=8, vocab=16, rms_eps=1e-5, rope_theta=1e4,
                           mask_id=15, eot_id=14, dtype="fp32")
     w = wl.make_weights(shape, seed=4, final_norm_gain=wl.spread_gain(shape))
