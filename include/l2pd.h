@@ -216,10 +216,11 @@ int64_t l2pd_collect_count(const l2pd_ctx *ctx);
  * mean over its samples and the s positions.  Arithmetic is fp32; a run is bit-reproducible on a given GPU.
  * d_c [N, s] float, d_y [N, s] uint8 (0 / 1): DEVICE.  d_w1 [s, s], d_b1 [s], d_w2 [s, s], d_b2 [s]: DEVICE fp32,
  * initial values in, trained values out.  h_losses: HOST [epochs * ceil(N / batch)] or NULL, the loss of every
- * update's batch measured before the update.  Runs on the current device, allocates and frees its scratch,
- * returns after the stream has finished.  Its launches take every SM for some 100 us each (one update, where that is
- * longer); kernels of other streams run between them.  s in [1, 64] (else L2PD_ERR_SHAPE); bad hyper-parameters L2PD_ERR_ARG;
- * L2PD_ERR_TIMEOUT when a bounded device-side wait ran out: the weights then keep their initial values.
+ * update's batch measured before the update.  Runs on the current device and returns after the stream has finished.
+ * Its launches take every SM for some 100 us each (one update, where that is longer); kernels of other streams run between
+ * them.  Of its scratch, at most 32 MB a device stay with the library for the next call, until l2pd_destroy.
+ * s in [1, 64] (else L2PD_ERR_SHAPE); bad hyper-parameters L2PD_ERR_ARG; L2PD_ERR_TIMEOUT when a bounded device-side wait ran
+ * out: the weights then keep their initial values.
  */
 typedef struct {
   float lr, beta1, beta2, eps, weight_decay;   /* the paper gives lr = 0.001; AdamW's published defaults: 0.9, 0.999, 1e-8, 0.01 */
@@ -325,7 +326,9 @@ float l2pd_last_step_ms(const l2pd_ctx *ctx);
 
 const char *l2pd_last_error(const l2pd_ctx *ctx);   /* never NULL; "" when there is none; ctx = NULL: what failed in
                                                         the calling thread's last context-free call (GEMM, LM head, ...) */
-void l2pd_destroy(l2pd_ctx *ctx);                   /* NULL is allowed */
+/* Also gives back the scratch that filter training keeps on the context's device; NULL is allowed and gives it back on
+ * every device (a process that trains without a context). */
+void l2pd_destroy(l2pd_ctx *ctx);
 
 /*
  * Stand-alone kernels of the step, exported for kernel-level tests and timing.

@@ -949,13 +949,20 @@ l2pd_status l2pd_set_collect(l2pd_ctx *c, float *d_c, uint8_t *d_y, int64_t capa
 int64_t l2pd_collect_count(const l2pd_ctx *c) { return c ? c->collect_n : 0; }
 
 // Scratch of the filter training: stream-ordered, from a pool of the library's own for each device that keeps at most 32 MB
-// between calls (a cudaMalloc and cudaFree pair took 0.7 ms of every call) and gives it back when a context is destroyed.
-static cudaMemPool_t train_pool(int dev) {
-  static cudaMemPool_t pools[64] = {};
-  static std::mutex mu;
-  if (dev < 0 || dev >= 64) return nullptr;
-  std::lock_guard<std::mutex> lock(mu);
-  if (!pools[dev]) {
+// between calls (cudaMalloc and cudaFree take 0.6 ms of every call, a pool made and destroyed by the call the same) and gives
+// it back in l2pd_destroy.
+namespace {
+constexpr int MAX_DEVICES = 64;
+struct TrainPools { std::mutex mu; cudaMemPool_t of[MAX_DEVICES] = {}; };
+TrainPools &train_pools() {
+  static TrainPools p;
+  return p;
+}
+cudaMemPool_t train_pool(int dev) {
+  if (dev < 0 || dev >= MAX_DEVICES) return nullptr;
+  TrainPools &p = train_pools();
+  std::lock_guard<std::mutex> lock(p.mu);
+  if (!p.of[dev]) {
     cudaMemPoolProps pr = {};
     pr.allocType = cudaMemAllocationTypePinned;
     pr.location.type = cudaMemLocationTypeDevice;
@@ -964,10 +971,18 @@ static cudaMemPool_t train_pool(int dev) {
     cudaMemPool_t q = nullptr;
     if (cudaMemPoolCreate(&q, &pr) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     if (cudaMemPoolSetAttribute(q, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) { cudaMemPoolDestroy(q); cudaGetLastError(); return nullptr; }
-    pools[dev] = q;
+    p.of[dev] = q;
   }
-  return pools[dev];
+  return p.of[dev];
 }
+// Gives back what the pools hold and no call uses: the one of `dev`, or all of them (-1).
+void train_pools_trim(int dev) {
+  TrainPools &p = train_pools();
+  std::lock_guard<std::mutex> lock(p.mu);
+  for (int i = 0; i < MAX_DEVICES; ++i)
+    if (p.of[i] && (dev < 0 || dev == i)) cudaMemPoolTrimTo(p.of[i], 0);
+}
+}  // namespace
 
 // What the test hook sets: updates per launch (0: chosen), the bound of a meeting's wait, and a launch whose meetings are one
 // arrival short (-1: none).
@@ -1127,10 +1142,10 @@ int64_t l2pd_chain_trace_read(l2pd_ctx *c, uint64_t *h_out, int64_t capacity, in
 }
 
 void l2pd_destroy(l2pd_ctx *c) {
-  if (!c) return;
+  if (!c) return train_pools_trim(-1);
   cudaSetDevice(c->device);
   cudaDeviceSynchronize();
-  if (cudaMemPool_t pool = train_pool(c->device)) cudaMemPoolTrimTo(pool, 0);
+  train_pools_trim(c->device);
   free_all(c);
   delete c;
 }

@@ -265,3 +265,20 @@ def test_gradients_of_small_batches_keep_their_accuracy(s, n, depth):
                 worst = max(worst, np.linalg.norm(a0.astype(np.float64) - a - want) / np.linalg.norm(want))
         errs.append(worst)
     assert np.median(errs) < 2.0 ** -23
+
+
+def test_the_kept_scratch_is_bounded_and_given_back():
+    """A training keeps at most 32 MB of device memory for the next; l2pd_destroy(NULL) gives it back without a context."""
+    import torch
+    b = _b()
+    C, Y = _data(64, 2000, seed=4)
+    c, y = torch.from_numpy(C).cuda(), torch.from_numpy(Y).cuda()
+    layers = [(np.eye(64, dtype=np.float32), np.zeros(64, np.float32))] * 4
+    b.filter_train_layers(layers, c, y, 2)
+    b.lib.l2pd_destroy(None)
+    free0 = torch.cuda.mem_get_info()[0]
+    b.filter_train_layers(layers, c, y, 2)
+    kept = free0 - torch.cuda.mem_get_info()[0]
+    assert 0 < kept <= 32 << 20
+    b.lib.l2pd_destroy(None)
+    assert torch.cuda.mem_get_info()[0] == free0
