@@ -7,6 +7,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <memory>
 #include <mutex>
 #include <new>
 #include <string>
@@ -1005,6 +1006,10 @@ static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t
   const int64_t per_epoch = (N + bs - 1) / bs, updates = per_epoch * t->epochs;
   // one allocation: theta, m, v | the blocks' gradient sums | losses | meeting counter, status
   const size_t n_sums = (size_t)filter_train_max_rows(N < bs ? N : bs, sms) * filter_train_row_floats(P), n_loss = (size_t)(updates > 0 ? updates : 1);
+  // what comes back to the host, losses and status in one copy: they lie behind one another
+  const size_t n_back = h_losses ? n_loss + 2 : 2;
+  std::unique_ptr<float[]> back(new (std::nothrow) float[n_back]);
+  if (!back) return L2PD_ERR_OOM;
   float *theta = nullptr;
   cudaMemPool_t pool = train_pool(dev);
   if (!pool || cudaMallocFromPoolAsync((void **)&theta, sizeof(float) * (3 * (size_t)P + n_sums + n_loss + 8), pool, st) != cudaSuccess) return L2PD_ERR_OOM;
@@ -1032,16 +1037,13 @@ static l2pd_status filter_train_impl(void *stream, int32_t s, int32_t L, int64_t
   }
   for (cudaEvent_t e : done) if (e) cudaEventDestroy(e);
   if (ok) ok = launch_filter_pack(st, w, b, s, L, theta, d_status, bar, false) == cudaSuccess;
-  // losses and status in one copy: they lie behind one another
-  const size_t n_back = h_losses ? n_loss + 2 : 2;
-  std::vector<float> back(n_back);
-  if (ok) ok = cudaMemcpyAsync(back.data(), losses + (n_loss + 2 - n_back), sizeof(float) * n_back, cudaMemcpyDeviceToHost, st) == cudaSuccess;
+  if (ok) ok = cudaMemcpyAsync(back.get(), losses + (n_loss + 2 - n_back), sizeof(float) * n_back, cudaMemcpyDeviceToHost, st) == cudaSuccess;
   ok = (cudaFreeAsync(theta, st) == cudaSuccess) && ok;
   ok = (cudaStreamSynchronize(st) == cudaSuccess) && ok;
   int32_t h_stat = DEV_OK;
   memcpy(&h_stat, &back[n_back - 1], 4);
   if (ok && h_stat != DEV_OK) return L2PD_ERR_TIMEOUT;
-  if (ok && h_losses && updates > 0) memcpy(h_losses, back.data(), sizeof(float) * updates);
+  if (ok && h_losses && updates > 0) memcpy(h_losses, back.get(), sizeof(float) * updates);
   return ok ? L2PD_OK : L2PD_ERR_CUDA;
 }
 

@@ -282,3 +282,28 @@ def test_the_kept_scratch_is_bounded_and_given_back():
     assert 0 < kept <= 32 << 20
     b.lib.l2pd_destroy(None)
     assert torch.cuda.mem_get_info()[0] == free0
+
+
+def test_losses_beyond_the_host_memory_are_an_error():
+    """The copy of the losses (32 MB here) cannot be allocated in a process whose address space is limited: the call says so,
+    before any launch, and nothing is thrown through the C interface."""
+    import subprocess
+    import sys
+    code = """
+import ctypes, resource
+import numpy as np, torch
+from paper_2509_25188_b200 import binding as b
+c, y = torch.zeros(1, 1, device="cuda"), torch.zeros(1, 1, dtype=torch.uint8, device="cuda")
+p = [torch.ones(1, device="cuda") for _ in range(4)]
+losses = np.zeros(8 << 20, np.float32)
+def train(epochs):
+    cfg = b.TrainConfig(1e-3, 0.9, 0.999, 1e-8, 0.01, epochs, 0)
+    return b.lib.l2pd_filter_train(None, 1, 1, c.data_ptr(), y.data_ptr(), *[t.data_ptr() for t in p], ctypes.byref(cfg), losses.ctypes.data)
+assert train(3) == 0
+torch.cuda.synchronize()
+size = int(next(l for l in open("/proc/self/status") if l.startswith("VmSize")).split()[1]) << 10
+resource.setrlimit(resource.RLIMIT_AS, (size + (16 << 20), resource.RLIM_INFINITY))
+print("status", train(8 << 20))
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "status -3" in r.stdout, r.stdout + r.stderr
