@@ -35,7 +35,7 @@ struct TrainArgs {
   const uint8_t *Y;        // [N, s] targets (0 / 1)
   int64_t N, batch;        // samples; samples per update (the last batch of an epoch may be shorter)
   int64_t u0, u1;          // this launch's updates
-  int per_epoch;           // updates per epoch
+  int64_t per_epoch;       // updates per epoch
   int s, n_layers, P;      // P parameters
   float *theta, *m, *v;    // packed per layer: W_k [s*s], b_k [s]
   float *gpart;            // a row per block: gradient sums, then the loss sum
@@ -459,7 +459,7 @@ cudaError_t launch_filter_train(cudaStream_t st, FilterTrainArgs &f, int64_t u0,
   if (f.n_layers < 1 || f.n_layers > MAX_LAYERS || f.s < 1 || f.s > MAX_S) return cudaErrorInvalidValue;
   TrainArgs a;
   a.C = f.C; a.Y = f.Y; a.N = f.N; a.batch = f.batch; a.u0 = u0; a.u1 = u1;
-  a.per_epoch = (int)((f.N + f.batch - 1) / f.batch);
+  a.per_epoch = (f.N + f.batch - 1) / f.batch;
   a.s = f.s; a.n_layers = f.n_layers; a.P = f.n_layers * (f.s * f.s + f.s);
   a.theta = f.theta; a.m = f.m; a.v = f.v; a.gpart = f.gpart; a.losses = f.losses;
   a.lr = f.h.lr; a.beta1 = f.h.beta1; a.beta2 = f.h.beta2; a.eps = f.h.eps; a.weight_decay = f.h.weight_decay;
