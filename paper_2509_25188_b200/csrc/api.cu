@@ -359,8 +359,12 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     c->tc_rows = T_rows;
   }
 
-  CKLK(L2PD_K_EMBED, launch_step_begin<T>(s, c->h_meta, n_slots, c->d_meta, c->d_row_slot, c->d_row_pos, c->d_tokens, c->P + c->G,
-                              (const T *)c->tok_emb, c->norm1[0], f.rms_eps, c->x, n, T_rows, d));
+  const bool described = n_slots <= STEP_META_BATCH;   // by the embedding's argument
+  for (int k = 0; !described && k < n_slots; k += STEP_META_BATCH)
+    CKLK(L2PD_K_OTHER, launch_build_row_map(s, c->h_meta, k, n_slots - k < STEP_META_BATCH ? n_slots - k : STEP_META_BATCH, c->d_meta,
+                                            c->d_row_slot, c->d_row_pos));
+  CKLK(L2PD_K_EMBED, launch_embed_rmsnorm<T>(s, described ? c->h_meta : nullptr, n_slots, c->d_meta, c->d_row_slot, c->d_row_pos,
+                                             c->d_tokens, c->P + c->G, (const T *)c->tok_emb, c->norm1[0], f.rms_eps, c->x, n, T_rows, d));
   if (c->cap) CK(cudaMemcpyAsync(c->cap, c->x, (size_t)T_rows * d * 4, cudaMemcpyDeviceToDevice, s));
 
   // The chained form of the layer loop: QKV of layer 0 alone, then per layer the attention kernel and ONE launch that

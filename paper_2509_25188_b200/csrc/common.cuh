@@ -75,12 +75,15 @@ template <> __device__ __forceinline__ bf16 from_f32<bf16>(float v) { return __f
 // ---- launchers implemented in the .cu files -------------------------------------------------------
 
 // elementwise.cu
-// A step's first kernels: the descriptions of its sequences (host memory) -> meta, the maps row -> slot and row -> position,
-// x = the rows' embeddings, n = RMSNorm(x)
+// A step's first kernel.  Up to STEP_META_BATCH sequences: the embedding, which takes their descriptions (h_meta, host memory)
+// as an argument and stores them and the maps row -> slot and row -> position; x = the rows' embeddings, n = RMSNorm(x).
+// More: launch_build_row_map for STEP_META_BATCH of them at a time, then the embedding with h_meta = nullptr.
+constexpr int STEP_META_BATCH = 64;
+cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, int slot0, int n, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos);
 template <typename T>
-cudaError_t launch_step_begin(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
-                              int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
-                              const float *gain, float eps, float *x, T *n, int rows, int d);
+cudaError_t launch_embed_rmsnorm(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
+                                 int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
+                                 const float *gain, float eps, float *x, T *n, int rows, int d);
 // n = RMSNorm(x).  With n_part > 0, first x += part[0] + part[1] + ... (slice s at part + s * part_stride elements,
 // added in that order) and x is written back: the fixed-order end of a K-split projection.
 template <typename T>

@@ -46,7 +46,7 @@ template <> struct Vec8<float> {
   __device__ __forceinline__ void set(int i, float f) { reinterpret_cast<float *>(&a)[i] = f; }
 };
 
-constexpr int META_BATCH = 64;
+constexpr int META_BATCH = STEP_META_BATCH;
 struct MetaBatch { SeqMeta m[META_BATCH]; };
 
 // x[row,:] = emb[token,:];  n[row,:] = x * g / sqrt(mean(x^2) + eps)
@@ -430,30 +430,26 @@ __global__ void gather_response_kernel(const int32_t *tokens, int P, int G, int3
 
 }  // namespace
 
-template <typename T>
-cudaError_t launch_step_begin(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
-                              int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
-                              const float *gain, float eps, float *x, T *n, int rows, int d) {
-  // The first launch is an ordinary one, which starts when all earlier work of the stream is complete: the kernels behind it
-  // read weights before their own wait.
+// A step's first launch, of these two, is an ordinary one, which starts when all earlier work of the stream is complete: the
+// kernels behind it read weights before their own wait.
+cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, int slot0, int n, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos) {
+  if (n < 1 || n > META_BATCH) return cudaErrorInvalidValue;
   MetaBatch b;
-  auto fill = [&](int slot0) {
-    const int k = n_slots - slot0 < META_BATCH ? n_slots - slot0 : META_BATCH;
-    for (int i = 0; i < k; ++i) b.m[i] = h_meta[slot0 + i];
-    return k;
-  };
-  if (n_slots <= META_BATCH) {
-    const int k = fill(0);
-    embed_rmsnorm_kernel<T><<<rows, 256, 0, st>>>(b, k, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
-    return cudaGetLastError();
-  }
-  for (int slot0 = 0; slot0 < n_slots; slot0 += META_BATCH) {
-    const int k = fill(slot0);
-    build_row_map_kernel<<<k, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return launch_kernel(embed_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, b, 0, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
+  for (int i = 0; i < n; ++i) b.m[i] = h_meta[slot0 + i];
+  build_row_map_kernel<<<n, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos);
+  return cudaGetLastError();
+}
+template <typename T>
+cudaError_t launch_embed_rmsnorm(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
+                                 int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
+                                 const float *gain, float eps, float *x, T *n, int rows, int d) {
+  MetaBatch b;
+  if (!h_meta)
+    return launch_kernel(embed_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, b, 0, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
+  if (n_slots < 1 || n_slots > META_BATCH) return cudaErrorInvalidValue;
+  for (int i = 0; i < n_slots; ++i) b.m[i] = h_meta[i];
+  embed_rmsnorm_kernel<T><<<rows, 256, 0, st>>>(b, n_slots, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
+  return cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_rmsnorm(cudaStream_t st, float *x, const float *gain, float eps, T *n,
@@ -507,8 +503,8 @@ cudaError_t launch_gather_response(cudaStream_t st, const int32_t *tokens, int B
 }
 
 #define INSTANTIATE(T)                                                                              \
-  template cudaError_t launch_step_begin<T>(cudaStream_t, const SeqMeta *, int, SeqMeta *, int32_t *, int32_t *, \
-                                            const int32_t *, int64_t, const T *, const float *, float, float *, T *, int, int); \
+  template cudaError_t launch_embed_rmsnorm<T>(cudaStream_t, const SeqMeta *, int, SeqMeta *, int32_t *, int32_t *, \
+                                               const int32_t *, int64_t, const T *, const float *, float, float *, T *, int, int); \
   template cudaError_t launch_rmsnorm<T>(cudaStream_t, float *, const float *, float, T *,           \
                                          int, int, const float *, int, int64_t);                     \
   template cudaError_t launch_rope_scatter<T>(cudaStream_t, const T *, const SeqMeta *,              \

@@ -411,3 +411,20 @@ def test_fp32_batches_beyond_a_grid_dimension(B):
     assert np.abs(out["logits"][0, 0] - want).max() <= 1e-4 * np.abs(want).max()
     assert np.array_equal(out["logits"], np.broadcast_to(out["logits"][:1], out["logits"].shape))
     assert (out["pred"] == want.argmax()).all() and out["unmask"].all() and (out["done"] == 1).all()
+
+
+def test_every_launch_of_a_step_is_counted():
+    """A launch describes up to 64 sequences: more of them take further launches, which the count and the timing list."""
+    shape, w = _tiny()
+    filt = wl.make_filter(4, 0.96, seed=0)
+    counts = {}
+    for B in (64, 65, 129):
+        dec = _b().Decoder(shape, w, filt, block_len=4, max_batch=B, max_seq=7)
+        dec.state_reset(wl.make_prompts(B, 3, shape, seed=4), 4)
+        dec.profile_enable(["other"])
+        before = dec.launch_count
+        dec.denoise_step(outputs=False)
+        counts[B] = (dec.launch_count - before, dec.profile_read().get("other", (0.0, 0))[1])
+        dec.close()
+    n = counts[64][0]
+    assert counts == {64: (n, 0), 65: (n + 2, 2), 129: (n + 3, 3)}
