@@ -167,8 +167,7 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__rest
   static_assert(KG >= 1 && KS % 4 == 0, "tiling");
   extern __shared__ __align__(16) float sm[];   // [F_STAGES][MATS][B][F_ROW]; the groups' sums at the end
   const int tid = threadIdx.x, grp = tid / TG, t = tid % TG, tx = t % (B / 4), ty = t / (B / 4);
-  const int m0 = (blockIdx.y + MAX_GRID_YZ * blockIdx.z) * B, n0 = blockIdx.x * B, n_st = (K + F_BK - 1) / F_BK;
-  if (m0 >= M) return;                          // row tiles beyond the grid's y go on in z
+  const int m0 = blockIdx.y * B, n0 = blockIdx.x * B, n_st = (K + F_BK - 1) / F_BK;
   auto load = [&](int st, bool act, bool wts) {
     float *d = sm + (st % F_STAGES) * MATS * MAT;
     for (int e = tid; e < B * (F_BK / 4); e += F_THREADS) {
@@ -266,15 +265,12 @@ __global__ void __launch_bounds__(F_THREADS) gemm_f32_kernel(const float *__rest
 constexpr int A_Q = 8, A_K = 64, A_THREADS = 16 * A_Q;
 __global__ void __launch_bounds__(A_THREADS) attention_f32_kernel(const float *__restrict__ q, const float *__restrict__ kc,
                                                             const float *__restrict__ vc, const SeqMeta *meta, float *out,
-                                                            int64_t kv_seq_stride, int H, int dh, int bufs, int n_slots, int n_qt) {
+                                                            int64_t kv_seq_stride, int H, int dh, int bufs) {
   extern __shared__ __align__(16) float sm[];
   grid_dep_launch();
-  int slot = blockIdx.z, qt = blockIdx.x;
-  while (qt >= n_qt) { qt -= n_qt; slot += MAX_GRID_YZ; }   // more sequences than the grid's z has room for
-  if (slot >= n_slots) return;
   grid_dep_wait();
-  const SeqMeta m = meta[slot];
-  const int q0 = qt * A_Q, h = blockIdx.y, hd = H * dh, tid = threadIdx.x, r = tid >> 4, l = tid & 15;
+  const SeqMeta m = meta[blockIdx.z];
+  const int q0 = blockIdx.x * A_Q, h = blockIdx.y, hd = H * dh, tid = threadIdx.x, r = tid >> 4, l = tid & 15;
   if (q0 >= m.n_rows) return;
   const int stride = (dh + 3) / 4 * 4 + 4, sk = A_K + 4;
   float *const Q = sm, *const S = Q + A_Q * stride, *const KV = S + A_Q * sk;   // S [A_Q][sk], KV [bufs][K then V][A_K][stride]
@@ -447,8 +443,7 @@ cudaError_t launch_gemm_f32(cudaStream_t st, const float *A, const float *W, con
   const size_t smem = sizeof(float) * F_STAGES * (EPI == EPI_SWIGLU ? 3 : 2) * B * F_ROW;
   cudaError_t e = cudaFuncSetAttribute(gemm_f32_kernel<EPI, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const int mt = ceil_div(M, B), y = mt < MAX_GRID_YZ ? mt : MAX_GRID_YZ;
-  return launch_kernel(gemm_f32_kernel<EPI, B>, dim3(ceil_div(N, B), y, ceil_div(mt, y)), dim3(F_THREADS), smem, st, A, W, W2, C, bias, M, N, K);
+  return launch_kernel(gemm_f32_kernel<EPI, B>, dim3(ceil_div(N, B), ceil_div(M, B)), dim3(F_THREADS), smem, st, A, W, W2, C, bias, M, N, K);
 }
 
 }  // namespace
@@ -458,12 +453,13 @@ cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, c
                              const float *bias, int M, int N, int K) {
   if constexpr (std::is_same<T, float>::value) {
     const uintptr_t bits = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(W2);
-    if ((bits & 15) == 0 && (K & 3) == 0) {
-      // 32 x 32 tiles until 64 x 64 ones give every SM two blocks (SwiGLU, two weight tiles: no more than 32 x 32); 16 x 16 tiles
-      // as long as 32 x 32 ones fill at most every second SM.  Tiny decode of 96 rows, 32 x 32 alone 4.00 ms, 16 x 16 up to 37 blocks
-      // (O, down) 3.36, up to 74 (QKV and gate/up too) 3.13
-      auto blocks = [&](int b) { return (int64_t)ceil_div(N, b) * ceil_div(M, b); };
-      const int tile = blocks(64) >= 296 && epi != EPI_SWIGLU ? 64 : (blocks(32) <= 74 ? 16 : 32);
+    // 32 x 32 tiles until 64 x 64 ones give every SM two blocks (SwiGLU, two weight tiles: no more than 32 x 32); 16 x 16 tiles
+    // as long as 32 x 32 ones fill at most every second SM.  Tiny decode of 96 rows, 32 x 32 alone 4.00 ms, 16 x 16 up to 37 blocks
+    // (O, down) 3.36, up to 74 (QKV and gate/up too) 3.13
+    auto blocks = [&](int b) { return (int64_t)ceil_div(N, b) * ceil_div(M, b); };
+    const int tile = blocks(64) >= 296 && epi != EPI_SWIGLU ? 64 : (blocks(32) <= 74 ? 16 : 32);
+    // more row tiles than a grid's y (SwiGLU of 2.1 million rows): the plain kernel below with its 64-row tiles
+    if ((bits & 15) == 0 && (K & 3) == 0 && ceil_div(M, tile) <= MAX_GRID_YZ) {
       float *Cf = reinterpret_cast<float *>(C);
 #define L2PD_F32(E)                                                                                      \
   case E: return tile == 16 ? launch_gemm_f32<E, 16>(st, A, W, W2, Cf, bias, M, N, K)                    \
@@ -495,14 +491,16 @@ template <typename T>
 cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, const T *vc,
                                   const SeqMeta *meta, const int32_t *row_slot, T *out,
                                   int64_t kv_seq_stride, int rows, int H, int dh, int max_kv, int n_slots, int max_q) {
+  // the grid's z holds the sequences; of more of them, a block per row and head takes any number
   if constexpr (std::is_same<T, float>::value) {   // q, K and V are the library's own buffers: rows of H * dh floats, 16-byte aligned
-    auto bytes = [&](int bufs) { return (int)(sizeof(float) * ((size_t)(A_Q + 2 * bufs * A_K) * ((dh + 3) / 4 * 4 + 4) + A_Q * (A_K + 4))); };
-    const int bufs = max_kv > A_K && bytes(2) <= 200 * 1024 ? 2 : 1;
-    cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(bufs));
-    if (e != cudaSuccess) return e;
-    const int n_qt = ceil_div(max_q, A_Q), z = n_slots < MAX_GRID_YZ ? n_slots : MAX_GRID_YZ;
-    return launch_kernel(attention_f32_kernel, dim3(n_qt * ceil_div(n_slots, z), H, z), dim3(A_THREADS), (size_t)bytes(bufs), st, q, kc, vc,
-                         meta, out, kv_seq_stride, H, dh, bufs, n_slots, n_qt);
+    if (n_slots <= MAX_GRID_YZ) {
+      auto bytes = [&](int bufs) { return (int)(sizeof(float) * ((size_t)(A_Q + 2 * bufs * A_K) * ((dh + 3) / 4 * 4 + 4) + A_Q * (A_K + 4))); };
+      const int bufs = max_kv > A_K && bytes(2) <= 200 * 1024 ? 2 : 1;
+      cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(bufs));
+      if (e != cudaSuccess) return e;
+      return launch_kernel(attention_f32_kernel, dim3(ceil_div(max_q, A_Q), H, n_slots), dim3(A_THREADS), (size_t)bytes(bufs), st, q, kc, vc,
+                           meta, out, kv_seq_stride, H, dh, bufs);
+    }
   }
   size_t smem = (size_t)(dh + max_kv) * sizeof(float);
   if (smem > 48 * 1024) {
