@@ -290,22 +290,16 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
       }
     }
     const int max_ks = (c->ksum == nullptr || T_rows <= c->ksum_rows) ? 4 : 1;   // K slices need their partial-sum area
-    if (small_chain) {
-      c->pl_qkv = plan_gemm_pair_one_slab(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 1, CHAIN_TILE_N);
-      c->pl_o = plan_gemm_pair_one_slab(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, max_ks, CHAIN_TILE_N);
-      c->pl_down = plan_gemm_pair_one_slab(EPI_RESIDUAL, T_rows, d, F, c->num_sms, max_ks, CHAIN_TILE_N);
-      c->pl_gu = plan_gemm_pair_one_slab(EPI_SWIGLU, T_rows, F, d, c->num_sms, 1, CHAIN_TILE_N);
-    } else {
-      c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0);
-      c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks);
-      c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks);
-      c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0);
-      if (big_chain) {
-        c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0, 1, CHAIN_TILE_N, 2);
-        c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks, CHAIN_TILE_N, 2, c->pl_o.k_splits);
-        c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks, CHAIN_TILE_N, 2, c->pl_down.k_splits);
-        c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0, 1, CHAIN_TILE_N, 2);
-      }
+    c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0);
+    c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks);
+    c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks);
+    c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0);
+    if (small_chain || big_chain) {
+      const int slabs = big_chain ? 2 : 1, ks_o = big_chain ? c->pl_o.k_splits : 0, ks_d = big_chain ? c->pl_down.k_splits : 0;
+      c->pl_qkv = plan_gemm_chained(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, slabs, 1, CHAIN_TILE_N);
+      c->pl_o = plan_gemm_chained(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, slabs, max_ks, CHAIN_TILE_N, ks_o);
+      c->pl_down = plan_gemm_chained(EPI_RESIDUAL, T_rows, d, F, c->num_sms, slabs, max_ks, CHAIN_TILE_N, ks_d);
+      c->pl_gu = plan_gemm_chained(EPI_SWIGLU, T_rows, F, d, c->num_sms, slabs, 1, CHAIN_TILE_N);
     }
     int box = c->pl_qkv.tile_n / c->pl_qkv.cta_group;
     if (box != c->box_qkv) { l2pd_status r = encode_weight_maps(c, c->tb_qkv, c->wqkv, 3 * hd, d, box); if (r) return r; c->box_qkv = box; }

@@ -195,11 +195,8 @@ void set_standalone_error(const char *fmt, ...);
 // accumulators that the epilogue adds.  No plan asks for it by itself (one issuer keeps up with the weight stream:
 // 32 rows, QKV 20.2 us against 23.9); chained launches of few rows and explicit requests do.
 struct GemmPlan { int cta_group, tile_n, k_splits, slabs, k_interleave; };
-// max_tile_n caps the tile width (a kernel that chains several projections keeps one ring geometry for all of them)
-// force_slabs / force_ks: 0 = chosen
-GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits = 4, int max_tile_n = 256,
-                   int force_slabs = 0, int force_ks = 0);
-GemmPlan plan_gemm_pair_one_slab(int epi, int M, int N, int K, int num_sms, int max_k_splits, int max_tile_n);
+GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits = 4);
+GemmPlan plan_gemm_chained(int epi, int M, int N, int K, int num_sms, int slabs, int max_k_splits, int max_tile_n, int force_ks = 0);
 int effective_k_splits(int K, int k_splits);   // what the launcher makes of a requested K split
 struct GemmArgs {
   int epi;                 // EPI_STORE, EPI_RESIDUAL, EPI_SWIGLU, or EPI_LMHEAD

@@ -527,7 +527,7 @@ static double plan_cost(int M, int N, int K, int num_sms, int cg, int slabs, int
   return span;
 }
 
-GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits, int max_tile_n, int force_slabs, int force_ks) {
+GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits) {
   GemmPlan best{1, 256, 1, 1, 0};
   double best_cost = 1e300;
   const bool swiglu = epi == EPI_SWIGLU;
@@ -537,14 +537,11 @@ GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, 
     for (int slabs = 1; slabs <= 2; ++slabs) {
       // a second slab: the weight tile is read once for twice the rows
       if (slabs == 2 && (cg == 1 || epi == EPI_LMHEAD || M <= TILE_M * cg)) continue;
-      if (force_slabs && slabs != force_slabs) continue;
       for (int tn = 256; tn >= 64; tn -= step) {
         if (force_tile_n && tn != force_tile_n) continue;
-        if (!force_tile_n && tn > max_tile_n) continue;
         const int unit_n = swiglu ? tn / 2 : tn;
         const int max_ks = (epi == EPI_RESIDUAL) ? (max_k_splits < 4 ? max_k_splits : 4) : 1;
         for (int ks = 1; ks <= max_ks; ++ks) {
-          if (force_ks && ks != force_ks) continue;
           if (ks > 1 && ceil_div(K, TILE_K) < 8 * ks) break;
           const double c = plan_cost(M, N, K, num_sms, cg, slabs, unit_n, tn, ks, epi == EPI_RESIDUAL);
           if (c < best_cost - 1e-9) { best_cost = c; best = GemmPlan{cg, tn, ks, slabs, 0}; }
@@ -556,19 +553,30 @@ GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, 
   return best;
 }
 
-// The plan of a step of few rows inside a chained launch: SM pairs, one 256-row slab per unit, the two MMA issuers on
-// alternate k-blocks; tile width and K slices by the same cost model.
-GemmPlan plan_gemm_pair_one_slab(int epi, int M, int N, int K, int num_sms, int max_k_splits, int max_tile_n) {
-  GemmPlan best{2, max_tile_n < 176 ? max_tile_n : 176, 1, 1, 1};
+// The plan of a projection inside a chained launch: SM pairs, tiles at most max_tile_n wide, and either two row slabs per unit
+// or (at most 256 rows) one with the two MMA issuers on alternate k-blocks.  force_ks: 0 = chosen.  Modelled on the chained
+// kernel, whose loops decide per k-block and whose ring is shared by all its projections: a k-block takes the pipe's
+// 2 tile_n cycles per slab, 620 of its issuer (330 where two alternate) or its bytes at 58 a cycle; a unit adds 6000 and its
+// drain, exposed with two slabs.  Chained steps of four 8B layers, planned by the single launches' model -> by this: 256 rows
+// 1.039 -> 1.004 ms, 512 rows 1.336 -> 1.286 (gate/up in two rounds of 176 columns, not three of 112), 1536 rows 2.47 -> 2.42.
+GemmPlan plan_gemm_chained(int epi, int M, int N, int K, int num_sms, int slabs, int max_k_splits, int max_tile_n, int force_ks) {
+  GemmPlan best{2, max_tile_n < 176 ? max_tile_n : 176, 1, slabs, slabs == 1 ? 1 : 0};
   double best_cost = 1e300;
+  const bool is_residual = epi == EPI_RESIDUAL;
   for (int tn = 256; tn >= 64; tn -= 16) {
     if (tn > max_tile_n) continue;
     const int unit_n = epi == EPI_SWIGLU ? tn / 2 : tn;
-    const int max_ks = (epi == EPI_RESIDUAL) ? (max_k_splits < 4 ? max_k_splits : 4) : 1;
+    const int max_ks = is_residual ? (max_k_splits < 4 ? max_k_splits : 4) : 1;
     for (int ks = 1; ks <= max_ks; ++ks) {
-      if (ceil_div(K, TILE_K) < 8 * ks) break;
-      const double c = plan_cost(M, N, K, num_sms, 2, 1, unit_n, tn, ks, epi == EPI_RESIDUAL);
-      if (c < best_cost - 1e-9) { best_cost = c; best = GemmPlan{2, tn, ks, 1, 1}; }
+      if (force_ks && ks != force_ks) continue;
+      if (ks > 1 && ceil_div(K, TILE_K) < 8 * ks) break;
+      const double bytes = (double)slabs * A_STAGE_BYTES + 64.0 * tn;
+      const double per_kb = 1.06 * fmax(fmax(2.0 * tn * slabs, slabs == 1 ? 330.0 : 620.0), bytes / 58.0);
+      // bf16 stores leave an SM at 34 B a cycle, additions into X at 17, partial sums at 34
+      const double drain = (double)TILE_M * slabs * unit_n * (is_residual ? (ks > 1 ? 4.0 / 34.0 : 4.0 / 17.0) : 2.0 / 34.0) + 1500.0;
+      const int waves = ceil_div(ceil_div(M, 2 * TILE_M * slabs) * ceil_div(N, unit_n) * ks, num_sms / 2);
+      const double c = waves * (ceil_div(ceil_div(K, TILE_K), ks) * per_kb + 6000.0 + (slabs == 2 ? drain : 0.3 * drain)) + (slabs == 2 ? 0.0 : 0.7 * drain);
+      if (c < best_cost - 1e-9) { best_cost = c; best.tile_n = tn; best.k_splits = ks; }
     }
   }
   return best;

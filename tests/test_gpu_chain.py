@@ -37,7 +37,7 @@ def _steps(dec, prompts, G, n_steps, chain):
 @pytest.mark.parametrize("layers,B,P,G", [(3, 1, 256, 256),      # the 8B step shape: 512 rows, two row slabs per unit
                                           (2, 1, 300, 128),      # 428 rows: a ragged second slab
                                           (2, 2, 320, 192),      # two sequences, 1024 rows: two row tiles per projection
-                                          (2, 3, 256, 256)])     # 1536 rows: an output projection without K slices
+                                          (2, 3, 256, 256)])     # 1536 rows: three row tiles, the most that chain
 def test_chained_step_equals_unchained(layers, B, P, G):
     import torch
     from paper_2509_25188_b200 import binding
@@ -62,6 +62,29 @@ def test_chained_step_equals_unchained(layers, B, P, G):
         for k in ("logits", "conf", "pred", "p", "unmask", "masks_left", "l_eff", "done", "forced"):
             assert np.array_equal(sa[k], sb[k]), "chained and unchained steps differ in %s" % k
     assert np.array_equal(tok_a, tok_b)
+
+
+@pytest.mark.parametrize("B,P,G", [(1, 172, 128), (2, 172, 128)])   # 300 and 600 rows: one and two row tiles
+def test_chained_step_with_k_slices_equals_unchained(B, P, G):
+    """The 8B projections of these row counts have no K slices; the down projection of a narrow model with a long K has
+    three or four, whose partial sums the RMSNorm phase takes in.  All three modes agree bit for bit."""
+    from paper_2509_25188_b200 import binding
+    shape = wl.ModelShape(n_layers=3, d_model=512, n_heads=4, head_dim=128, d_ff=8192, vocab=1000, rms_eps=1e-5,
+                          rope_theta=500000.0, mask_id=999, eot_id=998, dtype="bf16")
+    dec = binding.Decoder(shape, _device_weights(shape), wl.make_filter(32, 0.96, seed=0), block_len=32, max_batch=B, max_seq=P + G)
+    prompts = wl.make_prompts(B, P, shape, seed=5)
+    dec.profile_enable(["other", "gemm_chain"])
+    plain, tok = _steps(dec, prompts, G, 3, chain=0)
+    # single launches: the last layer's slices are added by a kernel of its own, so there are slices
+    assert dec.profile_read().get("other", (0.0, 0))[1] == 3 and "gemm_chain" not in dec.profile_read()
+    for mode in (1, 2):
+        got, tok_m = _steps(dec, prompts, G, 3, chain=mode)
+        assert dec.profile_read().get("gemm_chain", (0.0, 0))[1] == 3 * 4              # (mode 1 chains: QKV and a launch per layer)
+        for a, b in zip(got, plain):
+            for k in ("logits", "conf", "pred", "p", "unmask", "masks_left", "l_eff", "done", "forced"):
+                assert np.array_equal(a[k], b[k]), "mode %d and mode 0 differ in %s" % (mode, k)
+        assert np.array_equal(tok_m, tok)
+    dec.close()
 
 
 def test_chain_trace_records_every_phase():
