@@ -223,7 +223,7 @@ l2pd_status encode_weight_maps(l2pd_ctx *c, std::vector<TmaDesc> &dst, const std
 template <typename T>
 l2pd_status run_gemm_simt(l2pd_ctx *c, cudaStream_t s, int kind, int epi, const void *A, const void *W,
                           const void *W2, void *out, const float *bias, int M, int N, int K) {
-  CKLK(kind, launch_simt_gemm<T>(s, epi, (const T *)A, (const T *)W, (const T *)W2, out, bias, M, N, K));
+  CKLK(kind, launch_simt_gemm<T>(s, epi, (const T *)A, (const T *)W, (const T *)W2, out, bias, M, N, K, c->num_sms));
   return L2PD_OK;
 }
 

@@ -112,7 +112,7 @@ cudaError_t launch_gather_response(cudaStream_t st, const int32_t *tokens, int B
 enum { EPI_STORE = 0, EPI_RESIDUAL = 1, EPI_SWIGLU = 2, EPI_STORE_F32 = 3, EPI_LMHEAD = 4, EPI_QKV_ROPE = 5 };
 template <typename T>
 cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, const T *W2, void *C,
-                             const float *bias, int M, int N, int K);
+                             const float *bias, int M, int N, int K, int num_sms);
 template <typename T>
 cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, const T *vc,
                                   const SeqMeta *meta, const int32_t *row_slot, T *out,

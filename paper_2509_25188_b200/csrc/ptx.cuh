@@ -62,8 +62,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Waits for the phase with the given parity to complete; false after `limit_ns` nanoseconds.  For a whole converged warp: every lane gets the same answer, so that the warp stays together behind it (the
-// warp-wide instructions that follow would wait for ever for a lane that gave up on its own).
+// Waits for the phase with the given parity to complete; false after `limit_ns` nanoseconds.  For a whole converged warp:
+// every lane gets the same answer, so that the warp stays together behind it (the warp-wide instructions that follow would
+// wait for ever for a lane that gave up on its own).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t limit_ns = 2000000000ull) {
   if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
   const uint64_t t0 = globaltimer();

@@ -450,14 +450,14 @@ cudaError_t launch_gemm_f32(cudaStream_t st, const float *A, const float *W, con
 
 template <typename T>
 cudaError_t launch_simt_gemm(cudaStream_t st, int epi, const T *A, const T *W, const T *W2, void *C,
-                             const float *bias, int M, int N, int K) {
+                             const float *bias, int M, int N, int K, int num_sms) {
   if constexpr (std::is_same<T, float>::value) {
     const uintptr_t bits = reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(W) | reinterpret_cast<uintptr_t>(W2);
     // 32 x 32 tiles until 64 x 64 ones give every SM two blocks (SwiGLU, two weight tiles: no more than 32 x 32); 16 x 16 tiles
-    // as long as 32 x 32 ones fill at most every second SM.  Tiny decode of 96 rows, 32 x 32 alone 4.00 ms, 16 x 16 up to 37 blocks
-    // (O, down) 3.36, up to 74 (QKV and gate/up too) 3.13
+    // as long as 32 x 32 ones fill at most every second SM.  Tiny decode of 96 rows on 148 SMs, 32 x 32 alone 4.00 ms, 16 x 16 up
+    // to 37 blocks (O, down) 3.36, up to 74 (QKV and gate/up too) 3.13
     auto blocks = [&](int b) { return (int64_t)ceil_div(N, b) * ceil_div(M, b); };
-    const int tile = blocks(64) >= 296 && epi != EPI_SWIGLU ? 64 : (blocks(32) <= 74 ? 16 : 32);
+    const int tile = blocks(64) >= 2 * num_sms && epi != EPI_SWIGLU ? 64 : (blocks(32) <= num_sms / 2 ? 16 : 32);
     // more row tiles than a grid's y (SwiGLU of 2.1 million rows): the plain kernel below with its 64-row tiles
     if ((bits & 15) == 0 && (K & 3) == 0 && ceil_div(M, tile) <= MAX_GRID_YZ) {
       float *Cf = reinterpret_cast<float *>(C);
@@ -518,9 +518,9 @@ cudaError_t launch_row_softmax_partials(cudaStream_t st, const float *logits, in
 }
 
 template cudaError_t launch_simt_gemm<float>(cudaStream_t, int, const float *, const float *,
-                                             const float *, void *, const float *, int, int, int);
+                                             const float *, void *, const float *, int, int, int, int);
 template cudaError_t launch_simt_gemm<bf16>(cudaStream_t, int, const bf16 *, const bf16 *, const bf16 *,
-                                            void *, const float *, int, int, int);
+                                            void *, const float *, int, int, int, int);
 template cudaError_t launch_simt_attention<float>(cudaStream_t, const float *, const float *,
                                                   const float *, const SeqMeta *, const int32_t *,
                                                   float *, int64_t, int, int, int, int, int, int);
