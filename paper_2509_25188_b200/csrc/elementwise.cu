@@ -134,10 +134,12 @@ __device__ __forceinline__ void store4(bf16 *p, float a, float b, float c, float
 // the summed row is written back to x.
 // Bound by the chain of latencies between two projections.  NPART is a compile-time count and a row's loads are issued before
 // its first store (which may alias them), the gain's before the wait for the kernel before: one trip to memory where five
-// followed one another.  ONE: at most a block to an SM, up to 80 registers; else 48 or 40, so that the blocks of an SM leave
-// the next projection the registers to start beside them (512 rows: with 88 it, and its first weights, started 7 us later).
+// followed one another.  ONE (up to 128 rows, one row tile of the projections): 64 to 80 registers; else 48 (of which 16 to 64
+// bytes are spilled with slices to add) or 40, so that the blocks of an SM leave the next projection the registers to start
+// beside them (512 rows: with 88 it, and its first weights, started 7 us later).  The line at 148 rows, a block per SM,
+// instead of 128: a step of 132 to 148 rows 2 % faster in bf16, 2 to 12 % slower in fp32 (d = 256 and 512).
 // From the previous kernel's end to the last store, slices to add: 125 rows 4.6 -> 3.1 us, 32 rows (beside the next weights'
-// stream) 5.0 -> 4.3, 512 rows 4.1 as before; a whole step of 306 rows at d = 1024, with the rotation below: 224 -> 212 us.
+// stream) 5.0 -> 4.3, 512 rows 4.1 as before; a whole step of 306 rows at d = 512, with the rotation below: 224 -> 212 us.
 template <typename T, int NPART, bool ONE>
 __global__ void __launch_bounds__(256, ONE ? 3 : NPART ? 5 : 6) rmsnorm_kernel(float *x, const float *gain, float eps, T *n, int d,
                                                                               const float *part, int64_t part_stride) {

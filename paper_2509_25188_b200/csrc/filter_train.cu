@@ -3,14 +3,15 @@
 // layers; Section 4.4: one to four, ReLU between consecutive layers) with AdamW (Section 4.1: learning rate 0.001).
 //
 // filter_train_kernel runs some 100 us of updates in one cooperative launch.  One update:
-//   gradient   every block walks tiles of T samples held in shared memory: forward through the layers, dz = sigmoid(z) - y, delta of the layers below
-//              (delta_{k-1} = (delta_k W_k) [x_k > 0]), then dW_k += delta_k^T x_k into accumulators its threads own;
-//              it ends by writing its sums (not yet divided by the batch's element count) and its loss sum to its own
+//   gradient   every block walks tiles of T samples held in shared memory: forward through the layers, dz = sigmoid(z) - y,
+//              delta of the layers below (delta_{k-1} = (delta_k W_k) [x_k > 0]), then dW_k += delta_k^T x_k into
+//              accumulators its threads own; it ends by writing its sums (not yet divided by the batch's element count) and its loss sum to its own
 //              row of `gpart`;
-//   meeting    all blocks meet at a counter in global memory (cooperative launch: all are resident; bounded wait);
-//   AdamW      a block takes 8 parameters at a time, its threads shares of the rows that are then added in order (a run is
-//              bit-reproducible on a given GPU), scales by 1 / (samples * s) and applies the update: decoupled weight
-//              decay, bias-corrected moments;
+//   meeting    all blocks meet at a counter in global memory (cooperative launch: all are resident; bounded wait; the
+//              counter runs on from launch to launch);
+//   AdamW      a block takes 8, 32 or all its threads' number of parameters at a time, the threads of one parameter shares
+//              of the rows, whose sums are then added in order (a run is bit-reproducible on a given GPU), scales by
+//              1 / (samples * s) and applies the update: decoupled weight decay, bias-corrected moments;
 //   meeting    and every block reads the new weights.
 // K = s <= 64 is too short a contraction, and fp32 too wide a type, for the tensor cores; what bounds the kernel is the
 // fp32 pipe (432 M multiply-adds for 84,480 samples of 32: 12 us) and, for small batches, the two meetings (~2 us each) and
@@ -19,7 +20,8 @@
 // vectors of a warp lie in different banks.  The next tile arrives (cp.async) while one is worked on.
 // Measured, one update, two launches of per-sample warps before -> this: 84,480 samples of 32 positions, two layers 100 -> 40 us
 // (tiles 30 us, which are bound by shared-memory loads at 40 % of the fp32 pipe); 1,024 samples of 64, four layers
-// 95 -> 21 us; a call without updates 1.0 -> 0.15 ms.
+// 72 -> 20 us; a call without updates 0.80 -> 0.10 ms.  Batches of at most 300 samples of s <= 24 are 1 to 2 us an update
+// slower than those two launches (300 of 8, one layer: 6.3 -> 7.4), which had no meetings.
 #include "common.cuh"
 #include "ptx.cuh"
 
@@ -347,7 +349,7 @@ __global__ void __launch_bounds__(TH, OCC) filter_train_kernel(const TrainArgs a
     target += gridDim.x;
     if (!meet(a.bar, target, a.status, a.limit_ns, &s_ok)) return;
 
-    // AdamW: 32 parameters per block and pass, a share of the rows per warp; entry P is the loss
+    // AdamW; entry P is the loss
     p1 *= (double)a.beta1; p2 *= (double)a.beta2;
     const float bc1 = (float)(1.0 - p1), bc2 = (float)(1.0 - p2), inv_count = (float)(1.0 / ((double)nb * s));
     // A block's pass: PW parameters x RG shares of the rows.  Few parameters and many rows: a sector of a row per load and

@@ -496,7 +496,8 @@ l2pd_status make_tma_out_tail(TmaDesc *out, void *ptr, bool fp32, int64_t rows, 
 //             issuer needs at least (300 with two slabs), and the bytes a CTA takes in at 95 B per cycle (measured alone:
 //             79-117 B, by how many CTAs share a tile).  A sixth of the ingest time comes on top of the rest: between two
 //             tilings that keep the pipe equally busy the one that moves fewer bytes lets the power cap hold a higher clock.
-//             From 4096 rows on, where the cap holds all the time, nearly a half: the down projection (K = 12288) then takes
+//             From 4096 rows on nearly a half (measured at 4096, 16384 and 20000 rows; smaller steps reach the cap too when
+//             run for seconds, which this line does not follow): the down projection (K = 12288) then takes
 //             two slabs, whose exposed drain its long main loop outweighs (16384-row step: 0.15 195, 0.45 191, 0.8 197 ms).
 //   unit      one slab: two accumulator buffers, ~400 cycles between units; two slabs: the drain is exposed.
 //   launch    7000 cycles from the CTA's start to its first MMA, and the last unit's drain.
