@@ -449,7 +449,7 @@ int filter_train_max_rows(int64_t batch, int sms) { return (int)(ceil_div64(batc
 // model of their time that holds within a fifth (the fixed part: meetings and phases).  Beside training at 84,480 x 32, two
 // layers, a decode step of the tiny model (20 kernels, 0.12 ms alone) takes 0.48 ms and the 512-row step of four 8B layers
 // (0.85 ms alone) 2.5 ms; with launches of 400 us 2.0 and 9.1 ms, of 80 ms each stands still for a launch or two.  The
-// training itself pays 2 % (38.9 -> 39.9 us an update; four layers, 1,024 x 64: 19.3 -> 20.0).
+// training itself pays 2 % (38.9 -> 39.9 us an update), 5 % of a call of 60 updates of 20 us (1.30 -> 1.37 ms).
 int64_t filter_train_updates_per_launch(int64_t batch, int s, int n_layers) {
   const double S = s <= 32 ? 32.0 : 64.0, macs = (double)batch * S * S * (3 * n_layers - 1);
   const double us = 5.0 + 3.0 * n_layers + macs / 14.4e6;
