@@ -11,8 +11,9 @@
 //   * EoTP (Section 3.3): the earliest committed [EoT] cuts the sequence; later positions leave
 //     the mask set and read as [EoT];
 //   * block advance / stop (Algorithm 3: no block after one that holds [EoT]).
-// One thread block per sequence taking part in the step (a warp per block row where possible).  Bound by its chain of
-// latencies: the two-layer filter's weights come to shared memory before the wait for the LM head, the tile records and the
+// One thread block per sequence taking part in the step.  What took longest was the merge (988 records of 32 rows in a step of the
+// 8B shape, 380 KB): a warp to a row read a 32-byte sector for each 4-byte value it wanted, eight times the bytes through one SM;
+// with lanes along the rows the kernel takes 16.0 us where it took 36.6.  Besides, it is bound by its chain of latencies: the two-layer filter's weights come to shared memory before the wait for the LM head, the tile records and the
 // sequence's description leave together, its state follows at once.  The summary and the device status go straight to
 // pinned host memory, so that nothing is left to copy behind the step's last kernel.  With the descriptions of a step's
 // sequences as an argument of its first kernel, a step of 306 rows at d = 512: 212 -> 202 us.
@@ -24,7 +25,16 @@ namespace {
 
 constexpr int MAX_S = 64;
 
+// folds the record (om, os, oi) into (mx, sum, ix); the lowest id on ties
+__device__ __forceinline__ void fold(float &mx, float &sum, int &ix, float om, float os, int oi) {
+  const float nm = fmaxf(mx, om);
+  sum = (mx == -INFINITY ? 0.f : sum * expf(mx - nm)) + (om == -INFINITY ? 0.f : os * expf(om - nm));
+  ix = (om > mx || (om == mx && oi < ix)) ? oi : ix;
+  mx = nm;
+}
+
 __global__ void __launch_bounds__(1024) decide_kernel(const __grid_constant__ DecideArgs a) {
+  extern __shared__ float recs[];                                // records of the merge: max, sum exp, argmax
   __shared__ float s_w[2][MAX_S * (MAX_S + 1)], s_b[2][MAX_S];   // the two-layer filter, rows of s + 1
   __shared__ float s_conf[MAX_S];
   __shared__ int s_pred[MAX_S];
@@ -56,20 +66,27 @@ __global__ void __launch_bounds__(1024) decide_kernel(const __grid_constant__ De
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
 
   // ---- confidence head: merge tile records, row r = slot*s + j -------------------------------
-  for (int j = warp; j < s; j += n_warps) {
-    float mx = -INFINITY, sum = 0.f;
-    int ix = 0x7fffffff;
-    {   // rows beyond the block's (padding of the records) are folded in too and dropped below: no wait for m
-      int r = slot * s + j;
-      // eight records per lane are requested before the first is folded in (the fold order is unchanged)
-      constexpr int U = 8;
-      for (int t0 = lane; t0 < a.n_tiles; t0 += 32 * U) {
+  // Lanes take rows, which are adjacent in memory, and the warps (half warps for up to 16 rows) take turns along the tiles; their
+  // records then meet in shared memory, where a warp folds those of a row.
+  {
+    const int rl = s > 16 ? 32 : 16, row = lane & (rl - 1), sub = warp * (32 / rl) + lane / rl, n_sub = n_warps * (32 / rl);
+    float *const rec_m = recs, *const rec_s = recs + n_sub * (rl + 1);
+    int *const rec_i = reinterpret_cast<int *>(recs + 2 * n_sub * (rl + 1));
+    const int n_rec = n_sub < a.n_tiles ? n_sub : a.n_tiles;
+    for (int j0 = 0; j0 < s; j0 += rl) {
+      // rows beyond the block's (padding of the records) are folded in too and dropped below: no wait for m
+      const bool on = j0 + row < s;
+      const int64_t r = (int64_t)slot * s + (on ? j0 + row : 0);
+      float mx = -INFINITY, sum = 0.f;
+      int ix = 0x7fffffff;
+      constexpr int U = 8;   // records requested before the first is folded in
+      for (int t0 = sub; t0 < a.n_tiles; t0 += n_sub * U) {
         float tm[U], ts[U];
         int ti[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          const int t = t0 + 32 * u;
-          const bool in = t < a.n_tiles;
+          const int t = t0 + n_sub * u;
+          const bool in = on && t < a.n_tiles;
           const int64_t o = (int64_t)(in ? t : t0) * a.rows_padded + r;
           tm[u] = in ? a.part_m[o] : -INFINITY;
           ts[u] = in ? a.part_s[o] : 0.f;
@@ -77,25 +94,28 @@ __global__ void __launch_bounds__(1024) decide_kernel(const __grid_constant__ De
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-          if (t0 + 32 * u >= a.n_tiles) break;
+          if (t0 + n_sub * u >= a.n_tiles) break;
           if (tm[u] > mx) { sum = sum * expf(mx - tm[u]) + ts[u]; mx = tm[u]; ix = ti[u]; }
           else { sum += ts[u] * expf(tm[u] - mx); if (tm[u] == mx && ti[u] < ix) ix = ti[u]; }
         }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        float om = __shfl_xor_sync(0xffffffffu, mx, o);
-        float os = __shfl_xor_sync(0xffffffffu, sum, o);
-        int oi = __shfl_xor_sync(0xffffffffu, ix, o);
-        float nm = fmaxf(mx, om);
-        float ns = (mx == -INFINITY ? 0.f : sum * expf(mx - nm)) + (om == -INFINITY ? 0.f : os * expf(om - nm));
-        int ni = (om > mx || (om == mx && oi < ix)) ? oi : ix;
-        mx = nm; sum = ns; ix = ni;
+      if (j0 > 0) __syncthreads();   // the records of the rows before have been read
+      rec_m[sub * (rl + 1) + row] = mx; rec_s[sub * (rl + 1) + row] = sum; rec_i[sub * (rl + 1) + row] = ix;
+      __syncthreads();
+      for (int j = warp; j < rl && j0 + j < s; j += n_warps) {
+        mx = -INFINITY; sum = 0.f; ix = 0x7fffffff;
+        for (int g = lane; g < n_rec; g += 32) fold(mx, sum, ix, rec_m[g * (rl + 1) + j], rec_s[g * (rl + 1) + j], rec_i[g * (rl + 1) + j]);
+        for (int o = 16; o > 0; o >>= 1) {
+          const float om = __shfl_xor_sync(0xffffffffu, mx, o), os = __shfl_xor_sync(0xffffffffu, sum, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, ix, o);
+          fold(mx, sum, ix, om, os, oi);
+        }
+        if (lane == 0) {
+          const bool live = j0 + j < m.n_blk_rows;
+          s_conf[j0 + j] = live ? 1.0f / sum : 0.f;
+          s_pred[j0 + j] = live ? ix : -1;
+        }
       }
-    }
-    if (lane == 0) {
-      bool live = j < m.n_blk_rows;
-      s_conf[j] = live ? 1.0f / sum : 0.f;
-      s_pred[j] = live ? ix : -1;
     }
   }
   int e = a.st.eot_pos[seq], l_eff = a.st.l_eff[seq], steps = 0, n_forced = 0;
@@ -237,10 +257,14 @@ __global__ void __launch_bounds__(1024) decide_kernel(const __grid_constant__ De
 }  // namespace
 
 cudaError_t launch_decide(cudaStream_t st, const DecideArgs &a, int n_slots) {
-  // one warp per block row for the merge of the tile records (the latency-bound part): up to 32 warps
+  // a warp per block row: up to 32 take turns along the tile records (the merge is the longest part)
   int threads = 32 * a.s;
   threads = threads < 256 ? 256 : (threads > 1024 ? 1024 : threads);
-  return launch_kernel(decide_kernel, dim3(n_slots), dim3(threads), 0, st, a);
+  const int rl = a.s > 16 ? 32 : 16;
+  const size_t smem = sizeof(float) * 3 * (threads / rl) * (rl + 1);
+  cudaError_t e = cudaFuncSetAttribute(decide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(decide_kernel, dim3(n_slots), dim3(threads), smem, st, a);
 }
 
 }  // namespace l2pd
