@@ -93,6 +93,22 @@ struct l2pd_ctx {
   GemmPlan pl_qkv{}, pl_o{}, pl_gu{}, pl_down{};
   int box_qkv = 0, box_o = 0, box_gu = 0, box_down = 0, tn_lm = 0;
 
+  // projections with the weights on the M side (gemm_wm.cu): a step's plan, its activation map (of x_rows rows, x_box to a load) and
+  // the layers' weight maps (w_box rows to a load)
+  struct WmGemm {
+    bool on = false;
+    WmPlan plan{};
+    int x_rows = 0, x_box = 0, w_box = 0;
+    TmaDesc x;
+    std::vector<TmaDesc> w;
+    std::vector<int> up_first;
+  } wm_qkv, wm_o, wm_gu, wm_down;
+  std::vector<TmaDesc> tw_qk, tw_v;        // the caller's QKV matrices: q and k rows, rotary halves interleaved; v rows
+  bool wm_gate_up = false;                 // every layer's gate and up matrices can be mapped as one
+  bool wm_qkv_rope = false;                // every layer's QKV matrix can be mapped with its halves interleaved
+  float *ss = nullptr;                     // sums of squares of the rows of x by feature tile, [tiles][max_rows]
+  int32_t *d_row_kv = nullptr;             // row -> row of the key/value store
+
   // several projections per launch (gemm_chain.cu): on when every projection of the step runs on SM pairs with
   // two row slabs per unit and K slices store partial sums
   int chain_mode = 0;                // l2pd_set_chain: 0 one launch per projection, 1 chained launches, 2 the chained form's tiling in single launches
@@ -135,6 +151,17 @@ bool pdl_enabled() {
 
 namespace {
 
+// Steps of few rows have their weights on the M side and no RMSNorm kernels (gemm_wm.cu): a step of 32 rows of the 8B shape 3.4 ->
+// 3.2 ms, its decode of 64 steps 261 -> 245 ms; of 64 rows even, of 125 rows 5 % slower (the epilogues pass 16 rows at a time, and
+// nothing overlaps them when a CTA has one unit).
+constexpr int LEAN_MAX_ROWS = 48;
+// Otherwise a projection takes that side where its model says so.  The model leaves out what its epilogues take of shared memory's
+// bandwidth from the MMAs: measured over 288 to 8192 rows, its cycles times 1.06 to 1.15 (mostly 1.1 to 1.12) compare with the other
+// orientation's.  With all projections forced to it, eight 8B layers: 288 rows 0.90 of the time, 320 0.95, 384 1.01, 512 1.04, 640
+// 0.93, 768 1.08, 1024 1.12, 1029 0.91, 4096 1.03; the 1029-row step of 32 layers with this rule 15.55 -> 13.81 ms.  Up to 256 rows
+// (1.03 to 1.11 times the time) it is not asked.
+constexpr int WM_MIN_ROWS = 256;
+constexpr double WM_MARGIN = 1.12;
 constexpr int CHAIN_TILE_N = 176;       // widest tile of a step that chains projections
 constexpr int CHAIN_MAX_ROWS = 1536;    // steps of more rows run one launch per projection (the launch is then a small part)
 constexpr int CHAIN_TRACE_STAMPS = 4;   // stamps per phase and CTA
@@ -266,6 +293,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
   const bool tc = (f.dtype == L2PD_BF16) && !c->force_simt;
   T *n = (T *)c->n, *qkv = (T *)c->qkv, *q = (T *)c->q, *att = (T *)c->att, *hbuf = (T *)c->h, *nf = (T *)c->nf;
 
+  bool lean = false;   // all projections with the weights on the M side, the RMSNorm between them in their epilogues
   if (tc) {
     // the tiling follows the row count of this step; weight tensor maps are re-encoded when the
     // box (rows of the weight tile one CTA loads) changes
@@ -290,10 +318,50 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
       }
     }
     const int max_ks = (c->ksum == nullptr || T_rows <= c->ksum_rows) ? 4 : 1;   // K slices need their partial-sum area
-    c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0);
-    c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks);
-    c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks);
-    c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0);
+    double cost_qkv, cost_o, cost_down, cost_gu;
+    c->pl_qkv = plan_gemm(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, 0, 1, &cost_qkv);
+    c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks, &cost_o);
+    c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks, &cost_down);
+    c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0, 1, &cost_gu);
+    lean = c->chain_mode == 0 && c->wm_gate_up && c->wm_qkv_rope && T_rows <= LEAN_MAX_ROWS;
+    // the rotation and the scatter are a kernel of their own where the projection does not do them
+    if (!c->fuse_rope) cost_qkv += 4000.0 + 12.0 * T_rows * hd / 3100.0;
+    auto wm_plan = [&](l2pd_ctx::WmGemm &g, int epi, int N, int K, double other, int ks) {
+      g.plan = plan_gemm_wm(epi, T_rows, N, K, c->num_sms, lean ? 4 : ks, lean);
+      g.on = lean || (T_rows > WM_MIN_ROWS && g.plan.cost * WM_MARGIN < other);
+    };
+    wm_plan(c->wm_qkv, EPI_QKV_ROPE, 3 * hd, d, cost_qkv, 1);
+    wm_plan(c->wm_o, EPI_RESIDUAL, d, hd, cost_o, c->ksum ? max_ks : 1);
+    wm_plan(c->wm_down, EPI_RESIDUAL, d, F, cost_down, c->ksum ? max_ks : 1);
+    wm_plan(c->wm_gu, EPI_SWIGLU, F, d, cost_gu, 1);
+    if (!c->wm_gate_up) c->wm_gu.on = false;
+    if (!c->wm_qkv_rope) c->wm_qkv.on = false;
+    // slices that a later kernel adds (in a lean step there are none)
+    if (c->wm_o.on) c->pl_o.k_splits = lean ? 1 : c->wm_o.plan.k_splits;
+    if (c->wm_down.on) c->pl_down.k_splits = lean ? 1 : c->wm_down.plan.k_splits;
+    if (c->chain_mode != 0) c->wm_qkv.on = c->wm_o.on = c->wm_down.on = c->wm_gu.on = false;
+    auto wm_maps = [&](l2pd_ctx::WmGemm &g, const void *act, int64_t K, const std::vector<const void *> *w, const std::vector<const void *> *up, int64_t N) -> l2pd_status {
+      if (!g.on) return L2PD_OK;
+      const int xb = g.plan.tile_t / g.plan.cta_group;
+      if (g.x_rows != T_rows || g.x_box != xb) {
+        if (l2pd_status e = make_tma_2d_bf16(&g.x, act, T_rows, K, xb)) return set_err(c, e, "tensor map encode failed (%d rows of activations)", T_rows);
+        g.x_rows = T_rows; g.x_box = xb;
+      }
+      if (w && g.w_box != g.plan.w_rows) {
+        g.w_box = 0;
+        g.w.resize(w->size()); g.up_first.resize(w->size());
+        for (size_t l = 0; l < w->size(); ++l)
+          if (l2pd_status e = up ? make_tma_gate_up(&g.w[l], (*w)[l], (*up)[l], N, K, g.plan.w_rows, &g.up_first[l])
+                                 : make_tma_2d_bf16(&g.w[l], (*w)[l], N, K, g.plan.w_rows))
+            return set_err(c, e, "tensor map encode failed (%lld x %lld weights)", (long long)N, (long long)K);
+        g.w_box = g.plan.w_rows;
+      }
+      return L2PD_OK;
+    };
+    if (l2pd_status e = wm_maps(c->wm_qkv, c->n, d, nullptr, nullptr, 0)) return e;
+    if (l2pd_status e = wm_maps(c->wm_o, c->att, hd, &c->wo, nullptr, d)) return e;
+    if (l2pd_status e = wm_maps(c->wm_gu, c->n, d, &c->w_gate, &c->w_up, F)) return e;
+    if (l2pd_status e = wm_maps(c->wm_down, c->h, F, &c->w_down, nullptr, d)) return e;
     if (small_chain || big_chain) {
       const int slabs = big_chain ? 2 : 1, ks_o = big_chain ? c->pl_o.k_splits : 0, ks_d = big_chain ? c->pl_down.k_splits : 0;
       c->pl_qkv = plan_gemm_chained(EPI_STORE, T_rows, 3 * hd, d, c->num_sms, slabs, 1, CHAIN_TILE_N);
@@ -356,8 +424,8 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
   const bool described = n_slots <= STEP_META_BATCH;   // by the embedding's argument
   for (int k = 0; !described && k < n_slots; k += STEP_META_BATCH)
     CKLK(L2PD_K_OTHER, launch_build_row_map(s, c->h_meta, k, n_slots - k < STEP_META_BATCH ? n_slots - k : STEP_META_BATCH, c->d_meta,
-                                            c->d_row_slot, c->d_row_pos));
-  CKLK(L2PD_K_EMBED, launch_embed_rmsnorm<T>(s, described ? c->h_meta : nullptr, n_slots, c->d_meta, c->d_row_slot, c->d_row_pos,
+                                            c->d_row_slot, c->d_row_pos, c->d_row_kv, f.max_seq));
+  CKLK(L2PD_K_EMBED, launch_embed_rmsnorm<T>(s, described ? c->h_meta : nullptr, n_slots, c->d_meta, c->d_row_slot, c->d_row_pos, c->d_row_kv, f.max_seq,
                                              c->d_tokens, c->P + c->G, (const T *)c->tok_emb, c->norm1[0], f.rms_eps, c->x, n, T_rows, d));
   if (c->cap) CK(cudaMemcpyAsync(c->cap, c->x, (size_t)T_rows * d * 4, cudaMemcpyDeviceToDevice, s));
 
@@ -457,14 +525,47 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     c->chain_trace_launches = f.n_layers + 1; c->chain_trace_phases = CHAIN_TRACE_PHASES; c->chain_trace_ctas = n_ctas;
   }
 
+  // the projections of layer l with the weights on the M side
+  auto wm_args = [&](int epi, int N, int K, const l2pd_ctx::WmGemm &g, int l) {
+    WmArgs a{};
+    a.epi = epi; a.T = T_rows; a.N = N; a.K = K; a.plan = g.plan; a.w = epi == EPI_QKV_ROPE ? &c->tw_qk[l] : &g.w[l]; a.x = &g.x;
+    a.status = c->d_status; a.ss_stride = (int)c->max_rows; a.eps = f.rms_eps; a.width = d;
+    return a;
+  };
+  auto wm_qkv = [&](int l, void *kc, void *vc) {
+    WmArgs a = wm_args(EPI_QKV_ROPE, 3 * hd, d, c->wm_qkv, l);
+    a.wv = &c->tw_v[l]; a.hd = hd; a.dh = dh; a.cs_table = c->cs_table; a.row_pos = c->d_row_pos;
+    if (c->fuse_rope) { a.q = (bf16 *)c->qkv; a.k = a.q + hd; a.v = a.k + hd; a.q_stride = a.kv_stride = 3 * hd; }
+    else { a.q = (bf16 *)c->q; a.k = (bf16 *)kc; a.v = (bf16 *)vc; a.q_stride = a.kv_stride = hd; a.kv_row = c->d_row_kv; a.natural = 1; }
+    if (lean && l > 0) { a.ss_in = c->ss; a.ss_n = ceil_div(d, c->wm_down.plan.w_rows); }   // (the embedding's rows are normalised)
+    return a;
+  };
+  auto wm_residual = [&](const l2pd_ctx::WmGemm &g, int K, int l, const float *gain) {
+    WmArgs a = wm_args(EPI_RESIDUAL, d, K, g, l);
+    a.xres = c->x;
+    if (lean) {
+      a.in_cluster = 1;
+      if (gain) { a.n = (bf16 *)c->n; a.gain = gain; a.ss_out = c->ss; }
+    } else { a.part = c->ksum; a.part_stride = (int64_t)round_up(T_rows, 512) * d; }
+    return a;
+  };
+  auto wm_gate_up = [&](int l) {
+    WmArgs a = wm_args(EPI_SWIGLU, F, d, c->wm_gu, l);
+    a.up_first = c->wm_gu.up_first[l]; a.out = (bf16 *)c->h; a.out_stride = F;
+    if (lean) { a.ss_in = c->ss; a.ss_n = ceil_div(d, c->wm_o.plan.w_rows); }
+    return a;
+  };
+  const bool wq = tc && c->wm_qkv.on, wo = tc && c->wm_o.on, wg = tc && c->wm_gu.on, wd = tc && c->wm_down.on;
+
   for (int l = 0; l < f.n_layers && !chain; ++l) {
     T *kc = (T *)c->kc + (f.kv_cache_mode ? (int64_t)l * c->kv_layer_stride : 0);
     T *vc = (T *)c->vc + (f.kv_cache_mode ? (int64_t)l * c->kv_layer_stride : 0);
-    l2pd_status r;
-    if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_QKV, c->fuse_rope ? EPI_QKV_ROPE : EPI_STORE, &c->ta_n, &c->tb_qkv[l], nullptr, c->tcw_qkv > 0 ? &c->tc_qkv : nullptr, qkv, T_rows, 3 * hd, d, c->pl_qkv);
+    l2pd_status r = L2PD_OK;
+    if (wq) CKLK(L2PD_K_GEMM_QKV, launch_gemm_wm(s, wm_qkv(l, kc, vc), c->num_sms));
+    else if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_QKV, c->fuse_rope ? EPI_QKV_ROPE : EPI_STORE, &c->ta_n, &c->tb_qkv[l], nullptr, c->tcw_qkv > 0 ? &c->tc_qkv : nullptr, qkv, T_rows, 3 * hd, d, c->pl_qkv);
     else r = run_gemm_simt<T>(c, s, L2PD_K_GEMM_QKV, EPI_STORE, n, c->wqkv[l], nullptr, qkv, nullptr, T_rows, 3 * hd, d);
     if (r) return r;
-    if (!(tc && c->fuse_rope))
+    if (!(tc && c->fuse_rope) && !wq)
       CKLK(L2PD_K_ROPE, launch_rope_scatter<T>(s, qkv, c->d_meta, c->d_row_slot, c->cs_table, q, kc, vc, c->kv_seq_stride, T_rows, H, dh));
     if (tc && c->fuse_rope) {
       CKLK(L2PD_K_ATTENTION, launch_attention_tc(s, c->tq_packed, c->tk_packed, c->tv_packed, c->d_meta, (bf16 *)att, hd, 0, 0, 1,
@@ -479,18 +580,21 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     } else {
       CKLK(L2PD_K_ATTENTION, launch_simt_attention<T>(s, q, kc, vc, c->d_meta, c->d_row_slot, att, c->kv_seq_stride, T_rows, H, dh, max_kv, n_slots, max_q_rows));
     }
-    if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_O, EPI_RESIDUAL, &c->ta_att, &c->tb_o[l], nullptr, c->tcw_o > 0 ? &c->tc_o : nullptr, c->x, T_rows, d, hd, c->pl_o);
+    if (wo) CKLK(L2PD_K_GEMM_O, launch_gemm_wm(s, wm_residual(c->wm_o, hd, l, c->norm2[l]), c->num_sms));
+    else if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_O, EPI_RESIDUAL, &c->ta_att, &c->tb_o[l], nullptr, c->tcw_o > 0 ? &c->tc_o : nullptr, c->x, T_rows, d, hd, c->pl_o);
     else r = run_gemm_simt<T>(c, s, L2PD_K_GEMM_O, EPI_RESIDUAL, att, c->wo[l], nullptr, c->x, nullptr, T_rows, d, hd);
     if (r) return r;
-    {
+    if (!lean) {
       const int ks = (tc && c->ksum) ? effective_k_splits(hd, c->pl_o.k_splits) : 1;
       CKLK(L2PD_K_RMSNORM, launch_rmsnorm<T>(s, c->x, c->norm2[l], f.rms_eps, n, T_rows, d, c->ksum, ks > 1 ? ks : 0,
                                             (int64_t)round_up(T_rows, 512) * d));
     }
-    if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_GATE_UP, EPI_SWIGLU, &c->ta_n, &c->tb_gate[l], &c->tb_up[l], c->tcw_h > 0 ? &c->tc_h : nullptr, hbuf, T_rows, F, d, c->pl_gu);
+    if (wg) CKLK(L2PD_K_GEMM_GATE_UP, launch_gemm_wm(s, wm_gate_up(l), c->num_sms));
+    else if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_GATE_UP, EPI_SWIGLU, &c->ta_n, &c->tb_gate[l], &c->tb_up[l], c->tcw_h > 0 ? &c->tc_h : nullptr, hbuf, T_rows, F, d, c->pl_gu);
     else r = run_gemm_simt<T>(c, s, L2PD_K_GEMM_GATE_UP, EPI_SWIGLU, n, c->w_gate[l], c->w_up[l], hbuf, nullptr, T_rows, F, d);
     if (r) return r;
-    if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_DOWN, EPI_RESIDUAL, &c->ta_h, &c->tb_down[l], nullptr, c->tcw_down > 0 ? &c->tc_down : nullptr, c->x, T_rows, d, F, c->pl_down);
+    if (wd) CKLK(L2PD_K_GEMM_DOWN, launch_gemm_wm(s, wm_residual(c->wm_down, F, l, l + 1 < f.n_layers ? c->norm1[l + 1] : nullptr), c->num_sms));
+    else if (tc) r = run_gemm_tc(c, s, L2PD_K_GEMM_DOWN, EPI_RESIDUAL, &c->ta_h, &c->tb_down[l], nullptr, c->tcw_down > 0 ? &c->tc_down : nullptr, c->x, T_rows, d, F, c->pl_down);
     else r = run_gemm_simt<T>(c, s, L2PD_K_GEMM_DOWN, EPI_RESIDUAL, hbuf, c->w_down[l], nullptr, c->x, nullptr, T_rows, d, F);
     if (r) return r;
     // the down projection's K slices: summed by the next layer's RMSNorm, or right here when x is read by something else
@@ -502,7 +606,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     }
     if (c->cap)
       CK(cudaMemcpyAsync(c->cap + (int64_t)(l + 1) * c->cap_stride, c->x, (size_t)T_rows * d * 4, cudaMemcpyDeviceToDevice, s));
-    if (l + 1 < f.n_layers)
+    if (l + 1 < f.n_layers && !lean)
       CKLK(L2PD_K_RMSNORM, launch_rmsnorm<T>(s, c->x, c->norm1[l + 1], f.rms_eps, n, T_rows, d, c->ksum, ks_pend > 1 ? ks_pend : 0,
                                             ks_stride));
   }
@@ -582,7 +686,7 @@ void free_all(l2pd_ctx *c) {
   cudaFree(c->x); cudaFree(c->n); cudaFree(c->qkv); cudaFree(c->q); cudaFree(c->att); cudaFree(c->h); cudaFree(c->nf);
   cudaFree(c->kc); cudaFree(c->vc); cudaFree(c->part); cudaFree(c->logits_f32);
   for (void *w : c->wqkv_perm) cudaFree(w);
-  cudaFree(c->d_row_pos); cudaFree(c->cs_table_t); cudaFree(c->ksum);
+  cudaFree(c->d_row_pos); cudaFree(c->d_row_kv); cudaFree(c->ss); cudaFree(c->cs_table_t); cudaFree(c->ksum);
   cudaFree(c->d_chain_bar); cudaFree(c->d_chain_trace); cudaFree(c->d_chain_tabs);
   if (c->h_chain_tabs) cudaFreeHost(c->h_chain_tabs);
   cudaFree(c->d_meta); cudaFree(c->d_row_slot); cudaFree(c->d_status); cudaFree(c->cs_table);
@@ -699,12 +803,14 @@ l2pd_status l2pd_init(const l2pd_config *cfg, const l2pd_weights *w, int device,
   A(dev_alloc(c, &c->d_meta, (int64_t)f.max_batch));
   A(dev_alloc(c, &c->d_row_slot, mr));
   A(dev_alloc(c, &c->d_row_pos, mr));
+  A(dev_alloc(c, &c->d_row_kv, mr));
   // L2PD_ATOMIC_KSPLIT=1: no partial-sum area; K slices add into x in completion order (not bit-reproducible)
   const char *ak = getenv("L2PD_ATOMIC_KSPLIT");
   if (f.dtype == L2PD_BF16 && !(ak && ak[0] == '1')) {
     c->ksum_rows = round_up(mr < 4096 ? mr : 4096, 512);   // a slice's area covers whole 512-row units
     A(dev_alloc(c, &c->ksum, 4 * c->ksum_rows * d));
   }
+  if (f.dtype == L2PD_BF16 && !c->force_simt) A(dev_alloc(c, &c->ss, (int64_t)ceil_div(d, 32) * mr));
   if (f.dtype == L2PD_BF16 && c->ksum && !c->force_simt) {
     c->chain_clusters = chain_max_clusters(c->num_sms);
     if (c->chain_clusters > 0) {
@@ -767,6 +873,20 @@ l2pd_status l2pd_init(const l2pd_config *cfg, const l2pd_weights *w, int device,
       if (make_tma_2d_bf16(&c->ta_q, c->q, mr, hd, 128) || make_tma_2d_bf16(&c->t_kstore, c->kc, store_rows, hd, 128) ||
           make_tma_2d_bf16(&c->t_vstore, c->vc, store_rows, hd, 128))
         return fail(L2PD_ERR_CUDA);
+    }
+    if (!c->force_simt) {
+      const int half = f.head_dim / 2;
+      c->tw_qk.resize(f.n_layers); c->tw_v.resize(f.n_layers);
+      c->wm_gate_up = c->wm_qkv_rope = true;
+      for (int l = 0; l < f.n_layers; ++l) {
+        if (make_tma_halves(&c->tw_qk[l], c->wqkv[l], d, (int64_t)half * d * 2, half / 8, half / 8, 2 * f.n_heads,
+                            (int64_t)f.head_dim * d * 2, 128 / f.head_dim) ||
+            make_tma_2d_bf16(&c->tw_v[l], (const bf16 *)c->wqkv[l] + (int64_t)2 * hd * d, hd, d, 128))
+          c->wm_qkv_rope = false;
+        TmaDesc probe;
+        int up_first;
+        if (make_tma_gate_up(&probe, c->w_gate[l], c->w_up[l], F, d, 128, &up_first)) c->wm_gate_up = false;
+      }
     }
     const char *nf = getenv("L2PD_NO_ROPE_FUSION");
     c->fuse_rope = c->attn_tc && !c->force_simt && f.kv_cache_mode == 0 && (f.head_dim & (f.head_dim - 1)) == 0 &&
@@ -1188,12 +1308,33 @@ static l2pd_status finish_standalone(cudaStream_t s, int32_t *status, int check)
   return L2PD_OK;
 }
 
+// The stand-alone GEMMs with the weights on the M side (gemm_wm.cu).
+static l2pd_status gemm_common_wm(void *stream, int epi, const void *A, const void *W, const void *W2, void *out, int M, int N, int K,
+                                  const WmPlan &pl, int sms, int check) {
+  int32_t *status = standalone_status();
+  if (!status) return L2PD_ERR_CUDA;
+  TmaDesc tx, tw;
+  l2pd_status r = make_tma_2d_bf16(&tx, A, M, K, pl.tile_t / pl.cta_group);
+  if (r) return r;
+  WmArgs g{};
+  if (epi == EPI_SWIGLU) { r = make_tma_gate_up(&tw, W, W2, N, K, pl.w_rows, &g.up_first); if (r) return r; }
+  else { r = make_tma_2d_bf16(&tw, W, N, K, pl.w_rows); if (r) return r; }
+  g.epi = epi; g.T = M; g.N = N; g.K = K; g.plan = pl; g.w = &tw; g.x = &tx;
+  g.out = (bf16 *)out; g.out_stride = N; g.xres = (float *)out; g.status = status;
+  g.in_cluster = epi == EPI_RESIDUAL && pl.k_splits > 1;
+  { cudaError_t e = launch_gemm_wm((cudaStream_t)stream, g, sms); if (e != cudaSuccess) return standalone_cuda_error("GEMM launch", e); }
+  return finish_standalone((cudaStream_t)stream, status, check);
+}
+
 static l2pd_status gemm_common(void *stream, int epi, const void *A, const void *W, const void *W2, void *out,
                                int M, int N, int K, int tile_n, int check) {
   if (!A || !W || !out || (epi == EPI_SWIGLU && !W2)) return L2PD_ERR_ARG;
   if (M < 1 || N < 8 || K < 8 || (N % 8) || (K % 8)) return L2PD_ERR_SHAPE;
   if (tile_n < 0) return L2PD_ERR_SHAPE;
   const int sms = device_sms();
+  // + 10000000 * orientation (1 = weights on the M side, width = rows of a tile, K slices in a cluster; 2 = rows on the M side)
+  const int want_or = tile_n / 10000000;
+  tile_n %= 10000000;
   // tile_n = width + 1000 * cta_group + 10000 * k_splits + 100000 * slabs + 1000000 * k_interleave (1 = on, 2 = off);
   // any part 0 = chosen automatically
   const int want_kil = tile_n / 1000000;
@@ -1203,7 +1344,21 @@ static l2pd_status gemm_common(void *stream, int epi, const void *A, const void 
   const int unit = 16;
   if (want_tn && (want_tn < 32 || want_tn > 256 || (want_tn % unit))) return L2PD_ERR_SHAPE;
   if (want_cg > 2 || want_ks > 8 || (want_ks > 1 && epi != EPI_RESIDUAL) || want_sl > 2) return L2PD_ERR_SHAPE;
-  GemmPlan pl = plan_gemm(epi, M, N, K, sms, want_tn);
+  double cost = 0.0;
+  GemmPlan pl = plan_gemm(epi, M, N, K, sms, want_tn, 4, &cost);
+  if (want_or == 1 || (want_or == 0 && !want_kil && tile_n == 0)) {
+    WmPlan wp = plan_gemm_wm(epi, M, N, K, sms, 4, true);
+    if (want_or == 1) {
+      if (want_tn) wp.tile_t = want_tn;
+      if (want_cg) wp.cta_group = want_cg;
+      wp.k_splits = want_ks ? effective_k_splits(K, want_ks) : 1;
+      wp.w_rows = 128;
+    }
+    TmaDesc probe;
+    int up_first = 0;
+    const bool can = epi != EPI_SWIGLU || make_tma_gate_up(&probe, W, W2, N, K, wp.w_rows, &up_first) == L2PD_OK;
+    if (can && (want_or == 1 || wp.cost * WM_MARGIN < cost)) return gemm_common_wm(stream, epi, A, W, W2, out, M, N, K, wp, sms, check);
+  }
   if (want_tn) pl.tile_n = want_tn;
   if (want_cg) pl.cta_group = want_cg;
   if (want_ks) pl.k_splits = want_ks;

@@ -76,13 +76,14 @@ template <> __device__ __forceinline__ bf16 from_f32<bf16>(float v) { return __f
 
 // elementwise.cu
 // A step's first kernel.  Up to STEP_META_BATCH sequences: the embedding, which takes their descriptions (h_meta, host memory)
-// as an argument and stores them and the maps row -> slot and row -> position; x = the rows' embeddings, n = RMSNorm(x).
+// as an argument and stores them and the maps row -> slot, position and row of the key/value store (max_seq to a sequence); x = the rows' embeddings, n = RMSNorm(x).
 // More: launch_build_row_map for STEP_META_BATCH of them at a time, then the embedding with h_meta = nullptr.
 constexpr int STEP_META_BATCH = 64;
-cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, int slot0, int n, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos);
+cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, int slot0, int n, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos,
+                                 int32_t *row_kv, int max_seq);
 template <typename T>
 cudaError_t launch_embed_rmsnorm(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
-                                 int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
+                                 int32_t *row_pos, int32_t *row_kv, int max_seq, const int32_t *tokens, int64_t tok_stride, const T *emb,
                                  const float *gain, float eps, float *x, T *n, int rows, int d);
 // n = RMSNorm(x).  With n_part > 0, first x += part[0] + part[1] + ... (slice s at part + s * part_stride elements,
 // added in that order) and x is written back: the fixed-order end of a K-split projection.
@@ -195,7 +196,7 @@ void set_standalone_error(const char *fmt, ...);
 // accumulators that the epilogue adds.  No plan asks for it by itself (one issuer keeps up with the weight stream:
 // 32 rows, QKV 20.2 us against 23.9); chained launches of few rows and explicit requests do.
 struct GemmPlan { int cta_group, tile_n, k_splits, slabs, k_interleave; };
-GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits = 4);
+GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits = 4, double *cost = nullptr);   // cost: modelled cycles
 GemmPlan plan_gemm_chained(int epi, int M, int N, int K, int num_sms, int slabs, int max_k_splits, int max_tile_n, int force_ks = 0);
 int effective_k_splits(int K, int k_splits);   // what the launcher makes of a requested K split
 struct GemmArgs {
@@ -225,6 +226,41 @@ cudaError_t launch_gemm_tcgen05(cudaStream_t st, const GemmArgs &g, int num_sms)
 cudaError_t launch_merge_partials(cudaStream_t st, const float *part_m, const float *part_s,
                                   const int32_t *part_i, int n_tiles, int rows_padded, int R,
                                   int32_t *pred, float *conf);
+
+// gemm_wm.cu : the same projections with the weights on the M side of the MMA and the rows on its N side.
+typedef CUresult (*TmaEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
+                                const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+TmaEncodeFn tma_encode_fn();
+// tile_t: rows of a tile (a multiple of 16, at most 256); w_rows: weight rows of a CTA; cost: modelled cycles
+struct WmPlan { int cta_group, tile_t, k_splits, w_rows; double cost; };
+WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits = 4, bool in_cluster = false);   // in_cluster: as WmArgs
+struct WmArgs {
+  int epi, T, N, K;           // rows, output features (SwiGLU: F), depth
+  WmPlan plan;
+  // weights: boxes of w_rows rows (make_tma_2d_bf16).  SwiGLU and the q and k part of QKV: make_tma_halves; QKV: wv maps the v part
+  const TmaDesc *w, *wv;
+  const TmaDesc *x;           // activations [T, K], box of tile_t / cta_group rows
+  bf16 *out; int64_t out_stride;              // STORE, SWIGLU
+  int up_first;               // SwiGLU: `w` starts at the up projection
+  // QKV: q row = row, k and v row = kv_row[row] (null: row); cs_table [position][dh / 2], row_pos [T].  natural: dimensions in
+  // their order, otherwise rotary pairs adjacent
+  bf16 *q, *k, *v; int64_t q_stride, kv_stride; const int32_t *kv_row, *row_pos; const float2 *cs_table; int hd, dh, natural;
+  // RESIDUAL: x += acc.  K slices: summed inside a cluster (in_cluster), or partial sums at part + slice * part_stride [T][N] that
+  // the caller adds, or atomics (part = null)
+  float *xres, *part; int64_t part_stride; int in_cluster;
+  // n != null: also n = bf16(x gain) and the sums of squares of each tile of w_rows features at ss_out[tile * ss_stride + row]
+  bf16 *n; const float *gain; float *ss_out;
+  // the other epilogues, ss_in != null: accumulator rows times 1 / sqrt(sum of ss_n tiles / width + eps)
+  const float *ss_in; int ss_n, ss_stride; float eps; int width;
+  int32_t *status;
+};
+cudaError_t launch_gemm_wm(cudaStream_t st, const WmArgs &g, int num_sms);
+// A matrix of 128-byte row pieces whose rows are interleaved in groups of eight: dims {K, 8, 2, groups, outer}, the second half of a
+// pair `half_bytes` behind the first, groups 8 rows apart; box {64, 8, 2, box_groups, box_outer}.
+l2pd_status make_tma_halves(TmaDesc *out, const void *ptr, int64_t K, int64_t half_bytes, int64_t groups, int box_groups, int64_t outer,
+                            int64_t outer_bytes, int box_outer);
+// The gate and up matrices [F, K], two allocations, as the halves; fails where they are the same one or 2^40 bytes apart.
+l2pd_status make_tma_gate_up(TmaDesc *out, const void *gate, const void *up, int64_t F, int64_t K, int box_rows, int *up_first);
 
 // gemm_chain.cu : several projections (cta_group 2, two row slabs per unit) and the RMSNorms between them in one
 // persistent launch; the phases run in the order given, the CTAs meeting at a counter in global memory between them.

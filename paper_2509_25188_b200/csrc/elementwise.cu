@@ -55,7 +55,7 @@ struct MetaBatch { SeqMeta m[META_BATCH]; };
 // maps, for the kernels that follow.
 template <typename T>
 __global__ void embed_rmsnorm_kernel(const __grid_constant__ MetaBatch b, int n_arg, const int32_t *tokens, int64_t tok_stride,
-                                     SeqMeta *meta, int32_t *row_slot, int32_t *row_pos, const T *emb, const float *gain,
+                                     SeqMeta *meta, int32_t *row_slot, int32_t *row_pos, int32_t *row_kv, int max_seq, const T *emb, const float *gain,
                                      float eps, float *x, T *n, int d) {
   grid_dep_launch();
   __shared__ float red[32];
@@ -69,6 +69,7 @@ __global__ void embed_rmsnorm_kernel(const __grid_constant__ MetaBatch b, int n_
     if (threadIdx.x == 0) {
       row_slot[row] = slot;
       row_pos[row] = m.pos0 + (row - m.row0);
+      row_kv[row] = m.seq * max_seq + m.pos0 + (row - m.row0);
       if (row == m.row0) meta[slot] = m;
     }
   } else {
@@ -368,7 +369,8 @@ __global__ void final_norm_gather_kernel(const float *x, const SeqMeta *meta, co
 
 // The first kernel of a step of more than META_BATCH sequences: stores their descriptions, META_BATCH to a launch, and the
 // maps from packed rows to them.  (Fewer: embed_rmsnorm_kernel does it.)
-__global__ void build_row_map_kernel(const __grid_constant__ MetaBatch b, int slot0, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos) {
+__global__ void build_row_map_kernel(const __grid_constant__ MetaBatch b, int slot0, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos,
+                                     int32_t *row_kv, int max_seq) {
   grid_dep_launch();
   const SeqMeta m = b.m[blockIdx.x];
   const int slot = slot0 + blockIdx.x;
@@ -376,6 +378,7 @@ __global__ void build_row_map_kernel(const __grid_constant__ MetaBatch b, int sl
   for (int i = threadIdx.x; i < m.n_rows; i += blockDim.x) {
     row_slot[m.row0 + i] = slot;
     row_pos[m.row0 + i] = m.pos0 + i;
+    row_kv[m.row0 + i] = m.seq * max_seq + m.pos0 + i;
   }
 }
 
@@ -434,23 +437,24 @@ __global__ void gather_response_kernel(const int32_t *tokens, int P, int G, int3
 
 // A step's first launch, of these two, is an ordinary one, which starts when all earlier work of the stream is complete: the
 // kernels behind it read weights before their own wait.
-cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, int slot0, int n, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos) {
+cudaError_t launch_build_row_map(cudaStream_t st, const SeqMeta *h_meta, int slot0, int n, SeqMeta *meta, int32_t *row_slot, int32_t *row_pos,
+                                 int32_t *row_kv, int max_seq) {
   if (n < 1 || n > META_BATCH) return cudaErrorInvalidValue;
   MetaBatch b;
   for (int i = 0; i < n; ++i) b.m[i] = h_meta[slot0 + i];
-  build_row_map_kernel<<<n, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos);
+  build_row_map_kernel<<<n, 256, 0, st>>>(b, slot0, meta, row_slot, row_pos, row_kv, max_seq);
   return cudaGetLastError();
 }
 template <typename T>
 cudaError_t launch_embed_rmsnorm(cudaStream_t st, const SeqMeta *h_meta, int n_slots, SeqMeta *meta, int32_t *row_slot,
-                                 int32_t *row_pos, const int32_t *tokens, int64_t tok_stride, const T *emb,
+                                 int32_t *row_pos, int32_t *row_kv, int max_seq, const int32_t *tokens, int64_t tok_stride, const T *emb,
                                  const float *gain, float eps, float *x, T *n, int rows, int d) {
   MetaBatch b;
   if (!h_meta)
-    return launch_kernel(embed_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, b, 0, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
+    return launch_kernel(embed_rmsnorm_kernel<T>, dim3(rows), dim3(256), 0, st, b, 0, tokens, tok_stride, meta, row_slot, row_pos, row_kv, max_seq, emb, gain, eps, x, n, d);
   if (n_slots < 1 || n_slots > META_BATCH) return cudaErrorInvalidValue;
   for (int i = 0; i < n_slots; ++i) b.m[i] = h_meta[i];
-  embed_rmsnorm_kernel<T><<<rows, 256, 0, st>>>(b, n_slots, tokens, tok_stride, meta, row_slot, row_pos, emb, gain, eps, x, n, d);
+  embed_rmsnorm_kernel<T><<<rows, 256, 0, st>>>(b, n_slots, tokens, tok_stride, meta, row_slot, row_pos, row_kv, max_seq, emb, gain, eps, x, n, d);
   return cudaGetLastError();
 }
 template <typename T>
@@ -505,7 +509,7 @@ cudaError_t launch_gather_response(cudaStream_t st, const int32_t *tokens, int B
 }
 
 #define INSTANTIATE(T)                                                                              \
-  template cudaError_t launch_embed_rmsnorm<T>(cudaStream_t, const SeqMeta *, int, SeqMeta *, int32_t *, int32_t *, \
+  template cudaError_t launch_embed_rmsnorm<T>(cudaStream_t, const SeqMeta *, int, SeqMeta *, int32_t *, int32_t *, int32_t *, int, \
                                                const int32_t *, int64_t, const T *, const float *, float, float *, T *, int, int); \
   template cudaError_t launch_rmsnorm<T>(cudaStream_t, float *, const float *, float, T *,           \
                                          int, int, const float *, int, int64_t);                     \

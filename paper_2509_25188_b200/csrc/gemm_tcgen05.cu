@@ -389,25 +389,6 @@ gemm_tcgen05_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_c
   gemm_body<EPI, 2>(&tmA, &tmB, &tmB2, &tmC, &tmCT, p, smem_raw, bars, &tmem_slot, &abort_flag);
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void *ptr = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-        qres == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(ptr);
-  }
-  return fn;
-}
-
 __global__ void merge_partials_kernel(const float *part_m, const float *part_s, const int32_t *part_i,
                                       int n_tiles, int rows_padded, int32_t *pred, float *conf) {
   grid_dep_launch();
@@ -436,13 +417,27 @@ __global__ void merge_partials_kernel(const float *part_m, const float *part_s, 
 
 }  // namespace
 
+TmaEncodeFn tma_encode_fn() {
+  static TmaEncodeFn fn = nullptr;
+  static bool tried = false;
+  if (!tried) {
+    tried = true;
+    void *ptr = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
+        qres == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<TmaEncodeFn>(ptr);
+  }
+  return fn;
+}
+
 l2pd_status make_tma_2d_bf16(TmaDesc *out, const void *ptr, int64_t rows, int64_t cols, int box_rows) {
   return make_tma_2d_bf16_strided(out, ptr, rows, cols, cols, box_rows);
 }
 
 l2pd_status make_tma_2d_bf16_strided(TmaDesc *out, const void *ptr, int64_t rows, int64_t cols, int64_t row_stride,
                                      int box_rows) {
-  EncodeTiledFn fn = get_encode_fn();
+  TmaEncodeFn fn = tma_encode_fn();
   if (!fn) return L2PD_ERR_CUDA;
   if ((reinterpret_cast<uintptr_t>(ptr) & 15) || (cols % 8) || (row_stride % 8) || row_stride < cols || box_rows < 1 ||
       box_rows > 256)
@@ -458,7 +453,7 @@ l2pd_status make_tma_2d_bf16_strided(TmaDesc *out, const void *ptr, int64_t rows
 }
 
 l2pd_status make_tma_out_3d(TmaDesc *out, void *ptr, bool fp32, int64_t rows, int64_t N, int tile_w) {
-  EncodeTiledFn fn = get_encode_fn();
+  TmaEncodeFn fn = tma_encode_fn();
   if (!fn) return L2PD_ERR_CUDA;
   const int es = fp32 ? 4 : 2;
   const int64_t full = N / tile_w;
@@ -475,7 +470,7 @@ l2pd_status make_tma_out_3d(TmaDesc *out, void *ptr, bool fp32, int64_t rows, in
 }
 
 l2pd_status make_tma_out_tail(TmaDesc *out, void *ptr, bool fp32, int64_t rows, int64_t N, int tail_w) {
-  EncodeTiledFn fn = get_encode_fn();
+  TmaEncodeFn fn = tma_encode_fn();
   if (!fn) return L2PD_ERR_CUDA;
   const int es = fp32 ? 4 : 2;
   if (tail_w < 1 || tail_w >= N || ((tail_w * es) % 16) || ((N * es) % 16) || rows < 1) return L2PD_ERR_SHAPE;
@@ -528,7 +523,7 @@ static double plan_cost(int M, int N, int K, int num_sms, int cg, int slabs, int
   return span;
 }
 
-GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits) {
+GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, int max_k_splits, double *cost) {
   GemmPlan best{1, 256, 1, 1, 0};
   double best_cost = 1e300;
   const bool swiglu = epi == EPI_SWIGLU;
@@ -551,6 +546,7 @@ GemmPlan plan_gemm(int epi, int M, int N, int K, int num_sms, int force_tile_n, 
     }
   }
   if (force_tile_n && best_cost > 1e299) best.tile_n = force_tile_n;
+  if (cost) *cost = best_cost;
   return best;
 }
 

@@ -109,6 +109,26 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint32_t bar, uint32_t parity
   return true;
 }
 
+// The same for a whole converged warp whose wait lasts thousands of cycles, with one answer for every lane: it sleeps between
+// polls, as mbar_wait_idle does.
+__device__ __forceinline__ bool mbar_wait_idle_or_abort(uint32_t bar, uint32_t parity, uint32_t sleep_ns, int *abort_flag, int32_t *status,
+                                                        int code, uint64_t limit_ns = 2000000000ull) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  volatile int *const ab = abort_flag;
+  const uint64_t t0 = globaltimer();
+  uint32_t spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    __nanosleep(sleep_ns);
+    if (__any_sync(0xffffffffu, *ab != 0)) return false;
+    if ((++spins & 0x3fu) == 0 && __any_sync(0xffffffffu, globaltimer() - t0 > limit_ns)) {
+      if (status) atomicCAS(status, 0, code);
+      *ab = 1;
+      return false;
+    }
+  }
+  return true;
+}
+
 // ---- thread-block clusters (pairs of CTAs sharing one MMA tile) -----------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
   uint32_t r;
@@ -157,6 +177,27 @@ __device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const CUtens
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "l"(policy)
       : "memory");
+}
+// The same two loads through a 5-D map.
+__device__ __forceinline__ void tma_load_5d_hint(uint32_t dst, const CUtensorMap *m, uint32_t bar, int c0, int c1, int c2, int c3, int c4,
+                                                 uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_pair_hint(uint32_t dst, const CUtensorMap *m, uint32_t bar, int c0, int c1, int c2, int c3,
+                                                      int c4, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(policy)
+      : "memory");
+}
+// Copies shared memory of this CTA to that of a CTA of the cluster (dst and bar are shared::cluster addresses of it), the bytes
+// counted on its mbarrier.  16-byte aligned addresses and size.
+__device__ __forceinline__ void bulk_copy_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
 // Tiled stores shared -> global through a 3-D tensor map (coordinates c0 innermost), tracked by the
 // issuing thread's bulk async-group; the reduce form adds the fp32 tile to what global memory holds.

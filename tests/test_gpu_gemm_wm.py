@@ -1,0 +1,79 @@
+"""The GEMM with the weights on the M side of the MMA, at the edges of its tiles, and the merge of the LM head's records, at the
+edges of the blocks of rows a warp takes; against the oracle's functions."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from oracle import l2pd_oracle as orc
+from paper_2509_25188_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+WM = 10_000_000   # tile code: weights on the M side; the width is the rows of a tile
+
+
+def _bf16(seed, stream, shape, std):
+    return wl.make_activations(seed, stream, shape, std, "bf16")
+
+
+def _close_bf16(got, want, sums):
+    # fp32 sums of K exact products, K 2^-24 of the sum of magnitudes at most, then one rounding to bf16 (2^-9, twice for the
+    # two roundings of a SwiGLU's factors in fp32 arithmetic of a few ulp)
+    assert (np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + sums).all()
+
+
+@pytest.mark.parametrize("M,N,K,tile", [(1, 128, 64, 1032), (15, 104, 72, 1032), (17, 256, 1032, 1032), (128, 136, 192, 1128),
+                                        (129, 520, 320, 1144), (257, 1040, 136, 2144), (300, 528, 1032, 2112), (513, 264, 512, 2256),
+                                        (1029, 2064, 320, 2176), (700, 1536, 128, 1064)])
+def test_gemm_with_rows_on_the_n_side(M, N, K, tile):
+    """One row, tiles with a ragged last chunk, several row tiles per weight tile, weight tiles with a ragged end, single CTAs and
+    pairs (the second CTA without features too), a K tail; gate and up matrices in either order of address."""
+    from paper_2509_25188_b200 import binding as b
+    A, W, W2 = _bf16(11, 0, (M, K), 1.0), _bf16(11, 1, (N, K), 0.05), _bf16(11, 2, (N, K), 0.05)
+    a, w, w2 = orc.widen(A), orc.widen(W), orc.widen(W2)
+    dA, dW, dW2 = b.to_device(A), b.to_device(W), b.to_device(W2)
+    want, up = orc.linear(a, W), orc.linear(a, W2)
+    mag, mag2 = np.abs(a) @ np.abs(w).T, np.abs(a) @ np.abs(w2).T
+    eps = (K + 4) * 2.0 ** -24
+    _close_bf16(b.gemm_bf16(dA, dW, WM + tile).float().cpu().numpy(), want, eps * mag)
+    # |silu'| < 1.1, so an error of the gate's sum moves the result by 1.1 |up| of it
+    for g, u, gm, um, dg, du in ((want, up, mag, mag2, dW, dW2), (up, want, mag2, mag, dW2, dW)):
+        _close_bf16(b.gemm_bf16_swiglu(dA, dg, du, WM + tile).float().cpu().numpy(), orc.silu(g) * u,
+                    eps * (1.1 * np.abs(u) * gm + np.abs(g) * um) + 2.0 ** -20 * np.abs(g * u))
+    X = wl.make_activations(11, 3, (M, N), 1.0, "fp32")
+    got = b.gemm_bf16_residual(dA, dW, b.to_device(X.copy()), WM + 10000 + tile).cpu().numpy()
+    assert (np.abs(got - (X.astype(np.float64) + want)) <= eps * (mag + np.abs(X))).all()
+
+
+@pytest.mark.parametrize("M,N,K,slices", [(1, 128, 1024, 4), (3, 520, 1032, 2), (5, 520, 4104, 4), (32, 4096, 2048, 4), (97, 1000, 1024, 2),
+                                          (125, 4096, 1024, 4), (128, 512, 2048, 4)])
+def test_k_slices_of_a_cluster(M, N, K, slices):
+    """Slices that meet in shared memory: CTAs without rows of their own, uneven shares, a ragged feature tile, a shorter last
+    slice.  The sum is taken in slice order, so that it repeats bit for bit."""
+    from paper_2509_25188_b200 import binding as b
+    A, W = _bf16(12, 0, (M, K), 1.0), _bf16(12, 1, (N, K), 0.05)
+    X = wl.make_activations(12, 2, (M, N), 1.0, "fp32")
+    a, dA, dW = orc.widen(A), b.to_device(A), b.to_device(W)
+    code = WM + 10000 * slices + 1000 + max(32, (M + 15) // 16 * 16)
+    got = [b.gemm_bf16_residual(dA, dW, b.to_device(X.copy()), code).cpu().numpy() for _ in range(2)]
+    bound = (K + 4) * 2.0 ** -24 * (np.abs(a) @ np.abs(orc.widen(W)).T + np.abs(X))
+    assert (np.abs(got[0] - (X.astype(np.float64) + orc.linear(a, W))) <= bound).all()
+    assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("block,vocab", [(1, 2000), (15, 2000), (16, 70), (17, 5000), (33, 2000), (64, 20000)])
+def test_merge_of_the_records_of_a_block(block, vocab):
+    """Fewer and more records than warps, one and several blocks of rows, the last of them ragged."""
+    from paper_2509_25188_b200 import binding as b
+    shape = wl.ModelShape(n_layers=1, d_model=128, n_heads=1, head_dim=128, d_ff=256, vocab=vocab, rms_eps=1e-5, rope_theta=10000.0,
+                          mask_id=vocab - 1, eot_id=vocab - 2, dtype="bf16")
+    dec = b.Decoder(shape, wl.make_weights(shape, seed=3, final_norm_gain=wl.spread_gain(shape)), None, block_len=block, max_batch=3,
+                    max_seq=7 + block, use_filter=False)
+    dec.state_reset(wl.make_prompts(3, 7, shape, seed=2), block)
+    out = dec.denoise_step(want_logits=True)
+    dec.close()
+    pred, conf, _ = orc.confidence_head(out["logits"].reshape(3 * block, vocab).astype(np.float64))
+    assert np.array_equal(out["pred"].reshape(-1), pred)
+    # sums of `vocab` exponentials in fp32, each a few ulp
+    assert np.abs(out["conf"].reshape(-1) - conf).max() <= 1e-5
