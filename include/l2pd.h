@@ -341,12 +341,14 @@ void l2pd_destroy(l2pd_ctx *ctx);
 
 /* C[M,N] (bf16) = A[M,K] (bf16, row-major) x W[N,K]^T (bf16, row-major); tcgen05 path.
  * K and N multiples of 8.  tile_n = width + 1000 * cta_group + 10000 * k_splits + 100000 * slabs
- * + 1000000 * k_interleave, every part optional (0 = chosen automatically): width a multiple of 16 in
+ * + 1000000 * k_interleave + 10000000 * orientation, every part optional (0 = chosen automatically): width a multiple of 16 in
  * [32, 256]; cta_group 1, or 2 for a pair of SMs on one 256-row tile; k_splits (residual epilogue only)
  * slices K, the slices adding into X with floating-point reductions whose order is not fixed; slabs 2
  * (pairs only) lets one unit cover two 256-row slabs against one load of the weight tile; k_interleave
  * 1 (one slab only) has two threads issue the MMAs of alternate k-blocks into two accumulators that the
  * epilogue adds (never chosen automatically), 2 says that it is not wanted.
+ * orientation 1 puts the weights on the M side of the MMA (width = rows of A to a tile; 2 or 4 K slices, for at most 128 rows,
+ * meet inside a cluster and are added in slice order), 2 keeps A there.
  * A and the output follow stream order.  The weights W are requested before the kernel launched
  * just ahead of this one in the stream has completed (programmatic dependent launch): that kernel
  * must not be the one that writes them. */
