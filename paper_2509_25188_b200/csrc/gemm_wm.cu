@@ -326,12 +326,13 @@ gemm_wm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         break;
       }
       if (ok && feats) {
-        uint32_t v[CH], vn[CH];
+        // a chunk's columns are asked for as soon as the ones before have left the registers for shared memory; nothing reads the
+        // registers between a load and its wait (they are undefined until then)
+        uint32_t v[CH];
         if (half * CH < t_end) ptx::tmem_ld_x16(taddr + half * CH, v);
         for (int c = half; c * CH < t_end; c += 2) {
           ptx::tmem_ld_wait();
           const bool more = (c + 2) * CH < t_end;
-          if (more) ptx::tmem_ld_x16(taddr + (c + 2) * CH, vn);
           float4 now[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) now[i] = ahead[i];
@@ -339,6 +340,7 @@ gemm_wm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
           for (int i = 0; i < CH; ++i)
             asm volatile("st.shared.b32 [%0], %1;" ::"r"(stg + (uint32_t)(i * ROW_F + lane) * 4u), "r"(v[i]) : "memory");
+          if (more) ptx::tmem_ld_x16(taddr + (c + 2) * CH, v);
           __syncwarp();
           const int tc = c * CH, n_rows = t_end - tc;       // rows of this chunk (>= 16: all)
           if (EPI == EPI_RESIDUAL) {
@@ -420,8 +422,6 @@ gemm_wm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
             }
           }
           __syncwarp();
-#pragma unroll
-          for (int i = 0; i < CH; ++i) v[i] = vn[i];
         }
       }
       ptx::tc_fence_before_sync();
