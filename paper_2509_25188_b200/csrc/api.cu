@@ -536,7 +536,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     WmArgs a = wm_args(EPI_QKV_ROPE, 3 * hd, d, c->wm_qkv, l);
     a.wv = &c->tw_v[l]; a.hd = hd; a.dh = dh; a.cs_table = c->cs_table; a.row_pos = c->d_row_pos;
     if (c->fuse_rope) { a.q = (bf16 *)c->qkv; a.k = a.q + hd; a.v = a.k + hd; a.q_stride = a.kv_stride = 3 * hd; }
-    else { a.q = (bf16 *)c->q; a.k = (bf16 *)kc; a.v = (bf16 *)vc; a.q_stride = a.kv_stride = hd; a.kv_row = c->d_row_kv; a.natural = 1; }
+    else { a.q = (bf16 *)c->q; a.k = (bf16 *)kc; a.v = (bf16 *)vc; a.q_stride = a.kv_stride = hd; a.kv_row = c->d_row_kv; a.natural = 1; a.round_first = !lean; }   // (not lean: the same bits as the other modes)
     if (lean && l > 0) { a.ss_in = c->ss; a.ss_n = ceil_div(d, c->wm_down.plan.w_rows); }   // (the embedding's rows are normalised)
     return a;
   };

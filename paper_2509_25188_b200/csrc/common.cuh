@@ -243,8 +243,8 @@ struct WmArgs {
   bf16 *out; int64_t out_stride;              // STORE, SWIGLU
   int up_first;               // SwiGLU: `w` starts at the up projection
   // QKV: q row = row, k and v row = kv_row[row] (null: row); cs_table [position][dh / 2], row_pos [T].  natural: dimensions in
-  // their order, otherwise rotary pairs adjacent
-  bf16 *q, *k, *v; int64_t q_stride, kv_stride; const int32_t *kv_row, *row_pos; const float2 *cs_table; int hd, dh, natural;
+  // their order, otherwise rotary pairs adjacent.  round_first: q and k are rounded to bf16 before the rotation as well as after it
+  bf16 *q, *k, *v; int64_t q_stride, kv_stride; const int32_t *kv_row, *row_pos; const float2 *cs_table; int hd, dh, natural, round_first;
   // RESIDUAL: x += acc.  K slices: summed inside a cluster (in_cluster), or partial sums at part + slice * part_stride [T][N] that
   // the caller adds, or atomics (part = null)
   float *xres, *part; int64_t part_stride; int in_cluster;

@@ -10,7 +10,8 @@
 // Epilogues
 //   EPI_STORE     C (bf16)  = acc
 //   EPI_QKV_ROPE  q, k rotated by the row's position (pairs (i, i + dh/2) of a head), v as it is; each part has a pointer of its
-//                 own, k and v go to row kv_row[row] of theirs (the key/value store)
+//                 own, k and v go to row kv_row[row] of theirs (the key/value store).  round_first: q and k are rounded to bf16 ahead
+//                 of the rotation too, so that the result is that of the two kernels this replaces, bit for bit
 //   EPI_RESIDUAL  X (fp32) += acc; K slices either add (atomics), store partial sums for a later sum in slice order, or are the
 //                 CTAs of a cluster, which exchange their sums through shared memory: each adds a share of the rows, in slice order
 //   EPI_SWIGLU    H (bf16)  = silu(acc_gate) * acc_up
@@ -69,7 +70,7 @@ struct Params {
   bf16 *out; int64_t out_stride;                  // STORE, SWIGLU
   bf16 *q, *k, *v; int64_t q_stride, kv_stride;   // QKV
   const int32_t *kv_row, *row_pos; const float2 *cs;
-  int hd, dh, natural;
+  int hd, dh, natural, round_first;
   int res_mode;
   float *x, *part; int64_t part_stride;
   bf16 *n; const float *gain; float *ss_out;      // n != null: leave bf16(x gain) and the sums of squares
@@ -405,7 +406,11 @@ gemm_wm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                 } else {
                   // dimensions dim0 .. dim0 + 3 and their partners
                   const float4 c01 = now[2 * it], c23 = now[2 * it + 1];
-                  const float xa[4] = {a.x * s, a.y * s, a.z * s, a.w * s}, xb[4] = {b.x * s, b.y * s, b.z * s, b.w * s};
+                  float xa[4] = {a.x * s, a.y * s, a.z * s, a.w * s}, xb[4] = {b.x * s, b.y * s, b.z * s, b.w * s};
+                  if (p.round_first) {   // as a projection that stores bf16 and a rotation kernel behind it
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) { xa[e] = __bfloat162float(__float2bfloat16_rn(xa[e])); xb[e] = __bfloat162float(__float2bfloat16_rn(xb[e])); }
+                  }
                   const float co[4] = {c01.x, c01.z, c23.x, c23.z}, si[4] = {c01.y, c01.w, c23.y, c23.w};
                   float ya[4], yb[4];
 #pragma unroll
@@ -636,7 +641,7 @@ cudaError_t launch_gemm_wm(cudaStream_t st, const WmArgs &g, int num_sms) {
   p.up_first = g.up_first;
   p.out = g.out; p.out_stride = g.out_stride;
   p.q = g.q; p.k = g.k; p.v = g.v; p.q_stride = g.q_stride; p.kv_stride = g.kv_stride; p.kv_row = g.kv_row; p.row_pos = g.row_pos;
-  p.cs = g.cs_table; p.hd = g.hd; p.dh = g.dh; p.natural = g.natural;
+  p.cs = g.cs_table; p.hd = g.hd; p.dh = g.dh; p.natural = g.natural; p.round_first = g.round_first;
   p.x = g.xres; p.part = g.part; p.part_stride = g.part_stride;
   p.n = g.n; p.gain = g.gain; p.ss_out = g.ss_out; p.ss_in = g.ss_in; p.ss_n = g.ss_in ? g.ss_n : 0; p.ss_stride = g.ss_stride;
   p.eps = g.eps; p.inv_width = g.width > 0 ? 1.0f / (float)g.width : 0.f;

@@ -1,0 +1,57 @@
+"""Which kernel a step's projections take, and what may not depend on it.  The form that ran is told from the launches of the kinds
+it does without (profile_read)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_2509_25188_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = ("logits", "conf", "pred", "p", "unmask", "masks_left", "l_eff", "done", "forced")
+
+
+def _shape(head_dim, n_heads, d, d_ff, layers=3):
+    return wl.ModelShape(n_layers=layers, d_model=d, n_heads=n_heads, head_dim=head_dim, d_ff=d_ff, vocab=1000, rms_eps=1e-5,
+                         rope_theta=10000.0, mask_id=999, eot_id=998, dtype="bf16")
+
+
+def _decoder(shape, w, s, B, max_seq, kv=0, filt=None):
+    from paper_2509_25188_b200 import binding
+    return binding.Decoder(shape, w, filt, block_len=s, max_batch=B, max_seq=max_seq, kv_cache=kv, use_filter=filt is not None,
+                           use_eotp=False)
+
+
+def _launches(dec, kind):
+    return dec.profile_read().get(kind, (0.0, 0))[1]
+
+
+@pytest.mark.parametrize("head_dim,heads,kv,B,P,G,steps,unfused", [
+    (128, 4, 2, 1, 172, 128, 1, False),    # 300 rows that fill the store
+    (128, 4, 1, 3, 172, 128, 2, False),    # 900, then 384 rows against it
+    (64, 8, 0, 2, 57, 96, 2, False),       # heads of 64: 306 rows
+    (64, 8, 2, 2, 172, 128, 1, False),
+    (64, 3, 0, 1, 193, 64, 2, False),      # q, k and v of 192 features: 257 rows
+    (128, 4, 0, 1, 268, 32, 2, True)])     # the rotation kept apart by the switch
+def test_modes_agree_where_the_rotation_is_not_fused(monkeypatch, head_dim, heads, kv, B, P, G, steps, unfused):
+    """With more than 256 rows the three modes agree bit for bit also where q and k pass through bf16 before they are rotated."""
+    if unfused:
+        monkeypatch.setenv("L2PD_NO_ROPE_FUSION", "1")
+    shape = _shape(head_dim, heads, 512 if heads > 3 else 256, 1376)
+    dec = _decoder(shape, wl.make_weights(shape, seed=0, final_norm_gain=wl.spread_gain(shape)), 32, B, P + G, kv)
+    prompts = wl.make_prompts(B, P, shape, seed=5)
+    got = []
+    for mode in (0, 1, 2):
+        dec.set_chain(mode)
+        dec.state_reset(prompts, G)
+        dec.profile_enable(["rope"])
+        got.append([dec.denoise_step(want_logits=True) for _ in range(steps)])
+        if not unfused:   # mode 0 rotates in the projection, the others in a kernel of its own
+            assert _launches(dec, "rope") == (0 if mode == 0 else steps * shape.n_layers)
+        assert dec.last_step_rows > 256
+    dec.close()
+    for mode in (1, 2):
+        for a, b in zip(got[0], got[mode]):
+            for k in FIELDS:
+                assert np.array_equal(a[k], b[k]), "mode %d and mode 0 differ in %s" % (mode, k)
