@@ -262,8 +262,8 @@ cudaError_t launch_decide(cudaStream_t st, const DecideArgs &a, int n_slots) {
   threads = threads < 256 ? 256 : (threads > 1024 ? 1024 : threads);
   const int rl = a.s > 16 ? 32 : 16;
   const size_t smem = sizeof(float) * 3 * (threads / rl) * (rl + 1);
-  cudaError_t e = cudaFuncSetAttribute(decide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  // beside the kernel's own arrays within what any launch may have: a limit set here would hold for every thread's launches
+  static_assert(sizeof(float) * (2 * MAX_S * (MAX_S + 1) + 11 * MAX_S + 4) + sizeof(float) * 3 * 32 * 33 <= 48 * 1024, "shared memory of the decision kernel");
   return launch_kernel(decide_kernel, dim3(n_slots), dim3(threads), smem, st, a);
 }
 
