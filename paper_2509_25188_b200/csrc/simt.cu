@@ -491,12 +491,15 @@ template <typename T>
 cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, const T *vc,
                                   const SeqMeta *meta, const int32_t *row_slot, T *out,
                                   int64_t kv_seq_stride, int rows, int H, int dh, int max_kv, int n_slots, int max_q) {
+  // The limits of shared memory are set to what a call can ask for at most: they belong to the kernel, not to the call, and a thread
+  // with smaller tiles would take them from under another's launch.
   // the grid's z holds the sequences; of more of them, a block per row and head takes any number
   if constexpr (std::is_same<T, float>::value) {   // q, K and V are the library's own buffers: rows of H * dh floats, 16-byte aligned
     if (n_slots <= MAX_GRID_YZ) {
       auto bytes = [&](int bufs) { return (int)(sizeof(float) * ((size_t)(A_Q + 2 * bufs * A_K) * ((dh + 3) / 4 * 4 + 4) + A_Q * (A_K + 4))); };
-      const int bufs = max_kv > A_K && bytes(2) <= 200 * 1024 ? 2 : 1;
-      cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes(bufs));
+      constexpr int most = 200 * 1024;   // (one buffer of the widest head: 140 KB)
+      const int bufs = max_kv > A_K && bytes(2) <= most ? 2 : 1;
+      cudaError_t e = cudaFuncSetAttribute(attention_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
       if (e != cudaSuccess) return e;
       return launch_kernel(attention_f32_kernel, dim3(ceil_div(max_q, A_Q), H, n_slots), dim3(A_THREADS), (size_t)bytes(bufs), st, q, kc, vc,
                            meta, out, kv_seq_stride, H, dh, bufs);
@@ -504,8 +507,7 @@ cudaError_t launch_simt_attention(cudaStream_t st, const T *q, const T *kc, cons
   }
   size_t smem = (size_t)(dh + max_kv) * sizeof(float);
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(simt_attention_kernel<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(simt_attention_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     if (e != cudaSuccess) return e;
   }
   return launch_kernel(simt_attention_kernel<T>, dim3(rows, H), dim3(128), smem, st, q, kc, vc, meta, row_slot, out,

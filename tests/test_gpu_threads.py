@@ -45,7 +45,9 @@ def _decodes(dec, prompts, G, n, want):
 
 @pytest.mark.parametrize("shapes", [
     # blocks of 16 and 32: other records of the decision kernel
-    [(dict(n_layers=1), 16, 16, 32), (dict(n_layers=1), 32, 16, 32)]])
+    [(dict(n_layers=1), 16, 16, 32), (dict(n_layers=1), 32, 16, 32)],
+    # heads of 32 and 256, one and several key tiles: other tiles of the fp32 attention
+    [(dict(n_layers=1), 16, 16, 32), (dict(n_layers=1, n_heads=1, head_dim=256), 16, 80, 32)]])
 def test_contexts_of_different_sizes_decode_at_once(shapes):
     from paper_2509_25188_b200 import binding
     decs, jobs = [], []
