@@ -417,7 +417,9 @@ __global__ void filter_pack_kernel(PackArgs a, int pack, int32_t *status, unsign
 template <int S, int T, int LM, int TH, int OCC>
 cudaError_t launch_train(cudaStream_t st, TrainArgs &a, int sms, int *blocks) {
   const size_t smem = sizeof(float) * (size_t)train_smem_floats<S, T>(a.n_layers);
-  cudaError_t e = cudaFuncSetAttribute(filter_train_kernel<S, T, LM, TH, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit of the deepest filter of this form: it belongs to the kernel, and another thread may be preparing another depth
+  cudaError_t e = cudaFuncSetAttribute(filter_train_kernel<S, T, LM, TH, OCC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(sizeof(float) * (size_t)train_smem_floats<S, T>(LM)));
   if (e != cudaSuccess) return e;
   int occ = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, filter_train_kernel<S, T, LM, TH, OCC>, TH, smem);

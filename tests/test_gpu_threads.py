@@ -62,3 +62,33 @@ def test_contexts_of_different_sizes_decode_at_once(shapes):
     _together(jobs)
     for dec in decs:
         dec.close()
+
+
+def test_filters_of_different_depths_train_at_once():
+    """Filters of three and four layers share a kernel; what they hold in shared memory differs in size.  One update a launch, so that
+    a call prepares a thousand of them."""
+    import ctypes
+    import torch
+    from paper_2509_25188_b200 import binding as b
+    s, n, epochs = 16, 32, 1000
+    rng = np.random.default_rng(0)
+    c = torch.from_numpy(rng.random((n, s), dtype=np.float32)).cuda()
+    y = (c > 0.6).to(torch.uint8)
+    cfg = b.TrainConfig(1e-3, 0.9, 0.999, 1e-8, 0.01, epochs, 0)
+
+    def job(depth):
+        layers = [((np.eye(s) + 0.1 * rng.standard_normal((s, s))).astype(np.float32), np.zeros(s, np.float32)) for _ in range(depth)]
+        want, _ = b.filter_train_layers(layers, c, y, epochs)
+        w, bias = [torch.from_numpy(q).cuda() for q, _ in layers], [torch.from_numpy(q).cuda() for _, q in layers]
+        pw, pb = ((ctypes.c_void_p * depth)(*[t.data_ptr() for t in ts]) for ts in (w, bias))
+        losses = np.zeros(epochs, np.float32)
+        torch.cuda.synchronize()
+
+        def run():
+            r = b.lib.l2pd_debug_filter_train(torch.cuda.current_stream().cuda_stream, s, depth, n, c.data_ptr(), y.data_ptr(), pw, pb,
+                                              ctypes.byref(cfg), losses.ctypes.data, 1, 2_000_000_000, -1)
+            assert r == 0, b.lib.l2pd_last_error(None).decode()
+            for t, u, (ww, wb) in zip(w, bias, want):
+                assert np.array_equal(t.cpu().numpy(), ww) and np.array_equal(u.cpu().numpy(), wb)
+        return run
+    _together([job(3), job(4)])
