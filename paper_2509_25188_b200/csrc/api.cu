@@ -326,20 +326,23 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     lean = c->chain_mode == 0 && c->wm_gate_up && c->wm_qkv_rope && T_rows <= LEAN_MAX_ROWS;
     // the rotation and the scatter are a kernel of their own where the projection does not do them
     if (!c->fuse_rope) cost_qkv += 4000.0 + 12.0 * T_rows * hd / 3100.0;
-    auto wm_plan = [&](l2pd_ctx::WmGemm &g, int epi, int N, int K, double other, int ks) {
+    // asked only where its answer can be taken: the search takes up to 12 us ahead of the step's first launch
+    auto wm_plan = [&](l2pd_ctx::WmGemm &g, int epi, int N, int K, double other, int ks, bool can) {
+      g.on = false;
+      if (!can || (!lean && T_rows <= WM_MIN_ROWS)) return;
       g.plan = plan_gemm_wm(epi, T_rows, N, K, c->num_sms, lean ? 4 : ks, lean);
-      g.on = lean || (T_rows > WM_MIN_ROWS && g.plan.cost * WM_MARGIN < other);
+      g.on = lean || g.plan.cost * WM_MARGIN < other;
     };
-    wm_plan(c->wm_qkv, EPI_QKV_ROPE, 3 * hd, d, cost_qkv, 1);
-    wm_plan(c->wm_o, EPI_RESIDUAL, d, hd, cost_o, c->ksum ? max_ks : 1);
-    wm_plan(c->wm_down, EPI_RESIDUAL, d, F, cost_down, c->ksum ? max_ks : 1);
-    wm_plan(c->wm_gu, EPI_SWIGLU, F, d, cost_gu, 1);
-    if (!c->wm_gate_up) c->wm_gu.on = false;
-    if (!c->wm_qkv_rope) c->wm_qkv.on = false;
+    const bool single = c->chain_mode == 0;
+    wm_plan(c->wm_qkv, EPI_QKV_ROPE, 3 * hd, d, cost_qkv, 1, single && c->wm_qkv_rope);
+    wm_plan(c->wm_gu, EPI_SWIGLU, F, d, cost_gu, 1, single && c->wm_gate_up);
+    // (the chained modes take these two's K slices)
+    wm_plan(c->wm_o, EPI_RESIDUAL, d, hd, cost_o, c->ksum ? max_ks : 1, true);
+    wm_plan(c->wm_down, EPI_RESIDUAL, d, F, cost_down, c->ksum ? max_ks : 1, true);
     // slices that a later kernel adds (in a lean step there are none)
     if (c->wm_o.on) c->pl_o.k_splits = lean ? 1 : c->wm_o.plan.k_splits;
     if (c->wm_down.on) c->pl_down.k_splits = lean ? 1 : c->wm_down.plan.k_splits;
-    if (c->chain_mode != 0) c->wm_qkv.on = c->wm_o.on = c->wm_down.on = c->wm_gu.on = false;
+    if (!single) c->wm_o.on = c->wm_down.on = false;
     auto wm_maps = [&](l2pd_ctx::WmGemm &g, const void *act, int64_t K, const std::vector<const void *> *w, const std::vector<const void *> *up, int64_t N) -> l2pd_status {
       if (!g.on) return L2PD_OK;
       const int xb = g.plan.tile_t / g.plan.cta_group;
