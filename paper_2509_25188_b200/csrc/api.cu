@@ -324,14 +324,16 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks, &cost_down);
     c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0, 1, &cost_gu);
     lean = c->chain_mode == 0 && c->wm_gate_up && c->wm_qkv_rope && T_rows <= LEAN_MAX_ROWS;
-    // the rotation and the scatter are a kernel of their own where the projection does not do them
-    if (!c->fuse_rope) cost_qkv += 4000.0 + 12.0 * T_rows * hd / 3100.0;
+    // The rotation and the scatter are a kernel of their own where the projection does not do them: its bytes, and 4000 cycles for
+    // its launch; 400 ahead of the warp-level attention (heads of 64), whose blocks come up under that kernel but not beside a
+    // projection, which has all of an SM's shared memory.
+    if (!c->fuse_rope) cost_qkv += (c->attn_tc ? 4000.0 : 400.0) + 12.0 * T_rows * hd / 3100.0;
     // asked only where its answer can be taken: the search takes up to 12 us ahead of the step's first launch
     auto wm_plan = [&](l2pd_ctx::WmGemm &g, int epi, int N, int K, double other, int ks, bool can) {
       g.on = false;
       if (!can || (!lean && T_rows <= WM_MIN_ROWS)) return;
       g.plan = plan_gemm_wm(epi, T_rows, N, K, c->num_sms, lean ? 4 : ks, lean);
-      g.on = lean || g.plan.cost * WM_MARGIN < other;
+      g.on = lean || (g.plan.cost * WM_MARGIN < other && g.plan.cost + wm_exposed_drain(epi, g.plan, T_rows, N, K, c->num_sms) < other);
     };
     const bool single = c->chain_mode == 0;
     wm_plan(c->wm_qkv, EPI_QKV_ROPE, 3 * hd, d, cost_qkv, 1, single && c->wm_qkv_rope);

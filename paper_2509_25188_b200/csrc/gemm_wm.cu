@@ -603,6 +603,20 @@ WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits,
   return best;
 }
 
+// The rotating epilogue takes 82 cycles a row of the tile (measured, d = 512, cycles a unit: 32 rows 3440, 96 8500, 176 14600), where
+// the plan reckons with 20, and hides only behind the next unit's k-blocks.  With few of them (a narrow model) it is what the
+// projection takes: 4096 rows at d = 512 16 us on the other side, 27 here; 2048 at d = 1024 19 and 29; 1029 at d = 4096 110 and 87.
+// A decision between the sides that knows of it, four layers, rows in one to sixteen sequences of 257 to 8192, against one that does
+// not: d = 512, heads of 64, 770 rows 238 -> 218 us, 4096 rows 433 -> 418; d = 1024, 4096 rows 735 -> 707, heads of 128 with a cache
+// 623 -> 594; d = 4096 as before.  (The tiles stay those of the plan.)
+double wm_exposed_drain(int epi, const WmPlan &pl, int T, int N, int K, int num_sms) {
+  if (epi != EPI_QKV_ROPE) return 0.0;
+  const int rounds = ceil_div(ceil_div(N, pl.w_rows * pl.cta_group) * ceil_div(T, pl.tile_t), num_sms / pl.cta_group);
+  const double drain = 82.0 * pl.tile_t, bytes = 128.0 * pl.w_rows + 128.0 * pl.tile_t / pl.cta_group;
+  const double loop = ceil_div(K, BK) * (fmax(fmax(2.0 * pl.tile_t * (pl.cta_group == 1 ? 1.13 : 1.0), 250.0), bytes / 95.0) + (T >= 4096 ? 0.45 : 0.15) * bytes / 95.0) + 400.0;
+  return (rounds - 1) * fmax(0.0, drain - loop) + drain - 20.0 * pl.tile_t;
+}
+
 l2pd_status make_tma_halves(TmaDesc *out, const void *ptr, int64_t K, int64_t half_bytes, int64_t groups, int box_groups, int64_t outer,
                             int64_t outer_bytes, int box_outer) {
   TmaEncodeFn fn = tma_encode_fn();

@@ -27,15 +27,16 @@ def _launches(dec, kind):
     return dec.profile_read().get(kind, (0.0, 0))[1]
 
 
-@pytest.mark.parametrize("head_dim,heads,kv,B,P,G,steps,unfused", [
-    (128, 4, 2, 1, 172, 128, 1, False),    # 300 rows that fill the store
-    (128, 4, 1, 3, 172, 128, 2, False),    # 900, then 384 rows against it
-    (64, 8, 0, 2, 57, 96, 2, False),       # heads of 64: 306 rows
-    (64, 8, 2, 2, 172, 128, 1, False),
-    (64, 3, 0, 1, 193, 64, 2, False),      # q, k and v of 192 features: 257 rows
-    (128, 4, 0, 1, 268, 32, 2, True)])     # the rotation kept apart by the switch
-def test_modes_agree_where_the_rotation_is_not_fused(monkeypatch, head_dim, heads, kv, B, P, G, steps, unfused):
-    """With more than 256 rows the three modes agree bit for bit also where q and k pass through bf16 before they are rotated."""
+@pytest.mark.parametrize("head_dim,heads,kv,B,P,G,steps,unfused,m_side", [
+    (128, 4, 2, 1, 172, 128, 1, False, True),    # 300 rows that fill the store
+    (128, 4, 1, 3, 172, 128, 2, False, True),    # 900, then 384 rows against it
+    (64, 8, 0, 2, 57, 96, 2, False, True),       # heads of 64: 306 rows
+    (64, 8, 2, 1, 172, 128, 1, False, True),
+    (64, 3, 0, 1, 193, 64, 2, False, False),     # q, k and v of 192 features: 257 rows
+    (128, 4, 0, 1, 268, 32, 2, True, False)])    # the rotation kept apart by the switch
+def test_modes_agree_where_the_rotation_is_not_fused(monkeypatch, head_dim, heads, kv, B, P, G, steps, unfused, m_side):
+    """With more than 256 rows the three modes agree bit for bit also where q and k pass through bf16 before they are rotated.
+    m_side: mode 0 rotates in a projection with the weights on the M side."""
     if unfused:
         monkeypatch.setenv("L2PD_NO_ROPE_FUSION", "1")
     shape = _shape(head_dim, heads, 512 if heads > 3 else 256, 1376)
@@ -47,11 +48,26 @@ def test_modes_agree_where_the_rotation_is_not_fused(monkeypatch, head_dim, head
         dec.state_reset(prompts, G)
         dec.profile_enable(["rope"])
         got.append([dec.denoise_step(want_logits=True) for _ in range(steps)])
-        if not unfused:   # mode 0 rotates in the projection, the others in a kernel of its own
-            assert _launches(dec, "rope") == (0 if mode == 0 else steps * shape.n_layers)
+        if not unfused:
+            assert _launches(dec, "rope") == (0 if mode == 0 and m_side else steps * shape.n_layers)
         assert dec.last_step_rows > 256
     dec.close()
     for mode in (1, 2):
         for a, b in zip(got[0], got[mode]):
             for k in FIELDS:
                 assert np.array_equal(a[k], b[k]), "mode %d and mode 0 differ in %s" % (mode, k)
+
+
+@pytest.mark.parametrize("head_dim,heads,kv,B,L,m_side", [
+    (64, 8, 0, 2, 153, True), (64, 8, 0, 2, 385, False),      # 306 and 770 rows
+    (128, 4, 1, 1, 300, True), (128, 4, 1, 8, 512, False)])   # 300 and 4096 rows, with a store
+def test_narrow_models_rotate_in_the_projection_only_where_that_is_faster(head_dim, heads, kv, B, L, m_side):
+    """d = 512: few k-blocks, behind which the rotating epilogue of large tiles does not hide (step of 4 layers, rotation inside and
+    apart: 306 rows 190 and 189 us, 770 rows 238 and 218; 300 rows with a store 188 and 196, 4096 rows 371 and 358)."""
+    shape = _shape(head_dim, heads, 512, 1376)
+    dec = _decoder(shape, wl.make_weights(shape, seed=0, final_norm_gain=1.0), 32, B, L, kv)
+    dec.state_reset(wl.make_prompts(B, L - 32, shape, seed=5), 32)
+    dec.profile_enable(["rope"])
+    dec.denoise_step(outputs=False)
+    assert _launches(dec, "rope") == (0 if m_side else shape.n_layers)
+    dec.close()
