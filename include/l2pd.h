@@ -347,8 +347,9 @@ void l2pd_destroy(l2pd_ctx *ctx);
  * (pairs only) lets one unit cover two 256-row slabs against one load of the weight tile; k_interleave
  * 1 (one slab only) has two threads issue the MMAs of alternate k-blocks into two accumulators that the
  * epilogue adds (never chosen automatically), 2 says that it is not wanted.
- * orientation 1 puts the weights on the M side of the MMA (width = rows of A to a tile; 2 or 4 K slices, for at most 128 rows,
- * meet inside a cluster and are added in slice order), 2 keeps A there.
+ * orientation 1 puts the weights on the M side of the MMA (width = rows of A to a tile; 2 or 4 K slices, on single CTAs with
+ * tiles of at most 128 rows and no more slices of tiles than SMs, meet inside a cluster and are added in slice order; neither
+ * slabs 2 nor k_interleave 1), 2 keeps A there.  What a part's value rules out is L2PD_ERR_SHAPE.
  * A and the output follow stream order.  The weights W are requested before the kernel launched
  * just ahead of this one in the stream has completed (programmatic dependent launch): that kernel
  * must not be the one that writes them. */

@@ -1348,16 +1348,19 @@ static l2pd_status gemm_common(void *stream, int epi, const void *A, const void 
             want_tn = tile_n % 1000;
   const int unit = 16;
   if (want_tn && (want_tn < 32 || want_tn > 256 || (want_tn % unit))) return L2PD_ERR_SHAPE;
-  if (want_cg > 2 || want_ks > 8 || (want_ks > 1 && epi != EPI_RESIDUAL) || want_sl > 2) return L2PD_ERR_SHAPE;
+  if (want_cg > 2 || want_ks > 8 || (want_ks > 1 && epi != EPI_RESIDUAL) || want_sl > 2 || want_or > 2) return L2PD_ERR_SHAPE;
+  if (want_or == 1 && (want_sl == 2 || want_kil == 1)) return L2PD_ERR_SHAPE;   // that side has neither
   double cost = 0.0;
   GemmPlan pl = plan_gemm(epi, M, N, K, sms, want_tn, 4, &cost);
   if (want_or == 1 || (want_or == 0 && !want_kil && tile_n == 0)) {
     WmPlan wp = plan_gemm_wm(epi, M, N, K, sms, 4, true);
     if (want_or == 1) {
-      if (want_tn) wp.tile_t = want_tn;
-      if (want_cg) wp.cta_group = want_cg;
       wp.k_splits = want_ks ? effective_k_splits(K, want_ks) : 1;
       wp.w_rows = 128;
+      const bool sliced = wp.k_splits > 1;   // open parts: single CTAs and a tile that the slices' exchange has room for
+      wp.cta_group = want_cg ? want_cg : sliced ? 1 : wp.cta_group;
+      wp.tile_t = want_tn ? want_tn : sliced ? (int)round_up(ceil_div(M, ceil_div(M, 128)), 16) : wp.tile_t;
+      if (sliced && !wm_slices_in_cluster(wp, M, N, sms)) return L2PD_ERR_SHAPE;
     }
     TmaDesc probe;
     int up_first = 0;

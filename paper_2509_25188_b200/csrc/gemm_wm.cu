@@ -551,7 +551,7 @@ cudaError_t launch(cudaStream_t st, const WmArgs &g, const Params &p, int grid, 
 }  // namespace
 
 // The exchange takes a cluster of single CTAs with one unit each; its shares and slices have room for EXCHANGE_ROWS rows.
-static bool slices_in_cluster(const WmPlan &pl, int T, int N, int num_sms) {
+bool wm_slices_in_cluster(const WmPlan &pl, int T, int N, int num_sms) {
   return pl.cta_group == 1 && pl.w_rows == MMA_ROWS && (pl.k_splits == 2 || pl.k_splits == 4) && pl.tile_t <= EXCHANGE_ROWS &&
          ceil_div(N, pl.w_rows) * ceil_div(T, pl.tile_t) * pl.k_splits <= num_sms;
 }
@@ -586,7 +586,7 @@ WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits,
         if (k_block * k_blocks * w_tiles * t_tiles / groups + fixed >= best.cost) continue;
         for (int ks = 1; ks <= max_ks; ++ks) {
           if (ks > 1 && (k_blocks < 8 * ks || effective_k_splits(K, ks) != ks)) break;
-          if (in_cluster && ks > 1 && !slices_in_cluster(WmPlan{cg, tt, ks, wr, 0.0}, T, N, num_sms)) continue;
+          if (in_cluster && ks > 1 && !wm_slices_in_cluster(WmPlan{cg, tt, ks, wr, 0.0}, T, N, num_sms)) continue;
           const int kb = ceil_div(k_blocks, ks);
           auto unit = [&](int active) {
             return kb * fmax(k_block, 128.0 * wr * cg * active / t_tiles / 3450.0 + traffic * bytes / 95.0) + 400.0;
@@ -670,7 +670,7 @@ cudaError_t launch_gemm_wm(cudaStream_t st, const WmArgs &g, int num_sms) {
   p.eps = g.eps; p.inv_width = g.width > 0 ? 1.0f / (float)g.width : 0.f;
   p.status = g.status;
   p.res_mode = ks == 1 ? RES_ADD : g.in_cluster ? RES_CLUSTER : g.part ? RES_PART : RES_ATOMIC;
-  if (p.res_mode == RES_CLUSTER && (!slices_in_cluster(g.plan, g.T, g.N, num_sms) || p.staging_off < 2 * EXCHANGE_ROWS * EXCHANGE_ROW_BYTES)) return cudaErrorInvalidValue;
+  if (p.res_mode == RES_CLUSTER && (!wm_slices_in_cluster(g.plan, g.T, g.N, num_sms) || p.staging_off < 2 * EXCHANGE_ROWS * EXCHANGE_ROW_BYTES)) return cudaErrorInvalidValue;
   if (g.epi == EPI_RESIDUAL && g.n && (!g.gain || !g.ss_out || (ks > 1 && !g.in_cluster))) return cudaErrorInvalidValue;
   if (g.epi == EPI_QKV_ROPE && ((g.dh != 64 && g.dh != 128) || g.N != 3 * g.hd || !g.wv || !g.cs_table || !g.row_pos)) return cudaErrorInvalidValue;
   const int units = p.w_tiles * p.t_tiles * ks, groups = num_sms / cg;

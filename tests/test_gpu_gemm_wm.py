@@ -77,3 +77,38 @@ def test_merge_of_the_records_of_a_block(block, vocab):
     assert np.array_equal(out["pred"].reshape(-1), pred)
     # sums of `vocab` exponentials in fp32, each a few ulp
     assert np.abs(out["conf"].reshape(-1) - conf).max() <= 1e-5
+
+
+@pytest.mark.parametrize("code,residual,M,N,K", [
+    (WM + 30000, True, 64, 512, 2048),               # three slices
+    (WM + 80000, True, 64, 512, 2048),               # eight
+    (WM + 42000, True, 64, 512, 2048),               # four slices on pairs
+    (WM + 40000 + 1144, True, 300, 512, 2048),       # four slices of tiles of 144 rows
+    (WM + 40000 + 1064, True, 64, 128 * 200, 2048),  # more slices than SMs
+    (WM + 200000, False, 300, 512, 512),             # two slabs of rows, which the weights' side has not
+    (WM + 1000000, False, 300, 512, 512),            # two issuing threads, neither
+    (3 * WM, False, 300, 512, 512),                  # no such orientation
+    (9 * WM + 2128, False, 300, 512, 512)])
+def test_unsupported_tile_codes_are_refused(code, residual, M, N, K):
+    """L2PD_ERR_SHAPE, nothing launched and nothing written."""
+    import torch
+    from paper_2509_25188_b200 import binding as b
+    A, W = torch.ones(M, K, dtype=torch.bfloat16, device="cuda"), torch.ones(N, K, dtype=torch.bfloat16, device="cuda")
+    X = torch.zeros(M, N, device="cuda")
+    with pytest.raises(b.L2pdError) as e:
+        b.gemm_bf16_residual(A, W, X, code) if residual else b.gemm_bf16(A, W, code)
+    assert e.value.status == -2
+    assert not X.any()
+
+
+@pytest.mark.parametrize("code,M", [(WM + 40000, 64), (WM + 20000, 300), (WM + 40000, 200), (WM + 100000 + 2000000, 300)])
+def test_tile_codes_that_leave_parts_open(code, M):
+    """Slices with the tile left open get single CTAs and a tile that their exchange has room for; one slab and no second issuer is
+    what this side has."""
+    from paper_2509_25188_b200 import binding as b
+    N, K = 512, 2048
+    A, W, X = _bf16(13, 0, (M, K), 1.0), _bf16(13, 1, (N, K), 0.05), wl.make_activations(13, 2, (M, N), 1.0, "fp32")
+    a = orc.widen(A)
+    got = b.gemm_bf16_residual(b.to_device(A), b.to_device(W), b.to_device(X.copy()), code).cpu().numpy()
+    bound = (K + 4) * 2.0 ** -24 * (np.abs(a) @ np.abs(orc.widen(W)).T + np.abs(X))
+    assert (np.abs(got - (X.astype(np.float64) + orc.linear(a, W))) <= bound).all()
