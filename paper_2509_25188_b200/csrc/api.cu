@@ -162,6 +162,10 @@ constexpr int LEAN_MAX_ROWS = 48;
 // (1.03 to 1.11 times the time) it is not asked.
 constexpr int WM_MIN_ROWS = 256;
 constexpr double WM_MARGIN = 1.12;
+// A stand-alone call has no neighbours to start and end beside: 2500 cycles more, and no K slices on its own accord (their exchange:
+// 1024 x 2816, 300 rows 6.8 -> 10.6 us, 2048 x 2048, 256 rows 9.8 -> 16.0).  Of 140 calls (N, K 512 to 12288, 257 to 4096 rows, all
+// epilogues) it takes the M side for 28, 2 of them slower (5 and 4 %), the others 1 to 18 % faster; without the 2500 32 are slower.
+constexpr double WM_ALONE = 2500.0;
 constexpr int CHAIN_TILE_N = 176;       // widest tile of a step that chains projections
 constexpr int CHAIN_MAX_ROWS = 1536;    // steps of more rows run one launch per projection (the launch is then a small part)
 constexpr int CHAIN_TRACE_STAMPS = 4;   // stamps per phase and CTA
@@ -328,12 +332,13 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     // its launch; 400 ahead of the warp-level attention (heads of 64), whose blocks come up under that kernel but not beside a
     // projection, which has all of an SM's shared memory.
     if (!c->fuse_rope) cost_qkv += (c->attn_tc ? 4000.0 : 400.0) + 12.0 * T_rows * hd / 3100.0;
-    // asked only where its answer can be taken: the search takes up to 12 us ahead of the step's first launch
+    // asked only where its answer can be taken, and for plans below what the other side costs: nothing hides the search, which is
+    // ahead of the step's first launch
     auto wm_plan = [&](l2pd_ctx::WmGemm &g, int epi, int N, int K, double other, int ks, bool can) {
       g.on = false;
       if (!can || (!lean && T_rows <= WM_MIN_ROWS)) return;
-      g.plan = plan_gemm_wm(epi, T_rows, N, K, c->num_sms, lean ? 4 : ks, lean);
-      g.on = lean || (g.plan.cost * WM_MARGIN < other && g.plan.cost + wm_exposed_drain(epi, g.plan, T_rows, N, K, c->num_sms) < other);
+      g.plan = plan_gemm_wm(epi, T_rows, N, K, c->num_sms, lean ? 4 : ks, lean, lean ? 1e300 : other / WM_MARGIN);
+      g.on = lean || (g.plan.cta_group && g.plan.cost + wm_exposed_drain(epi, g.plan, T_rows, N, K, c->num_sms) < other);
     };
     const bool single = c->chain_mode == 0;
     wm_plan(c->wm_qkv, EPI_QKV_ROPE, 3 * hd, d, cost_qkv, 1, single && c->wm_qkv_rope);
@@ -1352,8 +1357,8 @@ static l2pd_status gemm_common(void *stream, int epi, const void *A, const void 
   if (want_or == 1 && (want_sl == 2 || want_kil == 1)) return L2PD_ERR_SHAPE;   // that side has neither
   double cost = 0.0;
   GemmPlan pl = plan_gemm(epi, M, N, K, sms, want_tn, 4, &cost);
-  if (want_or == 1 || (want_or == 0 && !want_kil && tile_n == 0)) {
-    WmPlan wp = plan_gemm_wm(epi, M, N, K, sms, 4, true);
+  if (want_or == 1 || (want_or == 0 && !want_kil && tile_n == 0 && M > WM_MIN_ROWS)) {
+    WmPlan wp = plan_gemm_wm(epi, M, N, K, sms, 1, true, want_or == 1 ? 1e300 : cost / WM_MARGIN - WM_ALONE);
     if (want_or == 1) {
       wp.k_splits = want_ks ? effective_k_splits(K, want_ks) : 1;
       wp.w_rows = 128;
@@ -1365,7 +1370,7 @@ static l2pd_status gemm_common(void *stream, int epi, const void *A, const void 
     TmaDesc probe;
     int up_first = 0;
     const bool can = epi != EPI_SWIGLU || make_tma_gate_up(&probe, W, W2, N, K, wp.w_rows, &up_first) == L2PD_OK;
-    if (can && (want_or == 1 || wp.cost * WM_MARGIN < cost)) return gemm_common_wm(stream, epi, A, W, W2, out, M, N, K, wp, sms, check);
+    if (can && wp.cta_group) return gemm_common_wm(stream, epi, A, W, W2, out, M, N, K, wp, sms, check);
   }
   if (want_tn) pl.tile_n = want_tn;
   if (want_cg) pl.cta_group = want_cg;

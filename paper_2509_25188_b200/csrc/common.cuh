@@ -233,7 +233,8 @@ typedef CUresult (*TmaEncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, 
 TmaEncodeFn tma_encode_fn();
 // tile_t: rows of a tile (a multiple of 16, at most 256); w_rows: weight rows of a CTA; cost: modelled cycles
 struct WmPlan { int cta_group, tile_t, k_splits, w_rows; double cost; };
-WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits = 4, bool in_cluster = false);   // in_cluster: as WmArgs
+// in_cluster: as WmArgs.  limit: plans that cost no less are of no interest (without a cheaper one cta_group is 0)
+WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits = 4, bool in_cluster = false, double limit = 1e300);
 bool wm_slices_in_cluster(const WmPlan &pl, int T, int N, int num_sms);   // the plan's K slices can meet in clusters (WmArgs: in_cluster)
 // cycles that the plan's cost leaves out: what the rotating epilogue takes beyond the main loops that it could hide behind
 double wm_exposed_drain(int epi, const WmPlan &pl, int T, int N, int K, int num_sms);

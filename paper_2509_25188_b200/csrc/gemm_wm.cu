@@ -563,12 +563,13 @@ bool wm_slices_in_cluster(const WmPlan &pl, int T, int N, int num_sms) {
 // A step plans its four projections ahead of its first launch, which nothing hides: a row tile that several counts of tiles come
 // to is looked at once, and a tile whose k-blocks alone take longer than the best so far not at all (the plans are the same; 1024
 // rows: 95 -> 7 us, 306 rows 25 -> 7).
-WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits, bool in_cluster) {
-  WmPlan best{0, 0, 1, MMA_ROWS, 1e300};
+WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits, bool in_cluster, double limit) {
+  WmPlan best{0, 0, 1, MMA_ROWS, limit};
   const int rows = epi == EPI_SWIGLU ? 2 * N : N;
   const int max_ks = epi == EPI_RESIDUAL ? (max_k_splits < 4 ? max_k_splits : 4) : 1;
   const double traffic = T >= 4096 ? 0.45 : 0.15;
   const int k_blocks = ceil_div(K, BK);
+  if (8000.0 + 20.0 * 16 + 250.0 * k_blocks / max_ks >= limit) return best;   // no tile is below this
   for (int cg = 1; cg <= 2; ++cg) {
     if (cg == 2 && num_sms < 2) continue;
     const int groups = num_sms / cg;
@@ -582,8 +583,8 @@ WmPlan plan_gemm_wm(int epi, int T, int N, int K, int num_sms, int max_k_splits,
         const int t_tiles = ceil_div(T, tt);
         const double bytes = 128.0 * wr + 128.0 * tt / cg, pipe = 2.0 * tt * (cg == 1 ? 1.13 : 1.0);
         const double k_block = fmax(fmax(pipe, 250.0), bytes / 95.0) + traffic * bytes / 95.0, fixed = 8000.0 + 20.0 * tt;
-        // no split of K takes less than all k-blocks spread evenly over the CTAs
-        if (k_block * k_blocks * w_tiles * t_tiles / groups + fixed >= best.cost) continue;
+        // no split of K takes less than all k-blocks spread evenly over the CTAs, nor than one unit
+        if (k_block * k_blocks * fmax((double)w_tiles * t_tiles / groups, 1.0 / max_ks) + fixed >= best.cost) continue;
         for (int ks = 1; ks <= max_ks; ++ks) {
           if (ks > 1 && (k_blocks < 8 * ks || effective_k_splits(K, ks) != ks)) break;
           if (in_cluster && ks > 1 && !wm_slices_in_cluster(WmPlan{cg, tt, ks, wr, 0.0}, T, N, num_sms)) continue;

@@ -112,3 +112,59 @@ def test_tile_codes_that_leave_parts_open(code, M):
     got = b.gemm_bf16_residual(b.to_device(A), b.to_device(W), b.to_device(X.copy()), code).cpu().numpy()
     bound = (K + 4) * 2.0 ** -24 * (np.abs(a) @ np.abs(orc.widen(W)).T + np.abs(X))
     assert (np.abs(got - (X.astype(np.float64) + orc.linear(a, W))) <= bound).all()
+
+
+def _kernels(call):
+    """Names of the kernels that call() launches, from a capture of it (the driver's own account of the graph's nodes)."""
+    import ctypes as C
+    import torch
+
+    class Node(C.Structure):   # CUDA_KERNEL_NODE_PARAMS_v2
+        _fields_ = [("func", C.c_void_p), ("dims", C.c_uint * 7), ("params", C.c_void_p), ("extra", C.c_void_p), ("kern", C.c_void_p), ("ctx", C.c_void_p)]
+
+    cu = C.CDLL("libcuda.so.1")
+    call()                     # what a first call sets up is not capturable
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw, n, names = C.c_void_p(graph.raw_cuda_graph()), C.c_size_t(), []
+    assert cu.cuGraphGetNodes(raw, None, C.byref(n)) == 0
+    nodes = (C.c_void_p * n.value)()
+    assert cu.cuGraphGetNodes(raw, nodes, C.byref(n)) == 0
+    for node in nodes:
+        kind, p, name = C.c_int(), Node(), C.c_char_p()
+        assert cu.cuGraphNodeGetType(C.c_void_p(node), C.byref(kind)) == 0
+        if kind.value == 0:    # a kernel
+            assert cu.cuGraphKernelNodeGetParams_v2(C.c_void_p(node), C.byref(p)) == 0
+            f = cu.cuFuncGetName(C.byref(name), C.c_void_p(p.func)) if p.func else cu.cuKernelGetName(C.byref(name), C.c_void_p(p.kern))
+            assert f == 0
+            names.append(name.value.decode())
+    return names
+
+
+@pytest.mark.parametrize("epi,M,N,K,m_side", [
+    ("res", 160, 4096, 4096, False), ("res", 256, 2048, 2048, False), ("store", 64, 3072, 1024, False),   # few rows
+    ("res", 300, 1024, 2816, False),                                                                    # no slices unasked
+    ("store", 300, 1536, 512, False), ("swiglu", 257, 1376, 512, False),                                # few k-blocks
+    ("store", 1029, 12288, 4096, True), ("res", 1029, 2048, 5632, True), ("swiglu", 400, 12288, 4096, True)])
+def test_automatic_calls_take_the_faster_side(epi, M, N, K, m_side):
+    """us, rows on the M side and weights there: 160 x 4096 x 4096 11.8 and 14.3, 256 x 2048 x 2048 9.8 and 16.0, 64 x 3072 x 1024 5.9 and
+    6.6, 300 x 1024 x 2816 6.8 and 10.6, 300 x 1536 x 512 5.3 and 5.8, 257 x 1376 x 512 5.4 and 6.0; 1029 x 12288 x 4096 100 and 83, 1029 x 2048
+    x 5632 23.8 and 21.4, 400 x 12288 x 4096 (SwiGLU) 93 and 82."""
+    import torch
+    from paper_2509_25188_b200 import binding as b
+    A, W, U = (torch.zeros(r, K, dtype=torch.bfloat16, device="cuda") for r in (M, N, N))
+    X, C = torch.zeros(M, N, device="cuda"), torch.zeros(M, N, dtype=torch.bfloat16, device="cuda")
+
+    def call():
+        s = torch.cuda.current_stream().cuda_stream
+        if epi == "res":
+            r = b.lib.l2pd_gemm_bf16_residual(s, A.data_ptr(), W.data_ptr(), X.data_ptr(), M, N, K, 0, 0)
+        elif epi == "swiglu":
+            r = b.lib.l2pd_gemm_bf16_swiglu(s, A.data_ptr(), W.data_ptr(), U.data_ptr(), C.data_ptr(), M, N, K, 0, 0)
+        else:
+            r = b.lib.l2pd_gemm_bf16(s, A.data_ptr(), W.data_ptr(), C.data_ptr(), M, N, K, 0, 0)
+        assert r == 0
+    names = _kernels(call)
+    assert len(names) == 1 and ("gemm_wm" in names[0]) == m_side, names

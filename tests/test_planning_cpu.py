@@ -23,8 +23,8 @@ class RowPlan(ctypes.Structure):
 def _planners():
     from paper_2509_25188_b200 import build
     lib = ctypes.CDLL(build.build())
-    wm, row = lib._ZN4l2pd12plan_gemm_wmEiiiiiib, lib._ZN4l2pd9plan_gemmEiiiiiiiPd
-    wm.restype, wm.argtypes = Plan, [ctypes.c_int] * 6 + [ctypes.c_bool]
+    wm, row = lib._ZN4l2pd12plan_gemm_wmEiiiiiibd, lib._ZN4l2pd9plan_gemmEiiiiiiiPd
+    wm.restype, wm.argtypes = Plan, [ctypes.c_int] * 6 + [ctypes.c_bool, ctypes.c_double]
     row.restype, row.argtypes = RowPlan, [ctypes.c_int] * 7 + [ctypes.c_void_p]
     return wm, row
 
@@ -65,10 +65,13 @@ def test_the_search_finds_the_best_tiles(epi, N, K):
     wm, _ = _planners()
     for T in (1, 16, 17, 48, 257, 306, 1024, 1029, 4096, 16384):
         for in_cluster in (False, True):
-            p = wm(epi, T, N, K, SMS, 4, in_cluster)
+            p = wm(epi, T, N, K, SMS, 4, in_cluster, 1e300)
             cost, plan = _exhaustive(epi, T, N, K, 4, in_cluster)
             assert (p.cta_group, p.tile_t, p.k_splits, p.w_rows) == plan, (T, in_cluster)
             assert math.isclose(p.cost, cost, rel_tol=1e-12)
+            p = wm(epi, T, N, K, SMS, 4, in_cluster, 1.01 * cost)       # a limit above the best cost changes nothing
+            assert (p.cta_group, p.tile_t, p.k_splits, p.w_rows) == plan
+            assert wm(epi, T, N, K, SMS, 4, in_cluster, 0.99 * cost).cta_group == 0
 
 
 @pytest.mark.parametrize("T", [306, 1024, 16384])
@@ -84,6 +87,6 @@ def test_the_search_costs_little(T):
                 call(QKV), call(RESIDUAL)
             times.append(time.perf_counter() - t0)
         return min(times)
-    here = best(lambda epi: wm(epi, T, 4096, 4096, SMS, 4, False))
+    here = best(lambda epi: wm(epi, T, 4096, 4096, SMS, 4, False, 1e300))
     other = best(lambda epi: row(STORE if epi == QKV else epi, T, 4096, 4096, SMS, 0, 4, None))
     assert here < 4 * other
