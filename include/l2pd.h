@@ -410,7 +410,8 @@ l2pd_status l2pd_attention_bf16(void *stream, const void *q, const void *k, cons
  * comparisons only — the defaults are the product):
  *   L2PD_FORCE_SIMT=1       bf16 configurations run their GEMMs and attention on the CUDA-core cross-check kernels
  *   L2PD_ATTN_WARP=1        head size 128 keeps the warp-level (mma.sync) attention kernel instead of tcgen05
- *   L2PD_NO_ROPE_FUSION=1   rotary embedding as a separate kernel instead of the QKV epilogue
+ *   L2PD_NO_ROPE_FUSION=1   rotary embedding as a separate kernel instead of the QKV epilogue, whichever kernel that is (steps of
+ *                           at most 48 rows then have their RMSNorms as kernels too)
  *   L2PD_NO_PDL=1           kernels launched without programmatic dependent launch
  *   L2PD_ATOMIC_KSPLIT=1    K slices of the O / down projections add into x in completion order (not
  *                           bit-reproducible) instead of storing partial sums that are added in slice order

@@ -901,6 +901,7 @@ l2pd_status l2pd_init(const l2pd_config *cfg, const l2pd_weights *w, int device,
     const char *nf = getenv("L2PD_NO_ROPE_FUSION");
     c->fuse_rope = c->attn_tc && !c->force_simt && f.kv_cache_mode == 0 && (f.head_dim & (f.head_dim - 1)) == 0 &&
                    !(nf && nf[0] == '1');
+    if (nf && nf[0] == '1') c->wm_qkv_rope = false;
     if (c->fuse_rope) {
       bf16 *qkvb = (bf16 *)c->qkv;
       if (make_tma_2d_bf16_strided(&c->tq_packed, qkvb, mr, hd, 3 * hd, 128) ||

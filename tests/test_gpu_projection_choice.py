@@ -71,3 +71,21 @@ def test_narrow_models_rotate_in_the_projection_only_where_that_is_faster(head_d
     dec.denoise_step(outputs=False)
     assert _launches(dec, "rope") == (0 if m_side else shape.n_layers)
     dec.close()
+
+
+@pytest.mark.parametrize("P", [12, 268])   # 44 and 300 rows
+def test_switch_for_a_rotation_kernel_of_its_own(monkeypatch, P):
+    shape = _shape(128, 4, 512, 1376)
+    w = wl.make_weights(shape, seed=0, final_norm_gain=wl.spread_gain(shape))
+    prompts = wl.make_prompts(1, P, shape, seed=5)
+    logits = []
+    for switch, rotations in (("0", 0), ("1", shape.n_layers)):
+        monkeypatch.setenv("L2PD_NO_ROPE_FUSION", switch)
+        dec = _decoder(shape, w, 32, 1, P + 32)
+        dec.state_reset(prompts, 32)
+        dec.profile_enable(["rope"])
+        logits.append(dec.denoise_step(want_logits=True)["logits"][0])
+        assert _launches(dec, "rope") == rotations
+        dec.close()
+    # q and k are rounded to bf16 once more
+    assert np.abs(logits[1] - logits[0]).max() <= 2e-2 * np.abs(logits[0]).max()
