@@ -414,7 +414,8 @@ l2pd_status l2pd_attention_bf16(void *stream, const void *q, const void *k, cons
  *                           at most 48 rows then have their RMSNorms as kernels too)
  *   L2PD_NO_PDL=1           kernels launched without programmatic dependent launch
  *   L2PD_ATOMIC_KSPLIT=1    K slices of the O / down projections add into x in completion order (not
- *                           bit-reproducible) instead of storing partial sums that are added in slice order
+ *                           bit-reproducible) instead of storing partial sums, or meeting in a cluster, that are added in
+ *                           slice order (steps of at most 48 rows then have their RMSNorms as kernels)
  *   L2PD_DIRECT_STORES=1    stand-alone GEMM calls use per-thread stores in the epilogue instead of staged TMA stores
  */
 

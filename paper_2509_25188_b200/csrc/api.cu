@@ -327,7 +327,8 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     c->pl_o = plan_gemm(EPI_RESIDUAL, T_rows, d, hd, c->num_sms, 0, max_ks, &cost_o);
     c->pl_down = plan_gemm(EPI_RESIDUAL, T_rows, d, F, c->num_sms, 0, max_ks, &cost_down);
     c->pl_gu = plan_gemm(EPI_SWIGLU, T_rows, F, d, c->num_sms, 0, 1, &cost_gu);
-    lean = c->chain_mode == 0 && c->wm_gate_up && c->wm_qkv_rope && T_rows <= LEAN_MAX_ROWS;
+    // (its K slices meet in clusters, in order: not with slices that add in completion order, which have no partial-sum area)
+    lean = c->chain_mode == 0 && c->wm_gate_up && c->wm_qkv_rope && c->ksum && T_rows <= LEAN_MAX_ROWS;
     // The rotation and the scatter are a kernel of their own where the projection does not do them: its bytes, and 4000 cycles for
     // its launch; 400 ahead of the warp-level attention (heads of 64), whose blocks come up under that kernel but not beside a
     // projection, which has all of an SM's shared memory.
@@ -344,8 +345,8 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
     wm_plan(c->wm_qkv, EPI_QKV_ROPE, 3 * hd, d, cost_qkv, 1, single && c->wm_qkv_rope);
     wm_plan(c->wm_gu, EPI_SWIGLU, F, d, cost_gu, 1, single && c->wm_gate_up);
     // (the chained modes take these two's K slices)
-    wm_plan(c->wm_o, EPI_RESIDUAL, d, hd, cost_o, c->ksum ? max_ks : 1, true);
-    wm_plan(c->wm_down, EPI_RESIDUAL, d, F, cost_down, c->ksum ? max_ks : 1, true);
+    wm_plan(c->wm_o, EPI_RESIDUAL, d, hd, cost_o, max_ks, true);
+    wm_plan(c->wm_down, EPI_RESIDUAL, d, F, cost_down, max_ks, true);
     // slices that a later kernel adds (in a lean step there are none)
     if (c->wm_o.on) c->pl_o.k_splits = lean ? 1 : c->wm_o.plan.k_splits;
     if (c->wm_down.on) c->pl_down.k_splits = lean ? 1 : c->wm_down.plan.k_splits;

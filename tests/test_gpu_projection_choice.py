@@ -5,7 +5,9 @@ from __future__ import annotations
 import numpy as np
 import pytest
 
+from oracle import l2pd_oracle as orc
 from paper_2509_25188_b200 import workloads as wl
+from tests.helpers import lockstep, oracle_model
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +91,22 @@ def test_switch_for_a_rotation_kernel_of_its_own(monkeypatch, P):
         dec.close()
     # q and k are rounded to bf16 once more
     assert np.abs(logits[1] - logits[0]).max() <= 2e-2 * np.abs(logits[0]).max()
+
+
+@pytest.mark.parametrize("P,norms", [(12, 0), (268, 5)])   # 44 and 300 rows; RMSNorm kernels of a step of three layers
+def test_switch_for_k_slices_in_completion_order(monkeypatch, P, norms):
+    """Under the switch the slices add into x: no slices in a cluster (hence RMSNorm kernels), no partial sums to add (after the last
+    layer a kernel of its own adds them)."""
+    shape = _shape(128, 4, 512, 1376)
+    w = wl.make_weights(shape, seed=0, final_norm_gain=wl.spread_gain(shape))
+    m = oracle_model(shape, w)
+    prompts = wl.make_prompts(1, P, shape, seed=5)
+    for switch in ("0", "1"):
+        monkeypatch.setenv("L2PD_ATOMIC_KSPLIT", switch)
+        dec = _decoder(shape, w, 32, 1, P + 32)
+        dec.profile_enable(["rmsnorm", "other"])
+        lockstep(dec, m, None, orc.DecodeConfig(block_len=32, use_filter=False, use_eotp=False), prompts, 32, logit_rtol=2e-2,
+                 conf_atol=1e-3, p_margin=0.02, max_steps=1)
+        assert _launches(dec, "rmsnorm") == (5 if switch == "1" else norms)
+        assert _launches(dec, "other") == (1 if switch == "0" and norms else 0)
+        dec.close()
