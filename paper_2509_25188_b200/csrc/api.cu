@@ -106,7 +106,7 @@ struct l2pd_ctx {
   std::vector<TmaDesc> tw_qk, tw_v;        // the caller's QKV matrices: q and k rows, rotary halves interleaved; v rows
   bool wm_gate_up = false;                 // every layer's gate and up matrices can be mapped as one
   bool wm_qkv_rope = false;                // every layer's QKV matrix can be mapped with its halves interleaved
-  float *ss = nullptr;                     // sums of squares of the rows of x by feature tile, [tiles][max_rows]
+  float *ss = nullptr;                     // sums of squares of the rows of x by feature tile, [tiles][LEAN_MAX_ROWS]
   int32_t *d_row_kv = nullptr;             // row -> row of the key/value store
 
   // several projections per launch (gemm_chain.cu): on when every projection of the step runs on SM pairs with
@@ -540,7 +540,7 @@ l2pd_status forward_and_decide(l2pd_ctx *c, cudaStream_t s, int n_slots, int T_r
   auto wm_args = [&](int epi, int N, int K, const l2pd_ctx::WmGemm &g, int l) {
     WmArgs a{};
     a.epi = epi; a.T = T_rows; a.N = N; a.K = K; a.plan = g.plan; a.w = epi == EPI_QKV_ROPE ? &c->tw_qk[l] : &g.w[l]; a.x = &g.x;
-    a.status = c->d_status; a.ss_stride = (int)c->max_rows; a.eps = f.rms_eps; a.width = d;
+    a.status = c->d_status; a.ss_stride = LEAN_MAX_ROWS; a.eps = f.rms_eps; a.width = d;
     return a;
   };
   auto wm_qkv = [&](int l, void *kc, void *vc) {
@@ -821,7 +821,7 @@ l2pd_status l2pd_init(const l2pd_config *cfg, const l2pd_weights *w, int device,
     c->ksum_rows = round_up(mr < 4096 ? mr : 4096, 512);   // a slice's area covers whole 512-row units
     A(dev_alloc(c, &c->ksum, 4 * c->ksum_rows * d));
   }
-  if (f.dtype == L2PD_BF16 && !c->force_simt) A(dev_alloc(c, &c->ss, (int64_t)ceil_div(d, 32) * mr));
+  if (f.dtype == L2PD_BF16 && !c->force_simt) A(dev_alloc(c, &c->ss, (int64_t)ceil_div(d, 64) * LEAN_MAX_ROWS));   // (no plan has narrower feature tiles)
   if (f.dtype == L2PD_BF16 && c->ksum && !c->force_simt) {
     c->chain_clusters = chain_max_clusters(c->num_sms);
     if (c->chain_clusters > 0) {

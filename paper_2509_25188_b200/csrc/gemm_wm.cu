@@ -35,15 +35,12 @@
 // take alternate chunks of 16 rows).  The loops of the issuing warps follow gemm_tcgen05.cu.
 #include <math.h>
 
-#include <type_traits>
-
 #include "common.cuh"
 #include "gemm_device.cuh"
 #include "ptx.cuh"
 
 namespace l2pd {
 
-using gemm_dev::fail;
 using gemm_dev::silu_mul;
 
 namespace {

@@ -1,5 +1,6 @@
-"""Which kernel a step's projections take, and what may not depend on it.  The form that ran is told from the launches of the kinds
-it does without (profile_read)."""
+"""Which kernel a step's projections take, and what may not depend on it: the launch modes' agreement, the environment switches,
+lockstep decodes with the oracle at the row counts and head sizes that reach each form.  The form that ran is told from the launches
+of the kinds it does without (profile_read)."""
 from __future__ import annotations
 
 import numpy as np
@@ -109,4 +110,46 @@ def test_switch_for_k_slices_in_completion_order(monkeypatch, P, norms):
                  conf_atol=1e-3, p_margin=0.02, max_steps=1)
         assert _launches(dec, "rmsnorm") == (5 if switch == "1" else norms)
         assert _launches(dec, "other") == (1 if switch == "0" and norms else 0)
+        dec.close()
+
+
+@pytest.mark.parametrize("head_dim,heads,d,d_ff,kv,s,B,P,G,m_side", [
+    (64, 8, 512, 1376, 0, 32, 2, 110, 64, True),     # 348 rows, no cache; the down projection has two slices
+    (64, 3, 1024, 2816, 0, 32, 1, 268, 32, True),    # 300 rows, q, k and v of 192 features: v ends inside a tile
+    (64, 3, 256, 704, 0, 16, 1, 21, 16, True),       # the same in 37 rows
+    (64, 8, 512, 1376, 2, 16, 1, 270, 32, True),     # 302 rows, then 16 against the store
+    (64, 3, 256, 12288, 2, 8, 1, 272, 16, False),    # 288 rows, then 8; gate / up in tiles of 96 features, four slices of a cluster
+    (64, 8, 512, 1376, 1, 16, 2, 250, 16, False),    # 532 rows, then 32 from the block's start
+    (128, 2, 256, 12288, 2, 16, 1, 284, 32, True),   # 316 rows, then 16, heads of 128
+    (128, 4, 512, 1376, 2, 5, 1, 300, 10, True)])    # 310 rows, then 5
+def test_lockstep_where_the_weights_are_on_the_m_side(head_dim, heads, d, d_ff, kv, s, B, P, G, m_side):
+    """Logits and decisions against the oracle's; bf16 roundings of two layers (2e-2 of a row's largest logit, as everywhere).
+    m_side: the rotation is inside the projection in a block's first step too."""
+    shape = _shape(head_dim, heads, d, d_ff, layers=2)
+    w = wl.make_weights(shape, seed=1, final_norm_gain=wl.spread_gain(shape))
+    dec = _decoder(shape, w, s, B, P + G, kv)
+    dec.profile_enable(["rope", "rmsnorm"])
+    st = lockstep(dec, oracle_model(shape, w), None,
+                  orc.DecodeConfig(block_len=s, kv_cache=kv > 0, dual_cache=kv == 2, use_filter=False, use_eotp=False),
+                  wl.make_prompts(B, P, shape, seed=2), G, logit_rtol=2e-2, conf_atol=1e-3, p_margin=0.02, max_steps=s + 2)
+    rows = B * (P + G)
+    # steps of at most 48 rows have neither rotation nor RMSNorm kernels
+    first = sum(1 for i in range(st["steps"]) if kv == 0 or i in (0, s))
+    assert _launches(dec, "rope") == (0 if m_side else 2 * first)
+    assert _launches(dec, "rmsnorm") == (3 * first if rows > 48 else 0)
+    assert st["replay_checked"] > 0 and st["pred_checked"] > 0
+    dec.close()
+
+
+def test_partial_sums_and_sums_in_a_cluster_are_the_ones_that_ran():
+    """306 rows at d = 512: the down projection's slices leave partial sums, which a kernel adds after the last layer; 33 rows: sums
+    meet in clusters and no kernel adds or normalises.  (A plan without slices would take the test from the lockstep above.)"""
+    shape = _shape(64, 8, 512, 1376, layers=2)
+    w = wl.make_weights(shape, seed=1, final_norm_gain=wl.spread_gain(shape))
+    for P, added, norms in ((274, 1, 3), (1, 0, 0)):
+        dec = _decoder(shape, w, 32, 1, P + 32)
+        dec.state_reset(wl.make_prompts(1, P, shape, seed=2), 32)
+        dec.profile_enable(["other", "rmsnorm"])
+        dec.denoise_step(outputs=False)
+        assert (_launches(dec, "other"), _launches(dec, "rmsnorm")) == (added, norms)
         dec.close()
