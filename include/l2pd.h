@@ -292,8 +292,8 @@ l2pd_status l2pd_profile_read(const l2pd_ctx *ctx, int32_t kind, double *ms_tota
  * modes 1 and 2 give bit-identical results).  With more than 256 rows modes 1 and 2 use two row slabs per unit, tiles of at
  * most 176 columns and mode 0's K slices: all three modes agree bit for bit.  With at most 256 rows they use one 256-row slab
  * per unit with the two MMA-issuing warps on alternate k-blocks (key/value-cache configurations only).  May be called between
- * steps.  Single launches are the faster form (8B step, mode 0 / 1, at 1.9 GHz: 32 rows 3.4 / 5.6 ms, 256 rows 4.4 / 6.1,
- * 512 rows 6.3 / 8.7, 1029 rows 13.2 / 18.5; under the power cap 512 rows 7.5 / 9.7): programmatic dependent launch hides
+ * steps.  Single launches are the faster form (8B step, mode 0 / 1, at 1.9 GHz: 32 rows 3.3 / 5.6 ms, 256 rows 4.6 / 6.2,
+ * 512 rows 6.3 / 8.7, 1029 rows 11.8 / 17.8; under the power cap 512 rows 7.5 / 9.7): programmatic dependent launch hides
  * the launch and the ring fill of a projection behind the one before it.
  * l2pd_chain_trace_enable(ctx, 1) makes every chained launch of the following steps record, per phase and CTA,
  * the nanosecond timer at which the CTA opened the phase, had its first and its last accumulator ready (for an
@@ -416,7 +416,9 @@ l2pd_status l2pd_attention_bf16(void *stream, const void *q, const void *k, cons
  *   L2PD_ATOMIC_KSPLIT=1    K slices of the O / down projections add into x in completion order (not
  *                           bit-reproducible) instead of storing partial sums, or meeting in a cluster, that are added in
  *                           slice order (steps of at most 48 rows then have their RMSNorms as kernels)
- *   L2PD_DIRECT_STORES=1    stand-alone GEMM calls use per-thread stores in the epilogue instead of staged TMA stores
+ *   L2PD_DIRECT_STORES=1    stand-alone GEMM calls use per-thread stores in the epilogue instead of staged TMA stores (with the
+ *                           rows of A on the M side, which orientation 2 of the tile code makes sure of; the other side has
+ *                           no staged stores)
  */
 
 #ifdef __cplusplus

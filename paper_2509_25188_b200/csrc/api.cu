@@ -151,20 +151,21 @@ bool pdl_enabled() {
 
 namespace {
 
-// Steps of few rows have their weights on the M side and no RMSNorm kernels (gemm_wm.cu): a step of 32 rows of the 8B shape 3.4 ->
-// 3.2 ms, its decode of 64 steps 261 -> 245 ms; of 64 rows even, of 125 rows 5 % slower (the epilogues pass 16 rows at a time, and
+// Steps of few rows have their weights on the M side and no RMSNorm kernels (gemm_wm.cu): a step of 32 rows of the 8B shape 3.41 ->
+// 3.32 ms, its decode of 64 steps 267 -> 247 ms; of 64 rows even, of 125 rows 5 % slower (the epilogues pass 16 rows at a time, and
 // nothing overlaps them when a CTA has one unit).
 constexpr int LEAN_MAX_ROWS = 48;
 // Otherwise a projection takes that side where its model says so.  The model leaves out what its epilogues take of shared memory's
 // bandwidth from the MMAs: measured over 288 to 8192 rows, its cycles times 1.06 to 1.15 (mostly 1.1 to 1.12) compare with the other
 // orientation's.  With all projections forced to it, eight 8B layers: 288 rows 0.90 of the time, 320 0.95, 384 1.01, 512 1.04, 640
-// 0.93, 768 1.08, 1024 1.12, 1029 0.91, 4096 1.03; the 1029-row step of 32 layers with this rule 15.55 -> 13.81 ms.  Up to 256 rows
+// 0.93, 768 1.08, 1024 1.12, 1029 0.91, 4096 1.03; the 1029-row step of 32 layers with this rule 13.2 -> 11.8 ms (at 1.9 GHz;
+// under the power cap 15.8 -> 13.8).  Up to 256 rows
 // (1.03 to 1.11 times the time) it is not asked.
 constexpr int WM_MIN_ROWS = 256;
 constexpr double WM_MARGIN = 1.12;
 // A stand-alone call has no neighbours to start and end beside: 2500 cycles more, and no K slices on its own accord (their exchange:
-// 1024 x 2816, 300 rows 6.8 -> 10.6 us, 2048 x 2048, 256 rows 9.8 -> 16.0).  Of 140 calls (N, K 512 to 12288, 257 to 4096 rows, all
-// epilogues) it takes the M side for 28, 2 of them slower (5 and 4 %), the others 1 to 18 % faster; without the 2500 32 are slower.
+// 1024 x 2816, 300 rows 6.8 -> 10.6 us, 2048 x 2048, 256 rows 9.8 -> 16.0).  Of 220 calls (N, K 512 to 12288, 257 to 4096 rows, all
+// epilogues) it takes the M side for 30, 2 of them slower (5 and 4 %), the others up to 18 % faster; without the 2500 32 are slower.
 constexpr double WM_ALONE = 2500.0;
 constexpr int CHAIN_TILE_N = 176;       // widest tile of a step that chains projections
 constexpr int CHAIN_MAX_ROWS = 1536;    // steps of more rows run one launch per projection (the launch is then a small part)

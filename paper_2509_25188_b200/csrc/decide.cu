@@ -11,12 +11,13 @@
 //   * EoTP (Section 3.3): the earliest committed [EoT] cuts the sequence; later positions leave
 //     the mask set and read as [EoT];
 //   * block advance / stop (Algorithm 3: no block after one that holds [EoT]).
-// One thread block per sequence taking part in the step.  What took longest was the merge (988 records of 32 rows in a step of the
-// 8B shape, 380 KB): a warp to a row read a 32-byte sector for each 4-byte value it wanted, eight times the bytes through one SM;
-// with lanes along the rows the kernel takes 16.0 us where it took 36.6.  Besides, it is bound by its chain of latencies: the two-layer filter's weights come to shared memory before the wait for the LM head, the tile records and the
-// sequence's description leave together, its state follows at once.  The summary and the device status go straight to
-// pinned host memory, so that nothing is left to copy behind the step's last kernel.  With the descriptions of a step's
-// sequences as an argument of its first kernel, a step of 306 rows at d = 512: 212 -> 202 us.
+// One thread block per sequence taking part in the step.  What took longest was the merge (988 records of 32 rows in a step of
+// the 8B shape, 380 KB): a warp to a row read a 32-byte sector for each 4-byte value it wanted, eight times the bytes through one
+// SM; with lanes along the rows the kernel takes 16.0 us where it took 36.6.  Besides, it is bound by its chain of latencies: the
+// two-layer filter's weights come to shared memory before the wait for the LM head, the tile records and the sequence's
+// description leave together, its state follows at once.  The summary and the device status go straight to pinned host memory,
+// so that nothing is left to copy behind the step's last kernel.  With the descriptions of a step's sequences as an argument of
+// its first kernel, a step of 306 rows at d = 512: 212 -> 202 us.
 #include "common.cuh"
 
 namespace l2pd {

@@ -25,8 +25,8 @@
 // What bounds it: many rows, the tensor pipe and, beside it, shared memory, which the epilogue's staging takes some 6 % of; few
 // rows, the weights' way from HBM and what lies between two projections (32 rows: 1.3 us from a kernel's end to the next one's
 // release, 1.2 to its first MMA, the weights at 6.7 TB/s for gate/up, then 1.5 to 2 us of epilogue).  Stand-alone, rows on the M
-// side -> here (us): 1029 rows QKV 85.8 -> 70.5, gate/up 157 -> 141, down 87 -> 80; 343 rows down 38 -> 30; 512 rows, which are
-// whole slabs, QKV 37.4 -> 38.6, gate/up 69.6 -> 73.7.  Why 128-row weight tiles (96 or 64 where the plan finds them to share the
+// side -> here (us, back to back): 1029 rows QKV 91.4 -> 74.4, gate/up 167 -> 149, down 92.1 -> 83.7; 512 rows, which are whole
+// slabs, QKV 48.1 -> 50.2, gate/up 89.6 -> 94.0.  Why 128-row weight tiles (96 or 64 where the plan finds them to share the
 // last round better, gate/up of 32 rows: 3 % of a step): the MMA's M.  The cluster exchange replaced partial sums in global memory
 // that the CTA arriving last added (5 us behind the last accumulator at 32 rows, 10 at 125).
 //
